@@ -192,7 +192,7 @@ def pair_work(shape, W, H):
     c1, c2, c3 = shape.enc
     d1, d2, d3 = shape.dec
     lat = shape.latent
-    dense = {  # the plain form's direct convolutions (9 taps everywhere)
+    dense = {  # nine taps an output pixel everywhere
         "enc1": 2 * H1 * W1 * c1 * 9 * 2,
         "enc2": 2 * H2 * W2 * c2 * 9 * c1,
         "enc3": 2 * H3 * W3 * c3 * 9 * c2,
@@ -211,6 +211,8 @@ def pair_work(shape, W, H):
     out["tc_dec1"] = (2 * H2 * W2 * d1 * 4 * lat, "tensor")
     out["tc_dec2"] = (2 * H1 * W1 * d2 * 4 * d1, "tensor")
     out["tc_dec3"] = (2 * H0 * W0 * d3 * 4 * d2, "tensor")
+    for l in ("dec1", "dec2", "dec3"):  # the FP32 form folds its decoder taps too
+        out[l] = (out["tc_" + l][0], "alu")
     out["tc_dec3_final"] = (out["tc_dec3"][0] + dense["final"], "tensor")
     out["edge_up2fix"] = (2 * 6 * (upfix_pixels(H2, W2) * d1 * lat + upfix_pixels(H1, W1) * d2 * d1), "alu")
     out["edge_final"] = (2 * H0 * W0 * d3 + 2 * w * h + 4 * H0 * W0, "hbm")

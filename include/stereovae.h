@@ -58,7 +58,7 @@ typedef enum {
 } sv_status;
 
 /* Arithmetic of the refinement convolutions.
- * SV_FP32: FP32 CUDA-core direct convolutions (the plain method).
+ * SV_FP32: FP32 convolutions on the CUDA cores (the plain method).
  * SV_BF16: implicit-GEMM convolutions on the tcgen05 tensor cores, BF16 operands,
  *          FP32 accumulation; the last conv and the residual stay FP32.
  * SV_FP64_CHECK: FP64 CUDA-core convolutions, for gradient checks on small crops.
@@ -252,8 +252,8 @@ SV_API sv_status sv_pipeline(sv_ctx* ctx, const sv_pair* pairs, int n_pairs, flo
 
 /* Training forward of n_pairs pairs: z = mu + eps * exp(logvar / 2) (the
  * reparameterisation of Eq. 8 in its standard form).  Saves in the context what
- * sv_refine_backward needs (decoder activations and the latent; the encoder is
- * recomputed there).  On SV_BF16 contexts the encoder and decoder convolutions run on
+ * sv_refine_backward needs (activations and the latent; SV_BF16 and SV_FP64_CHECK contexts
+ * recompute the encoder there).  On SV_BF16 contexts the encoder and decoder convolutions run on
  * the tensor cores (BF16 operands, FP32 accumulation, FP32 master weights) and the
  * backward runs in FP32; SV_FP32 runs FP32 throughout, SV_FP64_CHECK FP64.  Element type of coarse, eps, disp_out, mu_out and logvar_out
  * is float for SV_FP32 / SV_BF16 contexts and double for SV_FP64_CHECK contexts.

@@ -1,5 +1,5 @@
-// backward.cu -- gradient kernels of the refinement network (FP32 and FP64), the
-// transpose of the bilinear x4 upsampling, the loss and Adam.
+// backward.cu -- gradient kernels of the FP64 check form (the FP32 gradients are in wgrad_f32.cu
+// and conv_f32.cu), the transpose of the bilinear x4 upsampling, the loss and Adam.
 //
 //   dgrad_kernel    input gradient of a 3x3 / 1x1 conv read through a view (stride 1,
 //                   stride 2, nearest x2 + crop): a gather over the taps and output pixels
@@ -17,7 +17,6 @@ namespace sv {
 
 namespace {
 
-__device__ __forceinline__ float atomic_add(float* a, float v) { return atomicAdd(a, v); }
 __device__ __forceinline__ double atomic_add(double* a, double v) { return atomicAdd(a, v); }
 
 // Input view V(vy, vx, ci) of the forward conv (zero outside), mode as in conv_direct.
@@ -155,12 +154,6 @@ __global__ void up4_bwd(const T* __restrict__ gU, const T* __restrict__ gx0, int
   gc[idx] = acc;
 }
 
-template <typename T>
-__global__ void add_inplace(T* a, const T* b, size_t n) {
-  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) a[i] += b[i];
-}
-
 // x0 = (L / 256, U / 256) materialised for the enc1 weight gradient.
 template <typename T>
 __global__ void build_x0(const uint8_t* L, int pitch, int W, int H, const T* coarse, int w, int h, T* x0) {
@@ -181,17 +174,31 @@ __global__ void build_x0(const uint8_t* L, int pitch, int W, int H, const T* coa
 // the slots in a fixed order, so the loss is bitwise reproducible.  Slot layout: for pair
 // i, kLossBlocks smooth-L1 partials then kLossBlocks KL partials.
 constexpr int kLossBlocks = 128;
+static_assert(2 * kLossBlocks == 256, "loss_finish takes one slot a thread");
 
+// blockIdx.y: pair; blockIdx.z: 0 the smooth-L1 term, 1 the KL term.
 template <typename T>
-__global__ void loss_rec(const T* __restrict__ Y, const float* __restrict__ gt, size_t P, double inv_npix,
-                         T* __restrict__ gY, double* __restrict__ slots) {
+__global__ void loss_partial(const LossJob<T>* __restrict__ jobs, double inv_npix, double kl_scale,
+                             double* __restrict__ all_slots) {
   __shared__ double red[256];
+  const LossJob<T>& J = jobs[blockIdx.y];
+  double* slots = all_slots + (size_t)blockIdx.y * 2 * kLossBlocks + blockIdx.z * kLossBlocks;
   double s = 0;
-  for (size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x; p < P; p += (size_t)gridDim.x * blockDim.x) {
-    const T e = Y[p] - (T)gt[p];
-    const T a = e < (T)0 ? -e : e;
-    s += a < (T)1 ? (double)((T)0.5 * e * e) : (double)(a - (T)0.5);
-    if (gY) gY[p] = (a < (T)1 ? e : (e > (T)0 ? (T)1 : (T)-1)) * (T)inv_npix;
+  if (blockIdx.z == 0) {
+    for (size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x; p < J.P; p += (size_t)gridDim.x * blockDim.x) {
+      const T e = J.Y[p] - (T)J.gt[p];
+      const T a = e < (T)0 ? -e : e;
+      s += a < (T)1 ? (double)((T)0.5 * e * e) : (double)(a - (T)0.5);
+      if (J.gY) J.gY[p] = (a < (T)1 ? e : (e > (T)0 ? (T)1 : (T)-1)) * (T)inv_npix;
+    }
+  } else {
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < J.n; i += (size_t)gridDim.x * blockDim.x) {
+      const T m = J.mu[i], l = J.lv[i];
+      const T el = exp(l);
+      s += (double)((T)0.5 * (m * m + el - (T)1 - l));
+      if (J.gmu) J.gmu[i] = (T)kl_scale * m;
+      if (J.glv) J.glv[i] = (T)kl_scale * (T)0.5 * (el - (T)1);
+    }
   }
   red[threadIdx.x] = s;
   __syncthreads();
@@ -202,40 +209,30 @@ __global__ void loss_rec(const T* __restrict__ Y, const float* __restrict__ gt, 
   if (threadIdx.x == 0) slots[blockIdx.x] = red[0];
 }
 
-template <typename T>
-__global__ void loss_kl(const T* __restrict__ mu, const T* __restrict__ lv, size_t n, double kl_scale,
-                        T* __restrict__ gmu, T* __restrict__ glv, double* __restrict__ slots) {
-  __shared__ double red[256];
-  double s = 0;
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const T m = mu[i], l = lv[i];
-    const T el = exp(l);
-    s += (double)((T)0.5 * (m * m + el - (T)1 - l));
-    if (gmu) gmu[i] = (T)kl_scale * m;
-    if (glv) glv[i] = (T)kl_scale * (T)0.5 * (el - (T)1);
-  }
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-    if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) slots[kLossBlocks + blockIdx.x] = red[0];
-}
-
+// One block of 256 threads: every thread adds its strided share of the slots, then a fixed tree
+// (one thread adding 2 x 128 slots a pair took 195 us for 16 pairs).
 template <typename T>
 __global__ void loss_finish(const double* slots, int n_pairs, double inv_npix, double inv_nlat, double kl_w, T* out) {
-  double rec = 0, kl = 0;
-  for (int i = 0; i < n_pairs; ++i)
-    for (int b = 0; b < kLossBlocks; ++b) {
-      rec += slots[(size_t)i * 2 * kLossBlocks + b];
-      kl += slots[(size_t)i * 2 * kLossBlocks + kLossBlocks + b];
+  __shared__ double red[2][256];
+  double v[2] = {0, 0};
+  const int t = threadIdx.x, term = t / kLossBlocks;  // 256 = 2 x kLossBlocks
+  for (int i = 0; i < n_pairs; ++i) v[term] += slots[(size_t)i * 2 * kLossBlocks + t];
+  red[0][t] = v[0];
+  red[1][t] = v[1];
+  __syncthreads();
+  for (int o = 128; o > 0; o >>= 1) {
+    if (t < o) {
+      red[0][t] += red[0][t + o];
+      red[1][t] += red[1][t + o];
     }
-  rec *= inv_npix;
-  kl *= inv_nlat;
-  out[0] = (T)(rec + kl_w * kl);
-  out[1] = (T)rec;
-  out[2] = (T)kl;
+    __syncthreads();
+  }
+  if (t == 0) {
+    const double rec = red[0][0] * inv_npix, kl = red[1][0] * inv_nlat;
+    out[0] = (T)(rec + kl_w * kl);
+    out[1] = (T)rec;
+    out[2] = (T)kl;
+  }
 }
 
 template <typename T>
@@ -294,32 +291,19 @@ cudaError_t launch_build_x0(const uint8_t* L, int pitch, int W, int H, const T* 
   return cudaGetLastError();
 }
 
-template <typename T>
-cudaError_t launch_add(T* a, const T* b, size_t n, cudaStream_t st) {
-  add_inplace<T><<<blocks(n), 256, 0, st>>>(a, b, n);
-  return cudaGetLastError();
-}
-
 size_t loss_slots_per_pair() { return 2 * kLossBlocks; }
 
 template <typename T>
-cudaError_t launch_loss_rec(const T* Y, const float* gt, size_t P, double inv_npix, T* gY, double* slots,
-                            cudaStream_t st) {
-  loss_rec<T><<<kLossBlocks, 256, 0, st>>>(Y, gt, P, inv_npix, gY, slots);
-  return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t launch_loss_kl(const T* mu, const T* lv, size_t n, double kl_scale, T* gmu, T* glv, double* slots,
-                           cudaStream_t st) {
-  loss_kl<T><<<kLossBlocks, 256, 0, st>>>(mu, lv, n, kl_scale, gmu, glv, slots);
+cudaError_t launch_loss_partial(const LossJob<T>* jobs, int n, double inv_npix, double kl_scale, double* slots,
+                                cudaStream_t st) {
+  loss_partial<T><<<dim3(kLossBlocks, n, 2), 256, 0, st>>>(jobs, inv_npix, kl_scale, slots);
   return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t launch_loss_finish(const double* slots, int n_pairs, double inv_npix, double inv_nlat, double kl_w, T* out,
                                cudaStream_t st) {
-  loss_finish<T><<<1, 1, 0, st>>>(slots, n_pairs, inv_npix, inv_nlat, kl_w, out);
+  loss_finish<T><<<1, 256, 0, st>>>(slots, n_pairs, inv_npix, inv_nlat, kl_w, out);
   return cudaGetLastError();
 }
 
@@ -331,20 +315,21 @@ cudaError_t launch_adam(float* p, T* m, T* v, const T* g, size_t n, double lr, d
   return cudaGetLastError();
 }
 
-#define SV_BWD_INST(T)                                                                                              \
-  template cudaError_t launch_dgrad<T>(const T*, int, int, int, const T*, int, int, const T*, int, int, int, int, T*, \
-                                       cudaStream_t);                                                                \
-  template cudaError_t launch_wgrad<T>(const T*, int, int, int, const T*, int, int, int, int, int, T*, T*,           \
-                                       cudaStream_t);                                                                \
-  template cudaError_t launch_latent_bwd<T>(const T*, const T*, const T*, const T*, const T*, size_t, T*, T*,       \
-                                            cudaStream_t);                                                           \
-  template cudaError_t launch_up4_bwd<T>(const T*, const T*, int, int, int, int, T*, cudaStream_t);                 \
-  template cudaError_t launch_build_x0<T>(const uint8_t*, int, int, int, const T*, int, int, T*, cudaStream_t);     \
-  template cudaError_t launch_add<T>(T*, const T*, size_t, cudaStream_t);                                           \
-  template cudaError_t launch_loss_rec<T>(const T*, const float*, size_t, double, T*, double*, cudaStream_t);        \
-  template cudaError_t launch_loss_kl<T>(const T*, const T*, size_t, double, T*, T*, double*, cudaStream_t);        \
-  template cudaError_t launch_loss_finish<T>(const double*, int, double, double, double, T*, cudaStream_t);         \
-  template cudaError_t launch_adam<T>(float*, T*, T*, const T*, size_t, double, double, double, double, int,        \
+// the check form's gathers
+template cudaError_t launch_dgrad<double>(const double*, int, int, int, const double*, int, int, const double*, int,
+                                          int, int, int, double*, cudaStream_t);
+template cudaError_t launch_wgrad<double>(const double*, int, int, int, const double*, int, int, int, int, int,
+                                          double*, double*, cudaStream_t);
+template cudaError_t launch_latent_bwd<double>(const double*, const double*, const double*, const double*,
+                                               const double*, size_t, double*, double*, cudaStream_t);
+template cudaError_t launch_build_x0<double>(const uint8_t*, int, int, int, const double*, int, int, double*,
+                                             cudaStream_t);
+
+#define SV_BWD_INST(T)                                                                                           \
+  template cudaError_t launch_up4_bwd<T>(const T*, const T*, int, int, int, int, T*, cudaStream_t);               \
+  template cudaError_t launch_loss_partial<T>(const LossJob<T>*, int, double, double, double*, cudaStream_t);     \
+  template cudaError_t launch_loss_finish<T>(const double*, int, double, double, double, T*, cudaStream_t);       \
+  template cudaError_t launch_adam<T>(float*, T*, T*, const T*, size_t, double, double, double, double, int,      \
                                       cudaStream_t);
 SV_BWD_INST(float)
 SV_BWD_INST(double)

@@ -1,5 +1,5 @@
-// conv_direct.cu -- plain refinement layers on CUDA cores, FP32 (the plain method) and
-// FP64 (gradient-check form).  Activations NHWC, weights [cout][ks][ks][cin].
+// conv_direct.cu -- refinement layers of the FP64 gradient-check form on CUDA cores (the FP32
+// form's are in conv_f32.cu).  Activations NHWC, weights [cout][ks][ks][cin].
 //
 //   conv_direct_kernel  3x3 / 1x1 convolution with the input read through a view:
 //                       stride 1, stride 2, or nearest x2 upsampling cropped to the
@@ -63,9 +63,6 @@ struct SrcEnc1 {
 };
 
 template <typename OutT, typename T> __device__ __forceinline__ OutT to_out(T v) { return (OutT)v; }
-template <> __device__ __forceinline__ __nv_bfloat16 to_out<__nv_bfloat16, float>(float v) {
-  return __float2bfloat16_rn(v);
-}
 
 // One CTA: TH x TW output pixels x COT output channels; input channels in chunks of CIC
 // staged channel-planar in shared memory ([ci][row][col]) with the weights [tap][ci][co].
@@ -123,7 +120,6 @@ conv_direct_kernel(Src src, int Ci, const T* __restrict__ wt, const T* __restric
 }
 
 template <typename T> struct Cfg;
-template <> struct Cfg<float> { static constexpr int COT = 32, CIC = 8; };
 template <> struct Cfg<double> { static constexpr int COT = 16, CIC = 8; };
 
 template <typename T, typename Src, int S, int KS, int CIC = Cfg<T>::CIC, typename OutT = T>
@@ -271,26 +267,15 @@ cudaError_t launch_latent(const T* e3, int H3, int W3, int Ci, const T* wmu, con
   return cudaGetLastError();
 }
 
-template cudaError_t launch_conv_direct<float>(const DirectConvArgs<float>&, int, int, cudaStream_t);
 template cudaError_t launch_conv_direct<double>(const DirectConvArgs<double>&, int, int, cudaStream_t);
-template cudaError_t launch_enc1<float, int16_t>(const uint8_t*, int, int, int, const int16_t*, int, int, const float*,
-                                                 const float*, int, float*, cudaStream_t);
-template cudaError_t launch_enc1<float, float>(const uint8_t*, int, int, int, const float*, int, int, const float*,
-                                               const float*, int, float*, cudaStream_t);
 template cudaError_t launch_enc1<double, double>(const uint8_t*, int, int, int, const double*, int, int, const double*,
                                                  const double*, int, double*, cudaStream_t);
 template cudaError_t launch_enc1<double, int16_t>(const uint8_t*, int, int, int, const int16_t*, int, int,
                                                   const double*, const double*, int, double*, cudaStream_t);
 template cudaError_t launch_final<double, int16_t, double>(const double*, int, int, int, const double*, const double*,
                                                            const int16_t*, int, int, double*, cudaStream_t);
-template cudaError_t launch_final<float, int16_t, float>(const float*, int, int, int, const float*, const float*,
-                                                         const int16_t*, int, int, float*, cudaStream_t);
-template cudaError_t launch_final<float, float, float>(const float*, int, int, int, const float*, const float*,
-                                                       const float*, int, int, float*, cudaStream_t);
 template cudaError_t launch_final<double, double, double>(const double*, int, int, int, const double*, const double*,
                                                           const double*, int, int, double*, cudaStream_t);
-template cudaError_t launch_latent<float>(const float*, int, int, int, const float*, const float*, const float*,
-                                          const float*, int, const float*, float*, float*, float*, cudaStream_t);
 template cudaError_t launch_latent<double>(const double*, int, int, int, const double*, const double*, const double*,
                                            const double*, int, const double*, double*, double*, double*, cudaStream_t);
 

@@ -2029,15 +2029,17 @@ sv_status Ctx::tc_launch(const TcRun& r, const unsigned char* tables, cudaStream
     prm.err = (int*)err_flag.p;
     prm.spin = spin_limit;
     if (tl && pl.layer == L_MU) {
-      // training: mu, logvar and the reparameterised z instead of z = mu
-      for (int i = 0; i < r.n; ++i) {
-        LaunchScope ls(*this, "train_latent", st);
-        if ((s = cuda(launch_train_latent_bf16(tl->e3[i], tl->P3[i], net.enc[2], W + net.w_off(L_MU), W + net.b_off(L_MU),
-                                               W + net.w_off(L_LV), W + net.b_off(L_LV), net.lat, tl->eps[i], tl->mu[i],
-                                               tl->lv[i], tl->z[i], st),
-                      "train latent")))
-          return s;
-      }
+      // training: mu, logvar and the reparameterised z instead of z = mu, in FP32
+      LaunchScope ls(*this, "train_latent", st);
+      const float* P = (const float*)f32_w.p;
+      if ((s = cuda(launch_f32_convert(tl->e3, tl->n, tl->max_e3, st), "convert e3"))) return s;
+      if ((s = cuda(launch_f32_conv(f32_l[L_MU], tl->mu, tl->n, tl->maxH3, tl->maxW3, P, W + net.b_off(L_MU), 4, st),
+                    "mu head")))
+        return s;
+      if ((s = cuda(launch_f32_conv(f32_l[L_LV], tl->lv, tl->n, tl->maxH3, tl->maxW3, P, W + net.b_off(L_LV), 4, st),
+                    "logvar head")))
+        return s;
+      if ((s = cuda(launch_f32_reparam(tl->lat, tl->n, tl->max_lat, st), "reparameterisation"))) return s;
       continue;
     }
     if (r.fused && pl.layer == L_DEC3) {

@@ -219,11 +219,8 @@ sv_status Ctx::refine_direct(const sv_pair& p, const void* coarse_map, bool coar
 #undef SV_SCOPE
 }
 
-template <> const float* Ctx::weights<float>() const { return (const float*)w32.p; }
 template <> const double* Ctx::weights<double>() const { return (const double*)w64.p; }
 
-template sv_status Ctx::refine_direct<float>(const sv_pair&, const void*, bool, const float*, float*, float*, float*,
-                                             float* const*, cudaStream_t);
 template sv_status Ctx::refine_direct<double>(const sv_pair&, const void*, bool, const double*, double*, double*,
                                               double*, double* const*, cudaStream_t);
 
@@ -237,6 +234,7 @@ sv_status Ctx::refresh_weight_copies_async(cudaStream_t st) {
     f32_to_f64<<<(unsigned)((n + 255) / 256), 256, 0, st>>>((const float*)w32.p, (double*)w64.p, n);
     if ((s = cuda(cudaGetLastError(), "weights to fp64"))) return s;
   }
+  if ((s = f32_pack(st))) return s;
   // (the FP8 form also runs its last decoder layer from the BF16 packs)
   if (cfg.precision == SV_BF16 || cfg.precision == SV_FP8)
     if ((s = pack_bf16_weights(st))) return s;
@@ -325,8 +323,10 @@ sv_status sv_create(const sv_config* cfg, int device, sv_ctx** out) {
   if (!s) s = c->cuda(cudaMemset(c->err_flag.p, 0, sizeof(int)), "zero error flag");
   if (!s) s = c->cuda(c->w32.ensure(n * sizeof(float)), "alloc weights");
   if (!s) s = c->cuda(cudaMemset(c->w32.p, 0, n * sizeof(float)), "zero weights");
+  if (!s) s = c->f32_plan();
   if (!s) s = c->refresh_weight_copies();
   if (s) {
+    c->release_all();
     delete c;
     return s;
   }

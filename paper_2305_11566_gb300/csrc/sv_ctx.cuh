@@ -5,6 +5,7 @@
 #include <string>
 #include <vector>
 
+#include "conv_f32.cuh"
 #include "sv_internal.cuh"
 
 namespace sv {
@@ -56,13 +57,14 @@ struct ZRun {
   int maxD = 1;
 };
 
-// Per-pair buffers of the training latent of the tensor-core form.
+// Device tables of the training latent of the tensor-core form (e3 converted to FP32, the two
+// heads, the reparameterisation), run between enc3 and dec1.
 struct TcTrainLatent {
-  std::vector<const __nv_bfloat16*> e3;
-  std::vector<int> P3;
-  std::vector<const float*> eps;
-  std::vector<float*> mu, lv;
-  std::vector<__nv_bfloat16*> z;
+  const F32Cvt* e3;
+  const F32Job *mu, *lv;
+  const F32Lat* lat;
+  size_t max_e3, max_lat;
+  int n, maxH3, maxW3;
 };
 
 // One captured batched step (coarse match + tensor-core refinement) and what it needs.
@@ -79,6 +81,12 @@ struct GraphEntry {
   long long last_use = 0;
 };
 
+// One pair's tensors of the FP32 form.  Training only: mu, lv and the copies of mu, lv (the
+// caller's, may be null) and eps.
+struct F32Tensors {
+  float *e1, *e2, *e3, *z, *d1, *d2, *d3, *mu, *lv, *mu_out, *lv_out, *eps_copy;
+};
+
 size_t t1_param_count();  // the paper's Table I network (t1net.cu)
 
 struct Ctx {
@@ -93,6 +101,13 @@ struct Ctx {
   DevBuf wfuse;                  // packed BF16 operands of the fused last decoder layer
   DevBuf wf8, wf8u, wf8s;        // FP8 form: packed E4M3 operands, unfolded decoder E4M3 weights, scales
   size_t f8_scale_ofs[6] = {0}, f8_unf_ofs[3] = {0}, f8_unf_scale_ofs[3] = {0};
+  DevBuf f32_w, f32_descs;       // FP32 form: packed weights and the table that packs them
+  DevBuf f32_act, f32_tab;       // FP32 form: activations of one group of pairs, job tables
+  F32Layer f32_l[L_COUNT];       // forward layers
+  F32Layer f32_t[L_COUNT];       // decoder layers of the training forward
+  F32Layer f32_g[L_COUNT];       // input gradients (L_MU: both latent heads)
+  int f32_n_descs = 0;
+  size_t f32_max_count = 0;
   DevBuf zpairs, zjobs;          // coarse-matcher tables
   DevBuf coarse_maps;            // int16 coarse maps of sv_pipeline
   DevBuf act[7];                 // activations e1 e2 e3 z d1 d2 d3 (direct path)
@@ -103,9 +118,10 @@ struct Ctx {
   DevBuf adam_m, adam_v;
   // differentiation form: state saved by the last training forward
   DevBuf train_saved, train_scratch, loss_acc, train_mu;
-  DevBuf wgrad_slots;            // per-CTA partial weight gradients of the FP32 backward
+  DevBuf wgrad_slots;            // per-block partial weight gradients of the FP32 backward
   std::vector<sv_pair> train_pairs;
   std::vector<const void*> train_coarse;
+  std::vector<F32Tensors> train_t;  // FP32 and BF16 contexts: the saved tensors (e1 .. e3 null when recomputed)
   std::vector<size_t> train_off;
   int train_elem = 0;
   bool train_ready = false;
@@ -183,6 +199,16 @@ struct Ctx {
   template <typename T>
   sv_status refine_direct(const sv_pair& p, const void* coarse_map, bool coarse_int16, const T* eps, T* Y, T* mu_out,
                           T* lv_out, T* const* saved, cudaStream_t st);
+  sv_status f32_plan();
+  sv_status f32_pack(cudaStream_t st);
+  sv_status f32_forward(const sv_pair* pairs, int n, const F32Tensors* t, const int16_t* const* coarse_i,
+                        const float* const* coarse_f, const float* const* eps, float* const* Y, cudaStream_t st);
+  sv_status f32_train_forward(const sv_pair* pairs, const void* const* coarse, const void* const* eps, int n,
+                              void* const* Y, void* const* mu, void* const* lv, cudaStream_t st);
+  sv_status f32_backward(const void* const* gY, const void* const* gmu_ext, const void* const* glv_ext, float* gparams,
+                         void* const* gcoarse, cudaStream_t st);
+  sv_status train_save_alloc(const sv_pair* pairs, int n, bool encoder, void* const* mu, void* const* lv);
+  sv_status f32_refine(const sv_pair* pairs, const int16_t* const* coarse, int n, float* const* out, cudaStream_t st);
   sv_status refine_infer(const sv_pair* pairs, const int16_t* const* coarse, int n, float* const* out,
                          cudaStream_t st);
   sv_status pipeline(const sv_pair* pairs, int n, float* const* out, cudaStream_t st);
@@ -264,6 +290,7 @@ struct Ctx {
     ev_free.clear();
     host_img.release(); host_out.release(); host_jobs.release(); err_flag.release(); tune_out.release();
     sgm_s.release(); sgm_c.release(); sgm_a.release(); sgm_tab.release(); x_codes.release(); x_maps.release();
+    f32_w.release(); f32_descs.release(); f32_act.release(); f32_tab.release();
     t1_act.release(); t1_tab.release(); loss_slots.release();
     w32.release(); w64.release(); wbf.release(); wfuse.release(); wf8.release(); wf8u.release(); wf8s.release(); zpairs.release(); zjobs.release();
     coarse_maps.release();

@@ -13,11 +13,7 @@ sv_status Ctx::refine_infer(const sv_pair* pairs, const int16_t* const* coarse, 
   if (cfg.precision == SV_BF16 || cfg.precision == SV_FP8) return refine_tc(pairs, coarse, n, out, st);
   if (cfg.precision == SV_FP64_CHECK)
     return fail(SV_ERR_UNSUPPORTED, "inference entry points produce FP32; use sv_refine_train on FP64_CHECK contexts");
-  for (int i = 0; i < n; ++i) {
-    sv_status s = refine_direct<float>(pairs[i], coarse[i], true, nullptr, out[i], nullptr, nullptr, nullptr, st);
-    if (s) return s;
-  }
-  return SV_OK;
+  return f32_refine(pairs, coarse, n, out, st);
 }
 
 sv_status Ctx::pipeline(const sv_pair* pairs, int n, float* const* out, cudaStream_t st) {

@@ -206,24 +206,21 @@ cudaError_t launch_edge_up2fix_f8(const UpFixPair* pairs, int n, int max_segment
                                   cudaStream_t st);
 cudaError_t launch_bf16_to_e4m3(const __nv_bfloat16* a, uint8_t* b, size_t n, cudaStream_t st);
 
-// Training latent of the tensor-core form: mu, logvar (FP32, caller's buffers) from BF16
-// e3 with FP32 weights, z = mu + eps exp(logvar / 2) stored as BF16 for the decoder.
-cudaError_t launch_train_latent_bf16(const __nv_bfloat16* e3, int P, int Ci, const float* wmu, const float* bmu,
-                                     const float* wlv, const float* blv, int lat, const float* eps, float* mu,
-                                     float* lv, __nv_bfloat16* z, cudaStream_t st);
-cudaError_t launch_bf16_to_f32(const __nv_bfloat16* a, float* b, size_t n, cudaStream_t st);
+// Input gradient of enc1 in FP32 (Ci = 2): d loss / d (L / 256, U / 256).
+cudaError_t launch_enc1_dgrad(const float* gout, int Ho, int Wo, int Co, const float* w, int Hi, int Wi, float* gin,
+                              cudaStream_t st);
 
-// FP32 gradients of a conv read through its input view (bwd_tiled.cu): dgrad writes (or adds
-// to) the input gradient, masked by the input activation's ReLU; wgrad adds the weight and
-// bias gradients, reducing per-CTA partial sums (slots, wgrad_slot_floats floats) in a fixed
-// order.
-cudaError_t launch_dgrad_tiled(const float* gout, int Ho, int Wo, int Co, const float* w, int ks, int mode,
-                               const float* mask_act, int Hi, int Wi, int Ci, int accumulate, float* gin,
-                               cudaStream_t st);
-cudaError_t launch_wgrad_tiled(const float* gout, int Ho, int Wo, int Co, const float* in, int Hi, int Wi, int Ci,
-                               int ks, int mode, float* gw, float* gb, float* slots, size_t slot_cap,
-                               cudaStream_t st);
-size_t wgrad_slot_floats(int Ho, int Wo, int Co, int Ci, int ks);
+// One pair of the loss: smooth-L1 of Y against gt, KL of (mu, lv); gradients where not null.
+template <typename T>
+struct LossJob {
+  const T* Y;
+  const float* gt;
+  T* gY;
+  size_t P;
+  const T *mu, *lv;
+  T *gmu, *glv;
+  size_t n;
+};
 
 // latent heads on the H3 x W3 grid: mu = 1x1(e3) + b; optionally logvar and z = mu + eps * exp(lv / 2).
 template <typename T>

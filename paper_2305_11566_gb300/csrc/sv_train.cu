@@ -1,9 +1,8 @@
 // sv_train.cu -- differentiation form: training forward (saves the decoder activations
-// and the latent), backward through every refinement layer and the fused bilinear
-// upsampling (the encoder is recomputed, not stored), loss and Adam.  FP32 for SV_FP32 /
-// SV_BF16 contexts, FP64 for SV_FP64_CHECK contexts.
+// and the latent) and backward (through every refinement layer and the fused bilinear
+// upsampling; the encoder is recomputed, not stored) of SV_FP64_CHECK contexts, loss and Adam of
+// every context.  The FP32 forward and backward are in sv_f32.cu.
 #include <algorithm>
-#include <type_traits>
 #include <vector>
 
 #include "sv_ctx.cuh"
@@ -25,11 +24,8 @@ template <typename T>
 cudaError_t launch_build_x0(const uint8_t* L, int pitch, int W, int H, const T* coarse, int w, int h, T* x0,
                             cudaStream_t st);
 template <typename T>
-cudaError_t launch_loss_rec(const T* Y, const float* gt, size_t P, double inv_npix, T* gY, double* acc,
-                            cudaStream_t st);
-template <typename T>
-cudaError_t launch_loss_kl(const T* mu, const T* lv, size_t n, double kl_scale, T* gmu, T* glv, double* acc,
-                           cudaStream_t st);
+cudaError_t launch_loss_partial(const LossJob<T>* jobs, int n, double inv_npix, double kl_scale, double* slots,
+                                cudaStream_t st);
 template <typename T>
 cudaError_t launch_loss_finish(const double* slots, int n_pairs, double inv_npix, double inv_nlat, double kl_w, T* out,
                                cudaStream_t st);
@@ -98,80 +94,6 @@ sv_status Ctx::train_forward(const sv_pair* pairs, const void* const* coarse, co
   return SV_OK;
 }
 
-// Training forward of the BF16 form: the tensor-core encoder and decoder (BF16 operands,
-// FP32 accumulation), the training latent in FP32 on CUDA cores, the final conv in FP32.
-// The decoder activations and the latent are saved as FP32 for the FP32 backward.
-sv_status Ctx::train_forward_bf16(const sv_pair* pairs, const void* const* coarse, const void* const* eps, int n,
-                                  void* const* Y, void* const* mu, void* const* lv, cudaStream_t st) {
-  using T = float;
-  sv_status s;
-  std::vector<size_t> off(n + 1, 0);
-  size_t lat_total = 0;
-  for (int i = 0; i < n; ++i) {
-    size_t sz[S_COUNT];
-    off[i + 1] = off[i] + saved_sizes<T>(net, Levels(pairs[i].height, pairs[i].width), sz);
-    lat_total += (sz[S_LV] + 1) / 2 * 2;
-  }
-  if ((s = cuda(train_saved.ensure(std::max<size_t>(off[n], 2) * sizeof(T)), "alloc saved activations"))) return s;
-  if ((s = cuda(train_mu.ensure(std::max<size_t>(lat_total, 2) * sizeof(T)), "alloc latent scratch"))) return s;
-  train_pairs.assign(pairs, pairs + n);
-  train_coarse.assign(coarse, coarse + n);
-  train_off = off;
-  train_elem = sizeof(T);
-  std::vector<float*> outs(n);
-  for (int i = 0; i < n; ++i) outs[i] = (float*)Y[i];
-  TcRun r;
-  if ((s = tc_prepare(pairs, nullptr, n, outs.data(), r, (const float* const*)coarse))) return s;
-  if ((s = cuda(tc_tables.ensure(r.host.size()), "alloc tables"))) return s;
-  if ((s = cuda(cudaMemcpyAsync(tc_tables.p, r.host.data(), r.host.size(), cudaMemcpyHostToDevice, st),
-                "upload tables")))
-    return s;
-  TcTrainLatent tl;
-  std::vector<T*> svb(n * S_COUNT);
-  size_t mo = 0;
-  for (int i = 0; i < n; ++i) {
-    const Levels lv_(pairs[i].height, pairs[i].width);
-    size_t sz[S_COUNT];
-    saved_sizes<T>(net, lv_, sz);
-    T* base = (T*)train_saved.p + off[i];
-    for (int k = 0; k < S_COUNT; ++k) {
-      svb[i * S_COUNT + k] = base;
-      base += (sz[k] + 1) / 2 * 2;
-    }
-    tl.e3.push_back((const __nv_bfloat16*)tc_act[2].p + tc_off[i][2]);
-    tl.P3.push_back(lv_.H[3] * lv_.W[3]);
-    tl.eps.push_back((const float*)eps[i]);
-    float* m = mu && mu[i] ? (float*)mu[i] : (float*)train_mu.p + mo;
-    mo += (sz[S_LV] + 1) / 2 * 2;
-    tl.mu.push_back(m);
-    tl.lv.push_back(svb[i * S_COUNT + S_LV]);
-    tl.z.push_back((__nv_bfloat16*)tc_act[3].p + tc_off[i][3]);
-  }
-  if ((s = tc_launch(r, (const unsigned char*)tc_tables.p, st, &tl))) return s;
-  for (int i = 0; i < n; ++i) {
-    const int acts[4] = {3, 4, 5, 6};
-    const int slots[4] = {S_Z, S_D1, S_D2, S_D3};
-    for (int k = 0; k < 4; ++k) {
-      LaunchScope _ls(*this, "save_bf16_to_f32", st);
-      if ((s = cuda(launch_bf16_to_f32((const __nv_bfloat16*)tc_act[acts[k]].p + tc_off[i][acts[k]],
-                                       svb[i * S_COUNT + slots[k]], tc_len[i][acts[k]], st),
-                    "save activations")))
-        return s;
-    }
-    size_t sz[S_COUNT];
-    saved_sizes<T>(net, Levels(pairs[i].height, pairs[i].width), sz);
-    if (lv && lv[i] &&
-        (s = cuda(cudaMemcpyAsync(lv[i], svb[i * S_COUNT + S_LV], sz[S_LV] * sizeof(T), cudaMemcpyDeviceToDevice, st),
-                  "copy logvar")))
-      return s;
-    if ((s = cuda(cudaMemcpyAsync(svb[i * S_COUNT + S_EPS], eps[i], sz[S_EPS] * sizeof(T), cudaMemcpyDeviceToDevice, st),
-                  "copy eps")))
-      return s;
-  }
-  train_ready = true;
-  return SV_OK;
-}
-
 template <typename T>
 sv_status Ctx::train_backward(const void* const* gY, const void* const* gmu_ext, const void* const* glv_ext, T* gparams,
                               void* const* gcoarse, cudaStream_t st) {
@@ -194,29 +116,12 @@ sv_status Ctx::train_backward(const void* const* gY, const void* const* gmu_ext,
     need = std::max(need, t);
   }
   if ((s = cuda(train_scratch.ensure(need * sizeof(T)), "alloc backward scratch"))) return s;
-  // FP32: the tiled gradient kernels (per-CTA weight-gradient slots, reduced in a fixed
-  // order); FP64 (the check form): the plain gather kernels
-  if constexpr (std::is_same<T, float>::value) {
-    size_t maxw = 0;
-    for (int l = 0; l < L_COUNT; ++l)
-      maxw = std::max(maxw, (size_t)net.cout(l) * net.ks(l) * net.ks(l) * net.cin(l) + net.cout(l));
-    if ((s = cuda(wgrad_slots.ensure(4 * 152 * maxw * sizeof(float)), "alloc weight-gradient slots"))) return s;
-  }
   auto DG = [&](const T* go, int Ho, int Wo, int Co, const T* wt, int ks, int mode, const T* mask, int Hi, int Wi, int Ci,
-                int accum, T* gi) -> cudaError_t {
-    if constexpr (std::is_same<T, float>::value)
-      return launch_dgrad_tiled(go, Ho, Wo, Co, wt, ks, mode, mask, Hi, Wi, Ci, accum, gi, st);
-    else
-      return launch_dgrad<T>(go, Ho, Wo, Co, wt, ks, mode, mask, Hi, Wi, Ci, accum, gi, st);
+                int accum, T* gi) {
+    return launch_dgrad<T>(go, Ho, Wo, Co, wt, ks, mode, mask, Hi, Wi, Ci, accum, gi, st);
   };
   auto WG = [&](const T* go, int Ho, int Wo, int Co, const T* in, int Hi, int Wi, int Ci, int ks, int mode, T* gw,
-                T* gb) -> cudaError_t {
-    if constexpr (std::is_same<T, float>::value)
-      return launch_wgrad_tiled(go, Ho, Wo, Co, in, Hi, Wi, Ci, ks, mode, gw, gb, (float*)wgrad_slots.p,
-                                wgrad_slots.n / sizeof(float), st);
-    else
-      return launch_wgrad<T>(go, Ho, Wo, Co, in, Hi, Wi, Ci, ks, mode, gw, gb, st);
-  };
+                T* gb) { return launch_wgrad<T>(go, Ho, Wo, Co, in, Hi, Wi, Ci, ks, mode, gw, gb, st); };
   for (int i = 0; i < n; ++i) {
     const sv_pair& p = train_pairs[i];
     const Levels lv(p.height, p.width);
@@ -323,27 +228,27 @@ sv_status Ctx::loss(const sv_pair* pairs, int n, const void* const* Y, const flo
                     cudaStream_t st) {
   sv_status s;
   const size_t per = loss_slots_per_pair();
-  if ((s = cuda(loss_acc.ensure(per * n * sizeof(double)), "alloc loss partials"))) return s;
+  if ((s = cuda(loss_acc.ensure(n * (per * sizeof(double) + sizeof(LossJob<T>))), "alloc loss partials"))) return s;
   double npix = 0, nlat = 0;
   for (int i = 0; i < n; ++i) {
     const Levels lv_(pairs[i].height, pairs[i].width);
     npix += (double)pairs[i].width * pairs[i].height;
     nlat += (double)lv_.H[3] * lv_.W[3] * net.lat;
   }
+  std::vector<LossJob<T>> jobs(n);
   for (int i = 0; i < n; ++i) {
-    double* acc = (double*)loss_acc.p + per * i;
     const Levels lv_(pairs[i].height, pairs[i].width);
-    const size_t P = (size_t)pairs[i].width * pairs[i].height, nl = (size_t)lv_.H[3] * lv_.W[3] * net.lat;
-    {
-      LaunchScope _ls(*this, "loss_rec", st);
-      if ((s = cuda(launch_loss_rec<T>((const T*)Y[i], gt[i], P, 1.0 / npix, gY && gY[i] ? (T*)gY[i] : nullptr, acc, st),
-                    "loss rec")))
-        return s;
-    }
-    LaunchScope _ls(*this, "loss_kl", st);
-    if ((s = cuda(launch_loss_kl<T>((const T*)mu[i], (const T*)lv[i], nl, kl_w / nlat, gmu && gmu[i] ? (T*)gmu[i] : nullptr,
-                                    glv && glv[i] ? (T*)glv[i] : nullptr, acc, st),
-                  "loss kl")))
+    jobs[i] = {(const T*)Y[i], gt[i], gY ? (T*)gY[i] : nullptr, (size_t)pairs[i].width * pairs[i].height,
+               (const T*)mu[i], (const T*)lv[i], gmu ? (T*)gmu[i] : nullptr, glv ? (T*)glv[i] : nullptr,
+               (size_t)lv_.H[3] * lv_.W[3] * net.lat};
+  }
+  LossJob<T>* d_jobs = (LossJob<T>*)((double*)loss_acc.p + per * n);
+  if ((s = cuda(cudaMemcpyAsync(d_jobs, jobs.data(), sizeof(LossJob<T>) * n, cudaMemcpyHostToDevice, st),
+                "upload loss table")))
+    return s;
+  {
+    LaunchScope _ls(*this, "loss_partial", st);
+    if ((s = cuda(launch_loss_partial<T>(d_jobs, n, 1.0 / npix, kl_w / nlat, (double*)loss_acc.p, st), "loss")))
       return s;
   }
   LaunchScope _ls(*this, "loss_finish", st);
@@ -370,12 +275,8 @@ sv_status Ctx::adam(const T* g, int step, double lr, double b1, double b2, doubl
   return refresh_weight_copies_async(st);
 }
 
-template sv_status Ctx::train_forward<float>(const sv_pair*, const void* const*, const void* const*, int, void* const*,
-                                             void* const*, void* const*, cudaStream_t);
 template sv_status Ctx::train_forward<double>(const sv_pair*, const void* const*, const void* const*, int, void* const*,
                                               void* const*, void* const*, cudaStream_t);
-template sv_status Ctx::train_backward<float>(const void* const*, const void* const*, const void* const*, float*,
-                                              void* const*, cudaStream_t);
 template sv_status Ctx::train_backward<double>(const void* const*, const void* const*, const void* const*, double*,
                                                void* const*, cudaStream_t);
 
@@ -408,7 +309,7 @@ sv_status sv_refine_train(sv_ctx* ctx, const sv_pair* pairs, const void* const* 
     return c->train_forward<double>(pairs, coarse, eps, n_pairs, disp_out, mu_out, logvar_out, (cudaStream_t)stream);
   if (c->cfg.precision == SV_BF16)
     return c->train_forward_bf16(pairs, coarse, eps, n_pairs, disp_out, mu_out, logvar_out, (cudaStream_t)stream);
-  return c->train_forward<float>(pairs, coarse, eps, n_pairs, disp_out, mu_out, logvar_out, (cudaStream_t)stream);
+  return c->f32_train_forward(pairs, coarse, eps, n_pairs, disp_out, mu_out, logvar_out, (cudaStream_t)stream);
 }
 
 sv_status sv_refine_backward(sv_ctx* ctx, const void* const* grad_disp, const void* const* grad_mu,
@@ -426,8 +327,7 @@ sv_status sv_refine_backward(sv_ctx* ctx, const void* const* grad_disp, const vo
   if (c->train_elem == (int)sizeof(double))
     return c->train_backward<double>(grad_disp, grad_mu, grad_logvar, (double*)grad_params, grad_coarse,
                                      (cudaStream_t)stream);
-  return c->train_backward<float>(grad_disp, grad_mu, grad_logvar, (float*)grad_params, grad_coarse,
-                                  (cudaStream_t)stream);
+  return c->f32_backward(grad_disp, grad_mu, grad_logvar, (float*)grad_params, grad_coarse, (cudaStream_t)stream);
 }
 
 sv_status sv_loss(sv_ctx* ctx, const sv_pair* pairs, int n_pairs, const void* const* disp, const float* const* gt,

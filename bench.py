@@ -225,7 +225,7 @@ def pair_work(shape, W, H):
 # 3 eighth resolution.
 T1_LAYERS = [("t1_fe1", 0, 5, 32, 1, 1), ("t1_fe2", 0, 5, 32, 1, 1), ("t1_en1", 1, 5, 16, 64, 2),
              ("t1_en1r", 0, 5, 8, 16, 2), ("t1_en2", 1, 5, 32, 24, 3), ("t1_en2r", 0, 5, 16, 32, 3),
-             ("t1_heads", 0, 1, 2, 48, 3), ("t1_d1", 0, 1, 32, 1, 3), ("t1_d1r", 0, 5, 16, 80, 3),
+             ("t1_latent", 0, 1, 2, 48, 3), ("t1_latent", 0, 1, 32, 1, 3), ("t1_d1r", 0, 5, 16, 80, 3),
              ("t1_d2", 2, 5, 16, 96, 2), ("t1_d2r", 0, 5, 8, 40, 2), ("t1_d", 2, 5, 16, 48, 1),
              ("t1_y", 2, 5, 1, 81, 0)]
 
@@ -238,7 +238,7 @@ def t1_work(W, H):
     for name, mode, k, co, ci, lev in T1_LAYERS:
         Ho, Wo = lv[lev]
         taps = k * k / 4.0 if mode == 2 else k * k
-        out[name] = 2.0 * Ho * Wo * co * ci * taps
+        out[name] = out.get(name, 0.0) + 2.0 * Ho * Wo * co * ci * taps
     return out
 
 

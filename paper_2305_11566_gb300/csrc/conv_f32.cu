@@ -130,13 +130,14 @@ struct F32Args {
 
 // The patch rows iy0 .. of one channel chunk, channel-planar; zero outside the input.
 template <class G, int PR, int PC>
-__device__ __forceinline__ void load_patch(float* dst, const float* src, int C, int iy0, int ix0, int Hi, int Wi) {
+__device__ __forceinline__ void load_patch(float* dst, const float* src, int C, int iy0, int ix0, int Hi, int Wi,
+                                           int nc = G::CIC) {  // nc: channels that exist (the others are zero)
   constexpr int SL = kThreads / G::CIC, CW = SL < 32 ? SL : 32, RG = SL / CW;
   const int t = threadIdx.x, ci = t % G::CIC, cc = (t / G::CIC) % CW, rg = t / (G::CIC * CW);
   const ptrdiff_t step = (ptrdiff_t)RG * Wi * C;
   for (int c = cc; c < PC; c += CW) {
     const int ix = ix0 + c;
-    const bool cok = (unsigned)ix < (unsigned)Wi;
+    const bool cok = (unsigned)ix < (unsigned)Wi && ci < nc;
     ptrdiff_t o = ((ptrdiff_t)(iy0 + rg) * Wi + ix) * C + ci;
     const int cd = G::SPLIT ? (c & 1 ? G::EVEN : 0) + (c >> 1) : c;  // (patch column 0 is odd)
     float* d = dst + ci * G::PLANE + rg * G::PITCH + cd;
@@ -525,7 +526,11 @@ __global__ void f32_pack_kernel(const F32PackDesc* __restrict__ descs, const flo
       return params[D.src + (((size_t)o * D.ks + ky) * D.ks + kx) * D.ci + ii];
     };
     float v = 0.f;
-    if (D.border) {
+    if (D.kind == FK_Y5) {
+      // one source of the last layer: output "channel" n is phase (n >> 1, n & 1)
+      const int ky = ((n >> 1) ? 3 : 4) - 2 * (r - (n >> 1)), kx = ((n & 1) ? 3 : 4) - 2 * (c - (n & 1));
+      if (k < D.co && ky >= 0 && ky <= 4 && kx >= 0 && kx <= 4) v = params[D.src + (ky * 5 + kx) * D.ci + D.N + k];
+    } else if (D.border) {
       v = D.kind == FK_DUP2 ? W(k, r, c, nn) : W(nn, r, c, k);
     } else if (D.kind == FK_UP2) {
       for (int ky = 0; ky < 3; ++ky)
@@ -694,6 +699,83 @@ f32_final_kernel(const F32Img* __restrict__ imgs, const float* __restrict__ w, c
   }
 }
 
+// FK_Y5: a thread owns 8 input positions along x and their four output phases; the phase pair
+// py = 1 has no tap in window row 0.  Channels go 4 a step (a one-channel source fills its step
+// with zeros); the packed weights are [step][tap][channel][phase].
+struct Y5Geo {
+  static constexpr int CIC = 4, TW = 32, TH = 32, S = 1, PR = 34, PC = 34, PITCH = 36;
+  static constexpr int PLANE = (PR * PITCH + 31 - 4) / 32 * 32 + 4, WF = 9 * CIC * 4, BUF = CIC * PLANE + WF;
+  static constexpr bool SPLIT = false;
+  static constexpr int EVEN = 0;
+};
+__global__ void __launch_bounds__(kThreads, 5)
+f32_y5_kernel(const F32Job* __restrict__ jobs, const float* __restrict__ w, const float* __restrict__ bias, int steps,
+              float scale, int tiles_x) {
+  using G = Y5Geo;
+  __shared__ __align__(16) float sm[2 * G::BUF];
+  const F32Job& J = jobs[blockIdx.z];
+  const int Y0 = (blockIdx.x / tiles_x) * G::TH, X0 = (blockIdx.x % tiles_x) * G::TW;
+  if (Y0 >= J.Hi || X0 >= J.Wi) return;
+  const int gx = threadIdx.x % 4, row = threadIdx.x / 4;
+  int s = 0, c0 = 0;
+  auto stage = [&](int ch) {
+    float* b = sm + (ch & 1) * G::BUF;
+    if (c0 >= J.ic[s]) { c0 = 0; ++s; }
+    load_patch<G, G::PR, G::PC>(b, J.in[s] + c0, J.ic[s], Y0 - 1, X0 - 1, J.Hi, J.Wi, J.ic[s] - c0);
+    c0 += G::CIC;
+    if (threadIdx.x < G::WF / 4) cp16(b + G::CIC * G::PLANE + 4 * threadIdx.x, w + (size_t)ch * G::WF + 4 * threadIdx.x);
+    cp_commit();
+  };
+  u64 acc[PX][2];
+#pragma unroll
+  for (int p = 0; p < PX; ++p) acc[p][0] = acc[p][1] = 0ull;
+  stage(0);
+  for (int ch = 0; ch < steps; ++ch) {
+    if (ch + 1 < steps) {
+      stage(ch + 1);
+      cp_wait<1>();
+    } else {
+      cp_wait<0>();
+    }
+    __syncthreads();
+    const float* pa = sm + (ch & 1) * G::BUF + row * G::PITCH + gx * PX;
+    const float* pw = sm + (ch & 1) * G::BUF + G::CIC * G::PLANE;
+#pragma unroll 1
+    for (int ci = 0; ci < G::CIC; ++ci)
+#pragma unroll
+      for (int r = 0; r < 3; ++r) {
+        float a[12];
+        load_row<G, 3>(pa + ci * G::PLANE + r * G::PITCH, a);
+        u64 v[10];
+#pragma unroll
+        for (int q = 0; q < 10; ++q) v[q] = dup2(a[q]);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          const ulonglong2 k = *reinterpret_cast<const ulonglong2*>(pw + ((r * 3 + c) * G::CIC + ci) * 4);
+#pragma unroll
+          for (int p = 0; p < PX; ++p) {
+            fma2(acc[p][0], v[p + c], k.x);
+            if (r > 0) fma2(acc[p][1], v[p + c], k.y);
+          }
+        }
+      }
+    __syncthreads();
+  }
+  const float b0 = bias[0];
+#pragma unroll
+  for (int py = 0; py < 2; ++py) {
+    const int oy = 2 * (Y0 + row) + py;
+    if (oy >= J.Ho) break;
+#pragma unroll
+    for (int p = 0; p < PX; ++p) {
+      const int ox = 2 * (X0 + gx * PX + p);
+      const float2 f = unpack2(acc[p][py]);
+      if (ox < J.Wo) J.out[(size_t)oy * J.Wo + ox] = (f.x + b0) * scale;
+      if (ox + 1 < J.Wo) J.out[(size_t)oy * J.Wo + ox + 1] = (f.y + b0) * scale;
+    }
+  }
+}
+
 __global__ void f32_reparam_kernel(const F32Lat* __restrict__ lat) {
   const F32Lat& q = lat[blockIdx.y];
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < q.n; i += (size_t)gridDim.x * blockDim.x) {
@@ -786,6 +868,43 @@ F32Layer f32_plan_layer(int kind, const F32Src* src, int n_src, std::vector<F32P
     total += (size_t)l.K * l.N * ty * tx;
   }
   return l;
+}
+
+F32Layer f32_plan_y5(size_t w_ofs, const int* ic, int n_ic, std::vector<F32PackDesc>& descs, size_t& total) {
+  F32Layer l;
+  l.kind = FK_Y5;
+  l.w[0] = total;
+  int channels = 0;
+  for (int i = 0; i < n_ic; ++i) channels += ic[i];
+  int c0 = 0;
+  for (int i = 0; i < n_ic; ++i) {
+    F32PackDesc d{};
+    d.src = w_ofs;
+    d.dst = total;
+    d.kind = FK_Y5;
+    d.ks = 5;
+    d.co = ic[i];     // channels of this source
+    d.ci = channels;  // channels of the layer
+    d.N = c0;         // first channel of this source
+    d.cic = Y5Geo::CIC;
+    d.K = d.Ktot = (ic[i] + d.cic - 1) / d.cic * d.cic;
+    d.bn = 4;
+    d.taps = 9;
+    d.tx = 3;
+    d.count = (size_t)d.K * 9 * 4;
+    descs.push_back(d);
+    total += d.count;
+    l.K += d.K;
+    c0 += ic[i];
+  }
+  return l;
+}
+
+cudaError_t launch_f32_y5(const F32Layer& l, const F32Job* jobs, int n, int maxHo, int maxWo, const float* packed,
+                          const float* bias, float scale, cudaStream_t st) {
+  const int tx = ((maxWo + 1) / 2 + Y5Geo::TW - 1) / Y5Geo::TW, ty = ((maxHo + 1) / 2 + Y5Geo::TH - 1) / Y5Geo::TH;
+  f32_y5_kernel<<<dim3(tx * ty, 1, n), kThreads, 0, st>>>(jobs, packed + l.w[0], bias, l.K / Y5Geo::CIC, scale, tx);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_f32_pack(const F32PackDesc* d, int n, size_t max_count, const float* params, float* packed,

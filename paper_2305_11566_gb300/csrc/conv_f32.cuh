@@ -19,8 +19,10 @@ namespace sv {
 //   FK_DUP2  input gradient of FK_UP2: 4x4 taps, stride 2
 //   FK_S1_5, FK_S2_5  5x5 stride 1 / 2;  FK_DE5  5x5 stride-2 deconvolution: four phases of
 //            3x3, 3x2, 2x3, 2x2 taps
+//   FK_Y5    the Table I network's last layer: 5x5 stride-2 deconvolution to one channel, the four
+//            output phases taken as four output channels of a 3x3 window
 //   FK_UP2X  nearest x2 + 3x3 on the upsampled grid, nine taps (the training forward)
-enum F32Kind { FK_S2 = 0, FK_P1, FK_UP2, FK_DS2, FK_DUP2, FK_S1_5, FK_S2_5, FK_DE5, FK_UP2X, FK_COUNT };
+enum F32Kind { FK_S2 = 0, FK_P1, FK_UP2, FK_DS2, FK_DUP2, FK_S1_5, FK_S2_5, FK_DE5, FK_UP2X, FK_Y5, FK_COUNT };
 
 // One pair's operands of a layer.  `in`: the input is the channel concatenation of up to four
 // NHWC tensors of Hi x Wi (widths ic, each a whole number of staged channel chunks).
@@ -103,6 +105,10 @@ cudaError_t launch_f32_enc1(const F32Img* imgs, int n, int maxH1, int maxW1, con
                             cudaStream_t st);
 // z = mu + eps exp(lv / 2), with copies of mu, lv and eps where asked for.
 cudaError_t launch_f32_reparam(const F32Lat* lat, int n, size_t max_n, cudaStream_t st);
+// FK_Y5: out = scale (sum + bias); the jobs' tensors are [Hi][Wi][ic] inputs, [Ho][Wo] outputs.
+F32Layer f32_plan_y5(size_t w_ofs, const int* ic, int n_ic, std::vector<F32PackDesc>& descs, size_t& total);
+cudaError_t launch_f32_y5(const F32Layer& l, const F32Job* jobs, int n, int maxHo, int maxWo, const float* packed,
+                          const float* bias, float scale, cudaStream_t st);
 cudaError_t launch_f32_convert(const F32Cvt* jobs, int n, size_t max_n, cudaStream_t st);
 cudaError_t launch_f32_final(const F32Img* imgs, int n, int maxH, int maxW, const float* w, const float* b, int C,
                              cudaStream_t st);

@@ -225,8 +225,8 @@ template sv_status Ctx::refine_direct<double>(const sv_pair&, const void*, bool,
                                               double*, double* const*, cudaStream_t);
 
 sv_status Ctx::refresh_weight_copies_async(cudaStream_t st) {
-  if (t1) return SV_OK;  // the Table I network runs on the FP32 master copy
   sv_status s;
+  if (t1) return f32_pack(st);  // the Table I network runs on the FP32 master copy and its packs
   const size_t n = net.count();
   if ((s = cuda(w64.ensure(n * sizeof(double)), "alloc fp64 weights"))) return s;
   {

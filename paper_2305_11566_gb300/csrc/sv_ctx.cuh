@@ -88,6 +88,7 @@ struct F32Tensors {
 };
 
 size_t t1_param_count();  // the paper's Table I network (t1net.cu)
+void t1_plan_layers(F32Layer* layers, std::vector<F32PackDesc>& descs, size_t& total);
 
 struct Ctx {
   sv_config cfg{};
@@ -106,6 +107,7 @@ struct Ctx {
   F32Layer f32_l[L_COUNT];       // forward layers
   F32Layer f32_t[L_COUNT];       // decoder layers of the training forward
   F32Layer f32_g[L_COUNT];       // input gradients (L_MU: both latent heads)
+  F32Layer t1_l[13];             // the Table I network's 5 x 5 layers
   int f32_n_descs = 0;
   size_t f32_max_count = 0;
   DevBuf zpairs, zjobs;          // coarse-matcher tables

@@ -24,7 +24,7 @@ constexpr size_t pad32(size_t v) { return (v + 31) / 32 * 32; }
 }  // namespace
 
 sv_status Ctx::f32_plan() {
-  if (t1 || (cfg.precision != SV_FP32 && cfg.precision != SV_BF16)) return SV_OK;
+  if (cfg.precision != SV_FP32 && cfg.precision != SV_BF16) return SV_OK;
   auto src = [&](int l) { return F32Src{net.w_off(l), net.ks(l), net.cout(l), net.cin(l)}; };
   std::vector<F32PackDesc> descs;
   size_t total = 0;
@@ -33,22 +33,26 @@ sv_status Ctx::f32_plan() {
     for (int k : layers) s.push_back(src(k));
     l = f32_plan_layer(kind, s.data(), (int)s.size(), descs, total);
   };
-  add(f32_l[L_ENC2], FK_S2, {L_ENC2});
-  add(f32_l[L_ENC3], FK_S2, {L_ENC3});
-  add(f32_l[L_MU], FK_P1, {L_MU});
-  add(f32_l[L_LV], FK_P1, {L_LV});
-  for (int l : {L_DEC1, L_DEC2, L_DEC3}) {
-    if (cfg.precision == SV_FP32) {  // (a BF16 context decodes on the tensor cores)
-      add(f32_l[l], FK_UP2, {l});
-      f32_t[l] = f32_l[l];  // the nine unsummed taps, also the summed form's edge weights
-      f32_t[l].kind = FK_UP2X;
-      f32_t[l].w[0] = f32_l[l].wb;
+  if (t1) {
+    t1_plan_layers(t1_l, descs, total);
+  } else {
+    add(f32_l[L_ENC2], FK_S2, {L_ENC2});
+    add(f32_l[L_ENC3], FK_S2, {L_ENC3});
+    add(f32_l[L_MU], FK_P1, {L_MU});
+    add(f32_l[L_LV], FK_P1, {L_LV});
+    for (int l : {L_DEC1, L_DEC2, L_DEC3}) {
+      if (cfg.precision == SV_FP32) {  // (a BF16 context decodes on the tensor cores)
+        add(f32_l[l], FK_UP2, {l});
+        f32_t[l] = f32_l[l];  // the nine unsummed taps, also the summed form's edge weights
+        f32_t[l].kind = FK_UP2X;
+        f32_t[l].w[0] = f32_l[l].wb;
+      }
+      add(f32_g[l], FK_DUP2, {l});
     }
-    add(f32_g[l], FK_DUP2, {l});
+    add(f32_g[L_MU], FK_P1, {L_MU, L_LV});
+    add(f32_g[L_ENC3], FK_DS2, {L_ENC3});
+    add(f32_g[L_ENC2], FK_DS2, {L_ENC2});
   }
-  add(f32_g[L_MU], FK_P1, {L_MU, L_LV});
-  add(f32_g[L_ENC3], FK_DS2, {L_ENC3});
-  add(f32_g[L_ENC2], FK_DS2, {L_ENC2});
   f32_n_descs = (int)descs.size();
   f32_max_count = 0;
   for (auto& d : descs) f32_max_count = std::max(f32_max_count, d.count);

@@ -3,40 +3,18 @@
 //
 //   t1_inputs_kernel   X_1 = 2 x 2 box mean of the left image / 256 and X_0 = 4 x bilinear x2 of
 //                      the coarse map / 256, both at half resolution
-//   t1_conv_kernel     one layer: 5 x 5 (or 1 x 1) conv, stride 1 or 2, or 5 x 5 stride-2
-//                      deconvolution, over the channel concatenation of up to four NHWC
-//                      tensors of the same size (the skip connections of Table I are read in
-//                      place, never copied); bias, optional leaky ReLU 0.1 and output scale
-//   t1_gauss_kernel    mu, sigma from the heads and the decoder input
-//                      (mu - 1) + eps exp(sigma - 1) (Eq. 8; eps = 0 at inference)
+//   t1_latent_kernel   heads -> mu, sigma, the decoder input (mu - 1) + eps exp(sigma - 1) (Eq. 8;
+//                      eps = 0 at inference) and D_1 of it, a thread a pixel
 //
-// Every layer is a direct convolution: a CTA stages a tile of the concatenated input for
-// CIC channels at a time and the matching weights in shared memory; each thread
-// accumulates COT output channels of one output pixel (conv) or of the four output
-// phases (2 y + py, 2 x + px) of one input position (deconv: each phase reads its own
-// taps ky = py (mod 2), kx = px (mod 2), so a warp's threads share one tap sequence).
+// The 5 x 5 layers run on conv_f32.cu (kinds FK_S1_5, FK_S2_5, FK_DE5, FK_Y5): the skip connections of
+// Table I are channel concatenations of up to four tensors, read in place.
 #include "sv_ctx.cuh"
 
 namespace sv {
 
 namespace {
 
-constexpr int kTW = 16, kTH = 8;  // thread tile
-
-struct T1Src {
-  const float* p[4];
-  int c[4];
-};
-
-// One layer of one pair.
-struct T1Job {
-  T1Src src;
-  int Hi, Wi;
-  float* out;
-  int Ho, Wo;
-};
-
-// Per-pair inputs of t1_inputs_kernel / t1_gauss_kernel.
+// Per-pair operands of t1_inputs_kernel / t1_latent_kernel.
 struct T1PairIO {
   const uint8_t* L;
   int pitch, W, H, w, h;
@@ -44,24 +22,14 @@ struct T1PairIO {
   const float* coarse_f;    // real-valued coarse map when non-null
   float* X0;                // [Hh][Wh]
   float* X1;                // [Hh][Wh]
-  const float* heads;       // [H8][W8][2]
+  const float* en2;         // [H8][W8][32]
+  const float* en2r;        // [H8][W8][16]
   const float* eps;         // [H8][W8] or null
-  float* g;                 // [H8][W8] decoder input
+  float* d1;                // [H8][W8][32]
   float* mu;                // [H8][W8] or null
   float* sigma;             // [H8][W8] or null
   int H8, W8;
 };
-
-__device__ __forceinline__ float src_at(const T1Src& s, size_t pix, int ci) {
-  if (ci < s.c[0]) return s.p[0][pix * s.c[0] + ci];
-  ci -= s.c[0];
-  if (ci < s.c[1]) return s.p[1][pix * s.c[1] + ci];
-  ci -= s.c[1];
-  if (ci < s.c[2]) return s.p[2][pix * s.c[2] + ci];
-  ci -= s.c[2];
-  if (ci < s.c[3]) return s.p[3][pix * s.c[3] + ci];
-  return 0.f;
-}
 
 __global__ void t1_inputs_kernel(const T1PairIO* __restrict__ io) {
   const T1PairIO& p = io[blockIdx.z];
@@ -88,104 +56,44 @@ __global__ void t1_inputs_kernel(const T1PairIO* __restrict__ io) {
   p.X0[(size_t)y * Wh + x] = ((1.f - fy) * top + fy * bot) * (4.0f / 256.0f);
 }
 
-__global__ void t1_gauss_kernel(const T1PairIO* __restrict__ io) {
+constexpr int kLatThreads = 128;
+__global__ void __launch_bounds__(kLatThreads)
+t1_latent_kernel(const T1PairIO* __restrict__ io, const float* __restrict__ wh, const float* __restrict__ bh,
+                 const float* __restrict__ wd, const float* __restrict__ bd) {
+  __shared__ float4 hs[2][12];  // head weights
+  __shared__ float4 ds[8], db[8];  // D_1 weights and bias
+  if (threadIdx.x < 24) hs[threadIdx.x / 12][threadIdx.x % 12] = reinterpret_cast<const float4*>(wh)[threadIdx.x];
+  if (threadIdx.x >= 32 && threadIdx.x < 64) {
+    const int t = threadIdx.x - 32;
+    reinterpret_cast<float*>(ds)[t] = wd[t];
+    reinterpret_cast<float*>(db)[t] = bd[t];
+  }
+  __syncthreads();
   const T1PairIO& p = io[blockIdx.y];
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= p.H8 * p.W8) return;
-  const float m = p.heads[2 * q], s = p.heads[2 * q + 1];
-  p.g[q] = (m - 1.0f) + (p.eps ? p.eps[q] * expf(s - 1.0f) : 0.0f);
+  float m = 0.f, s = 0.f;
+#pragma unroll
+  for (int c = 0; c < 12; ++c) {
+    const float4 v = c < 8 ? *reinterpret_cast<const float4*>(p.en2 + (size_t)q * 32 + 4 * c)
+                           : *reinterpret_cast<const float4*>(p.en2r + (size_t)q * 16 + 4 * (c - 8));
+    const float4 a = hs[0][c], b = hs[1][c];
+    m = fmaf(v.w, a.w, fmaf(v.z, a.z, fmaf(v.y, a.y, fmaf(v.x, a.x, m))));
+    s = fmaf(v.w, b.w, fmaf(v.z, b.z, fmaf(v.y, b.y, fmaf(v.x, b.x, s))));
+  }
+  m += bh[0];
+  s += bh[1];
+  const float g = (m - 1.0f) + (p.eps ? p.eps[q] * expf(s - 1.0f) : 0.0f);
   if (p.mu) p.mu[q] = m;
   if (p.sigma) p.sigma[q] = s;
-}
-
-// MODE 0: conv stride 1, 1: conv stride 2, 2: deconv stride 2 (outputs 2 i + k - 2, cropped).
-template <int MODE, int KS, int COT, int CIC>
-__global__ void __launch_bounds__(kTW * kTH)
-t1_conv_kernel(const T1Job* __restrict__ jobs, int groups, const float* __restrict__ wt, const float* __restrict__ bias,
-               int Ci, int Co, int act, float scale) {
-  constexpr int PAD = KS / 2;
-  constexpr int S = MODE == 1 ? 2 : 1;
-  constexpr int TR = MODE == 2 ? kTH + 2 : (kTH - 1) * S + KS;
-  constexpr int TC = MODE == 2 ? kTW + 2 : (kTW - 1) * S + KS;
-  constexpr int NP = MODE == 2 ? 4 : 1;  // output phases per thread
-  __shared__ float tile[CIC][TR][TC];
-  __shared__ __align__(16) float wsm[KS * KS][CIC][COT];
-  const T1Job& J = jobs[blockIdx.z / groups];
-  const int co0 = (blockIdx.z % groups) * COT;
-  const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * kTW + tx;
-  const int X0 = blockIdx.x * kTW, Y0 = blockIdx.y * kTH;
-  // whole-block exit when the tile lies beyond this pair's output
-  if (MODE == 2 ? (2 * X0 >= J.Wo || 2 * Y0 >= J.Ho) : (X0 >= J.Wo || Y0 >= J.Ho)) return;
-  const int ry0 = MODE == 2 ? Y0 - 1 : Y0 * S - PAD;  // input row / column of tile element 0
-  const int rx0 = MODE == 2 ? X0 - 1 : X0 * S - PAD;
-  float acc[NP][COT];
 #pragma unroll
-  for (int q = 0; q < NP; ++q)
-#pragma unroll
-    for (int c = 0; c < COT; ++c) acc[q][c] = 0.f;
-  for (int ci0 = 0; ci0 < Ci; ci0 += CIC) {
-    for (int e = tid; e < TR * TC * CIC; e += kTW * kTH) {
-      const int ci = e % CIC, rc = e / CIC;
-      const int r = rc / TC, c = rc - r * TC;
-      const int iy = ry0 + r, ix = rx0 + c;
-      float v = 0.f;
-      if (iy >= 0 && ix >= 0 && iy < J.Hi && ix < J.Wi && ci0 + ci < Ci) v = src_at(J.src, (size_t)iy * J.Wi + ix, ci0 + ci);
-      tile[ci][r][c] = v;
-    }
-    for (int e = tid; e < KS * KS * CIC * COT; e += kTW * kTH) {
-      const int co = e % COT, t = e / COT;
-      const int ci = t % CIC, tap = t / CIC;
-      const int gco = co0 + co, gci = ci0 + ci;
-      wsm[tap][ci][co] = (gco < Co && gci < Ci) ? wt[((size_t)gco * KS * KS + tap) * Ci + gci] : 0.f;
-    }
-    __syncthreads();
-    if constexpr (MODE == 2) {
-#pragma unroll
-      for (int py = 0; py < 2; ++py)
-#pragma unroll
-        for (int px = 0; px < 2; ++px)
-#pragma unroll
-          for (int ky = py; ky < KS; ky += 2)
-#pragma unroll
-            for (int kx = px; kx < KS; kx += 2) {
-              const int r = ty + (py + 2 - ky) / 2 + 1, c = tx + (px + 2 - kx) / 2 + 1;
-#pragma unroll
-              for (int ci = 0; ci < CIC; ++ci) {
-                const float v = tile[ci][r][c];
-                const float* wp = wsm[ky * KS + kx][ci];
-#pragma unroll
-                for (int co = 0; co < COT; ++co) acc[py * 2 + px][co] = fmaf(v, wp[co], acc[py * 2 + px][co]);
-              }
-            }
-    } else {
-#pragma unroll
-      for (int ky = 0; ky < KS; ++ky)
-#pragma unroll
-        for (int kx = 0; kx < KS; ++kx)
-#pragma unroll
-          for (int ci = 0; ci < CIC; ++ci) {
-            const float v = tile[ci][ty * S + ky][tx * S + kx];
-            const float* wp = wsm[ky * KS + kx][ci];
-#pragma unroll
-            for (int co = 0; co < COT; ++co) acc[0][co] = fmaf(v, wp[co], acc[0][co]);
-          }
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int q = 0; q < NP; ++q) {
-    const int oy = MODE == 2 ? 2 * (Y0 + ty) + (q >> 1) : Y0 + ty;
-    const int ox = MODE == 2 ? 2 * (X0 + tx) + (q & 1) : X0 + tx;
-    if (oy < J.Ho && ox < J.Wo) {
-      float* op = J.out + ((size_t)oy * J.Wo + ox) * Co + co0;
-#pragma unroll
-      for (int co = 0; co < COT; ++co)
-        if (co0 + co < Co) {
-          float v = acc[q][co] + bias[co0 + co];
-          if (act && v < 0.f) v *= 0.1f;
-          op[co] = v * scale;
-        }
-    }
+  for (int c = 0; c < 8; ++c) {
+    const float4 w = ds[c], b = db[c];
+    auto f = [&](float wv, float bv) {
+      const float v = fmaf(g, wv, 0.f) + bv;
+      return v < 0.f ? v * 0.1f : v;
+    };
+    *reinterpret_cast<float4*>(p.d1 + (size_t)q * 32 + 4 * c) = make_float4(f(w.x, b.x), f(w.y, b.y), f(w.z, b.z), f(w.w, b.w));
   }
 }
 
@@ -196,35 +104,6 @@ struct T1Layer {
 constexpr T1Layer kT1[13] = {{0, 5, 32, 1},  {0, 5, 32, 1},  {1, 5, 16, 64}, {0, 5, 8, 16}, {1, 5, 32, 24},
                              {0, 5, 16, 32}, {0, 1, 2, 48},  {0, 1, 32, 1},  {0, 5, 16, 80}, {2, 5, 16, 96},
                              {0, 5, 8, 40},  {2, 5, 16, 48}, {2, 5, 1, 81}};
-
-template <int MODE, int KS, int COT, int CIC>
-cudaError_t run_t1(const T1Job* jobs, int n, int gx, int gy, int Ci, int Co, const float* w, const float* b, int act,
-                   float scale, cudaStream_t st) {
-  const int groups = (Co + COT - 1) / COT;
-  t1_conv_kernel<MODE, KS, COT, CIC><<<dim3(gx, gy, n * groups), dim3(kTW, kTH), 0, st>>>(jobs, groups, w, b, Ci, Co,
-                                                                                        act, scale);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_t1_layer(int l, const T1Job* jobs, int n, int maxHo, int maxWo, const float* w, const float* b,
-                            cudaStream_t st) {
-  const T1Layer L = kT1[l];
-  const int gx = L.mode == 2 ? (maxWo + 2 * kTW - 1) / (2 * kTW) : (maxWo + kTW - 1) / kTW;
-  const int gy = L.mode == 2 ? (maxHo + 2 * kTH - 1) / (2 * kTH) : (maxHo + kTH - 1) / kTH;
-  const int act = l == 6 || l == 12 ? 0 : 1;
-  const float scale = l == 12 ? 256.0f : 1.0f;  // the output in pixels (256 Y)
-  switch (l) {
-    case 0: case 1: return run_t1<0, 5, 16, 1>(jobs, n, gx, gy, L.ci, L.co, w, b, act, scale, st);
-    case 2: case 4: return run_t1<1, 5, 16, 8>(jobs, n, gx, gy, L.ci, L.co, w, b, act, scale, st);
-    case 3: case 10: return run_t1<0, 5, 8, 8>(jobs, n, gx, gy, L.ci, L.co, w, b, act, scale, st);
-    case 5: case 8: return run_t1<0, 5, 16, 8>(jobs, n, gx, gy, L.ci, L.co, w, b, act, scale, st);
-    case 6: return run_t1<0, 1, 2, 8>(jobs, n, gx, gy, L.ci, L.co, w, b, act, scale, st);
-    case 7: return run_t1<0, 1, 16, 1>(jobs, n, gx, gy, L.ci, L.co, w, b, act, scale, st);
-    case 9: case 11: return run_t1<2, 5, 16, 8>(jobs, n, gx, gy, L.ci, L.co, w, b, act, scale, st);
-    case 12: return run_t1<2, 5, 1, 8>(jobs, n, gx, gy, L.ci, L.co, w, b, act, scale, st);
-  }
-  return cudaErrorInvalidValue;
-}
 
 }  // namespace
 
@@ -240,6 +119,18 @@ static size_t t1_w_off(int l) {
   return o;
 }
 
+// Packed weights of the 5 x 5 layers (the 1 x 1 layers 6 and 7 read the parameters).
+void t1_plan_layers(F32Layer* layers, std::vector<F32PackDesc>& descs, size_t& total) {
+  for (int l = 0; l < 12; ++l) {
+    if (l == 6 || l == 7) continue;
+    const int kind = kT1[l].mode == 0 ? FK_S1_5 : kT1[l].mode == 1 ? FK_S2_5 : FK_DE5;
+    const F32Src src{t1_w_off(l), 5, kT1[l].co, kT1[l].ci};
+    layers[l] = f32_plan_layer(kind, &src, 1, descs, total);
+  }
+  const int ic[4] = {16, 1, 32, 32};
+  layers[12] = f32_plan_y5(t1_w_off(12), ic, 4, descs, total);
+}
+
 // Forward pass of the Table I network for n pairs.  coarse_i / coarse_f: per pair coarse map
 // (one of them); eps (nullable): per pair [H8][W8] noise; Y: per pair H x W disparity in
 // pixels; mu / sigma (nullable arrays): per pair [H8][W8].
@@ -247,8 +138,8 @@ sv_status Ctx::t1_forward(const sv_pair* pairs, int n, const int16_t* const* coa
                           const float* const* eps, float* const* Y, float* const* mu, float* const* sigma,
                           cudaStream_t st) {
   if (n == 0) return SV_OK;
-  // per pair activation sizes (floats): X0, X1, FE1, FE2, EN1, EN1R, EN2, EN2R, heads, g, D1, D1R, D2, D2R, D
-  std::vector<std::array<size_t, 15>> off(n);
+  // per pair activation sizes (floats): X0, X1, FE1, FE2, EN1, EN1R, EN2, EN2R, D1, D1R, D2, D2R, D
+  std::vector<std::array<size_t, 13>> off(n);
   size_t total = 0;
   int maxH[4] = {0, 0, 0, 0}, maxW[4] = {0, 0, 0, 0};
   for (int i = 0; i < n; ++i) {
@@ -258,20 +149,20 @@ sv_status Ctx::t1_forward(const sv_pair* pairs, int n, const int16_t* const* coa
       maxW[k] = std::max(maxW[k], lv.W[k]);
     }
     const size_t P2 = (size_t)lv.H[1] * lv.W[1], P4 = (size_t)lv.H[2] * lv.W[2], P8 = (size_t)lv.H[3] * lv.W[3];
-    const size_t sz[15] = {P2, P2, P2 * 32, P2 * 32, P4 * 16, P4 * 8, P8 * 32, P8 * 16, P8 * 2, P8,
+    const size_t sz[13] = {P2, P2, P2 * 32, P2 * 32, P4 * 16, P4 * 8, P8 * 32, P8 * 16,
                            P8 * 32, P8 * 16, P4 * 16, P4 * 8, P2 * 16};
-    for (int k = 0; k < 15; ++k) {
+    for (int k = 0; k < 13; ++k) {
       off[i][k] = total;
       total += (sz[k] + 31) / 32 * 32;  // 128-byte aligned tensors
     }
   }
   sv_status s;
   if ((s = cuda(t1_act.ensure(total * sizeof(float)), "alloc Table I activations"))) return s;
-  const size_t io_bytes = sizeof(T1PairIO) * n, job_bytes = sizeof(T1Job) * n * 13;
+  const size_t io_bytes = sizeof(T1PairIO) * n, job_bytes = sizeof(F32Job) * n * 13;
   if ((s = cuda(t1_tab.ensure(io_bytes + job_bytes), "alloc Table I tables"))) return s;
   std::vector<unsigned char> host(io_bytes + job_bytes);
   T1PairIO* io = reinterpret_cast<T1PairIO*>(host.data());
-  T1Job* jobs = reinterpret_cast<T1Job*>(host.data() + io_bytes);
+  F32Job* jobs = reinterpret_cast<F32Job*>(host.data() + io_bytes);
   float* A = (float*)t1_act.p;
   for (int i = 0; i < n; ++i) {
     const sv_pair& p = pairs[i];
@@ -289,21 +180,22 @@ sv_status Ctx::t1_forward(const sv_pair* pairs, int n, const int16_t* const* coa
     q.coarse_f = coarse_f ? coarse_f[i] : nullptr;
     q.X0 = T(0);
     q.X1 = T(1);
-    q.heads = T(8);
+    q.en2 = T(6);
+    q.en2r = T(7);
     q.eps = eps ? eps[i] : nullptr;
-    q.g = T(9);
+    q.d1 = T(8);
     q.mu = mu ? mu[i] : nullptr;
     q.sigma = sigma ? sigma[i] : nullptr;
     q.H8 = lv.H[3];
     q.W8 = lv.W[3];
     // layer l of pair i: sources (concatenated in Table I's order), sizes, output
     auto job = [&](int l, std::initializer_list<std::pair<int, int>> srcs, int lin, int lout, float* out) {
-      T1Job& j = jobs[l * n + i];
-      j = T1Job{};
+      F32Job& j = jobs[l * n + i];
+      j = F32Job{};
       int k = 0;
       for (auto& sc : srcs) {
-        j.src.p[k] = T(sc.first);
-        j.src.c[k] = sc.second;
+        j.in[k] = T(sc.first);
+        j.ic[k] = sc.second;
         ++k;
       }
       j.Hi = lv.H[lin];
@@ -318,41 +210,44 @@ sv_status Ctx::t1_forward(const sv_pair* pairs, int n, const int16_t* const* coa
     job(3, {{4, 16}}, 2, 2, T(5));                            // EN_1_R <- EN_1
     job(4, {{4, 16}, {5, 8}}, 2, 3, T(6));                    // EN_2 <- EN_1 & EN_1_R
     job(5, {{6, 32}}, 3, 3, T(7));                            // EN_2_R <- EN_2
-    job(6, {{6, 32}, {7, 16}}, 3, 3, T(8));                   // heads <- EN_2 & EN_2_R
-    job(7, {{9, 1}}, 3, 3, T(10));                            // D_1 <- gaussian
-    job(8, {{10, 32}, {6, 32}, {7, 16}}, 3, 3, T(11));        // D_1_R <- D_1 & EN_2 & EN_2_R
-    job(9, {{10, 32}, {6, 32}, {7, 16}, {11, 16}}, 3, 2, T(12));  // D_2 <- D_1 & EN_2 & EN_2_R & D_1_R
-    job(10, {{12, 16}, {4, 16}, {5, 8}}, 2, 2, T(13));        // D_2_R <- D_2 & EN_1 & EN_1_R
-    job(11, {{12, 16}, {4, 16}, {5, 8}, {13, 8}}, 2, 1, T(14));  // D <- D_2 & EN_1 & EN_1_R & D_2_R
-    job(12, {{14, 16}, {0, 1}, {2, 32}, {3, 32}}, 1, 0, Y[i]);   // Y <- D & X_0 & FE_1 & FE_2
+    job(8, {{8, 32}, {6, 32}, {7, 16}}, 3, 3, T(9));             // D_1_R <- D_1 & EN_2 & EN_2_R
+    job(9, {{8, 32}, {6, 32}, {7, 16}, {9, 16}}, 3, 2, T(10));   // D_2 <- D_1 & EN_2 & EN_2_R & D_1_R
+    job(10, {{10, 16}, {4, 16}, {5, 8}}, 2, 2, T(11));           // D_2_R <- D_2 & EN_1 & EN_1_R
+    job(11, {{10, 16}, {4, 16}, {5, 8}, {11, 8}}, 2, 1, T(12));  // D <- D_2 & EN_1 & EN_1_R & D_2_R
+    job(12, {{12, 16}, {0, 1}, {2, 32}, {3, 32}}, 1, 0, Y[i]);   // Y <- D & X_0 & FE_1 & FE_2
   }
   if ((s = cuda(cudaMemcpyAsync(t1_tab.p, host.data(), host.size(), cudaMemcpyHostToDevice, st),
                 "upload Table I tables")))
     return s;
   const T1PairIO* d_io = (const T1PairIO*)t1_tab.p;
-  const T1Job* d_jobs = (const T1Job*)((unsigned char*)t1_tab.p + io_bytes);
+  const F32Job* d_jobs = (const F32Job*)((unsigned char*)t1_tab.p + io_bytes);
   const float* W = (const float*)w32.p;
   {
     LaunchScope ls(*this, "t1_inputs", st);
     t1_inputs_kernel<<<dim3((maxW[1] + 127) / 128, maxH[1], n), 128, 0, st>>>(d_io);
     if ((s = cuda(cudaGetLastError(), "Table I inputs"))) return s;
   }
-  static const char* names[13] = {"t1_fe1", "t1_fe2", "t1_en1", "t1_en1r", "t1_en2", "t1_en2r", "t1_heads",
-                                  "t1_d1", "t1_d1r", "t1_d2", "t1_d2r", "t1_d", "t1_y"};
+  static const char* names[13] = {"t1_fe1", "t1_fe2", "t1_en1", "t1_en1r", "t1_en2", "t1_en2r", "t1_latent",
+                                  "", "t1_d1r", "t1_d2", "t1_d2r", "t1_d", "t1_y"};
   static const int out_level[13] = {1, 1, 2, 2, 3, 3, 3, 3, 3, 2, 2, 1, 0};
+  const float* P = (const float*)f32_w.p;
+  auto B = [&](int l) { return W + t1_w_off(l) + (size_t)kT1[l].co * kT1[l].ks * kT1[l].ks * kT1[l].ci; };
   for (int l = 0; l < 13; ++l) {
-    if (l == 7) {
-      LaunchScope ls(*this, "t1_gauss", st);
-      t1_gauss_kernel<<<dim3((maxH[3] * maxW[3] + 255) / 256, n), 256, 0, st>>>(d_io);
-      if ((s = cuda(cudaGetLastError(), "Table I reparameterisation"))) return s;
-    }
+    if (l == 7) continue;  // D_1 is part of the latent kernel
     LaunchScope ls(*this, names[l], st);
-    const size_t wo = t1_w_off(l);
-    const size_t bo = wo + (size_t)kT1[l].co * kT1[l].ks * kT1[l].ks * kT1[l].ci;
-    if ((s = cuda(launch_t1_layer(l, d_jobs + (size_t)l * n, n, maxH[out_level[l]], maxW[out_level[l]], W + wo, W + bo,
-                                  st),
-                  names[l])))
-      return s;
+    cudaError_t e;
+    const F32Job* J = d_jobs + (size_t)l * n;
+    const int mH = maxH[out_level[l]], mW = maxW[out_level[l]];
+    if (l == 6) {
+      t1_latent_kernel<<<dim3((maxH[3] * maxW[3] + kLatThreads - 1) / kLatThreads, n), kLatThreads, 0, st>>>(
+          d_io, W + t1_w_off(6), B(6), W + t1_w_off(7), B(7));
+      e = cudaGetLastError();
+    } else if (l == 12) {
+      e = launch_f32_y5(t1_l[12], J, n, mH, mW, P, B(12), 256.0f, st);  // the output in pixels (256 Y)
+    } else {
+      e = launch_f32_conv(t1_l[l], J, n, mH, mW, P, B(l), 2, st);
+    }
+    if ((s = cuda(e, names[l]))) return s;
   }
   return SV_OK;
 }

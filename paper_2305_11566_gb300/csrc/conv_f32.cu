@@ -12,10 +12,9 @@
 // 1242 x 375, 32/64/128 net: 22.1 -> 3.8 ms (dec2 at 51, dec1 at 45 TFLOP/s of 80 on the FP32 pipes).
 //
 // Nearest-x2 layers run as four output phases of 2x2 taps (2.25x fewer multiply-adds than the
-// 3x3 window on the upsampled grid), their input gradient as 4x4 taps instead of 36.  Where an
-// odd size crops the last upsampled row or column, the summed weights hold one kernel row or
-// column too many there: tiles that touch that edge run the unsummed 3x3 taps with the cropped
-// taps left out.
+// 3x3 window on the upsampled grid).  Where an odd size crops the last upsampled row or column, the
+// summed weights hold one kernel row or column too many there: tiles that touch that edge run the
+// unsummed 3x3 taps with the cropped taps left out.
 #include "conv_f32.cuh"
 
 #include <algorithm>
@@ -62,14 +61,14 @@ template <> struct Kind<FK_S2> { static constexpr int TY = 3, TX = 3, S = 2, PH 
 template <> struct Kind<FK_P1> { static constexpr int TY = 1, TX = 1, S = 1, PH = 1, BT = 0; };
 template <> struct Kind<FK_UP2> { static constexpr int TY = 2, TX = 2, S = 1, PH = 4, BT = 9; };
 template <> struct Kind<FK_DS2> { static constexpr int TY = 2, TX = 2, S = 1, PH = 4, BT = 0; };
-template <> struct Kind<FK_DUP2> { static constexpr int TY = 4, TX = 4, S = 2, PH = 1, BT = 9; };
+template <> struct Kind<FK_DUP2> { static constexpr int TY = 3, TX = 3, S = 2, PH = 1, BT = 0; };
 template <> struct Kind<FK_S1_5> { static constexpr int TY = 5, TX = 5, S = 1, PH = 1, BT = 0; };
 template <> struct Kind<FK_S2_5> { static constexpr int TY = 5, TX = 5, S = 2, PH = 1, BT = 0; };
 template <> struct Kind<FK_DE5> { static constexpr int TY = 3, TX = 3, S = 1, PH = 4, BT = 0; };
 template <> struct Kind<FK_UP2X> { static constexpr int TY = 3, TX = 3, S = 1, PH = 1, BT = 0; };
 
 // Channels staged per step: kinds with a large stride-2 patch stage fewer.
-constexpr int kind_cic(int kind) { return kind == FK_P1 ? 16 : kind == FK_DUP2 || kind == FK_S1_5 || kind == FK_S2_5 ? 4 : 8; }
+constexpr int kind_cic(int kind) { return kind == FK_P1 ? 16 : kind == FK_S1_5 || kind == FK_S2_5 ? 4 : 8; }
 
 constexpr int imax(int a, int b) { return a > b ? a : b; }
 
@@ -106,6 +105,19 @@ struct Geo<FK_S2, CG_, CIC_> {
   static constexpr bool SPLIT = true;
 };
 
+// FK_DUP2: columns 2x - 1 .. 2x + 2 of the upsampled grid, split by parity, in one buffer.
+template <int CG_, int CIC_>
+struct Geo<FK_DUP2, CG_, CIC_> {
+  static constexpr int CG = CG_, CIC = CIC_, BN = 8 * CG, S = 2;
+  static constexpr int TW = CG >= 4 ? 16 : 32, GX = TW / PX, TH = kThreads / CG / GX;
+  static constexpr int PR = 2 * TH + 2, PC = 2 * TW + 2;
+  static constexpr int EVEN = TW + 4, PITCH = 2 * EVEN;
+  static constexpr int PLANE = (PR * PITCH + 31 - 4) / 32 * 32 + 4;
+  static constexpr int BUF = CIC * PLANE + 9 * CIC * BN, NBUF = 1;
+  static constexpr size_t SMEM = sizeof(float) * BUF;
+  static constexpr bool SPLIT = true;
+};
+
 // FK_UP2X: the patch holds the input pixels under the tile, (TH / 2 + 2) x (TW / 2 + 2); column 0 sits
 // at offset 3, so that a thread's four input pixels are one aligned vector.
 template <int CG_, int CIC_>
@@ -125,6 +137,7 @@ struct F32Args {
   size_t w[4], wb;
   const float* bias;
   int K, N, nb, tiles_x, act;
+  int accumulate;  // 1: added to the output
   int bias_first;  // 1: the sum starts at the bias (else the bias is added to it)
 };
 
@@ -244,39 +257,41 @@ struct UpEdge {
   }
 };
 
-// Edge form of FK_DUP2: input pixel (y, x) gathers the upsampled positions (2y + a, 2x + b); the
-// last row's a = 1 and the last column's b = 1 are cropped away when the grid is odd.
-template <class G>
-struct DupEdge {
-  static constexpr int PR = G::PR, PC = G::PC, TAPS = 9;
-  int drop;
-  bool last_row;
-  __device__ __forceinline__ void operator()(u64 (&acc)[PX][4], const float* pa, const float* pw) const {
-    constexpr int NV = G::NV, WS = G::CIC * G::BN;
-#pragma unroll 1
-    for (int ci = 0; ci < G::CIC; ++ci, pa += G::PLANE, pw += G::BN)
-#pragma unroll 1
-      for (int ak = 0; ak < 6; ++ak) {
-        const int a_ = ak / 3, ky = ak - 3 * a_;
-        if (a_ == 1 && last_row) continue;
-        float a[4 * NV];
-        load_row<G, NV>(pa + (a_ + 2 - ky) * G::PITCH, a);
-        const float* w = pw + ky * 3 * WS;
-        tap<G, 2>(acc, a, w);
-        tap<G, 1>(acc, a, w + WS);
-        tap<G, 0>(acc, a, w + 2 * WS);
-        tap_but<G, 3>(acc, a, w, drop);
-        tap_but<G, 2>(acc, a, w + WS, drop);
-        tap_but<G, 1>(acc, a, w + 2 * WS, drop);
-      }
+// The training step keeps one summation order, whatever tile computes it: FK_S2 and FK_UP2X kernel
+// row, kernel column, channel within a step of 8 channels; FK_DUP2 the four upsampled positions of an
+// input pixel, then the same; FK_DS2 the same over the taps a phase has.  A reordered sum flips a few
+// ReLUs, after one Adam step (whose update is +-lr for every weight) also through the weights, and
+// moves an FP32 gradient by up to 1e-4 of its norm on small batches; in this order the step gives the
+// same bits as one thread per pixel does.  So these kinds run the unsummed nine taps (dec2 of 8 pairs of
+// 256 x 128: 229 us against 105 us for the summed 2x2 form, which inference uses).
+template <class G, int OFS>
+__device__ __forceinline__ void tap_unit(u64 (&acc)[PX][4], const float* a, const float* w) {
+  const ulonglong2 w0 = *reinterpret_cast<const ulonglong2*>(w);
+  const ulonglong2 w1 = *reinterpret_cast<const ulonglong2*>(w + G::BN / 2);
+#pragma unroll
+  for (int p = 0; p < PX; ++p) {
+    const u64 v = dup2(a[p + OFS]);
+    fma2(acc[p][0], v, w0.x);
+    fma2(acc[p][1], v, w0.y);
+    fma2(acc[p][2], v, w1.x);
+    fma2(acc[p][3], v, w1.y);
   }
-};
+}
+// All channels of a step for one tap; drop: position left out (EDGE tiles).
+template <class G, int OFS, int NV, bool EDGE = false>
+__device__ __forceinline__ void columns(u64 (&acc)[PX][4], const float* pa, const float* w, int drop = -1) {
+#pragma unroll 2
+  for (int ci = 0; ci < G::CIC; ++ci) {
+    float a[4 * NV];
+    load_row<G, NV>(pa + ci * G::PLANE, a);
+    if constexpr (EDGE) {
+#pragma unroll
+      for (int p = 0; p < PX; ++p) a[p + OFS] = p == drop ? 0.f : a[p + OFS];
+    }
+    tap_unit<G, OFS>(acc, a, w + ci * G::BN);
+  }
+}
 
-// FK_S2 and FK_UP2X sum in the order kernel row, kernel column, channel within a step of 8
-// channels, so that the training forward gives the same activation bits whatever tile computes them
-// (a ReLU that flips by a reordered sum moves an FP32 gradient by up to 1e-4 of its norm on small
-// batches).  The training decoder therefore keeps the nine unsummed taps: 229 us for dec2 of 8 pairs of
-// 256 x 128 against 105 us folded, which inference uses.
 template <class G>
 struct OrderedS2 {
   static constexpr int PR = G::PR, PC = G::PC, TAPS = 9;
@@ -284,27 +299,53 @@ struct OrderedS2 {
     constexpr int WS = G::CIC * G::BN;
 #pragma unroll 1
     for (int ky = 0; ky < 3; ++ky, pa += G::PITCH, pw += 3 * WS) {
-#pragma unroll 2
-      for (int ci = 0; ci < G::CIC; ++ci) column<0, 2>(acc, pa + ci * G::PLANE, pw + ci * G::BN);
-#pragma unroll 2
-      for (int ci = 0; ci < G::CIC; ++ci) column<0, 2>(acc, pa + G::EVEN + ci * G::PLANE, pw + WS + ci * G::BN);
-#pragma unroll 2
-      for (int ci = 0; ci < G::CIC; ++ci) column<1, 3>(acc, pa + ci * G::PLANE, pw + 2 * WS + ci * G::BN);
+      columns<G, 0, 2>(acc, pa, pw);
+      columns<G, 0, 2>(acc, pa + G::EVEN, pw + WS);
+      columns<G, 1, 3>(acc, pa, pw + 2 * WS);
     }
   }
-  template <int OFS, int NV>
-  __device__ __forceinline__ void column(u64 (&acc)[PX][4], const float* pa, const float* w) const {
-    float a[4 * NV];
-    load_row<G, NV>(pa, a);
-    const ulonglong2 w0 = *reinterpret_cast<const ulonglong2*>(w);
-    const ulonglong2 w1 = *reinterpret_cast<const ulonglong2*>(w + G::BN / 2);
+};
+
+// FK_DUP2: input pixel (y, x) gathers the upsampled positions (2y + a, 2x + b) through the taps: row
+// 2y + a + 1 - ky, column 2x + b + 1 - kx.  The last row's a = 1 and the last column's b = 1 are cropped
+// away when the grid is odd.
+template <class G, bool EDGE>
+struct OrderedDup {
+  static constexpr int PR = G::PR, PC = G::PC, TAPS = 9;
+  int na, drop;  // na: 1 where a = 1 is cropped
+  __device__ __forceinline__ void operator()(u64 (&acc)[PX][4], const float* pa, const float* pw) const {
+    constexpr int WS = G::CIC * G::BN;
+#pragma unroll 1
+    for (int a = 0; a < (EDGE ? na : 2); ++a) {
+      const float* p = pa + (a + 2) * G::PITCH;
+#pragma unroll 1
+      for (int ky = 0; ky < 3; ++ky) {
+        const float *q = p - ky * G::PITCH, *w = pw + ky * 3 * WS;
+        columns<G, 1, 3>(acc, q, w);
+        columns<G, 0, 2>(acc, q + G::EVEN, w + WS);
+        columns<G, 0, 2>(acc, q, w + 2 * WS);
+      }
+#pragma unroll 1
+      for (int ky = 0; ky < 3; ++ky) {
+        const float *q = p - ky * G::PITCH, *w = pw + ky * 3 * WS;
+        columns<G, 1, 3, EDGE>(acc, q + G::EVEN, w, drop);
+        columns<G, 1, 3, EDGE>(acc, q, w + WS, drop);
+        columns<G, 0, 2, EDGE>(acc, q + G::EVEN, w + 2 * WS, drop);
+      }
+    }
+  }
+};
+
+// FK_DS2: window taps from the last to the first (kernel rows and columns ascending).
+template <class G, int TY, int TX>
+struct OrderedDs {
+  static constexpr int PR = G::TH - 1 + TY, PC = G::TW - 1 + TX, TAPS = TY * TX;
+  __device__ __forceinline__ void operator()(u64 (&acc)[PX][4], const float* pa, const float* pw) const {
+    constexpr int WS = G::CIC * G::BN;
 #pragma unroll
-    for (int p = 0; p < PX; ++p) {
-      const u64 v = dup2(a[p + OFS]);
-      fma2(acc[p][0], v, w0.x);
-      fma2(acc[p][1], v, w0.y);
-      fma2(acc[p][2], v, w1.x);
-      fma2(acc[p][3], v, w1.y);
+    for (int r = TY - 1; r >= 0; --r) {
+      if (TX == 2) columns<G, 1, 3>(acc, pa + r * G::PITCH, pw + (r * TX + 1) * WS);
+      columns<G, 0, 2>(acc, pa + r * G::PITCH, pw + r * TX * WS);
     }
   }
 };
@@ -444,14 +485,14 @@ __global__ void __launch_bounds__(kThreads, 4) f32_conv_kernel(const F32Job* __r
   } else if constexpr (KIND == FK_DUP2) {
     const bool er = (J.Hi & 1) && Y0 + G::TH >= GH, ec = (J.Wi & 1) && X0 + G::TW >= GW;
     if (er || ec)
-      run(DupEdge<G>{ec ? GW - 1 - xb : -1, er && y == GH - 1}, A.packed + A.wb, -1, -1);
+      run(OrderedDup<G, true>{er && y == GH - 1 ? 1 : 2, ec ? GW - 1 - xb : -1}, wm, -1, -1);
     else
-      run(Window<G, 4, 4>{}, wm, -1, -1);
+      run(OrderedDup<G, false>{2, -1}, wm, -1, -1);
   } else if constexpr (KIND == FK_DS2) {
-    if (phase == 0) run(Window<G, 1, 1>{}, wm, 0, 0);
-    else if (phase == 1) run(Window<G, 1, 2>{}, wm, 0, 0);
-    else if (phase == 2) run(Window<G, 2, 1>{}, wm, 0, 0);
-    else run(Window<G, 2, 2>{}, wm, 0, 0);
+    if (phase == 0) run(OrderedDs<G, 1, 1>{}, wm, 0, 0);
+    else if (phase == 1) run(OrderedDs<G, 1, 2>{}, wm, 0, 0);
+    else if (phase == 2) run(OrderedDs<G, 2, 1>{}, wm, 0, 0);
+    else run(OrderedDs<G, 2, 2>{}, wm, 0, 0);
   } else if constexpr (KIND == FK_DE5) {
     if (phase == 0) run(Window<G, 3, 3>{}, wm, -1, -1);
     else if (phase == 1) run(Window<G, 3, 2>{}, wm, -1, 0);
@@ -481,6 +522,10 @@ __global__ void __launch_bounds__(kThreads, 4) f32_conv_kernel(const F32Job* __r
         f.z = m.z > 0.f ? f.z : 0.f;
         f.w = m.w > 0.f ? f.w : 0.f;
       }
+      if (KIND == FK_P1 && A.accumulate) {
+        const float4 g = *reinterpret_cast<const float4*>(J.out + oo);
+        f = make_float4(g.x + f.x, g.y + f.y, g.z + f.z, g.w + f.w);
+      }
       *reinterpret_cast<float4*>(J.out + oo) = f;
     }
   }
@@ -491,7 +536,7 @@ cudaError_t run_conv(const F32Layer& l, const F32Job* jobs, int n, int maxHo, in
                      const float* bias, int act, cudaStream_t st) {
   using G = Geo<KIND, CG, CIC>;
   constexpr int PH = Kind<KIND>::PH, OS = PH == 4 ? 2 : 1;
-  F32Args a{packed, {l.w[0], l.w[1], l.w[2], l.w[3]}, l.wb, bias, l.K, l.N, l.N / G::BN, 0, act & 3, act & 4 ? 1 : 0};
+  F32Args a{packed, {l.w[0], l.w[1], l.w[2], l.w[3]}, l.wb, bias, l.K, l.N, l.N / G::BN, 0, act & 3, act & 8 ? 1 : 0, act & 4 ? 1 : 0};
   a.tiles_x = ((maxWo + OS - 1) / OS + G::TW - 1) / G::TW;
   const int tiles_y = ((maxHo + OS - 1) / OS + G::TH - 1) / G::TH;
   auto kern = f32_conv_kernel<KIND, CG, CIC>;
@@ -530,29 +575,22 @@ __global__ void f32_pack_kernel(const F32PackDesc* __restrict__ descs, const flo
       // one source of the last layer: output "channel" n is phase (n >> 1, n & 1)
       const int ky = ((n >> 1) ? 3 : 4) - 2 * (r - (n >> 1)), kx = ((n & 1) ? 3 : 4) - 2 * (c - (n & 1));
       if (k < D.co && ky >= 0 && ky <= 4 && kx >= 0 && kx <= 4) v = params[D.src + (ky * 5 + kx) * D.ci + D.N + k];
-    } else if (D.border) {
-      v = D.kind == FK_DUP2 ? W(k, r, c, nn) : W(nn, r, c, k);
-    } else if (D.kind == FK_UP2) {
+    } else if (D.kind == FK_UP2 && !D.border) {
       for (int ky = 0; ky < 3; ++ky)
         for (int kx = 0; kx < 3; ++kx)
           if (((ky + 1 - py) >> 1) == r && ((kx + 1 - px) >> 1) == c) v += W(nn, ky, kx, k);
     } else if (D.kind == FK_DUP2) {
-      for (int a = 0; a < 2; ++a)
-        for (int b = 0; b < 2; ++b) {
-          const int ky = a + 2 - r, kx = b + 2 - c;
-          if (ky >= 0 && ky < 3 && kx >= 0 && kx < 3) v += W(k, ky, kx, nn);
-        }
+      v = W(k, r, c, nn);
     } else if (D.kind == FK_DS2) {
       v = W(k, py ? 2 - 2 * r : 1, px ? 2 - 2 * c : 1, nn);
     } else if (D.kind == FK_DE5) {
       v = W(nn, (py ? 3 : 4) - 2 * r, (px ? 3 : 4) - 2 * c, k);
-    } else if (D.kind == FK_P1 && D.border == 0 && D.phase == 1) {  // gradient of a 1x1: transposed
+    } else if (D.kind == FK_P1 && D.phase == 1) {  // gradient of a 1x1: transposed
       v = W(k, 0, 0, nn);
     } else {
       v = W(nn, r, c, k);
     }
-    const size_t blk = (size_t)nblk * (D.Ktot / D.cic) + D.k0 / D.cic + chunk;
-    packed[D.dst + ((blk * D.taps + t) * D.cic + ci) * D.bn + n] = v;
+    packed[D.dst + i] = v;
   }
 }
 
@@ -699,6 +737,60 @@ f32_final_kernel(const F32Img* __restrict__ imgs, const float* __restrict__ w, c
   }
 }
 
+// The final conv of the training forward: the same layer summed in the training step's order
+// (8 channels a step; kernel row, kernel column, channel).  A thread owns 8 consecutive pixels and holds
+// a kernel row's 8 channels of them in registers; 32 x 32 pixels a block.
+struct FinalGeo {
+  static constexpr int CIC = 8, TW = 32, TH = 32, S = 1, PR = 34, PC = 34, PITCH = 36;
+  static constexpr int PLANE = (PR * PITCH + 31 - 4) / 32 * 32 + 4;
+  static constexpr bool SPLIT = false;
+  static constexpr int EVEN = 0;
+};
+__global__ void __launch_bounds__(kThreads, 4)
+f32_final_ordered_kernel(const F32Img* __restrict__ imgs, const float* __restrict__ w, const float* __restrict__ b,
+                         int C, int tiles_x) {
+  using G = FinalGeo;
+  __shared__ __align__(16) float sm[G::CIC * G::PLANE];
+  __shared__ float ws[9 * G::CIC];  // [tap][channel]
+  const F32Img& I = imgs[blockIdx.z];
+  const int Y0 = (blockIdx.x / tiles_x) * G::TH, X0 = (blockIdx.x % tiles_x) * G::TW;
+  if (Y0 >= I.H || X0 >= I.W) return;
+  const int gx = threadIdx.x % 4, row = threadIdx.x / 4;
+  float acc[PX];
+#pragma unroll
+  for (int p = 0; p < PX; ++p) acc[p] = 0.f;
+  for (int c0 = 0; c0 < C; c0 += G::CIC) {
+    __syncthreads();
+    load_patch<G, G::PR, G::PC>(sm, I.d3 + c0, C, Y0 - 1, X0 - 1, I.H, I.W);
+    cp_commit();
+    if (threadIdx.x < 9 * G::CIC) ws[threadIdx.x] = w[(threadIdx.x / G::CIC) * C + c0 + threadIdx.x % G::CIC];
+    cp_wait<0>();
+    __syncthreads();
+#pragma unroll 1
+    for (int ky = 0; ky < 3; ++ky) {
+      float a[G::CIC][12];
+#pragma unroll
+      for (int ci = 0; ci < G::CIC; ++ci) load_row<G, 3>(sm + ci * G::PLANE + (row + ky) * G::PITCH + gx * PX, a[ci]);
+#pragma unroll
+      for (int kx = 0; kx < 3; ++kx)
+#pragma unroll
+        for (int ci = 0; ci < G::CIC; ++ci) {
+          const float k = ws[(ky * 3 + kx) * G::CIC + ci];
+#pragma unroll
+          for (int p = 0; p < PX; ++p) acc[p] = fmaf(k, a[ci][p + kx], acc[p]);
+        }
+    }
+  }
+  const int y = Y0 + row;
+  if (y >= I.H) return;
+#pragma unroll
+  for (int p = 0; p < PX; ++p) {
+    const int x = X0 + gx * PX + p;
+    if (x >= I.W) break;
+    I.Y[(size_t)y * I.W + x] = upsample4_f(I.coarse_f, I.w, I.h, x, y) + (b[0] + acc[p]);
+  }
+}
+
 // FK_Y5: a thread owns 8 input positions along x and their four output phases; the phase pair
 // py = 1 has no tap in window row 0.  Channels go 4 a step (a one-channel source fills its step
 // with zeros); the packed weights are [step][tap][channel][phase].
@@ -823,17 +915,16 @@ cudaError_t launch_f32_reparam(const F32Lat* lat, int n, size_t max_n, cudaStrea
   return cudaGetLastError();
 }
 
-F32Layer f32_plan_layer(int kind, const F32Src* src, int n_src, std::vector<F32PackDesc>& descs, size_t& total) {
-  const bool grad = kind == FK_DS2 || kind == FK_DUP2 || (kind == FK_P1 && n_src > 1);
+F32Layer f32_plan_layer(int kind, bool grad, const F32Src& src, std::vector<F32PackDesc>& descs, size_t& total) {
   F32Layer l;
   l.kind = kind;
-  l.N = grad ? src[0].ci : src[0].co;
-  for (int i = 0; i < n_src; ++i) l.K += grad ? src[i].co : src[i].ci;
+  l.N = grad ? src.ci : src.co;
+  l.K = grad ? src.co : src.ci;
   l.cg = l.N % 64 == 0 ? 8 : l.N % 32 == 0 ? 4 : l.N % 16 == 0 ? 2 : 1;
   const int cic = std::min(kind_cic(kind), l.K), bn = 8 * l.cg;
   const int phases = kind == FK_UP2 || kind == FK_DS2 || kind == FK_DE5 ? 4 : 1;
-  static const int ty0[FK_COUNT] = {3, 1, 2, 1, 4, 5, 5, 3, 3};
-  const bool edge = kind == FK_UP2 || kind == FK_DUP2;
+  static const int ty0[FK_COUNT] = {3, 1, 2, 1, 3, 5, 5, 3, 3};
+  const bool edge = kind == FK_UP2;
   for (int ph = 0; ph < phases + (edge ? 1 : 0); ++ph) {
     const bool border = ph == phases;
     const int py = ph >> 1, px = ph & 1;
@@ -842,29 +933,23 @@ F32Layer f32_plan_layer(int kind, const F32Src* src, int n_src, std::vector<F32P
     if (kind == FK_DE5) { ty = 3 - py; tx = 3 - px; }
     if (border) ty = tx = 3;
     (border ? l.wb : l.w[ph]) = total;
-    int k0 = 0;
-    for (int i = 0; i < n_src; ++i) {
-      F32PackDesc d{};
-      d.src = src[i].w_ofs;
-      d.dst = total;
-      d.kind = kind;
-      d.phase = kind == FK_P1 ? (grad ? 1 : 0) : (border ? 0 : ph);
-      d.border = border;
-      d.ks = src[i].ks;
-      d.co = src[i].co;
-      d.ci = src[i].ci;
-      d.K = grad ? src[i].co : src[i].ci;
-      d.N = l.N;
-      d.Ktot = l.K;
-      d.k0 = k0;
-      d.cic = cic;
-      d.bn = bn;
-      d.taps = ty * tx;
-      d.tx = tx;
-      d.count = (size_t)d.K * d.N * d.taps;
-      k0 += d.K;
-      descs.push_back(d);
-    }
+    F32PackDesc d{};
+    d.src = src.w_ofs;
+    d.dst = total;
+    d.kind = kind;
+    d.phase = kind == FK_P1 ? (grad ? 1 : 0) : (border ? 0 : ph);
+    d.border = border;
+    d.ks = src.ks;
+    d.co = src.co;
+    d.ci = src.ci;
+    d.K = l.K;
+    d.N = l.N;
+    d.cic = cic;
+    d.bn = bn;
+    d.taps = ty * tx;
+    d.tx = tx;
+    d.count = (size_t)l.K * l.N * d.taps;
+    descs.push_back(d);
     total += (size_t)l.K * l.N * ty * tx;
   }
   return l;
@@ -887,7 +972,7 @@ F32Layer f32_plan_y5(size_t w_ofs, const int* ic, int n_ic, std::vector<F32PackD
     d.ci = channels;  // channels of the layer
     d.N = c0;         // first channel of this source
     d.cic = Y5Geo::CIC;
-    d.K = d.Ktot = (ic[i] + d.cic - 1) / d.cic * d.cic;
+    d.K = (ic[i] + d.cic - 1) / d.cic * d.cic;
     d.bn = 4;
     d.taps = 9;
     d.tx = 3;
@@ -949,7 +1034,12 @@ cudaError_t launch_f32_enc1(const F32Img* imgs, int n, int maxH1, int maxW1, con
 }
 
 cudaError_t launch_f32_final(const F32Img* imgs, int n, int maxH, int maxW, const float* w, const float* b, int C,
-                             cudaStream_t st) {
+                             bool ordered, cudaStream_t st) {
+  if (ordered) {
+    const int tx = (maxW + FinalGeo::TW - 1) / FinalGeo::TW, ty = (maxH + FinalGeo::TH - 1) / FinalGeo::TH;
+    f32_final_ordered_kernel<<<dim3(tx * ty, 1, n), kThreads, 0, st>>>(imgs, w, b, C, tx);
+    return cudaGetLastError();
+  }
   auto go = [&](auto kern, int no) {
     const int tx = (maxW + no - 1) / no, ty = (maxH + kFinRows - 1) / kFinRows;
     kern<<<dim3(tx * ty, 1, n), 256, 0, st>>>(imgs, w, b, C, tx);

@@ -16,7 +16,7 @@ namespace sv {
 //   FK_UP2   nearest x2 + 3x3 (decoder): four output phases of 2x2 taps, the weights that
 //            fall on one input pixel summed
 //   FK_DS2   input gradient of FK_S2: four phases of 1x1, 1x2, 2x1, 2x2 taps
-//   FK_DUP2  input gradient of FK_UP2: 4x4 taps, stride 2
+//   FK_DUP2  input gradient of the nearest-x2 layer: nine taps at each of the four upsampled positions
 //   FK_S1_5, FK_S2_5  5x5 stride 1 / 2;  FK_DE5  5x5 stride-2 deconvolution: four phases of
 //            3x3, 3x2, 2x3, 2x2 taps
 //   FK_Y5    the Table I network's last layer: 5x5 stride-2 deconvolution to one channel, the four
@@ -69,8 +69,7 @@ struct F32WJob {
   const float* g;  // [Ho][Wo][Co]
   const float* x;  // [Hi][Wi][Ci]
   int Hi, Wi, Ho, Wo;
-  int tile0;       // first tile of this pair in the launch
-  int btile0;      // FK_UP2: first border tile
+  int unit0, units;  // first slot of this pair in the launch, its slots
 };
 
 // One packed weight block; see f32_pack_kernel.
@@ -79,8 +78,7 @@ struct F32PackDesc {
   size_t dst;      // offset of the block in the packed buffer
   int kind, phase, border;
   int ks, co, ci;  // of the source layer
-  int K, N;        // contraction and output channels of the packed form (source extent)
-  int Ktot, k0;    // concatenated inputs: channels of the whole contraction, first of this source
+  int K, N;        // contraction and output channels of the packed form
   int cic, bn, taps, tx;
   size_t count;
 };
@@ -91,14 +89,15 @@ struct F32Layer {
   size_t w[4] = {0, 0, 0, 0}, wb = 0;
 };
 
-// Adds the pack descriptors of a layer (one or two sources along K) to `descs` and returns its
-// launch constants; `total` is the packed buffer's size so far in floats.
+// Adds the pack descriptors of a layer (grad: its input gradient) to `descs` and returns its launch
+// constants; `total` is the packed buffer's size so far in floats.
 struct F32Src { size_t w_ofs; int ks, co, ci; };
-F32Layer f32_plan_layer(int kind, const F32Src* src, int n_src, std::vector<F32PackDesc>& descs, size_t& total);
+F32Layer f32_plan_layer(int kind, bool grad, const F32Src& src, std::vector<F32PackDesc>& descs, size_t& total);
 cudaError_t launch_f32_pack(const F32PackDesc* d_descs, int n, size_t max_count, const float* params, float* packed,
                             cudaStream_t st);
 
-// act: 0 none, 1 ReLU, 2 leaky ReLU 0.1; + 4 (FK_P1): the sums start at the bias.  maxHo / maxWo: largest output of the jobs.
+// act: 0 none, 1 ReLU, 2 leaky ReLU 0.1; + 4 (FK_P1): the sums start at the bias; + 8 (FK_P1):
+// added to the output.  maxHo / maxWo: largest output of the jobs.
 cudaError_t launch_f32_conv(const F32Layer& l, const F32Job* jobs, int n, int maxHo, int maxWo, const float* packed,
                             const float* bias, int act, cudaStream_t st);
 cudaError_t launch_f32_enc1(const F32Img* imgs, int n, int maxH1, int maxW1, const float* w, const float* b, int C,
@@ -110,26 +109,26 @@ F32Layer f32_plan_y5(size_t w_ofs, const int* ic, int n_ic, std::vector<F32PackD
 cudaError_t launch_f32_y5(const F32Layer& l, const F32Job* jobs, int n, int maxHo, int maxWo, const float* packed,
                           const float* bias, float scale, cudaStream_t st);
 cudaError_t launch_f32_convert(const F32Cvt* jobs, int n, size_t max_n, cudaStream_t st);
+// ordered: summed in the training step's order (real-valued coarse maps).
 cudaError_t launch_f32_final(const F32Img* imgs, int n, int maxH, int maxW, const float* w, const float* b, int C,
-                             cudaStream_t st);
+                             bool ordered, cudaStream_t st);
 
-// Weight gradients: plan (fills the jobs' tile offsets), slots (scratch, p.slot_floats) and launch;
+// Weight gradients: plan (fills the jobs' slot ranges), slots (scratch, p.slot_floats) and launch;
 // gw / gb are added to.
 struct F32WPlan {
-  int kind = 0, co = 0, ci = 0, cgn = 0, ign = 0;
-  int n_tiles = 0, n_main = 0, n_btiles = 0, n_edge = 0;
-  size_t slot = 0, bslot = 0, edge_ofs = 0, slot_floats = 0;
+  int kind = 0, co = 0, ci = 0, units = 0;
+  size_t slot = 0, slot_floats = 0;
 };
 F32WPlan f32_wgrad_plan(int kind, int co, int ci, std::vector<F32WJob>& jobs);
 cudaError_t launch_f32_wgrad(const F32WPlan& p, const F32WJob* d_jobs, int n, float* gw, float* gb, float* slots,
                              cudaStream_t st);
-// Backward of the final conv (gd3, dW, db) and weight gradient of enc1; scratch of
-// f32_edge_slot_floats(C) floats.
-size_t f32_edge_slot_floats(int C);
-cudaError_t launch_f32_final_bwd(const F32Img* imgs, int n, int maxH, int maxW, const float* w, int C, float* gw,
-                                 float* gb, float* slots, cudaStream_t st);
-cudaError_t launch_f32_enc1_wgrad(const F32Img* imgs, int n, int maxH1, int maxW1, int C, float* gw, float* gb,
-                                  float* slots, cudaStream_t st);
+// Input gradient of the final conv (masked by d3's ReLU).
+cudaError_t launch_f32_final_dgrad(const F32Img* imgs, int n, int maxH, int maxW, const float* w, int C,
+                                   cudaStream_t st);
+// Weight gradients of the final conv (kind FK_WFINAL) and of enc1 (FK_WENC1).
+enum { FK_WFINAL = FK_COUNT, FK_WENC1 };
+cudaError_t launch_f32_edge_wgrad(const F32WPlan& p, const F32Img* imgs, const F32WJob* d_jobs, int n, float* gw,
+                                  float* gb, float* slots, cudaStream_t st);
 cudaError_t launch_f32_latent_bwd(const F32Lat* lat, int n, size_t max_n, cudaStream_t st);
 
 }  // namespace sv

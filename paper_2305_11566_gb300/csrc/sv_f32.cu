@@ -28,30 +28,28 @@ sv_status Ctx::f32_plan() {
   auto src = [&](int l) { return F32Src{net.w_off(l), net.ks(l), net.cout(l), net.cin(l)}; };
   std::vector<F32PackDesc> descs;
   size_t total = 0;
-  auto add = [&](F32Layer& l, int kind, std::initializer_list<int> layers) {
-    std::vector<F32Src> s;
-    for (int k : layers) s.push_back(src(k));
-    l = f32_plan_layer(kind, s.data(), (int)s.size(), descs, total);
-  };
+  auto add = [&](F32Layer& l, int kind, int layer) { l = f32_plan_layer(kind, false, src(layer), descs, total); };
+  auto add_grad = [&](int kind, int layer) { f32_g[layer] = f32_plan_layer(kind, true, src(layer), descs, total); };
   if (t1) {
     t1_plan_layers(t1_l, descs, total);
   } else {
-    add(f32_l[L_ENC2], FK_S2, {L_ENC2});
-    add(f32_l[L_ENC3], FK_S2, {L_ENC3});
-    add(f32_l[L_MU], FK_P1, {L_MU});
-    add(f32_l[L_LV], FK_P1, {L_LV});
+    add(f32_l[L_ENC2], FK_S2, L_ENC2);
+    add(f32_l[L_ENC3], FK_S2, L_ENC3);
+    add(f32_l[L_MU], FK_P1, L_MU);
+    add(f32_l[L_LV], FK_P1, L_LV);
     for (int l : {L_DEC1, L_DEC2, L_DEC3}) {
       if (cfg.precision == SV_FP32) {  // (a BF16 context decodes on the tensor cores)
-        add(f32_l[l], FK_UP2, {l});
+        add(f32_l[l], FK_UP2, l);
         f32_t[l] = f32_l[l];  // the nine unsummed taps, also the summed form's edge weights
         f32_t[l].kind = FK_UP2X;
         f32_t[l].w[0] = f32_l[l].wb;
       }
-      add(f32_g[l], FK_DUP2, {l});
+      add_grad(FK_DUP2, l);
     }
-    add(f32_g[L_MU], FK_P1, {L_MU, L_LV});
-    add(f32_g[L_ENC3], FK_DS2, {L_ENC3});
-    add(f32_g[L_ENC2], FK_DS2, {L_ENC2});
+    add_grad(FK_P1, L_MU);
+    add_grad(FK_P1, L_LV);
+    add_grad(FK_DS2, L_ENC3);
+    add_grad(FK_DS2, L_ENC2);
   }
   f32_n_descs = (int)descs.size();
   f32_max_count = 0;
@@ -167,7 +165,8 @@ sv_status Ctx::f32_forward(const sv_pair* pairs, int n, const F32Tensors* t, con
   if ((s = conv(L_DEC2, "dec2", 1, 1))) return s;
   if ((s = conv(L_DEC3, "dec3", 0, 1))) return s;
   LaunchScope ls(*this, "final", st);
-  return cuda(launch_f32_final(d_img, n, mH[0], mW[0], W + net.w_off(L_FINAL), W + net.b_off(L_FINAL), net.dec[2], st),
+  return cuda(launch_f32_final(d_img, n, mH[0], mW[0], W + net.w_off(L_FINAL), W + net.b_off(L_FINAL), net.dec[2],
+                               train, st),
               "final");
 }
 
@@ -420,13 +419,13 @@ sv_status Ctx::f32_backward(const void* const* gY, const void* const* gmu_ext, c
       G(L_DEC3, gd3, 0, t.d2, gd2, 1);
       G(L_DEC2, gd2, 1, t.d1, gd1, 2);
       G(L_DEC1, gd1, 2, nullptr, gz, 3);
+      Wg(L_FINAL, nullptr, 0, t.d3, 0);  // (g is the image table's gY)
+      Wg(L_ENC1, ge1, 1, nullptr, 0);    // (x is built from the images)
       Wg(L_DEC3, gd3, 0, t.d2, 1);
       Wg(L_DEC2, gd2, 1, t.d1, 2);
       Wg(L_DEC1, gd1, 2, t.z, 3);
-      F32Job h{};  // both latent heads as one contraction over [gmu, glv]
-      h.in[0] = gmu; h.ic[0] = net.lat; h.in[1] = glv; h.ic[1] = net.lat; h.mask = t.e3; h.out = ge3;
-      h.Hi = h.Ho = lv.H[3]; h.Wi = h.Wo = lv.W[3];
-      gj[L_MU].push_back(h);
+      G(L_MU, gmu, 3, t.e3, ge3, 3);
+      G(L_LV, glv, 3, t.e3, ge3, 3);
       Wg(L_MU, gmu, 3, t.e3, 3);
       Wg(L_LV, glv, 3, t.e3, 3);
       G(L_ENC3, ge3, 3, t.e2, ge2, 2);
@@ -444,17 +443,15 @@ sv_status Ctx::f32_backward(const void* const* gY, const void* const* gmu_ext, c
         Fw(L_ENC3, t.e2, 2, t.e3, 3);
       }
     }
-    static const int kinds[L_COUNT] = {-1, FK_S2, FK_S2, FK_P1, FK_P1, FK_UP2, FK_UP2, FK_UP2, -1};
+    static const int kinds[L_COUNT] = {FK_WENC1, FK_S2, FK_S2, FK_P1, FK_P1, FK_UP2, FK_UP2, FK_UP2, FK_WFINAL};
     F32WPlan wp[L_COUNT];
-    size_t slots = std::max(f32_edge_slot_floats(net.dec[2]), f32_edge_slot_floats(net.enc[0]));
+    size_t slots = 0;
     Tables tb;
     size_t og[L_COUNT], of[L_COUNT], ow[L_COUNT];
     const size_t o_img = tb.put(img), o_lat = tb.put(lat);
     for (int l = 0; l < L_COUNT; ++l) {
-      if (kinds[l] >= 0) {
-        wp[l] = f32_wgrad_plan(kinds[l], net.cout(l), net.cin(l), wj[l]);
-        slots = std::max(slots, wp[l].slot_floats);
-      }
+      wp[l] = f32_wgrad_plan(kinds[l], net.cout(l), net.cin(l), wj[l]);
+      slots = std::max(slots, wp[l].slot_floats);
       og[l] = tb.put(gj[l]);
       of[l] = tb.put(fj[l]);
       ow[l] = tb.put(wj[l]);
@@ -472,14 +469,16 @@ sv_status Ctx::f32_backward(const void* const* gY, const void* const* gmu_ext, c
     LaunchScope _ls(*this, name, st);       \
     if ((s = cuda((expr), name))) return s; \
   }
-    auto dgrad = [&](int l, int li) {
-      return launch_f32_conv(f32_g[l], (const F32Job*)(d + og[l]), m, mH[li], mW[li], P, nullptr, 0, st);
+    auto dgrad = [&](int l, int li, int act = 0) {
+      return launch_f32_conv(f32_g[l], (const F32Job*)(d + og[l]), m, mH[li], mW[li], P, nullptr, act, st);
     };
     auto wgrad = [&](int l) {
-      return launch_f32_wgrad(wp[l], (const F32WJob*)(d + ow[l]), m, GW(l), GB(l), sl, st);
+      const F32WJob* j = (const F32WJob*)(d + ow[l]);
+      if (l == L_FINAL || l == L_ENC1) return launch_f32_edge_wgrad(wp[l], d_img, j, m, GW(l), GB(l), sl, st);
+      return launch_f32_wgrad(wp[l], j, m, GW(l), GB(l), sl, st);
     };
-    SV_BW("bwd_final", launch_f32_final_bwd(d_img, m, mH[0], mW[0], W + net.w_off(L_FINAL), net.dec[2], GW(L_FINAL),
-                                            GB(L_FINAL), sl, st));
+    SV_BW("bwd_final_dgrad", launch_f32_final_dgrad(d_img, m, mH[0], mW[0], W + net.w_off(L_FINAL), net.dec[2], st));
+    SV_BW("bwd_final_wgrad", wgrad(L_FINAL));
     SV_BW("bwd_dec3_dgrad", dgrad(L_DEC3, 1));
     SV_BW("bwd_dec3_wgrad", wgrad(L_DEC3));
     SV_BW("bwd_dec2_dgrad", dgrad(L_DEC2, 2));
@@ -495,14 +494,15 @@ sv_status Ctx::f32_backward(const void* const* gY, const void* const* gmu_ext, c
       SV_BW("recompute_enc3", launch_f32_conv(f32_l[L_ENC3], (const F32Job*)(d + of[L_ENC3]), m, mH[3], mW[3], P,
                                               W + net.b_off(L_ENC3), 1, st));
     }
-    SV_BW("bwd_heads_dgrad", dgrad(L_MU, 3));
+    SV_BW("bwd_mu_dgrad", dgrad(L_MU, 3));
+    SV_BW("bwd_lv_dgrad", dgrad(L_LV, 3, 8));
     SV_BW("bwd_mu_wgrad", wgrad(L_MU));
     SV_BW("bwd_lv_wgrad", wgrad(L_LV));
     SV_BW("bwd_enc3_dgrad", dgrad(L_ENC3, 2));
     SV_BW("bwd_enc3_wgrad", wgrad(L_ENC3));
     SV_BW("bwd_enc2_dgrad", dgrad(L_ENC2, 1));
     SV_BW("bwd_enc2_wgrad", wgrad(L_ENC2));
-    SV_BW("bwd_enc1_wgrad", launch_f32_enc1_wgrad(d_img, m, mH[1], mW[1], net.enc[0], GW(L_ENC1), GB(L_ENC1), sl, st));
+    SV_BW("bwd_enc1_wgrad", wgrad(L_ENC1));
     for (int i = i0; want_coarse && i < i1; ++i) {
       if (!gcoarse[i]) continue;
       const sv_pair& p = train_pairs[i];

@@ -125,7 +125,7 @@ void t1_plan_layers(F32Layer* layers, std::vector<F32PackDesc>& descs, size_t& t
     if (l == 6 || l == 7) continue;
     const int kind = kT1[l].mode == 0 ? FK_S1_5 : kT1[l].mode == 1 ? FK_S2_5 : FK_DE5;
     const F32Src src{t1_w_off(l), 5, kT1[l].co, kT1[l].ci};
-    layers[l] = f32_plan_layer(kind, &src, 1, descs, total);
+    layers[l] = f32_plan_layer(kind, false, src, descs, total);
   }
   const int ic[4] = {16, 1, 32, 32};
   layers[12] = f32_plan_y5(t1_w_off(12), ic, 4, descs, total);

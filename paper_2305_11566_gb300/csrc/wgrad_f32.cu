@@ -1,19 +1,20 @@
 // wgrad_f32.cu -- weight gradients of the FP32 refinement layers on the CUDA cores, all pairs of
-// a call per launch, and the fused backward of the one- and two-channel layers.
+// a call per launch.
 //
-// dW[co][tap][ci] = sum over output pixels p of g(p, co) x(p S + tap, ci): one GEMM per tap whose
-// reduction runs over the pixels.  A warp owns one tap of a block of BCO output x BCI input
-// channels (8 x 8 in registers per lane; lanes left over split the pixels), so each staged pixel
-// costs a lane 4 vector loads for 64 multiply-adds; the block's warps share the staged g and x of
-// 64 pixels (cp.async, two buffers).  (One lane holding every tap of 4 x 2 channels needed
-// 10 loads for 72 multiply-adds.)  Nearest-x2 layers run on the folded form: output phase (py, px)
-// reads 2x2 input pixels, 16 phase-taps instead of 4 x 9, and the reduction adds each kernel
-// element's four phase-taps; the last row / column of an odd output, whose cropped neighbour the
-// folded taps would count, goes to extra blocks that take the nine taps one by one.
-// Every block writes its sums to its own slot; wgrad_f32_reduce adds the slots in a fixed order
-// (no atomics: the same call gives the same bits).  Backward of 16 pairs of 1242 x 375, 16/32/64 net:
-// dec3 + dec2 weight gradients 6.8 -> 1.6 ms, final conv's two gradients 2.5 -> 0.27 ms; the whole
-// training step (with the input gradients of conv_f32.cu) 31.0 -> 6.7 ms.
+// dW[co][ky][kx][ci] = sum over output pixels p of g(p, co) V(p S + k - pad, ci), V the layer's input
+// view.  The summation order is fixed and does not depend on the block shape (conv_f32.cu says
+// why the training step keeps one order): a pair's 8 x 16 output tiles go to `units` chains, tile t to
+// chain t mod units; a chain adds its tiles' pixels in row order, each weight in one accumulator; the
+// chains' sums are added in chain order, the pairs' in pair order.  No atomics.
+//
+// A block runs one chain for a block of output x input channels.  A warp owns one kernel row: a lane
+// holds COL output x 4 input channels x 3 kernel columns in registers and slides the three input
+// columns along the row, so a pixel costs it 2 loads of g and 0.5 (nearest x2), 1 or 2 (stride 2) of x
+// for 96 multiply-adds (one thread holding 4 x 2 channels x 9 taps loaded 10 vectors for 72).  g and
+// x of a few rows are staged by cp.async in two buffers.  16 pairs of 1242 x 375, 16/32/64 net: dec3 and dec2
+// 3.5 ms (6.8 before, one pair a launch) at 40 TFLOP/s, the FMA pipes 60 % busy; the whole training step with
+// the input gradients of conv_f32.cu 31.1 -> 11.1 ms.  Summing the folded phase-taps instead ran dec3 and
+// dec2 in 1.6 ms but moves the gradient's bits (see conv_f32.cu).
 #include "conv_f32.cuh"
 
 #include <algorithm>
@@ -45,170 +46,153 @@ __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_grou
 template <int N>
 __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N)); }
 
-constexpr int kTR = 4, kTC = 16;  // pixels of a tile (input pixels for FK_UP2)
+constexpr int kTR = 8, kTC = 16;  // pixels of a tile
 
-// Warps (= taps, or pixel groups of the 1x1 form), staged pixels of g and x per tile.
+// Kernel rows (= warps per channel block) and columns, tile rows staged per step, staged x.
 template <int KIND> struct WK;
-template <> struct WK<FK_S2> { static constexpr int NW = 9, NG = 64, XR = 9, XC = 33; };
-template <> struct WK<FK_P1> { static constexpr int NW = 8, NG = 64, XR = 4, XC = 16; };
-template <> struct WK<FK_UP2> { static constexpr int NW = 16, NG = 256, XR = 6, XC = 18; };
+template <> struct WK<FK_S2> { static constexpr int KR = 3, KC = 3, ROWS = 2, XR = 5, XC = 33; };
+template <> struct WK<FK_P1> { static constexpr int KR = 1, KC = 1, ROWS = 4, XR = 4, XC = 16; };
+template <> struct WK<FK_UP2> { static constexpr int KR = 3, KC = 3, ROWS = 4, XR = 4, XC = 10; };
 
-template <int KIND, int CGN, int IGN>
+// COL output channels per lane, CGN x IGN lanes of a warp, NB input-channel blocks (warps) per kernel row.
+template <int KIND, int COL_, int CGN_, int IGN_, int NB_>
 struct WG {
   using K = WK<KIND>;
-  static constexpr int BCO = 8 * CGN, BCI = 8 * IGN, KSP = 32 / (CGN * IGN), NT = 32 * K::NW;
-  // FK_UP2's edge tiles stage 64 pixels of g and their nine taps of x
-  static constexpr int GF = K::NG * BCO, XF = (KIND == FK_UP2 ? 64 * 9 : K::XR * K::XC) * BCI;
-  static constexpr int MAINF = GF + K::XR * K::XC * BCI, EDGEF = 64 * BCO + 64 * 9 * BCI;
-  static constexpr int BUF = KIND == FK_UP2 && EDGEF > MAINF ? EDGEF : MAINF;
+  static constexpr int COL = COL_, CGN = CGN_, IGN = IGN_, NB = NB_;
+  static constexpr int BCO = COL * CGN, WCI = 4 * IGN, BCI = WCI * NB, NT = 32 * K::KR * NB;
+  static constexpr int NG = K::ROWS * kTC;
+  static constexpr int GF = NG * BCO, XF = K::XR * K::XC * BCI, BUF = GF + XF;
   static constexpr size_t SMEM = 2 * sizeof(float) * BUF;
+  static constexpr int WARPS = K::KR * NB, MINB = COL == 8 ? (WARPS > 6 ? 1 : WARPS > 3 ? 2 : 4) : (WARPS > 6 ? 2 : WARPS > 3 ? 3 : 6);
 };
 
-struct WArgs {
-  int n, Co, Ci, n_tiles, n_main, n_btiles, n_edge;  // tiles and blocks of the main and edge parts
-  size_t slot, bslot, edge_ofs;  // floats of a main / edge slot; first edge slot
-  float* slots;
-};
-
-__device__ __forceinline__ int tiles_of(int h, int w) { return ((h + kTR - 1) / kTR) * ((w + kTC - 1) / kTC); }
-
-template <int KIND, int CGN, int IGN>
-__global__ void __launch_bounds__(WG<KIND, CGN, IGN>::NT, KIND == FK_UP2 ? 1 : 2)
-wgrad_f32_kernel(const F32WJob* __restrict__ jobs, const WArgs A) {
-  using G = WG<KIND, CGN, IGN>;
+template <int KIND, int COL, int CGN, int IGN, int NB>
+__global__ void __launch_bounds__(WG<KIND, COL, CGN, IGN, NB>::NT, WG<KIND, COL, CGN, IGN, NB>::MINB)
+wgrad_f32_kernel(const F32WJob* __restrict__ jobs, int n, int Co, int Ci, size_t slot, float* __restrict__ slots) {
+  using G = WG<KIND, COL, CGN, IGN, NB>;
   using K = WK<KIND>;
-  constexpr int BCO = G::BCO, BCI = G::BCI, KSP = G::KSP;
+  constexpr int BCO = G::BCO, BCI = G::BCI, KC = K::KC;
   extern __shared__ __align__(16) float wf_sm[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int cg = lane % CGN, ig = lane / CGN % IGN, ks = lane / (CGN * IGN);
-  const int nci = A.Ci / BCI, co0 = ((int)blockIdx.y / nci) * BCO, ci0 = ((int)blockIdx.y % nci) * BCI;
-  const bool edge = KIND == FK_UP2 && (int)blockIdx.x >= A.n_main;
-  const int b = edge ? blockIdx.x - A.n_main : blockIdx.x, nb = edge ? A.n_edge : A.n_main;
-  const int nt = edge ? A.n_btiles : A.n_tiles;
-  const int t0 = (int)((long long)nt * b / nb), t1 = (int)((long long)nt * (b + 1) / nb);
-  u64 acc[8][4];
+  const int ky = warp % K::KR, cib = warp / K::KR;
+  const int cg = lane % CGN, ig = lane / CGN % IGN;  // (fewer than 32 lanes: the others repeat)
+  const int nci = (Ci + BCI - 1) / BCI, co0 = ((int)blockIdx.y / nci) * BCO, ci0 = ((int)blockIdx.y % nci) * BCI;
+  int job = 0;
+  while (job + 1 < n && (int)blockIdx.x >= jobs[job + 1].unit0) ++job;
+  const F32WJob& J = jobs[job];
+  const int Ho = J.Ho, Wo = J.Wo, Hi = J.Hi, Wi = J.Wi;
+  const int tiles_x = (Wo + kTC - 1) / kTC, ntiles = tiles_x * ((Ho + kTR - 1) / kTR);
+  const int t0 = blockIdx.x - J.unit0;
+  constexpr int STEPS = kTR / K::ROWS;
+  const int nsteps = (ntiles - t0 + J.units - 1) / J.units * STEPS;
+  u64 acc[KC][COL][2];
 #pragma unroll
-  for (int j = 0; j < 8; ++j)
+  for (int k = 0; k < KC; ++k)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) acc[j][q] = 0ull;
-  float4 bacc = make_float4(0.f, 0.f, 0.f, 0.f);  // bias gradient: lane l the channels 4 l .. of g
-  const bool want_bias = ci0 == 0;
+    for (int j = 0; j < COL; ++j) acc[k][j][0] = acc[k][j][1] = 0ull;
+  float4 bacc = make_float4(0.f, 0.f, 0.f, 0.f);  // bias gradient: lanes of the last warp, 4 channels each
+  const bool bias_lane = ci0 == 0 && warp == G::WARPS - 1 && lane < BCO / 4;
 
-  int job = 0;  // pair of the tile being staged
-  auto stage = [&](int t, int buf) {
-    while (job + 1 < A.n && t >= (edge ? jobs[job + 1].btile0 : jobs[job + 1].tile0)) ++job;
-    const F32WJob& J = jobs[job];
-    float* gs = wf_sm + buf * G::BUF;
-    if (!edge) {
-      float* xs = gs + G::GF;
-      const int Hp = KIND == FK_UP2 ? J.Ho / 2 : J.Ho, Wp = KIND == FK_UP2 ? J.Wo / 2 : J.Wo;  // tiled grid
-      const int tx = (Wp + kTC - 1) / kTC, tl = t - J.tile0;
-      const int Y0 = tl / tx * kTR, X0 = tl % tx * kTC;
+  auto stage = [&](int step) {
+    const int t = t0 + step / STEPS * J.units;
+    const int Y0 = t / tiles_x * kTR + step % STEPS * K::ROWS, X0 = t % tiles_x * kTC;
+    float* gs = wf_sm + (step & 1) * G::BUF;
+    float* xs = gs + G::GF;
 #pragma unroll 4
-      for (int e = threadIdx.x; e < K::NG * (BCO / 4); e += G::NT) {
-        const int c = e % (BCO / 4), p = e / (BCO / 4);
-        int oy, ox;
-        bool ok;
-        if (KIND == FK_UP2) {  // p = row of 8, column of 32 output pixels
-          oy = 2 * Y0 + p / 32;
-          ox = 2 * X0 + p % 32;
-          ok = oy < 2 * Hp && ox < 2 * Wp;
-        } else {
-          oy = Y0 + p / kTC;
-          ox = X0 + p % kTC;
-          ok = oy < Hp && ox < Wp;
-        }
-        cp16z(gs + p * BCO + 4 * c, ok ? J.g + ((size_t)oy * J.Wo + ox) * A.Co + co0 + 4 * c : J.g, ok);
-      }
-      const int iy0 = KIND == FK_S2 ? 2 * Y0 - 1 : KIND == FK_UP2 ? Y0 - 1 : Y0;
-      const int ix0 = KIND == FK_S2 ? 2 * X0 - 1 : KIND == FK_UP2 ? X0 - 1 : X0;
+    for (int e = threadIdx.x; e < G::NG * (BCO / 4); e += G::NT) {
+      const int c = e % (BCO / 4), p = e / (BCO / 4);
+      const int oy = Y0 + p / kTC, ox = X0 + p % kTC;
+      const bool ok = oy < Ho && ox < Wo;
+      cp16z(gs + p * BCO + 4 * c, ok ? J.g + ((size_t)oy * Wo + ox) * Co + co0 + 4 * c : J.g, ok);
+    }
+    const int iy0 = KIND == FK_S2 ? 2 * Y0 - 1 : KIND == FK_UP2 ? Y0 / 2 - 1 : Y0;
+    const int ix0 = KIND == FK_S2 ? 2 * X0 - 1 : KIND == FK_UP2 ? X0 / 2 - 1 : X0;
 #pragma unroll 4
-      for (int e = threadIdx.x; e < K::XR * K::XC * (BCI / 4); e += G::NT) {
-        const int c = e % (BCI / 4), p = e / (BCI / 4), r = p / K::XC, q = p - r * K::XC;
-        const int iy = iy0 + r, ix = ix0 + q;
-        const bool ok = iy >= 0 && ix >= 0 && iy < J.Hi && ix < J.Wi;
-        cp16z(xs + p * BCI + 4 * c, ok ? J.x + ((size_t)iy * J.Wi + ix) * A.Ci + ci0 + 4 * c : J.x, ok);
-      }
-    } else if constexpr (KIND == FK_UP2) {
-      // edge pixels in order: the last row when Ho is odd, then the last column above it
-      float* xs = gs + 64 * BCO;
-      const int nrow = J.Ho & 1 ? J.Wo : 0, ncol = J.Wo & 1 ? J.Ho - (J.Ho & 1) : 0;
-      const int p0 = (t - J.btile0) * 64;
-      for (int e = threadIdx.x; e < 64 * (BCO / 4); e += G::NT) {
-        const int c = e % (BCO / 4), q = e / (BCO / 4), p = p0 + q;
-        const bool ok = p < nrow + ncol;
-        const int oy = p < nrow ? J.Ho - 1 : p - nrow, ox = p < nrow ? p : J.Wo - 1;
-        cp16z(gs + q * BCO + 4 * c, ok ? J.g + ((size_t)oy * J.Wo + ox) * A.Co + co0 + 4 * c : J.g, ok);
-      }
-      for (int e = threadIdx.x; e < 64 * 9 * (BCI / 4); e += G::NT) {
-        const int c = e % (BCI / 4), m = e / (BCI / 4), q = m / 9, tp = m - 9 * q, p = p0 + q;
-        const int oy = p < nrow ? J.Ho - 1 : p - nrow, ox = p < nrow ? p : J.Wo - 1;
-        const int vy = oy + tp / 3 - 1, vx = ox + tp % 3 - 1;
-        const bool ok = p < nrow + ncol && vy >= 0 && vx >= 0 && vy < J.Ho && vx < J.Wo;
-        cp16z(xs + m * BCI + 4 * c, ok ? J.x + ((size_t)(vy >> 1) * J.Wi + (vx >> 1)) * A.Ci + ci0 + 4 * c : J.x, ok);
-      }
+    for (int e = threadIdx.x; e < K::XR * K::XC * (BCI / 4); e += G::NT) {
+      const int c = e % (BCI / 4), p = e / (BCI / 4), r = p / K::XC, q = p - r * K::XC;
+      const int iy = iy0 + r, ix = ix0 + q;
+      const bool ok = iy >= 0 && ix >= 0 && iy < Hi && ix < Wi && ci0 + 4 * c < Ci;
+      cp16z(xs + p * BCI + 4 * c, ok ? J.x + ((size_t)iy * Wi + ix) * Ci + ci0 + 4 * c : J.x, ok);
     }
     cp_commit();
   };
-  auto madd = [&](const float* g, const float* x) {
-    const float4 g0 = *reinterpret_cast<const float4*>(g + cg * 4);
-    const float4 g1 = *reinterpret_cast<const float4*>(g + BCO / 2 + cg * 4);
-    const ulonglong2 x0 = *reinterpret_cast<const ulonglong2*>(x + ig * 4);
-    const ulonglong2 x1 = *reinterpret_cast<const ulonglong2*>(x + BCI / 2 + ig * 4);
-    const float gv[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
+  auto loadg = [&](const float* g, u64 (&gv)[COL]) {
+    const float4 a = *reinterpret_cast<const float4*>(g + cg * 4);
+    gv[0] = dup2(a.x); gv[1] = dup2(a.y); gv[2] = dup2(a.z); gv[3] = dup2(a.w);
+    if constexpr (COL == 8) {
+      const float4 b = *reinterpret_cast<const float4*>(g + BCO / 2 + cg * 4);
+      gv[4] = dup2(b.x); gv[5] = dup2(b.y); gv[6] = dup2(b.z); gv[7] = dup2(b.w);
+    }
+  };
+  auto madd = [&](u64 (&a)[COL][2], const u64 (&gv)[COL], const ulonglong2& x) {
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const u64 v = dup2(gv[j]);
-      fma2(acc[j][0], v, x0.x);
-      fma2(acc[j][1], v, x0.y);
-      fma2(acc[j][2], v, x1.x);
-      fma2(acc[j][3], v, x1.y);
+    for (int j = 0; j < COL; ++j) {
+      fma2(a[j][0], gv[j], x.x);
+      fma2(a[j][1], gv[j], x.y);
     }
   };
 
-  if (t0 < t1) stage(t0, 0);
-  for (int t = t0; t < t1; ++t) {
-    const int buf = (t - t0) & 1;
-    if (t + 1 < t1) {
-      stage(t + 1, buf ^ 1);
+  if (nsteps > 0) stage(0);
+  for (int step = 0; step < nsteps; ++step) {
+    if (step + 1 < nsteps) {
+      stage(step + 1);
       cp_wait<1>();
     } else {
       cp_wait<0>();
     }
     __syncthreads();
-    const float* gs = wf_sm + buf * G::BUF;
-    if (!edge) {
-      const float* xs = gs + G::GF;
-      if constexpr (KIND == FK_S2) {
-        const int ky = warp / 3, kx = warp % 3;
-        for (int r = 0; r < kTR; ++r) {
-          const float* gp = gs + r * kTC * BCO;
-          const float* xp = xs + ((2 * r + ky) * K::XC + kx) * BCI;
+    const int t = t0 + step / STEPS * J.units;
+    const int Y0 = t / tiles_x * kTR + step % STEPS * K::ROWS, X0 = t % tiles_x * kTC;
+    const float* gs = wf_sm + (step & 1) * G::BUF;
+    const float* xs = gs + G::GF + cib * G::WCI + ig * 4;
+    auto X = [&](int r, int c) { return *reinterpret_cast<const ulonglong2*>(xs + (r * K::XC + c) * BCI); };
+#pragma unroll 1
+    for (int r = 0; r < K::ROWS; ++r) {
+      const float* gr = gs + r * kTC * BCO;
+      if constexpr (KIND == FK_UP2) {
+        if (Y0 + r + ky - 1 >= Ho) continue;  // the cropped upsampled row adds nothing
+        const int xr = ((r + ky - 1) >> 1) + 1;
+        ulonglong2 xm = X(xr, 0), x0 = X(xr, 1);
 #pragma unroll 2
-          for (int c = ks; c < kTC; c += KSP) madd(gp + c * BCO, xp + 2 * c * BCI);
+        for (int c = 0; c < kTC / 2; ++c) {
+          const ulonglong2 xp = X(xr, c + 2);
+          u64 gv[COL];
+          loadg(gr + 2 * c * BCO, gv);
+          madd(acc[0], gv, xm);
+          madd(acc[1], gv, x0);
+          if (X0 + 2 * c + 1 < Wo) madd(acc[2], gv, x0);  // (else cropped)
+          loadg(gr + (2 * c + 1) * BCO, gv);
+          madd(acc[0], gv, x0);
+          madd(acc[1], gv, x0);
+          madd(acc[2], gv, xp);
+          xm = x0;
+          x0 = xp;
         }
-      } else if constexpr (KIND == FK_P1) {
+      } else if constexpr (KIND == FK_S2) {
+        const int xr = 2 * r + ky;
+        ulonglong2 xa = X(xr, 0);
 #pragma unroll 2
-        for (int p = warp * 8 + ks; p < warp * 8 + 8; p += KSP) madd(gs + p * BCO, xs + p * BCI);
+        for (int c = 0; c < kTC; ++c) {
+          const ulonglong2 xb = X(xr, 2 * c + 1), xc = X(xr, 2 * c + 2);
+          u64 gv[COL];
+          loadg(gr + c * BCO, gv);
+          madd(acc[0], gv, xa);
+          madd(acc[1], gv, xb);
+          madd(acc[2], gv, xc);
+          xa = xc;
+        }
       } else {
-        const int ph = warp >> 2, py = ph >> 1, px = ph & 1, dr = (warp >> 1 & 1) + py, dc = (warp & 1) + px;
-        for (int r = 0; r < kTR; ++r) {
-          const float* gp = gs + ((2 * r + py) * 32 + px) * BCO;
-          const float* xp = xs + ((r + dr) * K::XC + dc) * BCI;
-#pragma unroll 2
-          for (int c = ks; c < kTC; c += KSP) madd(gp + 2 * c * BCO, xp + c * BCI);
+#pragma unroll 4
+        for (int c = 0; c < kTC; ++c) {
+          u64 gv[COL];
+          loadg(gr + c * BCO, gv);
+          madd(acc[0], gv, X(r, c));
         }
-      }
-    } else if constexpr (KIND == FK_UP2) {
-      if (warp < 9) {
-        const float* xs = gs + 64 * BCO;
-#pragma unroll 2
-        for (int p = ks; p < 64; p += KSP) madd(gs + p * BCO, xs + (p * 9 + warp) * BCI);
       }
     }
-    if (want_bias && lane < BCO / 4) {
-      const int np = edge ? 64 : K::NG;
-      for (int p = warp; p < np; p += K::NW) {
+    if (bias_lane) {
+#pragma unroll 4
+      for (int p = 0; p < G::NG; ++p) {
         const float4 g = *reinterpret_cast<const float4*>(gs + p * BCO + 4 * lane);
         bacc.x += g.x;
         bacc.y += g.y;
@@ -218,279 +202,244 @@ wgrad_f32_kernel(const F32WJob* __restrict__ jobs, const WArgs A) {
     }
     __syncthreads();
   }
-  // lanes that split the pixels add up
+  float* out = slots + (size_t)blockIdx.x * slot;
+  constexpr int TAPS = K::KR * KC;
+  const int ci = ci0 + cib * G::WCI + ig * 4;
+  if (lane < CGN * IGN && ci < Ci) {
 #pragma unroll
-  for (int o = CGN * IGN; o < 32; o <<= 1)
+    for (int k = 0; k < KC; ++k)
 #pragma unroll
-    for (int j = 0; j < 8; ++j)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const u64 v = __shfl_xor_sync(0xffffffffu, acc[j][q], o);
-        asm("add.rn.f32x2 %0, %0, %1;" : "+l"(acc[j][q]) : "l"(v));
-      }
-  float* out = A.slots + (edge ? A.edge_ofs + (size_t)b * A.bslot : (size_t)b * A.slot);
-  // main FK_UP2 slots: [phase-tap][co][ci]; every other slot in the parameters' order
-  const int taps = KIND == FK_P1 ? 1 : KIND == FK_UP2 && !edge ? 16 : 9;
-  auto put = [&](int co, int ci, int t, float4 v) {
-    const size_t o = KIND == FK_UP2 && !edge ? ((size_t)t * A.Co + co) * A.Ci + ci : ((size_t)co * taps + t) * A.Ci + ci;
-    *reinterpret_cast<float4*>(out + o) = v;
-  };
-  if constexpr (KIND == FK_P1) {  // the warps split the pixels too: add them up in warp order
-    for (int w = 1; w < K::NW; ++w) {
-      if (warp == w && ks == 0)
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-#pragma unroll
-          for (int q = 0; q < 4; ++q) reinterpret_cast<u64*>(wf_sm)[(j * 4 + q) * (CGN * IGN) + cg + CGN * ig] = acc[j][q];
-      __syncthreads();
-      if (warp == 0 && ks == 0)
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const u64 v = reinterpret_cast<u64*>(wf_sm)[(j * 4 + q) * (CGN * IGN) + cg + CGN * ig];
-            asm("add.rn.f32x2 %0, %0, %1;" : "+l"(acc[j][q]) : "l"(v));
-          }
-      __syncthreads();
-    }
-  }
-  if (ks == 0 && (KIND == FK_P1 ? warp == 0 : !edge || warp < 9)) {
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const float2 u = unpack2(acc[j][2 * h]), v = unpack2(acc[j][2 * h + 1]);
-        put(co0 + (j >> 2) * (BCO / 2) + cg * 4 + (j & 3), ci0 + h * (BCI / 2) + ig * 4, KIND == FK_P1 ? 0 : warp,
-            make_float4(u.x, u.y, v.x, v.y));
+      for (int j = 0; j < COL; ++j) {
+        const int co = co0 + (j >> 2) * (BCO / 2) + cg * 4 + (j & 3);
+        const float2 u = unpack2(acc[k][j][0]), v = unpack2(acc[k][j][1]);
+        *reinterpret_cast<float4*>(out + ((size_t)co * TAPS + ky * KC + k) * Ci + ci) = make_float4(u.x, u.y, v.x, v.y);
       }
   }
-  if (want_bias) {
-    float4* bs = reinterpret_cast<float4*>(wf_sm);
-    __syncthreads();
-    if (lane < BCO / 4) bs[warp * (BCO / 4) + lane] = bacc;
-    __syncthreads();
-    if (threadIdx.x < BCO) {
-      float s = 0.f;
-      for (int w = 0; w < K::NW; ++w) s += wf_sm[w * BCO + threadIdx.x];
-      out[(size_t)taps * A.Co * A.Ci + co0 + threadIdx.x] = s;
-    }
-  }
+  if (bias_lane) *reinterpret_cast<float4*>(out + (size_t)TAPS * Co * Ci + co0 + 4 * lane) = bacc;
 }
 
-// gw[e] += the slots' sums (e < nWw), gb[e - nWw] likewise.  A block takes 32 elements; its 8
-// rows add every 8th slot, then each other, in a fixed order.  folded: main slots hold the 16
-// phase-taps of a nearest-x2 layer.
+// gw[e] += the pairs' sums (e < nWw), gb[e - nWw] likewise: a pair's chains in chain order, the pairs in
+// pair order.  A block takes 32 elements, its 8 rows one pair each.
 __global__ void __launch_bounds__(256)
-wgrad_f32_reduce(const float* __restrict__ slots, int n_main, size_t slot, int n_edge, size_t bslot, size_t edge_ofs,
-                 int nWw, int Co, int Ci, int taps, int folded, float* __restrict__ gw, float* __restrict__ gb) {
+wgrad_f32_reduce(const float* __restrict__ slots, const F32WJob* __restrict__ jobs, int n, size_t slot, int nW, int nWw,
+                 float* __restrict__ gw, float* __restrict__ gb) {
   __shared__ float part[8][32];
   const int e = blockIdx.x * 32 + threadIdx.x, y = threadIdx.y;
-  const int nW = nWw + Co;
-  float s = 0.f;
-  if (e < nW) {
-    if (folded) {
-      size_t o[4];
-      int no = 1;
-      if (e < nWw) {
-        const int ci = e % Ci, t = e / Ci % 9, co = e / (9 * Ci), ky = t / 3, kx = t % 3;
-        no = 4;
-        for (int ph = 0; ph < 4; ++ph) {
-          const int py = ph >> 1, px = ph & 1, r = (ky + 1 - py) >> 1, c = (kx + 1 - px) >> 1;
-          o[ph] = ((size_t)(ph * 4 + r * 2 + c) * Co + co) * Ci + ci;
-        }
-      } else {
-        o[0] = (size_t)16 * Co * Ci + (e - nWw);
-        o[1] = o[2] = o[3] = o[0];
-      }
-      for (int b = y; b < n_main; b += 8) {
-        const float* p = slots + (size_t)b * slot;
-        s += no == 4 ? (p[o[0]] + p[o[1]]) + (p[o[2]] + p[o[3]]) : p[o[0]];
-      }
-    } else {
-#pragma unroll 4
-      for (int b = y; b < n_main; b += 8) s += slots[(size_t)b * slot + e];
-    }
-    for (int b = y; b < n_edge; b += 8) s += slots[edge_ofs + (size_t)b * bslot + e];
-  }
-  part[y][threadIdx.x] = s;
-  __syncthreads();
-  if (y == 0 && e < nW) {
-    float t = part[0][threadIdx.x];
+  float tot = 0.f;
+  if (y == 0 && e < nW) tot = e < nWw ? gw[e] : gb[e - nWw];
+  for (int i0 = 0; i0 < n; i0 += 8) {
+    float s = 0.f;
+    if (i0 + y < n && e < nW) {
+      const float* p = slots + (size_t)jobs[i0 + y].unit0 * slot + e;
+      const int u = jobs[i0 + y].units;
+      int b = 0;
+      for (; b + 8 <= u; b += 8) {
+        float v[8];
 #pragma unroll
-    for (int j = 1; j < 8; ++j) t += part[j][threadIdx.x];
+        for (int j = 0; j < 8; ++j) v[j] = p[(size_t)(b + j) * slot];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) s += v[j];
+      }
+      for (; b < u; ++b) s += p[(size_t)b * slot];
+    }
+    part[y][threadIdx.x] = s;
+    __syncthreads();
+    if (y == 0)
+      for (int j = 0; j < 8 && i0 + j < n; ++j) tot += part[j][threadIdx.x];
+    __syncthreads();
+  }
+  if (y == 0 && e < nW) {
     if (e < nWw)
-      gw[e] += t;
+      gw[e] = tot;
     else
-      gb[e - nWw] += t;
+      gb[e - nWw] = tot;
   }
 }
 
-// Backward of the final conv (C channels -> 1): input gradient masked by d3's ReLU, and weight and bias
-// gradient, in one pass over d3.  C / 4 lanes hold a pixel's channels; a thread walks down the
-// rows of one column with the nine neighbouring output gradients from shared memory.  Bound by
-// reading d3 and writing its gradient once.
+// Input gradient of the final conv (C channels -> 1), masked by d3's ReLU.  C / 4 lanes hold a
+// pixel's channels; a thread walks down the rows of one column with the nine neighbouring output
+// gradients from shared memory.  Bound by reading d3 and writing its gradient once.
 constexpr int kFbRows = 16, kFbThreads = 256;
-__global__ void __launch_bounds__(kFbThreads, 2)
-f32_final_bwd_kernel(const F32Img* __restrict__ imgs, int n, const float* __restrict__ w, int C, int tiles_x,
-                     int tiles_y, float* __restrict__ slots) {
+__global__ void __launch_bounds__(kFbThreads)
+f32_final_dgrad_kernel(const F32Img* __restrict__ imgs, const float* __restrict__ w, int C, int tiles_x) {
   extern __shared__ __align__(16) float fb_sm[];
   const int L = C / 4, NC = kFbThreads / L;  // lanes of a pixel, columns of a tile
   const int l = threadIdx.x % L, col = threadIdx.x / L, P = NC + 2;
-  const bool on = col < NC;
-  float* gs = fb_sm;  // [kFbRows + 2][P]
-  float4 k[9], acc[9];
+  const F32Img& I = imgs[blockIdx.z];
+  const int Y0 = (blockIdx.x / tiles_x) * kFbRows, X0 = (blockIdx.x % tiles_x) * NC;
+  if (Y0 >= I.H || X0 >= I.W) return;
+  float4 k[9];
 #pragma unroll
-  for (int t = 0; t < 9; ++t) {
-    k[t] = *reinterpret_cast<const float4*>(w + t * C + 4 * l);
-    acc[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int t = 0; t < 9; ++t) k[t] = *reinterpret_cast<const float4*>(w + t * C + 4 * l);
+  for (int e = threadIdx.x; e < (kFbRows + 2) * P; e += kFbThreads) {
+    const int r = e / P, c = e - r * P, y = Y0 - 1 + r, x = X0 - 1 + c;
+    fb_sm[e] = y >= 0 && x >= 0 && y < I.H && x < I.W ? I.gY[(size_t)y * I.W + x] : 0.f;
   }
-  float bacc = 0.f;
-  const int nt = n * tiles_x * tiles_y;
-  for (int t = blockIdx.x; t < nt; t += gridDim.x) {
-    const F32Img& I = imgs[t / (tiles_x * tiles_y)];
-    const int tl = t % (tiles_x * tiles_y), Y0 = tl / tiles_x * kFbRows, X0 = tl % tiles_x * NC;
-    if (Y0 >= I.H || X0 >= I.W) continue;
-    __syncthreads();
-    for (int e = threadIdx.x; e < (kFbRows + 2) * P; e += kFbThreads) {
-      const int r = e / P, c = e - r * P, y = Y0 - 1 + r, x = X0 - 1 + c;
-      gs[e] = y >= 0 && x >= 0 && y < I.H && x < I.W ? I.gY[(size_t)y * I.W + x] : 0.f;
-    }
-    __syncthreads();
-    const int x = X0 + col;
-    if (!on || x >= I.W) continue;
-    const int rows = min(kFbRows, I.H - Y0);
-    const size_t base = ((size_t)Y0 * I.W + x) * C + 4 * l, step = (size_t)I.W * C;
+  __syncthreads();
+  const int x = X0 + col;
+  if (col >= NC || x >= I.W) return;
+  const int rows = min(kFbRows, I.H - Y0);
+  const size_t base = ((size_t)Y0 * I.W + x) * C + 4 * l, step = (size_t)I.W * C;
 #pragma unroll 1
-    for (int r0 = 0; r0 < rows; r0 += 4) {
-      float4 v[4];
+  for (int r0 = 0; r0 < rows; r0 += 4) {
+    float4 v[4];
 #pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (r0 + j < rows) v[j] = __ldcs(reinterpret_cast<const float4*>(I.d3 + base + (r0 + j) * step));
+    for (int j = 0; j < 4; ++j)
+      if (r0 + j < rows) v[j] = *reinterpret_cast<const float4*>(I.d3 + base + (r0 + j) * step);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        if (r0 + j >= rows) break;
-        const int r = r0 + j;
-        float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int j = 0; j < 4; ++j) {
+      if (r0 + j >= rows) break;
+      const int r = r0 + j;
+      float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int ky = 0; ky < 3; ++ky)
-#pragma unroll
-          for (int kx = 0; kx < 3; ++kx) {
-            // output (y + 1 - ky, x + 1 - kx) read this pixel through tap (ky, kx)
-            const float g = gs[(r + 2 - ky) * P + col + 2 - kx];
-            const int q = ky * 3 + kx;
-            d.x = fmaf(g, k[q].x, d.x);
-            d.y = fmaf(g, k[q].y, d.y);
-            d.z = fmaf(g, k[q].z, d.z);
-            d.w = fmaf(g, k[q].w, d.w);
-            acc[q].x = fmaf(g, v[j].x, acc[q].x);
-            acc[q].y = fmaf(g, v[j].y, acc[q].y);
-            acc[q].z = fmaf(g, v[j].z, acc[q].z);
-            acc[q].w = fmaf(g, v[j].w, acc[q].w);
-            if (q == 4 && l == 0) bacc += g;
-          }
-        d.x = v[j].x > 0.f ? d.x : 0.f;
-        d.y = v[j].y > 0.f ? d.y : 0.f;
-        d.z = v[j].z > 0.f ? d.z : 0.f;
-        d.w = v[j].w > 0.f ? d.w : 0.f;
-        *reinterpret_cast<float4*>(I.gd3 + base + r * step) = d;
+      for (int q = 0; q < 9; ++q) {
+        // output (y + 1 - ky, x + 1 - kx) read this pixel through tap (ky, kx)
+        const float g = fb_sm[(r + 2 - q / 3) * P + col + 2 - q % 3];
+        d.x = fmaf(g, k[q].x, d.x);
+        d.y = fmaf(g, k[q].y, d.y);
+        d.z = fmaf(g, k[q].z, d.z);
+        d.w = fmaf(g, k[q].w, d.w);
       }
+      d.x = v[j].x > 0.f ? d.x : 0.f;
+      d.y = v[j].y > 0.f ? d.y : 0.f;
+      d.z = v[j].z > 0.f ? d.z : 0.f;
+      d.w = v[j].w > 0.f ? d.w : 0.f;
+      *reinterpret_cast<float4*>(I.gd3 + base + r * step) = d;
     }
-  }
-  // the columns of a block add up in column order, tap by tap
-  float* slot = slots + (size_t)blockIdx.x * (9 * C + 1);
-  float4* red = reinterpret_cast<float4*>(fb_sm);
-#pragma unroll
-  for (int t = 0; t < 9; ++t) {
-    __syncthreads();
-    if (on) red[threadIdx.x] = acc[t];
-    __syncthreads();
-    if (threadIdx.x < C) {
-      float s = 0.f;
-      for (int c = 0; c < NC; ++c) s += fb_sm[c * C + threadIdx.x];
-      slot[t * C + threadIdx.x] = s;
-    }
-  }
-  __syncthreads();
-  if (on && l == 0) fb_sm[col] = bacc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float s = 0.f;
-    for (int c = 0; c < NC; ++c) s += fb_sm[c];
-    slot[9 * C] = s;
   }
 }
 
-// Weight and bias gradient of enc1 (2 channels -> C, stride 2): the input patch (L / 256,
-// U / 256) of a tile is built in shared memory, C / 4 lanes hold a pixel's output gradient and every
-// lane sums its 4 output channels x 18 taps.
-constexpr int kEwRows = 8, kEwThreads = 256;
-__global__ void __launch_bounds__(kEwThreads, 2)
-f32_enc1_wgrad_kernel(const F32Img* __restrict__ imgs, int n, int C, int tiles_x, int tiles_y,
-                      float* __restrict__ slots) {
-  extern __shared__ __align__(16) float ew_sm[];
-  const int L = C / 4, NC = kEwThreads / L;
-  const int l = threadIdx.x % L, col = threadIdx.x / L, P = 2 * NC + 1;
-  const bool on = col < NC;
-  float2* xs = reinterpret_cast<float2*>(ew_sm);  // [2 kEwRows + 1][P]
-  float4 acc[18], bacc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-  for (int t = 0; t < 18; ++t) acc[t] = make_float4(0.f, 0.f, 0.f, 0.f);
-  const int nt = n * tiles_x * tiles_y;
-  for (int t = blockIdx.x; t < nt; t += gridDim.x) {
-    const F32Img& I = imgs[t / (tiles_x * tiles_y)];
-    const int tl = t % (tiles_x * tiles_y), Y0 = tl / tiles_x * kEwRows, X0 = tl % tiles_x * NC;
-    if (Y0 >= I.H1 || X0 >= I.W1) continue;
-    __syncthreads();
-    for (int e = threadIdx.x; e < (2 * kEwRows + 1) * P; e += kEwThreads) {
-      const int r = e / P, c = e - r * P, vy = 2 * Y0 - 1 + r, vx = 2 * X0 - 1 + c;
-      float2 v = make_float2(0.f, 0.f);
-      if (vy >= 0 && vx >= 0 && vy < I.H && vx < I.W) {
-        v.x = (float)I.L[(size_t)vy * I.pitch + vx] * (1.0f / 256.0f);
-        v.y = upsample4_f(I.coarse_f, I.w, I.h, vx, vy) * (1.0f / 256.0f);
-      }
-      xs[e] = v;
+// Weight gradient of the final conv: a lane owns one kernel row, 4 input channels and their three
+// kernel columns, and reads d3 and the output gradient of its chain's rows straight from memory (the
+// lanes of a pixel read whole sectors; the three kernel rows and neighbouring tiles meet in the
+// caches).  3 C / 4 lanes run a chain; the bias is one more lane.
+__global__ void __launch_bounds__(256)
+f32_final_wgrad_kernel(const F32Img* __restrict__ imgs, const F32WJob* __restrict__ jobs, int n, int units, int C,
+                       int lanes, size_t slot, float* __restrict__ slots) {
+  const int per = blockDim.x / lanes;  // chains of a block
+  const int u = blockIdx.x * per + threadIdx.x / lanes, l = threadIdx.x % lanes;
+  if (threadIdx.x / lanes >= per || u >= units) return;
+  int job = 0;
+  while (job + 1 < n && u >= jobs[job + 1].unit0) ++job;
+  const F32WJob& J = jobs[job];
+  const int H = J.Ho, W = J.Wo;
+  const int tiles_x = (W + kTC - 1) / kTC, ntiles = tiles_x * ((H + kTR - 1) / kTR);
+  const float* g = imgs[job].gY;
+  float* out = slots + (size_t)u * slot;
+  if (l == 3 * C / 4) {
+    float s = 0.f;
+    for (int t = u - J.unit0; t < ntiles; t += J.units) {
+      const int Y0 = t / tiles_x * kTR, X0 = t % tiles_x * kTC, ye = min(Y0 + kTR, H), xe = min(X0 + kTC, W);
+      for (int y = Y0; y < ye; ++y)
+        for (int x = X0; x < xe; ++x) s += g[(size_t)y * W + x];
     }
-    __syncthreads();
-    const int x = X0 + col;
-    if (!on || x >= I.W1) continue;
-    const int rows = min(kEwRows, I.H1 - Y0);
-    const float* g0 = I.ge1 + ((size_t)Y0 * I.W1 + x) * C + 4 * l;
-#pragma unroll 2
-    for (int r = 0; r < rows; ++r) {
-      const float4 g = *reinterpret_cast<const float4*>(g0 + (size_t)r * I.W1 * C);
-      bacc.x += g.x;
-      bacc.y += g.y;
-      bacc.z += g.z;
-      bacc.w += g.w;
+    out[9 * C] = s;
+    return;
+  }
+  const int ky = l / (C / 4), c4 = 4 * (l % (C / 4));
+  float4 acc[3] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
+  for (int t = u - J.unit0; t < ntiles; t += J.units) {
+    const int Y0 = t / tiles_x * kTR, X0 = t % tiles_x * kTC, ye = min(Y0 + kTR, H);
+    for (int y = Y0; y < ye; ++y) {
+      const int vy = y + ky - 1;
+      if (vy < 0 || vy >= H) continue;
+      const float* x = J.x + ((size_t)vy * W + X0) * C + c4;
+      const float* gr = g + (size_t)y * W + X0;
+      const int m = W - X0;  // columns of the row that exist
+      float4 v[kTC + 2];
+      float gv[kTC];
 #pragma unroll
-      for (int t9 = 0; t9 < 9; ++t9) {
-        const float2 v = xs[(2 * r + t9 / 3) * P + 2 * col + t9 % 3];
-        float4 &a = acc[2 * t9], &c = acc[2 * t9 + 1];
-        a.x = fmaf(g.x, v.x, a.x);
-        a.y = fmaf(g.y, v.x, a.y);
-        a.z = fmaf(g.z, v.x, a.z);
-        a.w = fmaf(g.w, v.x, a.w);
-        c.x = fmaf(g.x, v.y, c.x);
-        c.y = fmaf(g.y, v.y, c.y);
-        c.z = fmaf(g.z, v.y, c.z);
-        c.w = fmaf(g.w, v.y, c.w);
-      }
+      for (int j = 0; j < kTC + 2; ++j)
+        v[j] = (j > 0 || X0 > 0) && j - 1 < m ? *reinterpret_cast<const float4*>(x + (j - 1) * C)
+                                              : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int j = 0; j < kTC; ++j) gv[j] = j < m ? gr[j] : 0.f;
+#pragma unroll
+      for (int j = 0; j < kTC; ++j)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          acc[k].x = fmaf(gv[j], v[j + k].x, acc[k].x);
+          acc[k].y = fmaf(gv[j], v[j + k].y, acc[k].y);
+          acc[k].z = fmaf(gv[j], v[j + k].z, acc[k].z);
+          acc[k].w = fmaf(gv[j], v[j + k].w, acc[k].w);
+        }
     }
   }
-  float* slot = slots + (size_t)blockIdx.x * (19 * C);
-  float4* red = reinterpret_cast<float4*>(ew_sm);
 #pragma unroll
-  for (int t = 0; t < 19; ++t) {
-    __syncthreads();
-    if (on) red[threadIdx.x] = t < 18 ? acc[t < 18 ? t : 0] : bacc;
-    __syncthreads();
-    if (threadIdx.x < C) {
-      float s = 0.f;
-      for (int c = 0; c < NC; ++c) s += ew_sm[c * C + threadIdx.x];
-      if (t < 18)
-        slot[(size_t)threadIdx.x * 18 + t] = s;
-      else
-        slot[(size_t)18 * C + threadIdx.x] = s;
+  for (int k = 0; k < 3; ++k) *reinterpret_cast<float4*>(out + (ky * 3 + k) * C + c4) = acc[k];
+}
+
+// Weight and bias gradient of enc1 (2 channels -> C, stride 2): a warp's chain builds the network input
+// (L / 256, U / 256) under its tile in shared memory; a lane owns one kernel row and 4 output
+// channels: 4 x 3 columns x 2 channels.
+constexpr int kEwWarps = 4, kEwR = 2 * kTR + 1, kEwC = 2 * kTC + 1;
+__global__ void __launch_bounds__(32 * kEwWarps)
+f32_enc1_wgrad_kernel(const F32Img* __restrict__ imgs, const F32WJob* __restrict__ jobs, int n, int units, int C,
+                      size_t slot, float* __restrict__ slots) {
+  __shared__ float2 sm[kEwWarps][kEwR][kEwC];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, u = blockIdx.x * kEwWarps + warp;
+  if (u >= units) return;
+  int job = 0;
+  while (job + 1 < n && u >= jobs[job + 1].unit0) ++job;
+  const F32WJob& J = jobs[job];
+  const F32Img& I = imgs[job];
+  const int tiles_x = (I.W1 + kTC - 1) / kTC, ntiles = tiles_x * ((I.H1 + kTR - 1) / kTR);
+  float* out = slots + (size_t)u * slot;
+  const int q0 = C / 4;
+  // 3 q0 (kernel row, 4 channels) tasks, 32 at a time
+  for (int base = 0; base < 3 * q0; base += 32) {
+    const int task = base + lane;
+    const bool on = task < 3 * q0;
+    const int ky = on ? task / q0 : 0, c4 = on ? 4 * (task % q0) : 0;
+    float4 acc[6], bacc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int k = 0; k < 6; ++k) acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int t = u - J.unit0; t < ntiles; t += J.units) {
+      const int Y0 = t / tiles_x * kTR, X0 = t % tiles_x * kTC;
+      __syncwarp();
+      for (int e = lane; e < kEwR * kEwC; e += 32) {
+        const int r = e / kEwC, c = e - r * kEwC, vy = 2 * Y0 - 1 + r, vx = 2 * X0 - 1 + c;
+        float2 v = make_float2(0.f, 0.f);
+        if (vy >= 0 && vx >= 0 && vy < I.H && vx < I.W) {
+          v.x = (float)I.L[(size_t)vy * I.pitch + vx] * (1.0f / 256.0f);
+          v.y = upsample4_f(I.coarse_f, I.w, I.h, vx, vy) * (1.0f / 256.0f);
+        }
+        sm[warp][r][c] = v;
+      }
+      __syncwarp();
+      const int ye = min(kTR, I.H1 - Y0), xe = min(kTC, I.W1 - X0);
+      for (int y = 0; on && y < ye; ++y) {
+        const float* g = I.ge1 + ((size_t)(Y0 + y) * I.W1 + X0) * C + c4;
+        const float2* xr = sm[warp][2 * y + ky];
+        float2 xa = xr[0];
+#pragma unroll 4
+        for (int x = 0; x < xe; ++x) {
+          const float4 gv = *reinterpret_cast<const float4*>(g + (size_t)x * C);
+          const float2 xb = xr[2 * x + 1], xc = xr[2 * x + 2];
+          auto madd = [&](float4& a, float v) {
+            a.x = fmaf(gv.x, v, a.x);
+            a.y = fmaf(gv.y, v, a.y);
+            a.z = fmaf(gv.z, v, a.z);
+            a.w = fmaf(gv.w, v, a.w);
+          };
+          madd(acc[0], xa.x); madd(acc[1], xa.y);
+          madd(acc[2], xb.x); madd(acc[3], xb.y);
+          madd(acc[4], xc.x); madd(acc[5], xc.y);
+          bacc.x += gv.x; bacc.y += gv.y; bacc.z += gv.z; bacc.w += gv.w;
+          xa = xc;
+        }
+      }
+    }
+    if (on) {
+#pragma unroll
+      for (int k = 0; k < 6; ++k) {
+        const float v[4] = {acc[k].x, acc[k].y, acc[k].z, acc[k].w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) out[(size_t)(c4 + j) * 18 + ky * 6 + k] = v[j];
+      }
+      if (ky == 0) {
+        out[18 * C + c4] = bacc.x; out[18 * C + c4 + 1] = bacc.y; out[18 * C + c4 + 2] = bacc.z; out[18 * C + c4 + 3] = bacc.w;
+      }
     }
   }
 }
@@ -505,67 +454,63 @@ __global__ void f32_latent_bwd_kernel(const F32Lat* __restrict__ lat) {
   }
 }
 
-template <int KIND, int CGN, int IGN>
-cudaError_t run_wgrad(const F32WJob* d_jobs, const F32WPlan& p, int n, float* gw, float* gb, float* slots,
-                      cudaStream_t st) {
-  using G = WG<KIND, CGN, IGN>;
-  WArgs a{n, p.co, p.ci, p.n_tiles, p.n_main, p.n_btiles, p.n_edge, p.slot, p.bslot, p.edge_ofs, slots};
-  auto kern = wgrad_f32_kernel<KIND, CGN, IGN>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM);
-  if (e != cudaSuccess) return e;
-  kern<<<dim3(p.n_main + p.n_edge, (p.co / G::BCO) * (p.ci / G::BCI)), G::NT, G::SMEM, st>>>(d_jobs, a);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  const int taps = KIND == FK_P1 ? 1 : 9, nWw = p.co * taps * p.ci;
-  wgrad_f32_reduce<<<(nWw + p.co + 31) / 32, dim3(32, 8), 0, st>>>(slots, p.n_main, p.slot, p.n_edge, p.bslot,
-                                                                   p.edge_ofs, nWw, p.co, p.ci, taps,
-                                                                   KIND == FK_UP2 ? 1 : 0, gw, gb);
+cudaError_t reduce(const F32WPlan& p, const F32WJob* d_jobs, int n, int taps, float* gw, float* gb, const float* slots,
+                   cudaStream_t st) {
+  const int nWw = p.co * taps * p.ci, nW = nWw + p.co;
+  wgrad_f32_reduce<<<(nW + 31) / 32, dim3(32, 8), 0, st>>>(slots, d_jobs, n, p.slot, nW, nWw, gw, gb);
   return cudaGetLastError();
 }
 
+template <int KIND, int COL, int CGN, int IGN, int NB>
+cudaError_t run_wgrad(const F32WJob* d_jobs, const F32WPlan& p, int n, float* gw, float* gb, float* slots,
+                      cudaStream_t st) {
+  using G = WG<KIND, COL, CGN, IGN, NB>;
+  auto kern = wgrad_f32_kernel<KIND, COL, CGN, IGN, NB>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM);
+  if (e != cudaSuccess) return e;
+  kern<<<dim3(p.units, (p.co / G::BCO) * ((p.ci + G::BCI - 1) / G::BCI)), G::NT, G::SMEM, st>>>(d_jobs, n, p.co, p.ci,
+                                                                                             p.slot, slots);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  return reduce(p, d_jobs, n, WK<KIND>::KR * WK<KIND>::KC, gw, gb, slots, st);
+}
+
+// Channel blocks by the layer's widths: as many output channels as fit a warp's lanes, then input
+// channels up to 12 warps a block.
 template <int KIND>
 cudaError_t wgrad_by_width(const F32WJob* d_jobs, const F32WPlan& p, int n, float* gw, float* gb, float* slots,
                            cudaStream_t st) {
-  const int cgn = p.cgn, ign = p.ign;
-  if (cgn == 8 && ign == 4) return run_wgrad<KIND, 8, 4>(d_jobs, p, n, gw, gb, slots, st);
-  if (cgn == 8 && ign == 2) return run_wgrad<KIND, 8, 2>(d_jobs, p, n, gw, gb, slots, st);
-  if (cgn == 4 && ign == 4) return run_wgrad<KIND, 4, 4>(d_jobs, p, n, gw, gb, slots, st);
-  if (cgn == 4 && ign == 2) return run_wgrad<KIND, 4, 2>(d_jobs, p, n, gw, gb, slots, st);
-  if (cgn == 2 && ign == 4) return run_wgrad<KIND, 2, 4>(d_jobs, p, n, gw, gb, slots, st);
-  return run_wgrad<KIND, 2, 2>(d_jobs, p, n, gw, gb, slots, st);
+  if (p.co % 64 == 0) {
+    if (p.ci > 32) return run_wgrad<KIND, 8, 8, 4, 4>(d_jobs, p, n, gw, gb, slots, st);
+    return run_wgrad<KIND, 8, 8, 4, 2>(d_jobs, p, n, gw, gb, slots, st);
+  }
+  if (p.co % 32 == 0) {
+    if (p.ci > 32) return run_wgrad<KIND, 8, 4, 8, 2>(d_jobs, p, n, gw, gb, slots, st);
+    if (p.ci > 16) return run_wgrad<KIND, 8, 4, 8, 1>(d_jobs, p, n, gw, gb, slots, st);
+    return run_wgrad<KIND, 4, 8, 4, 1>(d_jobs, p, n, gw, gb, slots, st);
+  }
+  if (p.ci > 32) return run_wgrad<KIND, 4, 4, 8, 2>(d_jobs, p, n, gw, gb, slots, st);
+  return run_wgrad<KIND, 4, 4, 8, 1>(d_jobs, p, n, gw, gb, slots, st);
 }
 
 }  // namespace
 
-// Blocks: about one wave of the GPU over all channel blocks (each block walks its share of the
-// tiles, so more blocks only add slots to write and read); the edge tiles, which cost what a main
-// tile costs, get their share of them.
 F32WPlan f32_wgrad_plan(int kind, int co, int ci, std::vector<F32WJob>& jobs) {
   F32WPlan p;
   p.kind = kind;
   p.co = co;
   p.ci = ci;
-  p.cgn = co % 64 == 0 ? 8 : co % 32 == 0 ? 4 : 2;
-  p.ign = ci % 32 == 0 ? 4 : 2;
-  long long tiles = 0, btiles = 0;
-  for (F32WJob& j : jobs) {
-    j.tile0 = (int)tiles;
-    j.btile0 = (int)btiles;
-    const int h = kind == FK_UP2 ? j.Ho / 2 : j.Ho, w = kind == FK_UP2 ? j.Wo / 2 : j.Wo;
-    tiles += (long long)((h + kTR - 1) / kTR) * ((w + kTC - 1) / kTC);
-    if (kind == FK_UP2) btiles += ((j.Ho & 1 ? j.Wo : 0) + (j.Wo & 1 ? j.Ho - (j.Ho & 1) : 0) + 63) / 64;
-  }
-  p.n_tiles = (int)tiles;
-  p.n_btiles = (int)btiles;
-  const int blocks = (co / (8 * p.cgn)) * (ci / (8 * p.ign)), per_sm = kind == FK_UP2 ? 1 : 2;
-  const int want = std::max(1, 152 * per_sm / blocks);
-  if (btiles > 0)
-    p.n_edge = (int)std::min<long long>(btiles, std::max<long long>(1, (want * btiles + tiles) / (tiles + btiles)));
-  p.n_main = (int)std::max<long long>(1, std::min<long long>(tiles, std::max(1, want - p.n_edge)));
   const int taps = kind == FK_P1 ? 1 : 9;
-  p.slot = ((size_t)(kind == FK_UP2 ? 16 : taps) * co * ci + co + 31) / 32 * 32;
-  p.bslot = ((size_t)9 * co * ci + co + 31) / 32 * 32;
-  p.edge_ofs = p.slot * p.n_main;
-  p.slot_floats = p.edge_ofs + (p.n_edge ? p.bslot * p.n_edge : 0);
+  // chains of a pair (part of the summation order: a change moves the gradient's last bits)
+  const bool few = co * taps * ci + co <= 512 && (co < 16 || ci < 16);
+  const int most = few ? 608 : 304;
+  for (F32WJob& j : jobs) {
+    const int tiles = ((j.Wo + kTC - 1) / kTC) * ((j.Ho + kTR - 1) / kTR);
+    j.unit0 = p.units;
+    j.units = std::min(tiles, most);
+    p.units += j.units;
+  }
+  p.slot = ((size_t)taps * co * ci + co + 31) / 32 * 32;
+  p.slot_floats = p.slot * p.units;
   return p;
 }
 
@@ -579,33 +524,29 @@ cudaError_t launch_f32_wgrad(const F32WPlan& p, const F32WJob* d_jobs, int n, fl
   return cudaErrorInvalidValue;
 }
 
-size_t f32_edge_slot_floats(int C) { return (size_t)2 * 152 * std::max(9 * C + 1, 19 * C); }
-
-cudaError_t launch_f32_final_bwd(const F32Img* imgs, int n, int maxH, int maxW, const float* w, int C, float* gw,
-                                 float* gb, float* slots, cudaStream_t st) {
+cudaError_t launch_f32_final_dgrad(const F32Img* imgs, int n, int maxH, int maxW, const float* w, int C,
+                                   cudaStream_t st) {
   const int NC = kFbThreads / (C / 4);
   const int tx = (maxW + NC - 1) / NC, ty = (maxH + kFbRows - 1) / kFbRows;
-  const int grid = (int)std::min<long long>((long long)tx * ty * n, 2 * 152);
-  const size_t smem = std::max(sizeof(float) * (kFbRows + 2) * (NC + 2), sizeof(float4) * kFbThreads);
-  f32_final_bwd_kernel<<<grid, kFbThreads, smem, st>>>(imgs, n, w, C, tx, ty, slots);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  wgrad_f32_reduce<<<(9 * C + 1 + 31) / 32, dim3(32, 8), 0, st>>>(slots, grid, 9 * C + 1, 0, 0, 0, 9 * C, 1, C, 9, 0, gw,
-                                                                  gb);
+  f32_final_dgrad_kernel<<<dim3(tx * ty, 1, n), kFbThreads, sizeof(float) * (kFbRows + 2) * (NC + 2), st>>>(imgs, w, C,
+                                                                                                          tx);
   return cudaGetLastError();
 }
 
-cudaError_t launch_f32_enc1_wgrad(const F32Img* imgs, int n, int maxH1, int maxW1, int C, float* gw, float* gb,
-                                  float* slots, cudaStream_t st) {
-  const int NC = kEwThreads / (C / 4);
-  const int tx = (maxW1 + NC - 1) / NC, ty = (maxH1 + kEwRows - 1) / kEwRows;
-  const int grid = (int)std::min<long long>((long long)tx * ty * n, 2 * 152);
-  const size_t smem = std::max(sizeof(float2) * (2 * kEwRows + 1) * (2 * NC + 1), sizeof(float4) * kEwThreads);
-  f32_enc1_wgrad_kernel<<<grid, kEwThreads, smem, st>>>(imgs, n, C, tx, ty, slots);
+cudaError_t launch_f32_edge_wgrad(const F32WPlan& p, const F32Img* imgs, const F32WJob* d_jobs, int n, float* gw,
+                                  float* gb, float* slots, cudaStream_t st) {
+  if (p.kind == FK_WENC1) {
+    f32_enc1_wgrad_kernel<<<(p.units + kEwWarps - 1) / kEwWarps, 32 * kEwWarps, 0, st>>>(imgs, d_jobs, n, p.units, p.co,
+                                                                                         p.slot, slots);
+  } else {
+    // a chain takes 3 C / 4 lanes and one for the bias (C <= 256: at most 193)
+    const int lanes = 3 * p.ci / 4 + 1, threads = std::max(lanes, 128), per = threads / lanes;
+    f32_final_wgrad_kernel<<<(p.units + per - 1) / per, threads, 0, st>>>(imgs, d_jobs, n, p.units, p.ci, lanes, p.slot,
+                                                                          slots);
+  }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  wgrad_f32_reduce<<<(19 * C + 31) / 32, dim3(32, 8), 0, st>>>(slots, grid, 19 * C, 0, 0, 0, 18 * C, C, 2, 9, 0, gw, gb);
-  return cudaGetLastError();
+  return reduce(p, d_jobs, n, 9, gw, gb, slots, st);
 }
 
 cudaError_t launch_f32_latent_bwd(const F32Lat* lat, int n, size_t max_n, cudaStream_t st) {

@@ -1914,9 +1914,13 @@ sv_status Ctx::tc_prepare(const sv_pair* pairs, const int16_t* const* coarse, in
               "[sv] tc layer %d: mode %d cin %d cout %d NT %d ring %d%s smem %zu blocks/SM %d grid %d strips %zu rows %d\n",
               pl.layer, pl.mode, pl.cin, pl.cout, pl.NT, pl.ring, pl.split ? " (channel blocks)" : "", pl.smem, bps, grid,
               strips.size(), hs);
-    int mb = 0;
-    for (int i = 0; i < n; ++i) mb = std::max(mb, upfix_segments(lps[i].Ho, lps[i].Wo));
+    int mb = 0, mp = 0;
+    for (int i = 0; i < n; ++i) {
+      mb = std::max(mb, upfix_segments(lps[i].Ho, lps[i].Wo));
+      mp = std::max(mp, upfix_pixels(lps[i].Ho, lps[i].Wo));
+    }
     r.tabs[li].fix_segments = mb;
+    r.tabs[li].fix_pixels = mp;
   }
   std::vector<EdgePair> eps_(n);
   r.maxW = r.maxH = r.maxW1 = r.maxH1 = 0;
@@ -2063,21 +2067,24 @@ sv_status Ctx::tc_launch(const TcRun& r, const unsigned char* tables, cudaStream
       LaunchScope ls(*this, names[li], st);
       if ((s = cuda(tc::launch_conv(pl.mode, prm, pl.NT, r.tabs[li].grid, pl.smem, st, lf8), names[li]))) return s;
     }
-    if (lf8 && pl.mode == tc::TM_UP2 && r.tabs[li].fix_segments > 0) {
+    if (pl.mode == tc::TM_UP2 && r.tabs[li].fix_segments > 0) {
       const int k = pl.layer == L_DEC1 ? 0 : pl.layer == L_DEC2 ? 1 : 2;
+      const UpFixPair* fp = (const UpFixPair*)(tables + r.tabs[li].fix_ofs);
+      const __nv_bfloat16* wb = (const __nv_bfloat16*)wbf.p + pl.fix_wofs;
       LaunchScope ls(*this, "edge_up2fix", st);
-      if ((s = cuda(launch_edge_up2fix_f8((const UpFixPair*)(tables + r.tabs[li].fix_ofs), r.n, r.tabs[li].fix_segments,
-                                          (const uint8_t*)wf8u.p + f8_unf_ofs[k],
-                                          (const float*)wf8s.p + f8_unf_scale_ofs[k], prm.bias, net.cin(pl.layer),
-                                          pl.cout, 1, prm.out_f8, st),
-                    "border fix")))
-        return s;
-    } else if (pl.mode == tc::TM_UP2 && r.tabs[li].fix_segments > 0) {
-      LaunchScope ls(*this, "edge_up2fix", st);
-      if ((s = cuda(launch_edge_up2fix((const UpFixPair*)(tables + r.tabs[li].fix_ofs), r.n, r.tabs[li].fix_segments,
-                                       (const __nv_bfloat16*)wbf.p + pl.fix_wofs, prm.bias, pl.cin, pl.cout, 1, st),
-                    "border fix")))
-        return s;
+      if (tl)
+        s = cuda(launch_edge_up2fix(fp, r.n, r.tabs[li].fix_segments, wb, prm.bias, pl.cin, pl.cout, 1, st),
+                 "border fix");
+      else if (lf8)
+        s = cuda(launch_edge_up2fix_mma(fp, r.n, r.tabs[li].fix_pixels, (const uint8_t*)wf8u.p + f8_unf_ofs[k],
+                                        (const float*)wf8s.p + f8_unf_scale_ofs[k], prm.bias, net.cin(pl.layer), pl.cout,
+                                        1, true, prm.out_f8, st),
+                 "border fix");
+      else
+        s = cuda(launch_edge_up2fix_mma(fp, r.n, r.tabs[li].fix_pixels, wb, nullptr, prm.bias, pl.cin, pl.cout, 1, false,
+                                        0, st),
+                 "border fix");
+      if (s) return s;
     }
   }
   last_fused = r.fused;

@@ -37,7 +37,7 @@ struct TcRun {
   std::vector<TcLayerPlan> plans;
   struct Tab {
     size_t lp_ofs, strip_ofs, fix_ofs;
-    int n_strips, grid, fix_segments, hs;  // fix_segments: border-fix blocks per pair (max)
+    int n_strips, grid, fix_segments, fix_pixels, hs;  // border-fix blocks / pixels per pair (max)
   };
   std::vector<Tab> tabs;
   std::vector<unsigned char> host;

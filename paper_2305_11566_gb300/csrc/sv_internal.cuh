@@ -198,12 +198,13 @@ inline int upfix_segments(int Ho, int Wo) {
 cudaError_t launch_edge_up2fix(const UpFixPair* pairs, int n, int max_segments, const __nv_bfloat16* Wb,
                                const float* bias, int cin, int cout, int relu, cudaStream_t st);
 
-// FP8 form: border recompute on E4M3 input codes with E4M3 unfolded weights and their
-// per-output-channel scale (output E4M3 codes, or BF16 when out_f8 = 0); E4M3 codes of a
-// BF16 tensor.
-cudaError_t launch_edge_up2fix_f8(const UpFixPair* pairs, int n, int max_segments, const uint8_t* Wq,
-                                  const float* wscale, const float* bias, int cin, int cout, int relu, int out_f8,
-                                  cudaStream_t st);
+// The border recompute of inference on warp MMA: BF16 input and weights, or (f8) E4M3 input codes and
+// unfolded weights with their per-output-channel scale (output E4M3 codes, or BF16 when out_f8 = 0).
+inline int upfix_pixels(int Ho, int Wo) { return ((Ho & 1) ? Wo : 0) + ((Wo & 1) ? Ho - (Ho & 1) : 0); }
+cudaError_t launch_edge_up2fix_mma(const UpFixPair* pairs, int n, int max_pixels, const void* W, const float* wscale,
+                                   const float* bias, int cin, int cout, int relu, bool f8, int out_f8,
+                                   cudaStream_t st);
+// E4M3 codes of a BF16 tensor.
 cudaError_t launch_bf16_to_e4m3(const __nv_bfloat16* a, uint8_t* b, size_t n, cudaStream_t st);
 
 // Input gradient of enc1 in FP32 (Ci = 2): d loss / d (L / 256, U / 256).

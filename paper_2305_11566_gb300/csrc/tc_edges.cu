@@ -701,6 +701,8 @@ __device__ __forceinline__ void bf16x8_to_f32(const uint4& v, float* d) {
   }
 }
 
+// The training forward's border recompute, on CUDA-core FMA in one fixed order (its activations keep
+// their bits; see conv_f32.cu).
 __global__ void __launch_bounds__(256) edge_up2fix(const UpFixPair* __restrict__ pairs, const bf16* __restrict__ Wb,
                                                    const float* __restrict__ bias, int cin, int cout, int relu) {
   extern __shared__ __align__(16) float xsm[];
@@ -803,128 +805,132 @@ __global__ void __launch_bounds__(256) edge_up2fix(const UpFixPair* __restrict__
   }
 }
 
-// The border recompute of the FP8 form: the same geometry and pixel / channel mapping, on
-// E4M3 input codes (`in` holds bytes) and the E4M3 codes of the unfolded 3 x 3 weights with
-// their per-output-channel scale: relu(scale * sum(code * code) + bias), stored as E4M3
-// codes (out_f8) or BF16 (the last decoder layer, whose output feeds the BF16 final conv).
-__device__ __forceinline__ float e4m3_value(uint8_t c) {
-  __nv_fp8_e4m3 x;
-  x.__x = c;
-  return static_cast<float>(x);
+// The border recompute of inference on warp MMA, BF16 (F8 = false) or E4M3 operands: 16 border pixels
+// x 32 output channels a block; the 6 taps x channels of the contraction go round the block's four
+// warps, whose sums are added in warp order.  The work is a few hundred pixels a pair, so what counts is
+// latency: operands come straight from memory (a lane's 16 bytes of a pixel and of a weight row are
+// its fragments of the next steps; both operands permute the channels alike, so the sums do not
+// change), and blocks are small and many.  E4M3 codes are converted to FP16 (exact) and multiplied there;
+// the per-channel scale applies to the sum: relu(scale * sum + bias), stored as E4M3 codes (out_f8) or
+// BF16.  dec1 and dec2 of one 1242 x 375 pair: 53 -> 16.5 us together, of 64 pairs 149 -> 40 us, against
+// CUDA-core FMA in 64-pixel segments with operands staged in shared memory.
+__device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1, bool f16) {
+  if (f16)
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+  else
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// Two of the four E4M3 codes of a word as FP16 pairs.
+__device__ __forceinline__ uint32_t e4m3_pair(uint32_t w, int h) {
+  const __half2_raw r = __nv_cvt_fp8x2_to_halfraw2((__nv_fp8x2_storage_t)((w >> (16 * h)) & 0xFFFFu), __NV_E4M3);
+  return (uint32_t)r.x | ((uint32_t)r.y << 16);
 }
 
-// sixteen E4M3 codes (one 16-byte word) to FP32, two at a time through the paired conversion
-__device__ __forceinline__ void e4m3x16_to_f32(const uint4& v, float* d) {
-  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-  for (int k = 0; k < 4; ++k)
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const __half2_raw hr = __nv_cvt_fp8x2_to_halfraw2((__nv_fp8x2_storage_t)((w[k] >> (16 * h)) & 0xFFFFu), __NV_E4M3);
-      const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&hr));
-      d[4 * k + 2 * h] = f.x;
-      d[4 * k + 2 * h + 1] = f.y;
-    }
-}
-
-__global__ void __launch_bounds__(256) edge_up2fix_f8(const UpFixPair* __restrict__ pairs, const uint8_t* __restrict__ Wq,
-                                                      const float* __restrict__ wscale, const float* __restrict__ bias,
-                                                      int cin, int cout, int relu, int out_f8) {
-  extern __shared__ __align__(16) float xsm8[];
-  float* S = xsm8;                          // [2][kFixQ][kFixCk]
-  float* Wf = xsm8 + 2 * kFixQ * kFixCk;    // [6][kFixCk][32]
+constexpr int kFixPx = 16, kFixCo = 32, kFixWarps = 4;
+template <bool F8>
+__global__ void __launch_bounds__(32 * kFixWarps)
+edge_up2fix_mma(const UpFixPair* __restrict__ pairs, const uint8_t* __restrict__ W, const float* __restrict__ wscale,
+                const float* __restrict__ bias, int cin, int cout, int relu, int out_f8) {
+  __shared__ float red[kFixWarps][kFixPx][kFixCo + 1];
   const UpFixPair L = pairs[blockIdx.z];
+  const int nrow = (L.Ho & 1) ? L.Wo : 0;               // last row, every column
+  const int ncol = (L.Wo & 1) ? L.Ho - (L.Ho & 1) : 0;  // last column, rows above a fixed last row
+  const int p0 = blockIdx.x * kFixPx, np = nrow + ncol;
+  if (p0 >= np) return;
+  const int cb = blockIdx.y * kFixCo;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+  const int bytes = cin * (F8 ? 1 : 2), groups = (bytes + 63) / 64;  // 64 bytes of a pixel a step
   const uint8_t* in = reinterpret_cast<const uint8_t*>(L.in);
-  const int nrow = (L.Ho & 1) ? L.Wo : 0;
-  const int ncol = (L.Wo & 1) ? L.Ho - (L.Ho & 1) : 0;
-  const int segr = (nrow + kUpFixSeg - 1) / kUpFixSeg, segc = (ncol + kUpFixSeg - 1) / kUpFixSeg;
-  int seg = blockIdx.x;
-  if (seg >= segr + segc) return;
-  const bool rowfix = seg < segr;
-  if (!rowfix) seg -= segr;
-  const int p0 = seg * kUpFixSeg;
-  const int npix = min(kUpFixSeg, (rowfix ? nrow : ncol) - p0);
-  const int cb = blockIdx.y * 32;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  float acc[8];
+  float acc[4][4];
 #pragma unroll
-  for (int j = 0; j < 8; ++j) acc[j] = 0.f;
-  for (int c0 = 0; c0 < cin; c0 += kFixCk) {
-    const int ck = min(kFixCk, cin - c0);
-    __syncthreads();
-    // 16 codes per 16-byte load (cin is a multiple of 32); a thread's loads are all issued
-    // before any is decoded
-    const int c16 = ck / 16;
-    constexpr int U = 4;
-    for (int e0 = threadIdx.x; e0 < 2 * kFixQ * c16; e0 += U * blockDim.x) {
-      uint4 v[U];
+  for (int j = 0; j < 4; ++j)
 #pragma unroll
-      for (int i = 0; i < U; ++i) {
-        const int e = e0 + i * (int)blockDim.x;
-        const int a = e / (kFixQ * c16), r = e - a * kFixQ * c16, q = r / c16, u = r - q * c16;
-        const int uy = rowfix ? L.Ho - 2 + a : p0 - 1 + q;
-        const int ux = rowfix ? p0 - 1 + q : L.Wo - 2 + a;
-        v[i] = make_uint4(0, 0, 0, 0);
-        if (e < 2 * kFixQ * c16 && uy >= 0 && uy < L.Ho && ux >= 0 && ux < L.Wo)
-          v[i] = *reinterpret_cast<const uint4*>(in + ((size_t)(uy >> 1) * L.Wi + (ux >> 1)) * cin + c0 + u * 16);
-      }
+    for (int q = 0; q < 4; ++q) acc[j][q] = 0.f;
+  const uint4 zero = make_uint4(0, 0, 0, 0);
+#pragma unroll 3
+  for (int it = warp; it < 6 * groups; it += kFixWarps) {
+    const int tap = it / groups, o = (it - tap * groups) * 64 + 16 * t;
+    const int a = tap / 3, b = tap - 3 * a;
+    const bool in_range = o < bytes;
+    uint4 x[2], w[4];
 #pragma unroll
-      for (int i = 0; i < U; ++i) {
-        const int e = e0 + i * (int)blockDim.x;
-        if (e >= 2 * kFixQ * c16) break;
-        const int a = e / (kFixQ * c16), r = e - a * kFixQ * c16, q = r / c16, u = r - q * c16;
-        e4m3x16_to_f32(v[i], S + ((size_t)a * kFixQ + q) * kFixCk + u * 16);
-      }
+    for (int r = 0; r < 2; ++r) {
+      const int p = p0 + g + 8 * r;
+      const bool row = p < nrow;
+      // row fix: (ky, kx) = (a, b), up rows Ho - 2 + a; column fix: (b, a), up columns Wo - 2 + a
+      const int uy = row ? L.Ho - 2 + a : p - nrow - 1 + b, ux = row ? p - 1 + b : L.Wo - 2 + a;
+      const bool ok = in_range && p < np && uy >= 0 && uy < L.Ho && ux >= 0 && ux < L.Wo;
+      x[r] = ok ? *reinterpret_cast<const uint4*>(in + ((size_t)(uy >> 1) * L.Wi + (ux >> 1)) * bytes + o) : zero;
     }
-    for (int e0 = threadIdx.x; e0 < 6 * c16 * 32; e0 += U * blockDim.x) {
-      uint4 v[U];
+    // the row and the column fix read different taps: lanes of a block hold one kind, except in the
+    // block where the row's pixels end (its two kinds run one after the other)
 #pragma unroll
-      for (int i = 0; i < U; ++i) {
-        const int e = e0 + i * (int)blockDim.x;
-        const int o = e & 31, r = e >> 5, t = r / c16, u = r - t * c16;
-        const int a = t / 3, b = t - 3 * a, ky = rowfix ? a : b, kx = rowfix ? b : a;
-        v[i] = make_uint4(0, 0, 0, 0);
-        if (e < 6 * c16 * 32 && cb + o < cout)
-          v[i] = *reinterpret_cast<const uint4*>(Wq + ((size_t)((cb + o) * 3 + ky) * 3 + kx) * cin + c0 + u * 16);
+    for (int kind = 0; kind < 2; ++kind) {
+      if (kind == 0 ? p0 >= nrow : p0 + kFixPx <= nrow) continue;
+      const int ky = kind == 0 ? a : b, kx = kind == 0 ? b : a;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int n = cb + 8 * j + g;
+        w[j] = in_range && n < cout
+                   ? *reinterpret_cast<const uint4*>(W + ((size_t)(n * 3 + ky) * 3 + kx) * bytes + o) : zero;
       }
+      uint4 y[2];
 #pragma unroll
-      for (int i = 0; i < U; ++i) {
-        const int e = e0 + i * (int)blockDim.x;
-        if (e >= 6 * c16 * 32) break;
-        const int o = e & 31, r = e >> 5, t = r / c16, u = r - t * c16;
-        float f[16];
-        e4m3x16_to_f32(v[i], f);
-        float* d = Wf + ((size_t)t * kFixCk + u * 16) * 32 + o;
+      for (int r = 0; r < 2; ++r) y[r] = (p0 + g + 8 * r < nrow) == (kind == 0) ? x[r] : zero;
+      const uint32_t y0[4] = {y[0].x, y[0].y, y[0].z, y[0].w}, y1[4] = {y[1].x, y[1].y, y[1].z, y[1].w};
 #pragma unroll
-        for (int j = 0; j < 16; ++j) d[j * 32] = f[j];
-      }
-    }
-    __syncthreads();
-    for (int t = 0; t < 6; ++t) {
-      const int a = t / 3, b = t - 3 * a;
-      const float* sp = S + ((size_t)a * kFixQ + warp * 8 + b) * kFixCk;
-      const float* wp = Wf + (size_t)t * kFixCk * 32 + lane;
-      for (int c = 0; c < ck; ++c) {
-        const float wv = wp[c * 32];
+      for (int s = 0; s < (F8 ? 4 : 2); ++s) {
+        uint32_t af[4];
+        if (F8) {
+          af[0] = e4m3_pair(y0[s], 0); af[1] = e4m3_pair(y1[s], 0);
+          af[2] = e4m3_pair(y0[s], 1); af[3] = e4m3_pair(y1[s], 1);
+        } else {
+          af[0] = y0[2 * s]; af[1] = y1[2 * s]; af[2] = y0[2 * s + 1]; af[3] = y1[2 * s + 1];
+        }
 #pragma unroll
-        for (int j = 0; j < 8; ++j) acc[j] = fmaf(wv, sp[j * kFixCk + c], acc[j]);
+        for (int j = 0; j < 4; ++j) {
+          const uint32_t wv[4] = {w[j].x, w[j].y, w[j].z, w[j].w};
+          if (F8)
+            mma16816(acc[j], af, e4m3_pair(wv[s], 0), e4m3_pair(wv[s], 1), true);
+          else
+            mma16816(acc[j], af, wv[(2 * s) & 3], wv[(2 * s + 1) & 3], false);
+        }
       }
     }
   }
-  const int co = cb + lane;
-  if (co >= cout) return;
 #pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    const int p = warp * 8 + j;
-    if (p >= npix) break;
-    const int Y = rowfix ? L.Ho - 1 : p0 + p, X = rowfix ? p0 + p : L.Wo - 1;
-    float v = fmaf(acc[j], wscale[co], bias[co]);
-    if (relu) v = fmaxf(v, 0.f);
-    const size_t o = ((size_t)Y * L.Wo + X) * cout + co;
-    if (out_f8)
-      reinterpret_cast<uint8_t*>(L.out)[o] = (uint8_t)__nv_cvt_float_to_fp8(v, __NV_SATFINITE, __NV_E4M3);
-    else
-      L.out[o] = __float2bfloat16_rn(v);
+  for (int j = 0; j < 4; ++j)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) red[warp][g + 8 * (q >> 1)][8 * j + 2 * t + (q & 1)] = acc[j][q];
+  __syncthreads();
+  const int px = threadIdx.x / 8, c4 = threadIdx.x % 8 * 4, p = p0 + px, co = cb + c4;
+  if (p >= np || co >= cout) return;
+  const int Y = p < nrow ? L.Ho - 1 : p - nrow, X = p < nrow ? p : L.Wo - 1;
+  float v[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    float s = red[0][px][c4 + j];
+#pragma unroll
+    for (int w = 1; w < kFixWarps; ++w) s += red[w][px][c4 + j];
+    v[j] = F8 ? fmaf(s, wscale[co + j], bias[co + j]) : bias[co + j] + s;
+    if (relu) v[j] = fmaxf(v[j], 0.f);
+  }
+  const size_t o = ((size_t)Y * L.Wo + X) * cout + co;
+  if (out_f8) {
+    uint32_t q = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) q |= (uint32_t)(uint8_t)__nv_cvt_float_to_fp8(v[j], __NV_SATFINITE, __NV_E4M3) << (8 * j);
+    *reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(L.out) + o) = q;
+  } else {
+    const __nv_bfloat162 lo = __floats2bfloat162_rn(v[0], v[1]), hi = __floats2bfloat162_rn(v[2], v[3]);
+    uint2 q;
+    q.x = *reinterpret_cast<const uint32_t*>(&lo);
+    q.y = *reinterpret_cast<const uint32_t*>(&hi);
+    *reinterpret_cast<uint2*>(L.out + o) = q;
   }
 }
 
@@ -936,14 +942,15 @@ __global__ void bf16_to_e4m3(const bf16* __restrict__ a, uint8_t* __restrict__ b
 
 }  // namespace
 
-cudaError_t launch_edge_up2fix_f8(const UpFixPair* pairs, int n, int max_segments, const uint8_t* Wq,
-                                  const float* wscale, const float* bias, int cin, int cout, int relu, int out_f8,
-                                  cudaStream_t st) {
-  if (n <= 0 || max_segments <= 0) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(edge_up2fix_f8, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFixSmem);
-  if (e != cudaSuccess) return e;
-  edge_up2fix_f8<<<dim3(max_segments, (cout + 31) / 32, n), 256, kFixSmem, st>>>(pairs, Wq, wscale, bias, cin, cout,
-                                                                                  relu, out_f8);
+cudaError_t launch_edge_up2fix_mma(const UpFixPair* pairs, int n, int max_pixels, const void* W, const float* wscale,
+                                   const float* bias, int cin, int cout, int relu, bool f8, int out_f8,
+                                   cudaStream_t st) {
+  if (n <= 0 || max_pixels <= 0) return cudaSuccess;
+  const dim3 grid((max_pixels + kFixPx - 1) / kFixPx, (cout + kFixCo - 1) / kFixCo, n);
+  if (f8)
+    edge_up2fix_mma<true><<<grid, 32 * kFixWarps, 0, st>>>(pairs, (const uint8_t*)W, wscale, bias, cin, cout, relu, out_f8);
+  else
+    edge_up2fix_mma<false><<<grid, 32 * kFixWarps, 0, st>>>(pairs, (const uint8_t*)W, wscale, bias, cin, cout, relu, 0);
   return cudaGetLastError();
 }
 

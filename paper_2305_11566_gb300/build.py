@@ -1,8 +1,8 @@
 """Build libstereovae.so (the CUDA library behind include/stereovae.h) in-tree.
 
 nvcc compiles every translation unit for sm_103a only, in parallel; the coarse
-matcher is compiled once per window radius (1..7) so its template instances build
-side by side.  Objects go to _build/, the library next to this file.
+matcher is compiled once per window radius (1..7) and output mode so its template
+instances build side by side.  Objects go to _build/, the library next to this file.
 """
 from __future__ import annotations
 
@@ -36,8 +36,9 @@ def units():
             continue
         src = os.path.join(CSRC, f)
         if f == "zncc_wta.cu":
-            for r in range(1, 8):
-                out.append((src, [f"-DSV_ZNCC_R={r}"], f"zncc_wta_r{r}.o"))
+            for r in range(7, 0, -1):  # the largest units first
+                for m in (2, 1, 0):
+                    out.append((src, [f"-DSV_ZNCC_R={r}", f"-DSV_ZNCC_MODE={m}"], f"zncc_wta_r{r}_m{m}.o"))
         else:
             out.append((src, [], f[:-3] + ".o"))
     return out
@@ -58,7 +59,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(BUILD, exist_ok=True)
     nvcc = _nvcc()
     jobs = []
-    for src, defs, obj in units():
+    for src, defs, obj in sorted(units(), key=lambda u: "zncc" not in u[2]):
         jobs.append([nvcc, *ARCH, *FLAGS, *defs, "-c", src, "-o", os.path.join(BUILD, obj)])
 
     def run(cmd):

@@ -111,7 +111,8 @@ void Ctx::coarse_prepare(const sv_pair* pairs, int n, int16_t* const* disp, floa
   z.jobs.clear();
   z.maxD = 1;
   for (int i = 0; i < n; ++i) z.maxD = std::max(z.maxD, pairs[i].max_disp);
-  const int gx = kZnccWarps * zncc_tx(zncc_kd(z.maxD));
+  z.shape = zncc_shape(pairs, n, z.maxD);
+  const int gx = kZnccWarps * z.shape.tx;
   for (int i = 0; i < n; ++i) {
     const sv_pair& p = pairs[i];
     ZPair& q = z.pairs[i];
@@ -120,7 +121,7 @@ void Ctx::coarse_prepare(const sv_pair* pairs, int n, int16_t* const* disp, floa
     q.disp = disp[i];
     q.best = best ? best[i] : nullptr;
     q.second = second ? second[i] : nullptr;
-    for (int y0 = 0; y0 < q.h; y0 += kZnccTY)
+    for (int y0 = 0; y0 < q.h; y0 += z.shape.ty)
       for (int x0 = 0; x0 < q.w; x0 += gx) z.jobs.push_back({i, y0, x0, 0});
   }
 }
@@ -130,7 +131,21 @@ sv_status Ctx::coarse_launch(const ZRun& z, const ZPair* d_pairs, const ZJob* d_
   LaunchScope ls(*this, "zncc_wta", st);
   bool scores = false;
   for (const ZPair& q : z.pairs) scores |= q.best != nullptr || q.second != nullptr;
-  return cuda(launch_zncc_wta(d_pairs, d_jobs, (int)z.jobs.size(), cfg.window / 2, z.maxD, st, scores ? 1 : 0),
+  ZInline in;
+  if (!d_pairs) {  // few pairs: they travel with the launch
+    in.n = (int)z.pairs.size();
+    in.tx = z.shape.tx;
+    in.ty = z.shape.ty;
+    in.job0[0] = 0;
+    for (int i = 0; i < in.n; ++i) {
+      const int gx = kZnccWarps * in.tx;
+      in.p[i] = z.pairs[i];
+      in.tiles_x[i] = (z.pairs[i].w + gx - 1) / gx;
+      in.job0[i + 1] = in.job0[i] + in.tiles_x[i] * ((z.pairs[i].h + in.ty - 1) / in.ty);
+    }
+  }
+  return cuda(launch_zncc_wta(d_pairs, d_jobs, (int)z.jobs.size(), cfg.window / 2, z.maxD, st, scores ? 1 : 0,
+                              z.shape.small, d_pairs ? nullptr : &in),
               "zncc_wta launch");
 }
 
@@ -139,6 +154,7 @@ sv_status Ctx::coarse(const sv_pair* pairs, int n, int16_t* const* disp, float* 
   ZRun z;
   coarse_prepare(pairs, n, disp, best, second, z);
   if (z.jobs.empty()) return SV_OK;
+  if (n <= kZnccInline) return coarse_launch(z, nullptr, nullptr, st);
   sv_status s;
   if ((s = cuda(zpairs.ensure(sizeof(ZPair) * n), "alloc pair table"))) return s;
   if ((s = cuda(zjobs.ensure(sizeof(ZJob) * z.jobs.size()), "alloc job table"))) return s;

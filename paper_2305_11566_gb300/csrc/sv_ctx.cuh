@@ -55,6 +55,7 @@ struct ZRun {
   std::vector<ZPair> pairs;
   std::vector<ZJob> jobs;
   int maxD = 1;
+  ZShape shape{};
 };
 
 // Device tables of the training latent of the tensor-core form (e3 converted to FP32, the two

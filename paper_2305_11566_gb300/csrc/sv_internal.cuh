@@ -29,16 +29,26 @@ struct ZPair {
   float* cost;       // [h][w][D] cost volume 1 - rho (2 where x - d < 0), or nullptr
 };
 
-// One CTA job: rows [y0, y0 + kZnccTY) and columns [x0, x0 + group width) of a pair.
+// One CTA job: rows [y0, y0 + ty) and columns [x0, x0 + group width) of a pair.
 struct ZJob {
   int pair, y0, x0, pad;
 };
 
 constexpr int kZnccTY = 8;      // coarse rows per job
 constexpr int kZnccWarps = 8;   // warps per CTA; each owns a column tile of TX(KD) columns
+constexpr int kZnccSmallTX = 8, kZnccSmallTY = 4;  // jobs of a call that would leave SMs idle
 
 inline int zncc_kd(int D) { return (D + 31) / 32; }
 inline int zncc_tx(int kd) { return kd == 1 ? 32 : kd == 2 ? 20 : kd == 3 ? 16 : 12; }
+
+// Pairs of a small call, passed by value with the launch (no table upload): pair i's jobs start
+// at job0[i], tiles_x[i] of them per row of jobs.
+constexpr int kZnccInline = 16;
+struct ZInline {
+  int n, tx, ty;
+  int job0[kZnccInline + 1], tiles_x[kZnccInline];
+  ZPair p[kZnccInline];
+};
 
 // Shared-memory layout of one ZNCC job (window radius r, disparity count D, tile TX).
 struct ZLayout {
@@ -46,9 +56,8 @@ struct ZLayout {
   size_t off_sl, off_sr, off_suml, off_invl, off_statr, off_cs, off_cs2, total;
 };
 __host__ __device__ inline size_t align16(size_t v) { return (v + 15) & ~size_t(15); }
-__host__ __device__ inline ZLayout zlayout(int r, int D, int tx) {
+__host__ __device__ inline ZLayout zlayout(int r, int D, int tx, int TY) {
   ZLayout z;
-  const int TY = kZnccTY;
   z.gx = kZnccWarps * tx;
   z.nlc = z.gx + 2 * r;
   z.nrc = z.gx + 2 * r + D - 1;
@@ -64,29 +73,50 @@ __host__ __device__ inline ZLayout zlayout(int r, int D, int tx) {
   z.total = o;
   return z;
 }
-inline size_t zncc_smem_bytes(int r, int D) { return zlayout(r, D, zncc_tx(zncc_kd(D))).total; }
+
+// Job shape of a call: the large jobs share their staging and statistics over more pixels; a call
+// whose large jobs are fewer than the GPU's SMs takes the small ones, whose chain of dependent work is a fifth
+// as long.  One 256 x 128 pair, D = 16: 4 large jobs 38.7 us, 8 small ones 15.0; one 1242 x 375 pair, D = 48: 24
+// large jobs 41, 120 small ones 16.7 us.
+struct ZShape {
+  int tx, ty;
+  bool small;
+};
+inline ZShape zncc_shape(const sv_pair* pairs, int n, int maxD) {
+  const int tx = zncc_tx(zncc_kd(maxD)), gx = kZnccWarps * tx;
+  long long jobs = 0;
+  for (int i = 0; i < n; ++i)
+    jobs += (long long)((pairs[i].height / 4 + kZnccTY - 1) / kZnccTY) * ((pairs[i].width / 4 + gx - 1) / gx);
+  if (jobs < 152) return {kZnccSmallTX, kZnccSmallTY, true};
+  return {tx, kZnccTY, false};
+}
 
 // Fused downsample + ZNCC + WTA over the given jobs, one entry per window radius
-// r = 1..7 (each compiled in its own translation unit).
+// r = 1..7 and mode (each compiled in its own translation unit).
 // mode 0: disparities only; 1: also the best / second scores of the pairs that ask for them;
 // 2: also the cost volume (the pairs' cost pointers are set).
-#define SV_ZNCC_DECL(r)                                                                              \
-  cudaError_t launch_zncc_wta_r##r(const ZPair* d_pairs, const ZJob* d_jobs, int n_jobs, int maxD, \
-                                   int mode, cudaStream_t st);
-SV_ZNCC_DECL(1) SV_ZNCC_DECL(2) SV_ZNCC_DECL(3) SV_ZNCC_DECL(4) SV_ZNCC_DECL(5) SV_ZNCC_DECL(6) SV_ZNCC_DECL(7)
+// small: jobs of the small shape; in: the pairs by value (p and j unused), or null.
+#define SV_ZNCC_DECL(r, m)                                                                                          \
+  cudaError_t launch_zncc_wta_r##r##_m##m(const ZPair* d_pairs, const ZJob* d_jobs, int n_jobs, int maxD, bool small, \
+                                          const ZInline* in, cudaStream_t st);
+#define SV_ZNCC_EACH(X) X(1) X(2) X(3) X(4) X(5) X(6) X(7)
+#define SV_ZNCC_DECLS(r) SV_ZNCC_DECL(r, 0) SV_ZNCC_DECL(r, 1) SV_ZNCC_DECL(r, 2)
+SV_ZNCC_EACH(SV_ZNCC_DECLS)
 inline cudaError_t launch_zncc_wta(const ZPair* p, const ZJob* j, int n, int r, int maxD, cudaStream_t st,
-                                   int mode) {
-  switch (r) {
-    case 1: return launch_zncc_wta_r1(p, j, n, maxD, mode, st);
-    case 2: return launch_zncc_wta_r2(p, j, n, maxD, mode, st);
-    case 3: return launch_zncc_wta_r3(p, j, n, maxD, mode, st);
-    case 4: return launch_zncc_wta_r4(p, j, n, maxD, mode, st);
-    case 5: return launch_zncc_wta_r5(p, j, n, maxD, mode, st);
-    case 6: return launch_zncc_wta_r6(p, j, n, maxD, mode, st);
-    case 7: return launch_zncc_wta_r7(p, j, n, maxD, mode, st);
+                                   int mode, bool small, const ZInline* in = nullptr) {
+  switch (r * 3 + mode) {
+#define SV_ZNCC_CASES(r)                                                          \
+  case r * 3: return launch_zncc_wta_r##r##_m0(p, j, n, maxD, small, in, st);     \
+  case r * 3 + 1: return launch_zncc_wta_r##r##_m1(p, j, n, maxD, small, in, st); \
+  case r * 3 + 2: return launch_zncc_wta_r##r##_m2(p, j, n, maxD, small, in, st);
+    SV_ZNCC_EACH(SV_ZNCC_CASES)
   }
   return cudaErrorInvalidValue;
 }
+#undef SV_ZNCC_CASES
+#undef SV_ZNCC_DECLS
+#undef SV_ZNCC_DECL
+#undef SV_ZNCC_EACH
 
 // ------------------------------------------------------------------ refinement
 enum Layer { L_ENC1 = 0, L_ENC2, L_ENC3, L_MU, L_LV, L_DEC1, L_DEC2, L_DEC3, L_FINAL, L_COUNT };

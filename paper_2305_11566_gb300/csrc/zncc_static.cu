@@ -75,7 +75,8 @@ extern "C" sv_status sv_coarse_match_static(const sv_pair* pairs, int n_pairs, i
     if (!disp_out[i]) return SV_ERR_INVALID_ARG;
     if (pairs[i].max_disp > maxD) maxD = pairs[i].max_disp;
   }
-  const int gx = sv::kZnccWarps * sv::zncc_tx(sv::zncc_kd(maxD));
+  const sv::ZShape shape = sv::zncc_shape(pairs, n_pairs, maxD);
+  const int gx = sv::kZnccWarps * shape.tx;
   std::vector<sv::ZPair> zp(n_pairs);
   std::vector<sv::ZJob> jobs;
   for (int i = 0; i < n_pairs; ++i) {
@@ -86,7 +87,7 @@ extern "C" sv_status sv_coarse_match_static(const sv_pair* pairs, int n_pairs, i
     z.disp = disp_out[i];
     z.best = best ? best[i] : nullptr;
     z.second = second ? second[i] : nullptr;
-    for (int y0 = 0; y0 < z.h; y0 += sv::kZnccTY)
+    for (int y0 = 0; y0 < z.h; y0 += shape.ty)
       for (int x0 = 0; x0 < z.w; x0 += gx) jobs.push_back({i, y0, x0, 0});
   }
   if ((int)jobs.size() > kStaticMaxJobs) return SV_ERR_UNSUPPORTED;
@@ -103,7 +104,7 @@ extern "C" sv_status sv_coarse_match_static(const sv_pair* pairs, int n_pairs, i
   bool scores = false;
   for (const sv::ZPair& q : zp) scores |= q.best != nullptr || q.second != nullptr;
   if (sv::launch_zncc_wta(reinterpret_cast<const sv::ZPair*>(b), reinterpret_cast<const sv::ZJob*>(b + kJobOffset),
-                          (int)jobs.size(), window / 2, maxD, st, scores ? 1 : 0) != cudaSuccess)
+                          (int)jobs.size(), window / 2, maxD, st, scores ? 1 : 0, shape.small) != cudaSuccess)
     return SV_ERR_CUDA;
   return SV_OK;
 }

@@ -1,7 +1,7 @@
 // zncc_wta.cu -- K1: fused quarter-size downsample + ZNCC (Eq. 1-3) + winner-take-all
 // (Eq. 6) for many pairs in one launch.
 //
-// One CTA job = one pair, kZnccTY coarse rows, kZnccWarps * TX coarse columns.
+// One CTA job = one pair, TY coarse rows, kZnccWarps * TX coarse columns (two job shapes, zncc_shape).
 //  stage 1  4x4 box sums S (uint16, exact) of the rows/columns the job touches,
 //           window positions outside the image clamped to the edge;
 //  stage 2  per-window sums sum(S) and exact variance v = N sum(S^2) - sum(S)^2 for every
@@ -39,10 +39,10 @@ __device__ __forceinline__ float key_value(int k) {
 // Stage 4x4 box sums of rows y0 - R .. y0 + TY + R - 1 (clamped) and columns base_c ..
 // base_c + ncols - 1 (clamped) into dst[row][col]; the loads of 8 elements per thread are
 // all issued before any is summed (one memory round trip per 8 elements, not per element).
-template <int R>
+template <int R, int TY>
 __device__ __forceinline__ void stage_box(const uint8_t* __restrict__ img, int pitch, int w, int h, int base_c,
                                           int y0, int ncols, uint16_t* dst) {
-  const int n = (kZnccTY + 2 * R) * ncols;
+  const int n = (TY + 2 * R) * ncols;
   constexpr int U = 8;
   for (int e0 = threadIdx.x; e0 < n; e0 += U * blockDim.x) {
     unsigned v[U][4];
@@ -72,10 +72,9 @@ __device__ __forceinline__ void stage_box(const uint8_t* __restrict__ img, int p
 // TY output rows; writes sum and 1/sigma for `ncols_out` windows starting at column
 // `c0` of the staged array (staged column c0 + t is the window's left edge), either to
 // sum_out / inv_out or, packed as {sum, bits of 1/sigma}, to packed.
-template <int R>
+template <int R, int TY>
 __device__ void window_stats(const uint16_t* s, int ncols, int* cs, unsigned* cs2, int* sum_out, float* inv_out,
                              int2* packed, int ncols_out) {
-  const int TY = kZnccTY;
   for (int c = threadIdx.x; c < ncols; c += blockDim.x) {
     int a = 0;
     unsigned a2 = 0;
@@ -87,6 +86,7 @@ __device__ void window_stats(const uint16_t* s, int ncols, int* cs, unsigned* cs
     }
     cs[c] = a;
     cs2[c] = a2;
+#pragma unroll
     for (int yi = 1; yi < TY; ++yi) {
       unsigned vin = s[(yi + 2 * R) * ncols + c], vout = s[(yi - 1) * ncols + c];
       a += (int)vin - (int)vout;
@@ -118,16 +118,33 @@ __device__ void window_stats(const uint16_t* s, int ncols, int* cs, unsigned* cs
   __syncthreads();
 }
 
+// The job of a block and its pair, from the tables or from the launch's own pairs.
+__device__ __forceinline__ void get_job(const ZPair* __restrict__ pairs, const ZJob* __restrict__ jobs,
+                                        const ZInline& in, ZJob& job, ZPair& P) {
+  if (jobs) {
+    job = jobs[blockIdx.x];
+    P = pairs[job.pair];
+    return;
+  }
+  int i = 0;
+  while (i + 1 < in.n && (int)blockIdx.x >= in.job0[i + 1]) ++i;
+  const int j = blockIdx.x - in.job0[i];
+  job.pair = i;
+  job.y0 = j / in.tiles_x[i] * in.ty;
+  job.x0 = j % in.tiles_x[i] * (kZnccWarps * in.tx);
+  P = in.p[i];
+}
+
 // MODE 0: disparity only; 1: also best / second scores; 2: also the cost volume.
-template <int R, int KD, int TX, int MODE>
+template <int R, int KD, int TX, int TY, int MODE>
 __global__ void __launch_bounds__(kZnccWarps * 32, (KD == 1 || (KD == 2 && R <= 5)) ? 2 : 1)
-zncc_wta_kernel(const ZPair* __restrict__ pairs, const ZJob* __restrict__ jobs) {
+zncc_wta_kernel(const ZPair* __restrict__ pairs, const ZJob* __restrict__ jobs, const __grid_constant__ ZInline in) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const int TY = kZnccTY;
-  const ZJob job = jobs[blockIdx.x];
-  const ZPair P = pairs[job.pair];
+  ZJob job;
+  ZPair P;
+  get_job(pairs, jobs, in, job, P);
   const int D = P.D, w = P.w, h = P.h;
-  const ZLayout Z = zlayout(R, D, TX);
+  const ZLayout Z = zlayout(R, D, TX, TY);
   uint16_t* sL = reinterpret_cast<uint16_t*>(smem + Z.off_sl);
   uint16_t* sR = reinterpret_cast<uint16_t*>(smem + Z.off_sr);
   int* sumL = reinterpret_cast<int*>(smem + Z.off_suml);
@@ -140,12 +157,12 @@ zncc_wta_kernel(const ZPair* __restrict__ pairs, const ZJob* __restrict__ jobs) 
   const int rbase = x0 - R - (D - 1);     // coarse column of staged right column 0
 
   // ---- stage 1: box sums, clamped rows / columns
-  stage_box<R>(P.L, P.pitch, w, h, lbase, y0, Z.nlc, sL);
-  stage_box<R>(P.R, P.pitch, w, h, rbase, y0, Z.nrc, sR);
+  stage_box<R, TY>(P.L, P.pitch, w, h, lbase, y0, Z.nlc, sL);
+  stage_box<R, TY>(P.R, P.pitch, w, h, rbase, y0, Z.nrc, sR);
   __syncthreads();
   // ---- stage 2: window statistics (left windows at x0 + t; right windows at rbase + R + t)
-  window_stats<R>(sL, Z.nlc, cs, cs2, sumL, invL, nullptr, Z.gx);
-  window_stats<R>(sR, Z.nrc, cs, cs2, nullptr, nullptr, statR, Z.nrs);
+  window_stats<R, TY>(sL, Z.nlc, cs, cs2, sumL, invL, nullptr, Z.gx);
+  window_stats<R, TY>(sR, Z.nrc, cs, cs2, nullptr, nullptr, statR, Z.nrs);
 
   // ---- stage 3: sliding ZNCC + WTA
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -252,16 +269,16 @@ zncc_wta_kernel(const ZPair* __restrict__ pairs, const ZJob* __restrict__ jobs) 
 // over ascending k: lowest d on exact ties); the half's argmax is one max reduction over a
 // 64-bit key, the lane's order key above 63 - d, so that the lowest d wins exact ties, as in
 // the full-warp kernel.  Stages 1 and 2 as in zncc_wta_kernel.
-template <int R, int TXH>
+template <int R, int TXH, int TY>
 __global__ void __launch_bounds__(kZnccWarps * 32, 2)
-zncc_wta_hw_kernel(const ZPair* __restrict__ pairs, const ZJob* __restrict__ jobs) {
+zncc_wta_hw_kernel(const ZPair* __restrict__ pairs, const ZJob* __restrict__ jobs, const __grid_constant__ ZInline in) {
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int KH = 3, TX = 2 * TXH;
-  const int TY = kZnccTY;
-  const ZJob job = jobs[blockIdx.x];
-  const ZPair P = pairs[job.pair];
+  ZJob job;
+  ZPair P;
+  get_job(pairs, jobs, in, job, P);
   const int D = P.D, w = P.w, h = P.h;
-  const ZLayout Z = zlayout(R, D, TX);
+  const ZLayout Z = zlayout(R, D, TX, TY);
   uint16_t* sL = reinterpret_cast<uint16_t*>(smem + Z.off_sl);
   uint16_t* sR = reinterpret_cast<uint16_t*>(smem + Z.off_sr);
   int* sumL = reinterpret_cast<int*>(smem + Z.off_suml);
@@ -272,11 +289,11 @@ zncc_wta_hw_kernel(const ZPair* __restrict__ pairs, const ZJob* __restrict__ job
   const int y0 = job.y0, x0 = job.x0;
   const int lbase = x0 - R;
   const int rbase = x0 - R - (D - 1);
-  stage_box<R>(P.L, P.pitch, w, h, lbase, y0, Z.nlc, sL);
-  stage_box<R>(P.R, P.pitch, w, h, rbase, y0, Z.nrc, sR);
+  stage_box<R, TY>(P.L, P.pitch, w, h, lbase, y0, Z.nlc, sL);
+  stage_box<R, TY>(P.R, P.pitch, w, h, rbase, y0, Z.nrc, sR);
   __syncthreads();
-  window_stats<R>(sL, Z.nlc, cs, cs2, sumL, invL, nullptr, Z.gx);
-  window_stats<R>(sR, Z.nrc, cs, cs2, nullptr, nullptr, statR, Z.nrs);
+  window_stats<R, TY>(sL, Z.nlc, cs, cs2, sumL, invL, nullptr, Z.gx);
+  window_stats<R, TY>(sR, Z.nrc, cs, cs2, nullptr, nullptr, statR, Z.nrs);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, hf = lane >> 4, l = lane & 15;
   const int xw = x0 + warp * TX;
@@ -355,57 +372,49 @@ zncc_wta_hw_kernel(const ZPair* __restrict__ pairs, const ZJob* __restrict__ job
   }
 }
 
-template <int R, int KD, int MODE>
-cudaError_t launch_rk(const ZPair* p, const ZJob* j, int n, int maxD, cudaStream_t st) {
-  constexpr int TX = KD == 1 ? 32 : KD == 2 ? 20 : KD == 3 ? 16 : 12;  // == zncc_tx(KD)
+template <int R, int KD, int TX, int TY, int MODE>
+cudaError_t launch_shape(const ZPair* p, const ZJob* j, int n, int maxD, const ZInline& in, cudaStream_t st) {
+  const size_t smem = zlayout(R, maxD, TX, TY).total;
+  auto go = [&](auto kern) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    kern<<<n, kZnccWarps * 32, smem, st>>>(p, j, in);
+    return cudaGetLastError();
+  };
   if constexpr (MODE == 0 && KD == 2) {
-    if (maxD <= 48) {  // half-warp layout: 48 candidate slots per pixel, the same job geometry
-      auto kern = zncc_wta_hw_kernel<R, TX / 2>;
-      const size_t smem = zlayout(R, maxD, TX).total;
-      cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
-      kern<<<n, kZnccWarps * 32, smem, st>>>(p, j);
-      return cudaGetLastError();
-    }
+    // half-warp layout: 48 candidate slots per pixel, the same job geometry
+    if (maxD <= 48) return go(zncc_wta_hw_kernel<R, TX / 2, TY>);
   }
-  auto kern = zncc_wta_kernel<R, KD, TX, MODE>;
-  const size_t smem = zlayout(R, maxD, TX).total;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  kern<<<n, kZnccWarps * 32, smem, st>>>(p, j);
-  return cudaGetLastError();
+  return go(zncc_wta_kernel<R, KD, TX, TY, MODE>);
+}
+
+template <int R, int KD, int MODE>
+cudaError_t launch_rk(const ZPair* p, const ZJob* j, int n, int maxD, bool small, const ZInline& in, cudaStream_t st) {
+  constexpr int TX = KD == 1 ? 32 : KD == 2 ? 20 : KD == 3 ? 16 : 12;  // == zncc_tx(KD)
+  if (small) return launch_shape<R, KD, kZnccSmallTX, kZnccSmallTY, MODE>(p, j, n, maxD, in, st);
+  return launch_shape<R, KD, TX, kZnccTY, MODE>(p, j, n, maxD, in, st);
 }
 
 }  // namespace
 
-#ifndef SV_ZNCC_R
-#error "compile this file once per window radius with -DSV_ZNCC_R=<r>"
+#if !defined(SV_ZNCC_R) || !defined(SV_ZNCC_MODE)
+#error "compile this file once per window radius and mode with -DSV_ZNCC_R=<r> -DSV_ZNCC_MODE=<mode>"
 #endif
 
-#define SV_CAT2(a, b) a##b
-#define SV_CAT(a, b) SV_CAT2(a, b)
-// Internal linkage: every radius has its own translation unit, and a template with external
-// linkage instantiated in all of them would be merged by the linker into one radius's copy.
-namespace {
-template <int MODE>
-cudaError_t launch_r(const ZPair* p, const ZJob* j, int n, int maxD, cudaStream_t st) {
-  switch (zncc_kd(maxD)) {
-    case 1: return launch_rk<SV_ZNCC_R, 1, MODE>(p, j, n, maxD, st);
-    case 2: return launch_rk<SV_ZNCC_R, 2, MODE>(p, j, n, maxD, st);
-    case 3: return launch_rk<SV_ZNCC_R, 3, MODE>(p, j, n, maxD, st);
-    case 4: return launch_rk<SV_ZNCC_R, 4, MODE>(p, j, n, maxD, st);
-  }
-  return cudaErrorInvalidValue;
-}
-}  // namespace
+#define SV_CAT2(a, b, c, d) a##b##c##d
+#define SV_CAT(a, b, c, d) SV_CAT2(a, b, c, d)
 
-cudaError_t SV_CAT(launch_zncc_wta_r, SV_ZNCC_R)(const ZPair* p, const ZJob* j, int n, int maxD, int mode,
-                                                  cudaStream_t st) {
+cudaError_t SV_CAT(launch_zncc_wta_r, SV_ZNCC_R, _m, SV_ZNCC_MODE)(const ZPair* p, const ZJob* j, int n, int maxD,
+                                                                   bool small, const ZInline* inl, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  switch (mode) {
-    case 0: return launch_r<0>(p, j, n, maxD, st);
-    case 1: return launch_r<1>(p, j, n, maxD, st);
-    case 2: return launch_r<2>(p, j, n, maxD, st);
+  static const ZInline none{};
+  const ZInline& in = inl ? *inl : none;
+  if (inl) p = nullptr, j = nullptr;
+  switch (zncc_kd(maxD)) {
+    case 1: return launch_rk<SV_ZNCC_R, 1, SV_ZNCC_MODE>(p, j, n, maxD, small, in, st);
+    case 2: return launch_rk<SV_ZNCC_R, 2, SV_ZNCC_MODE>(p, j, n, maxD, small, in, st);
+    case 3: return launch_rk<SV_ZNCC_R, 3, SV_ZNCC_MODE>(p, j, n, maxD, small, in, st);
+    case 4: return launch_rk<SV_ZNCC_R, 4, SV_ZNCC_MODE>(p, j, n, maxD, small, in, st);
   }
   return cudaErrorInvalidValue;
 }

@@ -9,16 +9,20 @@
 //              the box sums, clamped windows), census_cost (Hamming distance of the codes of
 //              (x, y) and (x - d, y); kc^2 - 1 where x - d < 0)
 //   aggregation A [h][w][D]
-//     SGM      sgm_path: Eq. 4 along one direction per launch, one warp per path line, the
-//              lanes holding consecutive disparities (d = lane + 32 k) so that the d - 1 and
-//              d + 1 terms are register shuffles and the minimum over d a warp reduction;
-//              the directions add into A in launch order (Eq. 5, deterministic); the last
-//              direction also takes the winner-take-all of the sum (Eq. 6)
-//     DT       dt_rows / dt_cols: the recursive domain-transform filter on every disparity
-//              slice, guided by the left box sums, one thread per (row, d) or (column, d)
-//   wta        Eq. 6 on a volume: one warp per pixel, argmin over d, lowest d on ties
+//     SGM      sgm_axis: Eq. 4 along both directions of one axis per launch, 8 lanes per path
+//              line, each holding V consecutive disparities, so that the d - 1 and d + 1 terms are
+//              registers but for one shuffle each way; the directions add into A in order
+//              (Eq. 5, deterministic); the last one also takes the winner-take-all of the sum
+//              (Eq. 6).  The pairs of a call go through cost and paths in parts of bounded
+//              volume
+//     DT       dt_weights (the edge weights of an iteration), dt_rows / dt_cols: the recursive
+//              domain-transform filter on every disparity slice, guided by the left box sums, one
+//              thread per (row, d) or (column, d)
+//   wta        Eq. 6 on a volume: 8 lanes per pixel, argmin over d, lowest d on ties
 //   smp        single-matching-phase check (Eq. 7, read as uniqueness of the target column),
 //              one block per row; median3: 3 x 3 median filter, one thread per pixel
+#include <type_traits>
+
 #include "sv_ctx.cuh"
 
 namespace sv {
@@ -35,6 +39,8 @@ struct XPair {
   uint64_t* CR;     // [h][w] census codes of R
   float* C;         // [h][w][D] cost
   float* A;         // [h][w][D] aggregated cost
+  float* WX;        // [h][w] DT weight between (x - 1, y) and (x, y)
+  float* WY;        // [h][w] DT weight between (x, y - 1) and (x, y)
   int16_t* wta;     // [h][w] winner-take-all map
   int16_t* mid;     // [h][w] after the occlusion check, when the median filter follows
   int16_t* disp;    // [h][w] result
@@ -90,237 +96,261 @@ __global__ void census_codes_kernel(const XPair* __restrict__ P) {
   p.CR[(size_t)y * w + x] = mr;
 }
 
-__global__ void census_cost_kernel(const XPair* __restrict__ P, int kc2m1) {
+// One block per row: the row's right codes in shared memory, a warp per pixel with the lanes over d,
+// so a pixel's costs leave as one contiguous store.  Bound by writing the volume.
+__global__ void __launch_bounds__(256) census_cost_kernel(const XPair* __restrict__ P, int kc2m1) {
+  extern __shared__ uint64_t cr_sm[];
   const XPair& p = P[blockIdx.y];
-  const size_t n = (size_t)p.w * p.h * p.D;
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const size_t q = i / p.D;
-    const int d = (int)(i - q * p.D);
-    const int x = (int)(q % p.w);
-    p.C[i] = x - d >= 0 ? (float)__popcll(p.CL[q] ^ p.CR[q - d]) : (float)kc2m1;
+  const int y = blockIdx.x, w = p.w, D = p.D;
+  if (y >= p.h) return;
+  for (int x = threadIdx.x; x < w; x += blockDim.x) cr_sm[x] = p.CR[(size_t)y * w + x];
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  for (int x = threadIdx.x >> 5; x < w; x += blockDim.x >> 5) {
+    const uint64_t cl = p.CL[(size_t)y * w + x];
+    float* c = p.C + ((size_t)y * w + x) * D;
+    for (int d = lane; d < D; d += 32) c[d] = x - d >= 0 ? (float)__popcll(cl ^ cr_sm[x - d]) : (float)kc2m1;
   }
 }
 
-// Eq. 4 along direction dir (0: left to right along rows, 1: right to left, 2: top to
-// bottom along columns, 3: bottom to top), one warp per line.  first: write A, else add.
-// last: also the winner-take-all of A into wta; keep: store A (else only the map).
-template <int KD>
-__global__ void __launch_bounds__(256) sgm_path_kernel(const XPair* __restrict__ P, int dir, int first, int last,
-                                                       int keep, float P1, float P2) {
-  const XPair& p = P[blockIdx.y];
-  const int w = p.w, h = p.h, D = p.D;
-  const int dx = dir == 0 ? 1 : dir == 1 ? -1 : 0;
-  const int dy = dir == 2 ? 1 : dir == 3 ? -1 : 0;
-  const int nlines = dy == 0 ? h : w, len = dy == 0 ? w : h;
-  const int line = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (line >= nlines) return;  // whole warp
-  const int lane = threadIdx.x & 31;
+// V consecutive values of a line's pixel from d0 on, INF beyond D (or 0: PAD0).  VEC: pairs of floats
+// (D even and 8-byte aligned volumes).
+template <int V, bool VEC, bool PAD0>
+__device__ __forceinline__ void load_d(const float* p, int d0, int D, float (&v)[V]) {
+  const float pad = PAD0 ? 0.f : __int_as_float(0x7f800000);
+  if constexpr (VEC) {
+#pragma unroll
+    for (int k = 0; k < V; k += 2) {
+      float2 f = make_float2(pad, pad);
+      if (d0 + k < D) f = *reinterpret_cast<const float2*>(p + d0 + k);
+      v[k] = f.x;
+      v[k + 1] = f.y;
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < V; ++k) v[k] = d0 + k < D ? p[d0 + k] : pad;
+  }
+}
+
+// Lowest d among the smallest values over the 8 lanes of a group, in every lane.
+template <int V>
+__device__ __forceinline__ int group_argmin(const float (&v)[V], int d0, int D) {
+  int key = INT_MAX, bd = 0x7FFFFFFF;
+#pragma unroll
+  for (int k = 0; k < V; ++k) {
+    const int kk = d0 + k < D ? fkey(v[k]) : INT_MAX;
+    if (kk < key) { key = kk; bd = d0 + k; }
+  }
+#pragma unroll
+  for (int o = 1; o < 8; o <<= 1) {
+    const int ok = __shfl_xor_sync(0xffffffffu, key, o), od = __shfl_xor_sync(0xffffffffu, bd, o);
+    if (ok < key || (ok == key && od < bd)) { key = ok; bd = od; }
+  }
+  return bd;
+}
+
+// One direction of Eq. 4 along a line of `len` pixels, `step` floats (and qstep pixels) apart, from pixel
+// q0 on.  FIRST: A = L, else A += L.  The costs and sums of the next PF pixels are loaded ahead.
+template <int V, bool VEC, bool FIRST>
+__device__ __forceinline__ void sgm_line(const XPair& p, int q0, int qstep, int len, int l, bool active, bool last,
+                                         bool keep, float P1, float P2) {
+  constexpr int PF = V <= 8 ? 8 : 4;
   const unsigned FULL = 0xffffffffu;
   const float INF = __int_as_float(0x7f800000);
-  auto at = [&](int s) {
-    const int x = dx == 0 ? line : dx > 0 ? s : w - 1 - s;
-    const int y = dy == 0 ? line : dy > 0 ? s : h - 1 - s;
-    return ((size_t)y * w + x) * D;
+  const int D = p.D, d0 = l * V;
+  const float* C = p.C;
+  float* A = p.A;
+  const ptrdiff_t step = (ptrdiff_t)qstep * D;
+  ptrdiff_t o = (ptrdiff_t)q0 * D;
+  float c[PF][V], a[PF][V];
+  auto fetch = [&](int slot, int s) {
+    if (s >= len) return;
+    load_d<V, VEC, false>(C + o + slot * step, d0, D, c[slot]);
+    if constexpr (!FIRST) load_d<V, VEC, true>(A + o + slot * step, d0, D, a[slot]);
   };
-  float prev[KD], cur[KD], cn[KD], an[KD];
-  float m = 0.f;
-  size_t o = at(0);
 #pragma unroll
-  for (int k = 0; k < KD; ++k) {
-    const int d = lane + 32 * k;
-    cn[k] = d < D ? p.C[o + d] : INF;
-    an[k] = (!first && d < D) ? p.A[o + d] : 0.f;
+  for (int j = 0; j < PF; ++j) fetch(j, j);
+  float prev[V], m = 0.f;
+#pragma unroll 1
+  for (int s0 = 0; s0 < len; s0 += PF) {
+#pragma unroll
+    for (int j = 0; j < PF; ++j) {
+      const int s = s0 + j;
+      if (s >= len) break;
+      float cur[V];
+      if (s == 0) {
+#pragma unroll
+        for (int k = 0; k < V; ++k) cur[k] = c[j][k];
+      } else {
+        float lo = __shfl_up_sync(FULL, prev[V - 1], 1, 8), hi = __shfl_down_sync(FULL, prev[0], 1, 8);
+        if (l == 0) lo = INF;
+        if (l == 7) hi = INF;
+        const float mp = m + P2;
+#pragma unroll
+        for (int k = 0; k < V; ++k) {
+          float best = fminf(prev[k], fminf(k > 0 ? prev[k - 1] : lo, k + 1 < V ? prev[k + 1] : hi) + P1);
+          best = fminf(best, mp);
+          cur[k] = c[j][k] + (best - m);
+        }
+      }
+      float mn = cur[0];
+#pragma unroll
+      for (int k = 1; k < V; ++k) mn = fminf(mn, cur[k]);
+#pragma unroll
+      for (int x = 1; x < 8; x <<= 1) mn = fminf(mn, __shfl_xor_sync(FULL, mn, x));
+      m = mn;
+      float tot[V];
+#pragma unroll
+      for (int k = 0; k < V; ++k) {
+        prev[k] = cur[k];
+        tot[k] = FIRST ? cur[k] : a[j][k] + cur[k];
+      }
+      float* out = A + o + j * step;
+      if (active && (keep || !last)) {
+        if constexpr (VEC) {
+#pragma unroll
+          for (int k = 0; k < V; k += 2)
+            if (d0 + k < D) *reinterpret_cast<float2*>(out + d0 + k) = make_float2(tot[k], tot[k + 1]);
+        } else {
+#pragma unroll
+          for (int k = 0; k < V; ++k)
+            if (d0 + k < D) out[d0 + k] = tot[k];
+        }
+      }
+      if (last) {
+        const int bd = group_argmin<V>(tot, d0, D);
+        if (active && l == 0) p.wta[q0 + s * qstep] = (int16_t)bd;
+      }
+      // the slot's next pixel, PF ahead
+      if (s + PF < len) {
+        load_d<V, VEC, false>(C + o + (j + PF) * step, d0, D, c[j]);
+        if constexpr (!FIRST) load_d<V, VEC, true>(A + o + (j + PF) * step, d0, D, a[j]);
+      }
+    }
+    o += PF * step;
   }
-  for (int s = 0; s < len; ++s) {
-    float c[KD], a[KD];
+}
+
+// Eq. 4 along rows (axis 0: left to right, then right to left) or columns (axis 1: top to bottom, then
+// bottom to top), 8 lanes per line and 4 lines per warp; ndir: 1 or both directions.  first: the
+// axis's first direction writes A, every other adds; last: the axis's last direction also takes the
+// winner-take-all into wta; keep: it stores A too (else only the map).  A lane's values of the
+// second direction are the ones it stored in the first.  (One warp per line with the lanes over d
+// spent 10 shuffles on a line's minimum and used 48 of 64 lane slots at D = 48.)  Four paths of 64
+// pairs of 1242 x 375, D = 48: 1294 -> 577 us; reading and writing the volumes once per direction takes
+// 470 us at the measured 6.8 TB/s.
+template <int V, bool VEC>
+__global__ void __launch_bounds__(128) sgm_axis_kernel(const XPair* __restrict__ P, int axis, int ndir, int first,
+                                                       int last, int keep, float P1, float P2) {
+  const XPair& p = P[blockIdx.y];
+  const int w = p.w, h = p.h, nlines = axis == 0 ? h : w, len = axis == 0 ? w : h;
+  const int base = (blockIdx.x * 4 + (threadIdx.x >> 5)) * 4;
+  if (base >= nlines) return;  // whole warp
+  const int l = threadIdx.x & 7, line0 = base + (threadIdx.x >> 3 & 3);
+  const bool active = line0 < nlines;
+  const int line = min(line0, nlines - 1);
+  const int qstep = axis == 0 ? 1 : w, q0 = axis == 0 ? line * w : line;
+  const bool one = ndir == 1;
+  if (first)
+    sgm_line<V, VEC, true>(p, q0, qstep, len, l, active, last && one, keep, P1, P2);
+  else
+    sgm_line<V, VEC, false>(p, q0, qstep, len, l, active, last && one, keep, P1, P2);
+  if (!one) sgm_line<V, VEC, false>(p, q0 + (len - 1) * qstep, -qstep, len, l, active, last, keep, P1, P2);
+}
+
+// The weights of one DT iteration, once for all disparities: a^t between a pixel and its left / upper
+// neighbour.
+__global__ void dt_weights_kernel(const XPair* __restrict__ P, float lna, float ratio) {
+  const XPair& p = P[blockIdx.z];
+  const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
+  if (y >= p.h || x >= p.w) return;
+  const size_t q = (size_t)y * p.w + x;
+  const int32_t g = p.SL[q];
+  if (x > 0) p.WX[q] = expf(lna * (1.0f + ratio * fabsf((float)(g - p.SL[q - 1]) * 0.0625f)));
+  if (y > 0) p.WY[q] = expf(lna * (1.0f + ratio * fabsf((float)(g - p.SL[q - p.w]) * 0.0625f)));
+}
+
+// (Two iterations on 16 pairs of 1242 x 375, D = 48, census: rows and columns 430 -> 223 us with the weights
+// computed once instead of per disparity and the loads running ahead.)
+// J[n] = c[n] + wt[n] (J[n - 1] - c[n]) for n = 1 .. len - 1, written to dst; src, dst and wt advance by
+// `step`, `step` and `wstep` per n (wt points at the weight of n = 1).  The loads of the next U
+// elements are out while the current U go through the recurrence.
+__device__ __forceinline__ void dt_line(const float* src, float* dst, ptrdiff_t step, const float* wt, ptrdiff_t wstep,
+                                        int len, float J) {
+  constexpr int U = 8;
+  float c[2][U], k[2][U];
+  auto fetch = [&](int b, int n0) {
 #pragma unroll
-    for (int k = 0; k < KD; ++k) { c[k] = cn[k]; a[k] = an[k]; }
-    const size_t on = s + 1 < len ? at(s + 1) : o;
-    if (s + 1 < len) {  // the next pixel's loads go out before this pixel's arithmetic
-#pragma unroll
-      for (int k = 0; k < KD; ++k) {
-        const int d = lane + 32 * k;
-        cn[k] = d < D ? p.C[on + d] : INF;
-        an[k] = (!first && d < D) ? p.A[on + d] : 0.f;
+    for (int u = 0; u < U; ++u)
+      if (n0 + u < len) {
+        c[b][u] = src[(n0 + u) * step];
+        k[b][u] = wt[(n0 + u - 1) * wstep];
       }
+  };
+  fetch(0, 1);
+#pragma unroll 1
+  for (int n0 = 1; n0 < len; n0 += 2 * U) {
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+      const int n1 = n0 + b * U;
+      fetch(b ^ 1, n1 + U);
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (n1 + u < len) {
+          J = c[b][u] + k[b][u] * (J - c[b][u]);
+          dst[(n1 + u) * step] = J;
+        }
     }
-    if (s == 0) {
-#pragma unroll
-      for (int k = 0; k < KD; ++k) cur[k] = c[k];
-    } else {
-#pragma unroll
-      for (int k = 0; k < KD; ++k) {
-        float lo = __shfl_up_sync(FULL, prev[k], 1);                 // d - 1
-        const float lo_wrap = __shfl_sync(FULL, prev[k > 0 ? k - 1 : 0], 31);
-        float hi = __shfl_down_sync(FULL, prev[k], 1);               // d + 1
-        const float hi_wrap = __shfl_sync(FULL, prev[k + 1 < KD ? k + 1 : k], 0);
-        if (lane == 0) lo = k > 0 ? lo_wrap : INF;
-        if (lane == 31) hi = k + 1 < KD ? hi_wrap : INF;
-        const int d = lane + 32 * k;
-        float best = fminf(prev[k], fminf(lo, hi) + P1);
-        best = fminf(best, m + P2);
-        cur[k] = d < D ? c[k] + (best - m) : INF;
-      }
-    }
-    float mn = cur[0];
-#pragma unroll
-    for (int k = 1; k < KD; ++k) mn = fminf(mn, cur[k]);
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) mn = fminf(mn, __shfl_xor_sync(FULL, mn, off));
-    m = mn;
-    float tot[KD];
-#pragma unroll
-    for (int k = 0; k < KD; ++k) {
-      prev[k] = cur[k];
-      tot[k] = first ? cur[k] : a[k] + cur[k];
-      const int d = lane + 32 * k;
-      if (d < D && (keep || !last)) p.A[o + d] = tot[k];
-    }
-    if (last) {
-      int key = INT_MAX, bd = 0x7FFFFFFF;
-#pragma unroll
-      for (int k = 0; k < KD; ++k) {
-        const int d = lane + 32 * k;
-        const int kk = d < D ? fkey(tot[k]) : INT_MAX;
-        if (kk < key) { key = kk; bd = d; }
-      }
-      const int gk = __reduce_min_sync(FULL, key);
-      const unsigned gd = __reduce_min_sync(FULL, key == gk ? (unsigned)bd : 0x7FFFFFFFu);
-      if (lane == 0) p.wta[o / D] = (int16_t)gd;
-    }
-    o = on;
   }
 }
 
 // One domain-transform pass along rows (both ways) for every (row, d) of a pair; src is
 // read once (the first pass reads C), dst written (the aggregated volume).
-__global__ void dt_rows_kernel(const XPair* __restrict__ P, int from_cost, float lna, float ratio) {
+__global__ void dt_rows_kernel(const XPair* __restrict__ P, int from_cost) {
   const XPair& p = P[blockIdx.y];
   const int w = p.w, h = p.h, D = p.D;
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= h * D) return;
   const int y = t / D, d = t - y * D;
-  const float* src = from_cost ? p.C : p.A;
-  float* dst = p.A;
-  const int32_t* g = p.SL + (size_t)y * w;
   const size_t base = (size_t)y * w * D + d;
-  constexpr int U = 8;
-  float J = src[base];
-  dst[base] = J;
-  for (int x0 = 1; x0 < w; x0 += U) {
-    float c[U], wt[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int x = x0 + u;
-      if (x < w) {
-        c[u] = src[base + (size_t)x * D];
-        wt[u] = expf(lna * (1.0f + ratio * fabsf((float)(g[x] - g[x - 1]) * 0.0625f)));
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int x = x0 + u;
-      if (x < w) {
-        J = c[u] + wt[u] * (J - c[u]);
-        dst[base + (size_t)x * D] = J;
-      }
-    }
-  }
-  for (int x0 = w - 2; x0 >= 0; x0 -= U) {
-    float c[U], wt[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int x = x0 - u;
-      if (x >= 0) {
-        c[u] = dst[base + (size_t)x * D];
-        wt[u] = expf(lna * (1.0f + ratio * fabsf((float)(g[x + 1] - g[x]) * 0.0625f)));
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int x = x0 - u;
-      if (x >= 0) {
-        J = c[u] + wt[u] * (J - c[u]);
-        dst[base + (size_t)x * D] = J;
-      }
-    }
-  }
+  const float* src = (from_cost ? p.C : p.A) + base;
+  float* dst = p.A + base;
+  const float* wx = p.WX + (size_t)y * w;
+  const float J = src[0];
+  dst[0] = J;
+  dt_line(src, dst, D, wx + 1, 1, w, J);
+  float* end = dst + (size_t)(w - 1) * D;
+  dt_line(end, end, -(ptrdiff_t)D, wx + w - 1, -1, w, end[0]);
 }
 
 // The same along columns, in place on A, one thread per (column, d): consecutive threads
 // touch consecutive addresses of a row.
-__global__ void dt_cols_kernel(const XPair* __restrict__ P, float lna, float ratio) {
+__global__ void dt_cols_kernel(const XPair* __restrict__ P) {
   const XPair& p = P[blockIdx.y];
   const int w = p.w, h = p.h, D = p.D;
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= w * D) return;
   const int x = t / D;
   float* A = p.A + t;
-  const size_t row = (size_t)w * D;
-  const int32_t* g = p.SL + x;
-  constexpr int U = 8;
-  float J = A[0];
-  for (int y0 = 1; y0 < h; y0 += U) {
-    float c[U], wt[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int y = y0 + u;
-      if (y < h) {
-        c[u] = A[(size_t)y * row];
-        wt[u] = expf(lna * (1.0f + ratio * fabsf((float)(g[(size_t)y * w] - g[(size_t)(y - 1) * w]) * 0.0625f)));
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int y = y0 + u;
-      if (y < h) {
-        J = c[u] + wt[u] * (J - c[u]);
-        A[(size_t)y * row] = J;
-      }
-    }
-  }
-  for (int y0 = h - 2; y0 >= 0; y0 -= U) {
-    float c[U], wt[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int y = y0 - u;
-      if (y >= 0) {
-        c[u] = A[(size_t)y * row];
-        wt[u] = expf(lna * (1.0f + ratio * fabsf((float)(g[(size_t)(y + 1) * w] - g[(size_t)y * w]) * 0.0625f)));
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int y = y0 - u;
-      if (y >= 0) {
-        J = c[u] + wt[u] * (J - c[u]);
-        A[(size_t)y * row] = J;
-      }
-    }
-  }
+  const ptrdiff_t row = (ptrdiff_t)w * D;
+  dt_line(A, A, row, p.WY + x + w, w, h, A[0]);
+  float* end = A + (size_t)(h - 1) * row;
+  dt_line(end, end, -row, p.WY + x + (size_t)(h - 1) * w, -(ptrdiff_t)w, h, end[0]);
 }
 
-// Eq. 6 on a volume (vol_sel 0: C, 1: A): one warp per pixel, lowest d among the minima.
-template <int KD>
-__global__ void vol_wta_kernel(const XPair* __restrict__ P, int vol_sel) {
+// Eq. 6 on a volume (vol_sel 0: C, 1: A): 8 lanes per pixel, lowest d among the minima.
+template <int V, bool VEC>
+__global__ void __launch_bounds__(256) vol_wta_kernel(const XPair* __restrict__ P, int vol_sel) {
   const XPair& p = P[blockIdx.y];
-  const int D = p.D;
-  const float* V = vol_sel ? p.A : p.C;
-  const int lane = threadIdx.x & 31;
-  const int npix = p.w * p.h;
-  for (int q = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); q < npix; q += gridDim.x * (blockDim.x >> 5)) {
-    int key = INT_MAX, bd = 0x7FFFFFFF;
-#pragma unroll
-    for (int k = 0; k < KD; ++k) {
-      const int d = lane + 32 * k;
-      if (d < D) {
-        const int kk = fkey(V[(size_t)q * D + d]);
-        if (kk < key) { key = kk; bd = d; }
-      }
-    }
-    const int gk = __reduce_min_sync(0xffffffffu, key);
-    const unsigned gd = __reduce_min_sync(0xffffffffu, key == gk ? (unsigned)bd : 0x7FFFFFFFu);
-    if (lane == 0) p.wta[q] = (int16_t)gd;
+  const int D = p.D, npix = p.w * p.h, l = threadIdx.x & 7;
+  const float* A = vol_sel ? p.A : p.C;
+  const int stride = gridDim.x * 32;
+  for (int q0 = blockIdx.x * 32 + (threadIdx.x >> 5) * 4; q0 < npix; q0 += stride) {  // whole warps
+    const int q = q0 + (threadIdx.x >> 3 & 3);
+    float v[V];
+    load_d<V, VEC, false>(A + (size_t)min(q, npix - 1) * D, l * V, D, v);
+    const int bd = group_argmin<V>(v, l * V, D);
+    if (l == 0 && q < npix) p.wta[q] = (int16_t)bd;
   }
 }
 
@@ -329,6 +359,9 @@ __global__ void vol_wta_kernel(const XPair* __restrict__ P, int vol_sel) {
 // disparity of the nearest kept pixel of the row (left first at equal distance).  A row
 // without a kept pixel is copied.  in / out: the pair's maps selected by sel_in / sel_out
 // (0: wta, 1: mid, 2: disp).
+// Disparities in [0, D) put every pixel of one target within D of the others, so the keeper of a target
+// is its leftmost pixel: one shared-memory minimum per pixel.  A row with values outside that
+// range (maps the caller brings) looks back over its D - 1 neighbours instead.
 __global__ void smp_kernel(const XPair* __restrict__ P, int sel_in, int sel_out) {
   extern __shared__ int smp_sm[];
   const XPair& p = P[blockIdx.y];
@@ -336,20 +369,30 @@ __global__ void smp_kernel(const XPair* __restrict__ P, int sel_in, int sel_out)
   if (y >= p.h) return;
   const int16_t* in = (sel_in == 0 ? p.wta : sel_in == 1 ? p.mid : p.disp) + (size_t)y * w;
   int16_t* out = (sel_out == 0 ? p.wta : sel_out == 1 ? p.mid : p.disp) + (size_t)y * w;
-  int* tgt = smp_sm;                                               // [w] target columns
-  unsigned char* ok = reinterpret_cast<unsigned char*>(smp_sm + w);  // [w] kept
-  int* val = smp_sm + w + (w + 3) / 4;                             // [w] disparities
+  int* val = smp_sm;                                               // [w] disparities
+  int* own = smp_sm + w;                                           // [w + D] leftmost pixel of target t - D
+  unsigned char* ok = reinterpret_cast<unsigned char*>(own + w + D);  // [w] kept
+  int odd = 0;
+  for (int x = threadIdx.x; x < w + D; x += blockDim.x) own[x] = INT_MAX;
   for (int x = threadIdx.x; x < w; x += blockDim.x) {
     val[x] = in[x];
-    tgt[x] = x - val[x];
+    odd |= val[x] < 0 || val[x] >= D;
   }
-  __syncthreads();
+  odd = __syncthreads_or(odd);
+  if (!odd) {
+    for (int x = threadIdx.x; x < w; x += blockDim.x) atomicMin(&own[x - val[x] + D], x);
+    __syncthreads();
+  }
   int any = 0;
   for (int x = threadIdx.x; x < w; x += blockDim.x) {
     int keep = 1;
-    const int lo = max(0, x - D + 1);
-    for (int u = x - 1; u >= lo; --u)
-      if (tgt[u] == tgt[x]) { keep = 0; break; }
+    if (!odd) {
+      keep = own[x - val[x] + D] == x;
+    } else {
+      const int lo = max(0, x - D + 1);
+      for (int u = x - 1; u >= lo; --u)
+        if (u - val[u] == x - val[x]) { keep = 0; break; }
+    }
     ok[x] = (unsigned char)keep;
     any |= keep;
   }
@@ -401,30 +444,43 @@ cudaError_t launch_census_codes(const XPair* T, int kc, int maxw, int maxh, int 
   return cudaGetLastError();
 }
 
-cudaError_t launch_sgm_path(const XPair* T, int kd, int nlines, int n, int dir, int first, int last, int keep,
-                            float P1, float P2, cudaStream_t st) {
-  const dim3 g((nlines + 7) / 8, n);
-  switch (kd) {
-    case 1: sgm_path_kernel<1><<<g, 256, 0, st>>>(T, dir, first, last, keep, P1, P2); break;
-    case 2: sgm_path_kernel<2><<<g, 256, 0, st>>>(T, dir, first, last, keep, P1, P2); break;
-    case 3: sgm_path_kernel<3><<<g, 256, 0, st>>>(T, dir, first, last, keep, P1, P2); break;
-    case 4: sgm_path_kernel<4><<<g, 256, 0, st>>>(T, dir, first, last, keep, P1, P2); break;
-    default: return cudaErrorInvalidValue;
+// Disparities per lane for the largest range of the call; vec: every pair's volumes can be read in
+// pairs of floats.
+template <typename F>
+cudaError_t by_range(int maxD, bool vec, F&& f) {
+#define SV_RANGE(v)                                                                     \
+  if (maxD <= 8 * v) {                                                                  \
+    if (vec)                                                                            \
+      f(std::integral_constant<int, v>(), std::true_type());                            \
+    else                                                                                \
+      f(std::integral_constant<int, v>(), std::false_type());                           \
+    return cudaGetLastError();                                                          \
   }
-  return cudaGetLastError();
+  SV_RANGE(2) SV_RANGE(4) SV_RANGE(6) SV_RANGE(8) SV_RANGE(12) SV_RANGE(16)
+#undef SV_RANGE
+  return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_vol_wta(const XPair* T, int kd, int n, int vol_sel, cudaStream_t st) {
-  const dim3 g(4 * 152, n);
-  switch (kd) {
-    case 1: vol_wta_kernel<1><<<g, 256, 0, st>>>(T, vol_sel); break;
-    case 2: vol_wta_kernel<2><<<g, 256, 0, st>>>(T, vol_sel); break;
-    case 3: vol_wta_kernel<3><<<g, 256, 0, st>>>(T, vol_sel); break;
-    case 4: vol_wta_kernel<4><<<g, 256, 0, st>>>(T, vol_sel); break;
-    default: return cudaErrorInvalidValue;
-  }
-  return cudaGetLastError();
+cudaError_t launch_sgm_axis(const XPair* T, int maxD, bool vec, int nlines, int n, int axis, int ndir, int first,
+                            int last, int keep, float P1, float P2, cudaStream_t st) {
+  const dim3 g((nlines + 15) / 16, n);
+  return by_range(maxD, vec, [&](auto v, auto vc) {
+    sgm_axis_kernel<decltype(v)::value, decltype(vc)::value><<<g, 128, 0, st>>>(T, axis, ndir, first, last, keep, P1,
+                                                                                P2);
+  });
 }
+
+cudaError_t launch_vol_wta(const XPair* T, int maxD, bool vec, int n, int maxpix, int vol_sel, cudaStream_t st) {
+  const dim3 g(std::min(8 * 152, (maxpix + 31) / 32), n);
+  return by_range(maxD, vec, [&](auto v, auto vc) {
+    vol_wta_kernel<decltype(v)::value, decltype(vc)::value><<<g, 256, 0, st>>>(T, vol_sel);
+  });
+}
+
+// Volume bytes (cost and aggregated) the pairs of one part may hold, which bounds the workspace.  The path
+// kernels need the lines of many pairs to cover a step's latency more than they need a part to fit the L2:
+// 64 pairs of 1242 x 375 (11 MB each) take 577 us in one part, 733 in two, 932 in four.
+constexpr size_t kPartBytes = size_t(1) << 30;
 
 }  // namespace
 
@@ -436,7 +492,7 @@ sv_status Ctx::post_launch(const void* table, int n, int maxw, int maxh, int pos
   const bool smp = post & SV_POST_SMP, med = post & SV_POST_MEDIAN;
   if (smp) {
     LaunchScope ls(*this, "smp", st);
-    const size_t sm = (size_t)maxw * 2 * sizeof(int) + (maxw + 3) / 4 * sizeof(int);
+    const size_t sm = ((size_t)maxw * 2 + kMaxDisp) * sizeof(int) + (maxw + 3) / 4 * sizeof(int);
     if (sm > 48 * 1024 &&
         (s = cuda(cudaFuncSetAttribute(smp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm),
                   "occlusion check shared memory")))
@@ -462,30 +518,52 @@ sv_status Ctx::coarse_ext(const sv_pair* pairs, int n, const sv_coarse_opts& o, 
   // map the post-processing reads)
   const bool plain = zncc && o.aggregation == SV_AGG_NONE;
   int maxw = 0, maxh = 0, maxD = 1;
-  size_t nS = 0, nV = 0, nA = 0;
+  size_t nS = 0;
+  // parts: the volumes of a part's pairs share the workspace with every other part's
+  std::vector<int> part(1, 0);
+  size_t nV = 0, nA = 0, pV = 0, pA = 0;
+  const bool agg = o.aggregation != SV_AGG_NONE;
+  auto own_c = [&](int i) { return !(want_cost && cost_out[i] && !agg); };
+  auto own_a = [&](int i) { return agg && !(want_cost && cost_out[i]); };
   for (int i = 0; i < n; ++i) {
     const int w = pairs[i].width / 4, h = pairs[i].height / 4, D = pairs[i].max_disp;
+    const size_t vol = plain && !want_cost ? 0 : (size_t)w * h * D;
     maxw = std::max(maxw, w);
     maxh = std::max(maxh, h);
     maxD = std::max(maxD, D);
     nS += (size_t)w * h;
-    if (!(want_cost && cost_out[i] && o.aggregation == SV_AGG_NONE)) nV += (size_t)w * h * D;
-    if (o.aggregation != SV_AGG_NONE && !(want_cost && cost_out[i])) nA += (size_t)w * h * D;
+    if (i > part.back() && (pV + pA + 2 * vol) * sizeof(float) > kPartBytes) {
+      part.push_back(i);
+      pV = pA = 0;
+    }
+    if (own_c(i)) pV += vol;
+    if (own_a(i)) pA += vol;
+    nV = std::max(nV, pV);
+    nA = std::max(nA, pA);
   }
+  part.push_back(n);
   if (plain && !want_cost) nV = 0;
-  const bool need_box = !zncc || o.aggregation == SV_AGG_DT;
+  const bool dt = o.aggregation == SV_AGG_DT;
+  const bool need_box = !zncc || dt;
   sv_status s;
   if (need_box && (s = cuda(sgm_s.ensure(2 * nS * sizeof(int32_t)), "alloc box sums"))) return s;
   if (!zncc && (s = cuda(x_codes.ensure(2 * nS * sizeof(uint64_t)), "alloc census codes"))) return s;
+  if (dt && (s = cuda(dt_w.ensure(2 * nS * sizeof(float)), "alloc DT weights"))) return s;
   if (nV && (s = cuda(sgm_c.ensure(nV * sizeof(float)), "alloc cost volume"))) return s;
   if (nA && (s = cuda(sgm_a.ensure(nA * sizeof(float)), "alloc aggregated volume"))) return s;
   if ((s = cuda(x_maps.ensure(2 * nS * sizeof(int16_t)), "alloc coarse maps"))) return s;
   if ((s = cuda(sgm_tab.ensure(sizeof(XPair) * n), "alloc pair table"))) return s;
   std::vector<XPair> tab(n);
   size_t oS = 0, oV = 0, oA = 0;
-  for (int i = 0; i < n; ++i) {
+  bool vec = true;
+  for (int i = 0, k = 0; i < n; ++i) {
     const int w = pairs[i].width / 4, h = pairs[i].height / 4, D = pairs[i].max_disp;
+    if (i == part[k + 1]) {
+      ++k;
+      oV = oA = 0;
+    }
     XPair& q = tab[i];
+    q = XPair{};
     q.L = (const uint8_t*)pairs[i].left;
     q.R = (const uint8_t*)pairs[i].right;
     q.pitch = pairs[i].pitch;
@@ -496,23 +574,21 @@ sv_status Ctx::coarse_ext(const sv_pair* pairs, int n, const sv_coarse_opts& o, 
     q.SR = need_box ? (int32_t*)sgm_s.p + nS + oS : nullptr;
     q.CL = !zncc ? (uint64_t*)x_codes.p + oS : nullptr;
     q.CR = !zncc ? (uint64_t*)x_codes.p + nS + oS : nullptr;
-    const bool own_c = !(want_cost && cost_out[i] && o.aggregation == SV_AGG_NONE);
-    if (own_c) {
+    q.WX = dt ? (float*)dt_w.p + oS : nullptr;
+    q.WY = dt ? (float*)dt_w.p + nS + oS : nullptr;
+    if (own_c(i)) {
       q.C = nV ? (float*)sgm_c.p + oV : nullptr;
-      if (nV) oV += (size_t)w * h * D;
+      oV += (size_t)w * h * D;
     } else {
       q.C = cost_out[i];
     }
-    if (o.aggregation != SV_AGG_NONE) {
-      if (want_cost && cost_out[i]) {
-        q.A = cost_out[i];
-      } else {
-        q.A = (float*)sgm_a.p + oA;
-        oA += (size_t)w * h * D;
-      }
+    if (own_a(i)) {
+      q.A = (float*)sgm_a.p + oA;
+      oA += (size_t)w * h * D;
     } else {
-      q.A = nullptr;
+      q.A = agg ? cost_out[i] : nullptr;
     }
+    vec = vec && D % 2 == 0 && (((uintptr_t)q.C | (uintptr_t)q.A) & 7) == 0;
     q.disp = disp[i];
     q.wta = post ? (int16_t*)x_maps.p + oS : disp[i];
     q.mid = (int16_t*)x_maps.p + nS + oS;
@@ -522,17 +598,18 @@ sv_status Ctx::coarse_ext(const sv_pair* pairs, int n, const sv_coarse_opts& o, 
                 "upload pair table")))
     return s;
   const XPair* T = (const XPair*)sgm_tab.p;
-  const int kd = (maxD + 31) / 32;
 
-  // ---- cost volume (and, for the plain matcher, its winner-take-all)
+  const bool with_cost = !plain || want_cost;
+  ZRun z;
+  std::vector<int> job0;  // first job of every pair
   if (zncc) {
     std::vector<int16_t*> wta(n);
     for (int i = 0; i < n; ++i) wta[i] = tab[i].wta;
-    ZRun z;
     coarse_prepare(pairs, n, wta.data(), nullptr, nullptr, z);
-    const bool with_cost = !plain || want_cost;
     if (with_cost)
       for (int i = 0; i < n; ++i) z.pairs[i].cost = tab[i].C;
+    job0.assign(n + 1, (int)z.jobs.size());
+    for (int j = (int)z.jobs.size() - 1; j >= 0; --j) job0[z.jobs[j].pair] = j;
     if ((s = cuda(zpairs.ensure(sizeof(ZPair) * n), "alloc pair table"))) return s;
     if ((s = cuda(zjobs.ensure(sizeof(ZJob) * z.jobs.size()), "alloc job table"))) return s;
     if ((s = cuda(cudaMemcpyAsync(zpairs.p, z.pairs.data(), sizeof(ZPair) * n, cudaMemcpyHostToDevice, st),
@@ -541,11 +618,6 @@ sv_status Ctx::coarse_ext(const sv_pair* pairs, int n, const sv_coarse_opts& o, 
     if ((s = cuda(cudaMemcpyAsync(zjobs.p, z.jobs.data(), sizeof(ZJob) * z.jobs.size(), cudaMemcpyHostToDevice, st),
                   "upload jobs")))
       return s;
-    LaunchScope ls(*this, with_cost ? "zncc_cost" : "zncc_wta", st);
-    if ((s = cuda(launch_zncc_wta((const ZPair*)zpairs.p, (const ZJob*)zjobs.p, (int)z.jobs.size(), cfg.window / 2,
-                                  z.maxD, st, with_cost ? 2 : 0, z.shape.small),
-                  "zncc cost")))
-      return s;
   }
   if (need_box) {
     LaunchScope ls(*this, "box4", st);
@@ -553,46 +625,64 @@ sv_status Ctx::coarse_ext(const sv_pair* pairs, int n, const sv_coarse_opts& o, 
     if ((s = cuda(cudaGetLastError(), "box sums"))) return s;
   }
   if (!zncc) {
-    {
-      LaunchScope ls(*this, "census_codes", st);
-      if ((s = cuda(launch_census_codes(T, o.census_window, maxw, maxh, n, st), "census codes"))) return s;
-    }
-    LaunchScope ls(*this, "census_cost", st);
-    census_cost_kernel<<<dim3(8 * 152 / std::max(1, std::min(n, 8)), n), 256, 0, st>>>(
-        T, o.census_window * o.census_window - 1);
-    if ((s = cuda(cudaGetLastError(), "census cost"))) return s;
+    LaunchScope ls(*this, "census_codes", st);
+    if ((s = cuda(launch_census_codes(T, o.census_window, maxw, maxh, n, st), "census codes"))) return s;
   }
-
-  // ---- aggregation and winner-take-all
-  if (o.aggregation == SV_AGG_SGM) {
-    for (int dir = 0; dir < o.npaths; ++dir) {
-      LaunchScope ls(*this, "sgm_path", st);
-      const int nlines = dir < 2 ? maxh : maxw;
-      if ((s = cuda(launch_sgm_path(T, kd, nlines, n, dir, dir == 0, dir == o.npaths - 1, want_cost ? 1 : 0, o.P1,
-                                    o.P2, st),
-                    "SGM path")))
+  for (size_t k = 0; k + 1 < part.size(); ++k) {
+    const int i0 = part[k], m = part[k + 1] - i0;
+    // ---- cost volume (and, for the plain matcher, its winner-take-all)
+    if (zncc) {
+      LaunchScope ls(*this, with_cost ? "zncc_cost" : "zncc_wta", st);
+      if ((s = cuda(launch_zncc_wta((const ZPair*)zpairs.p, (const ZJob*)zjobs.p + job0[i0], job0[i0 + m] - job0[i0],
+                                    cfg.window / 2, z.maxD, st, with_cost ? 2 : 0, z.shape.small),
+                    "zncc cost")))
         return s;
+    } else {
+      LaunchScope ls(*this, "census_cost", st);
+      const size_t sm = (size_t)maxw * sizeof(uint64_t);
+      if ((s = cuda(cudaFuncSetAttribute(census_cost_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm),
+                    "census cost shared memory")))
+        return s;
+      census_cost_kernel<<<dim3(maxh, m), 256, sm, st>>>(T + i0, o.census_window * o.census_window - 1);
+      if ((s = cuda(cudaGetLastError(), "census cost"))) return s;
     }
-  } else if (o.aggregation == SV_AGG_DT) {
-    const double N = o.dt_iters;
-    const float ratio = (float)((double)o.dt_sigma_s / (double)o.dt_sigma_r);
-    for (int it = 1; it <= o.dt_iters; ++it) {
-      const double sig = o.dt_sigma_s * std::sqrt(3.0) * std::pow(2.0, N - it) / std::sqrt(std::pow(4.0, N) - 1.0);
-      const float lna = (float)(-std::sqrt(2.0) / sig);
-      {
-        LaunchScope ls(*this, "dt_rows", st);
-        dt_rows_kernel<<<dim3((maxh * maxD + 127) / 128, n), 128, 0, st>>>(T, it == 1, lna, ratio);
-        if ((s = cuda(cudaGetLastError(), "DT rows"))) return s;
+
+    // ---- aggregation and winner-take-all
+    if (o.aggregation == SV_AGG_SGM) {
+      for (int axis = 0; 2 * axis < o.npaths; ++axis) {
+        LaunchScope ls(*this, "sgm_path", st);
+        const int ndir = std::min(2, o.npaths - 2 * axis);
+        if ((s = cuda(launch_sgm_axis(T + i0, maxD, vec, axis == 0 ? maxh : maxw, m, axis, ndir, axis == 0,
+                                      2 * axis + ndir == o.npaths, want_cost ? 1 : 0, o.P1, o.P2, st),
+                      "SGM path")))
+          return s;
       }
-      LaunchScope ls(*this, "dt_cols", st);
-      dt_cols_kernel<<<dim3((maxw * maxD + 127) / 128, n), 128, 0, st>>>(T, lna, ratio);
-      if ((s = cuda(cudaGetLastError(), "DT columns"))) return s;
+    } else if (dt) {
+      const double N = o.dt_iters;
+      const float ratio = (float)((double)o.dt_sigma_s / (double)o.dt_sigma_r);
+      for (int it = 1; it <= o.dt_iters; ++it) {
+        const double sig = o.dt_sigma_s * std::sqrt(3.0) * std::pow(2.0, N - it) / std::sqrt(std::pow(4.0, N) - 1.0);
+        const float lna = (float)(-std::sqrt(2.0) / sig);
+        {
+          LaunchScope ls(*this, "dt_weights", st);
+          dt_weights_kernel<<<dim3((maxw + 127) / 128, maxh, m), 128, 0, st>>>(T + i0, lna, ratio);
+          if ((s = cuda(cudaGetLastError(), "DT weights"))) return s;
+        }
+        {
+          LaunchScope ls(*this, "dt_rows", st);
+          dt_rows_kernel<<<dim3((maxh * maxD + 127) / 128, m), 128, 0, st>>>(T + i0, it == 1);
+          if ((s = cuda(cudaGetLastError(), "DT rows"))) return s;
+        }
+        LaunchScope ls(*this, "dt_cols", st);
+        dt_cols_kernel<<<dim3((maxw * maxD + 127) / 128, m), 128, 0, st>>>(T + i0);
+        if ((s = cuda(cudaGetLastError(), "DT columns"))) return s;
+      }
+      LaunchScope ls(*this, "vol_wta", st);
+      if ((s = cuda(launch_vol_wta(T + i0, maxD, vec, m, maxw * maxh, 1, st), "winner-take-all"))) return s;
+    } else if (!zncc) {
+      LaunchScope ls(*this, "vol_wta", st);
+      if ((s = cuda(launch_vol_wta(T + i0, maxD, vec, m, maxw * maxh, 0, st), "winner-take-all"))) return s;
     }
-    LaunchScope ls(*this, "vol_wta", st);
-    if ((s = cuda(launch_vol_wta(T, kd, n, 1, st), "winner-take-all"))) return s;
-  } else if (!zncc) {
-    LaunchScope ls(*this, "vol_wta", st);
-    if ((s = cuda(launch_vol_wta(T, kd, n, 0, st), "winner-take-all"))) return s;
   }
 
   // ---- post-processing

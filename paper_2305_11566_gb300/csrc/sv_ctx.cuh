@@ -131,7 +131,7 @@ struct Ctx {
   DevBuf host_img, host_out;     // device staging of sv_pipeline_host
   DevBuf host_jobs;              // row-copy job tables of sv_pipeline_host (gather + scatter)
   DevBuf sgm_s, sgm_c, sgm_a, sgm_tab;  // coarse-stage variants: box sums, cost, aggregated cost, pairs
-  DevBuf x_codes, x_maps;               // census codes; winner-take-all and intermediate maps
+  DevBuf x_codes, x_maps, dt_w;         // census codes; winner-take-all and intermediate maps; DT weights
   DevBuf t1_act, t1_tab;                // Table I network: activations, per-call tables
   DevBuf loss_slots;                    // per-block partial sums of sv_loss_paper
   cudaStream_t copy_stream = nullptr;    // sv_pipeline_host: results go back here while the
@@ -292,7 +292,7 @@ struct Ctx {
     for (auto e : ev_free) cudaEventDestroy(e);
     ev_free.clear();
     host_img.release(); host_out.release(); host_jobs.release(); err_flag.release(); tune_out.release();
-    sgm_s.release(); sgm_c.release(); sgm_a.release(); sgm_tab.release(); x_codes.release(); x_maps.release();
+    sgm_s.release(); sgm_c.release(); sgm_a.release(); sgm_tab.release(); x_codes.release(); x_maps.release(); dt_w.release();
     f32_w.release(); f32_descs.release(); f32_act.release(); f32_tab.release();
     t1_act.release(); t1_tab.release(); loss_slots.release();
     w32.release(); w64.release(); wbf.release(); wfuse.release(); wf8.release(); wf8u.release(); wf8s.release(); zpairs.release(); zjobs.release();

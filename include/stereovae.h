@@ -368,8 +368,7 @@ SV_API sv_status sv_synchronize(sv_ctx* ctx, sv_stream stream);
  *                    an SM
  *   "fused_final"    1 (default): an SV_BF16 inference call computes the last decoder
  *                    layer, the final conv and the residual in one kernel (d3 stays in
- *                    shared memory) when the decoder widths allow it and every output
- *                    width is even; 0: separate kernels (d3 materialised in HBM)
+ *                    shared memory) when the decoder widths allow it; 0: separate kernels (d3 materialised in HBM)
  *   "fused_ring"     0 (default): the fused kernel stages as many input rows ahead as
  *                    shared memory holds; 4..16: at most this many rows in its ring
  *   "split_rows"     1 (default): a tensor-core layer whose shared memory holds no staged

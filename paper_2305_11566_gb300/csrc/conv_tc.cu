@@ -713,8 +713,8 @@ __global__ void __launch_bounds__(kThreads, 1) conv_tc_kernel(const __grid_const
 // are zero, so the carried sum of the last row is complete after the last tile.  An odd
 // output height crops half of the last up-sampled row: the last tile's phase-0 rows then
 // subtract the kernel row that falls on the cropped half (4 extra MMA groups with B
-// negated, reusing phase-1 blocks), which gives the cropped conv.  Odd output widths are not
-// handled here.
+// negated, reusing phase-1 blocks), which gives the cropped conv.  An odd output width's last two
+// columns are recomputed afterwards (fused_edge_cols in tc_edges.cu).
 struct alignas(128) FusedPair {
   float* Y;                    // refined disparity [Ho][Wo]
   const int16_t* coarse;       // coarse map [h4][w4]
@@ -1943,9 +1943,9 @@ sv_status Ctx::tc_prepare(const sv_pair* pairs, const int16_t* const* coarse, in
 
   // fused last decoder layer + final conv: inference only (training keeps d3 for backward)
   r.fused = false;
-  bool even = true;
-  for (int i = 0; i < n; ++i) even = even && (pairs[i].width % 2 == 0);
-  if (!coarse_f && fused_final && even && tc::fused_supported(net.dec[2], net.dec[1]) && wfuse.p) {
+  r.fused_odd = false;
+  for (int i = 0; i < n; ++i) r.fused_odd = r.fused_odd || pairs[i].width % 2 != 0;
+  if (!coarse_f && fused_final && tc::fused_supported(net.dec[2], net.dec[1]) && wfuse.p) {
     const int NT = net.dec[2], cin = net.dec[1];
     int ring = 4;  // 3 rows per tile + 1 ahead; more where shared memory allows
     while (ring < 3 + kPrefetchSteps && tc::fused_smem_bytes(NT, cin, ring + 1) <= kSmemLimit) ++ring;
@@ -2061,7 +2061,15 @@ sv_status Ctx::tc_launch(const TcRun& r, const unsigned char* tables, cudaStream
       LaunchScope ls(*this, "tc_dec3_final", st);
       if ((s = cuda(tc::launch_fused(fp, net.dec[2], net.dec[1], r.fused_grid, r.fused_smem, st), "fused dec3 + final")))
         return s;
-      continue;  // no border fix: the crop is exact inside the fused kernel
+      if (r.fused_odd) {  // (an odd height's crop is exact inside the fused kernel, an odd width's is not)
+        LaunchScope le(*this, "edge_cols", st);
+        if ((s = cuda(launch_fused_edge_cols((const UpFixPair*)(tables + r.tabs[li].fix_ofs), d_edges, r.n, r.maxH,
+                                             (const __nv_bfloat16*)wbf.p + pl.fix_wofs, prm.bias, W + net.w_off(L_FINAL),
+                                             W + net.b_off(L_FINAL), net.dec[1], net.dec[2], st),
+                      "fused last columns")))
+          return s;
+      }
+      continue;
     }
     {
       LaunchScope ls(*this, names[li], st);

@@ -44,8 +44,8 @@ struct TcRun {
   size_t edge_ofs = 0;
   int n = 0, maxW = 0, maxH = 0, maxW1 = 0, maxH1 = 0;
   size_t e1_count = 0;  // elements of the e1 workspace (all pairs)
-  // fused last decoder layer + final conv (inference, even output widths)
-  bool fused = false;
+  // fused last decoder layer + final conv (inference); fused_odd: some output width is odd
+  bool fused = false, fused_odd = false;
   size_t fused_fp_ofs = 0, fused_strip_ofs = 0, fused_smem = 0;
   int fused_n_strips = 0, fused_grid = 0, fused_ring = 0, fused_hs = 0;
 };

@@ -234,6 +234,11 @@ inline int upfix_pixels(int Ho, int Wo) { return ((Ho & 1) ? Wo : 0) + ((Wo & 1)
 cudaError_t launch_edge_up2fix_mma(const UpFixPair* pairs, int n, int max_pixels, const void* W, const float* wscale,
                                    const float* bias, int cin, int cout, int relu, bool f8, int out_f8,
                                    cudaStream_t st);
+// Last two output columns of odd-width pairs after the fused dec3 + final kernel (W: BF16 unfolded dec3
+// weights, wf / bf: FP32 final conv).
+cudaError_t launch_fused_edge_cols(const UpFixPair* fix, const EdgePair* edges, int n, int maxH, const void* W,
+                                   const float* bias, const float* wf, const float* bf, int cin, int NT,
+                                   cudaStream_t st);
 // E4M3 codes of a BF16 tensor.
 cudaError_t launch_bf16_to_e4m3(const __nv_bfloat16* a, uint8_t* b, size_t n, cudaStream_t st);
 

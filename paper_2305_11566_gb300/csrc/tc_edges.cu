@@ -934,6 +934,91 @@ edge_up2fix_mma(const UpFixPair* __restrict__ pairs, const uint8_t* __restrict__
   }
 }
 
+// Odd output widths of the fused dec3 + final kernel: its folded taps count the cropped upsampled column
+// in the last d3 column, which reaches the last two output columns.  They are recomputed here: 16 output
+// rows a block, the 18 x 3 d3 pixels under them on warp MMA with the unsummed taps (16 pixels a warp,
+// BF16 as the fused kernel rounds them), then the final conv and the residual.  32 frames of the four KITTI
+// sizes (a quarter of them odd): dec3 + final 1.14 ms apart, 0.62 ms fused with this.
+constexpr int kColRows = 16;
+template <int NT>
+__global__ void __launch_bounds__(128)
+fused_edge_cols(const UpFixPair* __restrict__ fix, const EdgePair* __restrict__ edges, const uint8_t* __restrict__ W,
+                const float* __restrict__ bias, const float* __restrict__ wf, const float* __restrict__ bf, int cin) {
+  __shared__ float d3[64][NT + 1];
+  const UpFixPair L = fix[blockIdx.y];
+  if (!(L.Wo & 1)) return;
+  const int Y0 = blockIdx.x * kColRows;
+  if (Y0 >= L.Ho) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+  const int bytes = cin * 2, groups = (bytes + 63) / 64;
+  const uint8_t* in = reinterpret_cast<const uint8_t*>(L.in);
+  int oy[2], ox[2];
+  bool valid[2];
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    const int p = warp * 16 + g + 8 * r;
+    oy[r] = Y0 - 1 + p / 3;
+    ox[r] = L.Wo - 3 + p % 3;
+    valid[r] = p < 3 * (kColRows + 2) && oy[r] >= 0 && oy[r] < L.Ho && ox[r] >= 0;
+  }
+  float acc[NT / 8][4];
+#pragma unroll
+  for (int j = 0; j < NT / 8; ++j)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) acc[j][q] = 0.f;
+  const uint4 zero = make_uint4(0, 0, 0, 0);
+#pragma unroll 6
+  for (int it = 0; it < 9 * groups; ++it) {
+    const int tap = it / groups, o = (it - tap * groups) * 64 + 16 * t, ky = tap / 3, kx = tap - 3 * ky;
+    const bool in_range = o < bytes;
+    uint4 x[2], w[NT / 8];
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      const int vy = oy[r] + ky - 1, vx = ox[r] + kx - 1;
+      const bool ok = in_range && valid[r] && vy >= 0 && vx >= 0 && vy < L.Ho && vx < L.Wo;
+      x[r] = ok ? *reinterpret_cast<const uint4*>(in + ((size_t)(vy >> 1) * L.Wi + (vx >> 1)) * bytes + o) : zero;
+    }
+#pragma unroll
+    for (int j = 0; j < NT / 8; ++j)
+      w[j] = in_range ? *reinterpret_cast<const uint4*>(W + ((size_t)(8 * j + g) * 9 + tap) * bytes + o) : zero;
+    const uint32_t a0[4] = {x[0].x, x[1].x, x[0].y, x[1].y}, a1[4] = {x[0].z, x[1].z, x[0].w, x[1].w};
+#pragma unroll
+    for (int j = 0; j < NT / 8; ++j) {
+      mma16816(acc[j], a0, w[j].x, w[j].y, false);
+      mma16816(acc[j], a1, w[j].z, w[j].w, false);
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < NT / 8; ++j)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int c = 8 * j + 2 * t + (q & 1), r = q >> 1;
+      const float v = __bfloat162float(__float2bfloat16_rn(acc[j][q] + bias[c]));
+      d3[warp * 16 + g + 8 * r][c] = valid[r] ? fmaxf(v, 0.f) : 0.f;
+    }
+  __syncthreads();
+  // a thread: one output, a quarter of the channels
+  const int o = threadIdx.x >> 2, part = threadIdx.x & 3, row = o >> 1, col = o & 1;  // column Wo - 2 + col
+  float s = 0.f;
+#pragma unroll
+  for (int ky = 0; ky < 3; ++ky)
+#pragma unroll
+    for (int kx = 0; kx < 3; ++kx) {
+      if (col + kx > 2) continue;  // beyond the last column
+      const float* d = d3[(row + ky) * 3 + col + kx];
+      const float* w = wf + (ky * 3 + kx) * NT;
+#pragma unroll
+      for (int c = 0; c < NT / 4; ++c) s = fmaf(w[part * (NT / 4) + c], d[part * (NT / 4) + c], s);
+    }
+  s += __shfl_xor_sync(0xffffffffu, s, 1);
+  s += __shfl_xor_sync(0xffffffffu, s, 2);
+  const int Y = Y0 + row, X = L.Wo - 2 + col;
+  if (part == 0 && Y < L.Ho) {
+    const EdgePair& E = edges[blockIdx.y];
+    E.Y[(size_t)Y * L.Wo + X] = upsample4_f(E.coarse, E.w, E.h, X, Y) + (bf[0] + s);
+  }
+}
+
 // E4M3 codes of a BF16 activation (the first layer's output in the FP8 form).
 __global__ void bf16_to_e4m3(const bf16* __restrict__ a, uint8_t* __restrict__ b, size_t n) {
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -951,6 +1036,19 @@ cudaError_t launch_edge_up2fix_mma(const UpFixPair* pairs, int n, int max_pixels
     edge_up2fix_mma<true><<<grid, 32 * kFixWarps, 0, st>>>(pairs, (const uint8_t*)W, wscale, bias, cin, cout, relu, out_f8);
   else
     edge_up2fix_mma<false><<<grid, 32 * kFixWarps, 0, st>>>(pairs, (const uint8_t*)W, wscale, bias, cin, cout, relu, 0);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_fused_edge_cols(const UpFixPair* fix, const EdgePair* edges, int n, int maxH, const void* W,
+                                   const float* bias, const float* wf, const float* bf, int cin, int NT,
+                                   cudaStream_t st) {
+  const dim3 grid((maxH + kColRows - 1) / kColRows, n);
+  if (NT == 32)
+    fused_edge_cols<32><<<grid, 128, 0, st>>>(fix, edges, (const uint8_t*)W, bias, wf, bf, cin);
+  else if (NT == 16)
+    fused_edge_cols<16><<<grid, 128, 0, st>>>(fix, edges, (const uint8_t*)W, bias, wf, bf, cin);
+  else
+    return cudaErrorInvalidValue;
   return cudaGetLastError();
 }
 

@@ -63,3 +63,30 @@ def test_border_recompute(svlib, form, shape, W, H):
         assert err.max() <= top and err.mean() <= mean, (err.max(), err.mean())
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("W,H", [(61, 31), (253, 64), (255, 37), (257, 66), (509, 35), (1241, 75)])
+@pytest.mark.parametrize("form,shape", [("bf16", synth.NET_SMALL), ("bf16", synth.NET_WIDE), ("fp8", synth.NET_WIDE),
+                                        ("bf16", synth.NetShape((16, 32, 16), 16, (32, 32, 32)))],
+                         ids=["small", "wide", "fp8", "32-32"])
+def test_fused_tail_odd_widths(svlib, form, shape, W, H):
+    """The fused decoder tail at odd widths (mixed with an even one) against the separate kernels:
+    only BF16 rounding of d3 and of the summed weights lies between them (the forms' bars)."""
+    k, D = 3, 4
+    ctx = binding.Context(shape, k, form)
+    try:
+        ctx.set_weights(synth.he_normal_weights(shape, 7))
+        sizes = [(W, H), (W + 1, H), (W, H + 1)]
+        dps = [binding.to_device(synth.make_pair(w, h, 12.0, 700 + w + h), D) for w, h in sizes]
+        rng = np.random.default_rng(5)
+        maps = [torch.from_numpy(rng.integers(0, D, (h // 4, w // 4)).astype(np.int16)).cuda() for w, h in sizes]
+        fused = ctx.refine(dps, maps)
+        ctx.set_option("fused_final", 0)
+        apart = ctx.refine(dps, maps)
+        ctx.synchronize()
+        for (w, h), a, b in zip(sizes, fused, apart):
+            d = (a - b).abs()
+            assert d.max().item() <= 0.05 and d.mean().item() <= 0.01, (w, h, d.max().item())
+            assert d[:, -2:].mean().item() <= 0.01, (w, h)
+    finally:
+        ctx.close()

@@ -1739,6 +1739,50 @@ sv_status Ctx::pack_fp8_weights(cudaStream_t st) {
   return SV_OK;
 }
 
+// Strip height of a launch: `lanes` CTAs take the strips in turn, a CTA's time is its strips' rows plus
+// `extra` rows' worth per strip (halo, ring restart), and the launch lasts as long as its busiest CTA.
+// Every column of Hu rows is cut into equal strips, so candidates differ in how many rounds of
+// strips there are and how much of the last round idles.  Four strips per CTA of whatever height, the last
+// one of a column short, left 25-40 % of a launch in its tail (64 pairs of 1242 x 375: enc2 188 us against 137 at
+// 32 rows, dec1 489 against 305 at 4).
+struct StripCols { int Hu; long long cols; };
+static int pick_strip_rows(const std::vector<StripCols>& groups, int lanes, double extra) {
+  int maxHu = 1;
+  for (auto& g : groups) maxHu = std::max(maxHu, g.Hu);
+  int best = maxHu;
+  double best_cost = 1e300;
+  for (int hs = std::min(2, maxHu); hs <= maxHu; hs += hs < 64 ? 1 : hs / 8) {
+    long long strips = 0;
+    int tall = 1;
+    for (auto& g : groups) {
+      const int m = (g.Hu + hs - 1) / hs;
+      strips += m * g.cols;
+      tall = std::max(tall, (g.Hu + m - 1) / m);
+    }
+    const double cost = (double)((strips + lanes - 1) / lanes) * (tall + extra);
+    if (cost < best_cost - 1e-9) {
+      best_cost = cost;
+      best = hs;
+    }
+  }
+  return best;
+}
+static void add_cols(std::vector<StripCols>& groups, int Hu, long long cols) {
+  if (!groups.empty() && groups.back().Hu == Hu)
+    groups.back().cols += cols;
+  else
+    groups.push_back({Hu, cols});
+}
+// The strips of one column: equal heights, or (fixed) hs rows and a shorter last one.
+template <typename F>
+static void cut_column(int Hu, int hs, bool fixed, F&& f) {
+  const int m = (Hu + hs - 1) / hs;
+  for (int t = 0; t < m; ++t) {
+    const int i0 = fixed ? t * hs : (int)((long long)Hu * t / m), i1 = fixed ? std::min(Hu, i0 + hs) : (int)((long long)Hu * (t + 1) / m);
+    f(i0, i1 - i0);
+  }
+}
+
 // Host side of one tensor-core refinement call: activation workspaces (allocated here),
 // per-layer descriptor and strip tables (built here, uploaded by the caller) and launch
 // geometry.  Nothing is enqueued on a stream.
@@ -1868,7 +1912,7 @@ sv_status Ctx::tc_prepare(const sv_pair* pairs, const int16_t* const* coarse, in
                     : pl.layer == L_DEC2 ? 2 : 1;
     const int lout = pl.layer == L_ENC2 ? 2 : pl.layer == L_ENC3 ? 3 : pl.layer == L_MU ? 3 : pl.layer == L_DEC1 ? 2
                      : pl.layer == L_DEC2 ? 1 : 0;
-    long long units = 0;
+    std::vector<StripCols> groups;
     std::vector<UpFixPair> fix(n);
     for (int i = 0; i < n; ++i) {
       LayerPair& L = lps[i];
@@ -1879,7 +1923,7 @@ sv_status Ctx::tc_prepare(const sv_pair* pairs, const int16_t* const* coarse, in
       L.Ho = lv[i].H[lout]; L.Wo = lv[i].W[lout];
       if (pl.mode == tc::TM_UP2) { L.Hu = L.Hi; L.Wu = L.Wi; }
       else { L.Hu = L.Ho; L.Wu = L.Wo; }
-      units += (long long)L.Hu * ((L.Wu + 127) / 128);
+      add_cols(groups, L.Hu, (L.Wu + 127) / 128);
       bool okm;
       if (pl.mode == tc::TM_S2)
         okm = make_tmap(&L.tm[0], L.in + pl.cin, pl.cin, L.Wi / 2, L.Hi, L.Wi, 2, 129) &&
@@ -1893,15 +1937,12 @@ sv_status Ctx::tc_prepare(const sv_pair* pairs, const int16_t* const* coarse, in
     if (bps <= 0) return fail(SV_ERR_UNSUPPORTED, "layer %d: tensor-core kernel does not fit an SM", pl.layer);
     int grid = std::max(pl.G, (nsm * bps) / pl.G * pl.G);
     const int cpg = grid / pl.G;
-    // strip height: about four strips per CTA of a weight set, at least 2 rows, unless tuned
-    const long long want = std::max<long long>(1, (long long)cpg * 4);
-    int hs = (int)std::max<long long>(2, (units + want - 1) / want);
-    if (tc_strip_rows > 0) hs = tc_strip_rows;
-    if (tc_rows_override[li] > 0) hs = tc_rows_override[li];
+    const int fixed = tc_rows_override[li] > 0 ? tc_rows_override[li] : tc_strip_rows;
+    const int hs = fixed > 0 ? fixed : pick_strip_rows(groups, cpg, 0.5);
     std::vector<Strip> strips;
     for (int i = 0; i < n; ++i)
       for (int j0 = 0; j0 < lps[i].Wu; j0 += 128)
-        for (int i0 = 0; i0 < lps[i].Hu; i0 += hs) strips.push_back({i, j0, i0, std::min(hs, lps[i].Hu - i0)});
+        cut_column(lps[i].Hu, hs, fixed > 0, [&](int i0, int cnt) { strips.push_back({i, j0, i0, cnt}); });
     grid = (int)std::min<long long>(grid, (long long)pl.G * (long long)strips.size());
     r.tabs[li].lp_ofs = put(lps.data(), sizeof(LayerPair) * n);
     r.tabs[li].fix_ofs = put(fix.data(), sizeof(UpFixPair) * n);
@@ -1951,7 +1992,7 @@ sv_status Ctx::tc_prepare(const sv_pair* pairs, const int16_t* const* coarse, in
     while (ring < 3 + kPrefetchSteps && tc::fused_smem_bytes(NT, cin, ring + 1) <= kSmemLimit) ++ring;
     if (fused_ring > 0) ring = std::min(ring, fused_ring);
     std::vector<tc::FusedPair> fps(n);
-    long long units = 0;
+    std::vector<StripCols> groups;
     for (int i = 0; i < n; ++i) {
       tc::FusedPair& F = fps[i];
       memset(&F, 0, sizeof(F));
@@ -1965,16 +2006,15 @@ sv_status Ctx::tc_prepare(const sv_pair* pairs, const int16_t* const* coarse, in
       F.h4 = pairs[i].height / 4;
       if (!make_tmap(&F.tm, act(5, i), cin, F.Wu, F.Hu, F.Wu, 1, tc::kFusedNpx))
         return fail(SV_ERR_CUDA, "pair %d: cuTensorMapEncodeTiled failed (fused decoder)", i);
-      units += (long long)F.Hu * ((F.Wo + 1 + 253) / 254);
+      add_cols(groups, F.Hu, (F.Wo + 1 + 253) / 254);
     }
     const int grid0 = nsm;  // one CTA per SM (about 214 KB of shared memory each)
-    int hs = (int)std::max<long long>(2, (units + grid0 * 4LL - 1) / (grid0 * 4LL));
-    if (tc_strip_rows > 0) hs = tc_strip_rows;
-    if (tc_rows_override[5] > 0) hs = tc_rows_override[5];
+    const int fixed = tc_rows_override[5] > 0 ? tc_rows_override[5] : tc_strip_rows;
+    const int hs = fixed > 0 ? fixed : pick_strip_rows(groups, grid0, 1.5);  // (a strip starts with a halo tile)
     std::vector<tc::Strip> strips;
     for (int i = 0; i < n; ++i)
       for (int sx = 0; 254 * sx - 1 < fps[i].Wo; ++sx)
-        for (int i0 = 0; i0 < fps[i].Hu; i0 += hs) strips.push_back({i, 127 * sx - 1, i0, std::min(hs, fps[i].Hu - i0)});
+        cut_column(fps[i].Hu, hs, fixed > 0, [&](int i0, int cnt) { strips.push_back({i, 127 * sx - 1, i0, cnt}); });
     r.fused_fp_ofs = put(fps.data(), sizeof(tc::FusedPair) * n);
     r.fused_strip_ofs = put(strips.data(), sizeof(tc::Strip) * strips.size());
     r.fused_n_strips = (int)strips.size();

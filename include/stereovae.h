@@ -363,9 +363,8 @@ SV_API sv_status sv_synchronize(sv_ctx* ctx, sv_stream stream);
  *   "spin_limit"     clock cycles one device-side wait may spin before it gives up
  *                    (default 4e9, about 2 s)
  *   "tc_strip_rows"  rows per work item of the tensor-core convolutions (0 = automatic)
- *   "tc_ctas_per_sm" 0 (default): each tensor-core convolution stages as many input rows
- *                    ahead as shared memory holds; k = 1..4: fewer, so that k CTAs share
- *                    an SM
+ *   "tc_ctas_per_sm" k = 1..4: each tensor-core convolution stages as many input rows ahead
+ *                    as lets k CTAs share an SM; 0 (default): k is chosen per layer
  *   "fused_final"    1 (default): an SV_BF16 inference call computes the last decoder
  *                    layer, the final conv and the residual in one kernel (d3 stays in
  *                    shared memory) when the decoder widths allow it; 0: separate kernels (d3 materialised in HBM)

@@ -1818,20 +1818,36 @@ sv_status Ctx::tc_prepare(const sv_pair* pairs, const int16_t* const* coarse, in
       pl.smem = tc::smem_bytes(pl.mode, NT, pl.cin, pl.ring, false, pl.f8 != 0);
     }
   }
+  int nsm = 0;
   {
     // shallower rings so that k CTAs share an SM (k per layer from the autotuner, else the
-    // context option); one CTA's control overhead between its MMA batches is then
+    // context option, else by what fits); one CTA's control overhead between its MMA batches is then
     // covered by the other CTAs' MMAs
     int per_sm = 0, reserved = 0;
     cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, device);
     cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, device);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device);
     for (size_t li = 0; li < r.plans.size(); ++li) {
-      const int k = tc_ctas_override[li] > 0 ? tc_ctas_override[li] : tc_ctas_per_sm;
-      if (k <= 1) continue;
       TcLayerPlan& pl = r.plans[li];
-      const size_t budget = (size_t)per_sm / k - (size_t)reserved;
       const int RA = pl.mode == tc::TM_S2 ? 3 : pl.mode == tc::TM_UP2 ? 2 : 1;
       const int STEP = pl.mode == tc::TM_S2 ? 2 : 1;
+      int k = tc_ctas_override[li] > 0 ? tc_ctas_override[li] : tc_ctas_per_sm;
+      // untuned, with enough rows for it: as many as keep two row steps staged ahead of a tile (one for
+      // the one-tap latent).  16/32/64 net, 32 pairs of 1000 x 300: dec2 110 -> 76 us, enc2 38 -> 30;
+      // 32/64/128 net, 64 pairs of 1242 x 375: latent 66 -> 56; FP8 enc2 66 -> 47.  The FP8 decoder and
+      // latent, whose MMAs are half as long, lose instead (dec2 250 -> 291 us) and keep one
+      static const int unit_level[6] = {2, 3, 3, 3, 2, 1};
+      long long rows = 0;
+      for (int i = 0; i < n; ++i) {
+        const Levels l(pairs[i].height, pairs[i].width);
+        rows += (long long)l.H[unit_level[li]] * ((l.W[unit_level[li]] + 127) / 128);
+      }
+      const int least = RA + (pl.mode == tc::TM_P1 ? 1 : 2) * STEP;
+      const bool able = rows * pl.G >= 8LL * nsm && !(pl.f8 && pl.mode != tc::TM_S2);
+      for (int kk = 3; k == 0 && able && kk > 1; --kk)
+        if (tc::smem_bytes(pl.mode, pl.NT, pl.cin, least, false, pl.f8 != 0) <= (size_t)per_sm / kk - (size_t)reserved) k = kk;
+      if (k <= 1) continue;
+      const size_t budget = (size_t)per_sm / k - (size_t)reserved;
       while (pl.ring > RA + STEP && tc::smem_bytes(pl.mode, pl.NT, pl.cin, pl.ring, false, pl.f8 != 0) > budget) --pl.ring;
       pl.smem = tc::smem_bytes(pl.mode, pl.NT, pl.cin, pl.ring, false, pl.f8 != 0);
     }
@@ -1862,8 +1878,6 @@ sv_status Ctx::tc_prepare(const sv_pair* pairs, const int16_t* const* coarse, in
     pl.smem = tc::smem_bytes(pl.mode, pl.NT, pl.cin, units, true, pl.f8 != 0);
   }
   sv_status s;
-  int nsm = 0;
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device);
   std::vector<Levels> lv(n);
   size_t cnt[7] = {0};
   std::vector<std::array<size_t, 7>> off(n), lens;

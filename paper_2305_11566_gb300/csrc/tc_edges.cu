@@ -945,13 +945,20 @@ __global__ void __launch_bounds__(128)
 fused_edge_cols(const UpFixPair* __restrict__ fix, const EdgePair* __restrict__ edges, const uint8_t* __restrict__ W,
                 const float* __restrict__ bias, const float* __restrict__ wf, const float* __restrict__ bf, int cin) {
   __shared__ float d3[64][NT + 1];
+  extern __shared__ __align__(16) unsigned char col_w[];  // weights [9 NT rows][cin], rows 16 bytes apart in banks
   const UpFixPair L = fix[blockIdx.y];
   if (!(L.Wo & 1)) return;
   const int Y0 = blockIdx.x * kColRows;
   if (Y0 >= L.Ho) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
-  const int bytes = cin * 2, groups = (bytes + 63) / 64;
+  const int bytes = cin * 2, groups = (bytes + 63) / 64, pitch = bytes + 16;
   const uint8_t* in = reinterpret_cast<const uint8_t*>(L.in);
+  for (int e = threadIdx.x; e < 9 * NT * (bytes / 16); e += 128) {
+    const int r = e / (bytes / 16), c = e - r * (bytes / 16);
+    const unsigned dst = (unsigned)__cvta_generic_to_shared(col_w + r * pitch + c * 16);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(W + (size_t)r * bytes + c * 16));
+  }
+  asm volatile("cp.async.commit_group;");
   int oy[2], ox[2];
   bool valid[2];
 #pragma unroll
@@ -967,25 +974,35 @@ fused_edge_cols(const UpFixPair* __restrict__ fix, const EdgePair* __restrict__ 
 #pragma unroll
     for (int q = 0; q < 4; ++q) acc[j][q] = 0.f;
   const uint4 zero = make_uint4(0, 0, 0, 0);
-#pragma unroll 6
-  for (int it = 0; it < 9 * groups; ++it) {
-    const int tap = it / groups, o = (it - tap * groups) * 64 + 16 * t, ky = tap / 3, kx = tap - 3 * ky;
-    const bool in_range = o < bytes;
-    uint4 x[2], w[NT / 8];
+  constexpr int AHEAD = 6;  // input fragments loaded together
+  for (int i0 = 0; i0 < 9 * groups; i0 += AHEAD) {
+    uint4 x[AHEAD][2];
 #pragma unroll
-    for (int r = 0; r < 2; ++r) {
-      const int vy = oy[r] + ky - 1, vx = ox[r] + kx - 1;
-      const bool ok = in_range && valid[r] && vy >= 0 && vx >= 0 && vy < L.Ho && vx < L.Wo;
-      x[r] = ok ? *reinterpret_cast<const uint4*>(in + ((size_t)(vy >> 1) * L.Wi + (vx >> 1)) * bytes + o) : zero;
+    for (int u = 0; u < AHEAD; ++u) {
+      const int it = i0 + u, tap = it / groups, o = (it - tap * groups) * 64 + 16 * t, ky = tap / 3, kx = tap - 3 * ky;
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        const int vy = oy[r] + ky - 1, vx = ox[r] + kx - 1;
+        const bool ok = tap < 9 && o < bytes && valid[r] && vy >= 0 && vx >= 0 && vy < L.Ho && vx < L.Wo;
+        x[u][r] = ok ? *reinterpret_cast<const uint4*>(in + ((size_t)(vy >> 1) * L.Wi + (vx >> 1)) * bytes + o) : zero;
+      }
+    }
+    if (i0 == 0) {
+      asm volatile("cp.async.wait_group 0;");
+      __syncthreads();
     }
 #pragma unroll
-    for (int j = 0; j < NT / 8; ++j)
-      w[j] = in_range ? *reinterpret_cast<const uint4*>(W + ((size_t)(8 * j + g) * 9 + tap) * bytes + o) : zero;
-    const uint32_t a0[4] = {x[0].x, x[1].x, x[0].y, x[1].y}, a1[4] = {x[0].z, x[1].z, x[0].w, x[1].w};
+    for (int u = 0; u < AHEAD; ++u) {
+      const int it = i0 + u, tap = it / groups, o = (it - tap * groups) * 64 + 16 * t;
+      if (tap >= 9) break;
+      const uint32_t a0[4] = {x[u][0].x, x[u][1].x, x[u][0].y, x[u][1].y};
+      const uint32_t a1[4] = {x[u][0].z, x[u][1].z, x[u][0].w, x[u][1].w};
 #pragma unroll
-    for (int j = 0; j < NT / 8; ++j) {
-      mma16816(acc[j], a0, w[j].x, w[j].y, false);
-      mma16816(acc[j], a1, w[j].z, w[j].w, false);
+      for (int j = 0; j < NT / 8; ++j) {
+        const uint4 w = o < bytes ? *reinterpret_cast<const uint4*>(col_w + ((8 * j + g) * 9 + tap) * pitch + o) : zero;
+        mma16816(acc[j], a0, w.x, w.y, false);
+        mma16816(acc[j], a1, w.z, w.w, false);
+      }
     }
   }
 #pragma unroll
@@ -1043,13 +1060,14 @@ cudaError_t launch_fused_edge_cols(const UpFixPair* fix, const EdgePair* edges, 
                                    const float* bias, const float* wf, const float* bf, int cin, int NT,
                                    cudaStream_t st) {
   const dim3 grid((maxH + kColRows - 1) / kColRows, n);
-  if (NT == 32)
-    fused_edge_cols<32><<<grid, 128, 0, st>>>(fix, edges, (const uint8_t*)W, bias, wf, bf, cin);
-  else if (NT == 16)
-    fused_edge_cols<16><<<grid, 128, 0, st>>>(fix, edges, (const uint8_t*)W, bias, wf, bf, cin);
-  else
-    return cudaErrorInvalidValue;
-  return cudaGetLastError();
+  const size_t smem = (size_t)9 * NT * (cin * 2 + 16);
+  auto go = [&](auto kern) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    kern<<<grid, 128, smem, st>>>(fix, edges, (const uint8_t*)W, bias, wf, bf, cin);
+    return cudaGetLastError();
+  };
+  return NT == 32 ? go(fused_edge_cols<32>) : NT == 16 ? go(fused_edge_cols<16>) : cudaErrorInvalidValue;
 }
 
 cudaError_t launch_bf16_to_e4m3(const bf16* a, uint8_t* b, size_t n, cudaStream_t st) {

@@ -339,7 +339,7 @@ sv_status sv_create(const sv_config* cfg, int device, sv_ctx** out) {
   if (!s) s = c->cuda(cudaMemset(c->err_flag.p, 0, sizeof(int)), "zero error flag");
   if (!s) s = c->cuda(c->w32.ensure(n * sizeof(float)), "alloc weights");
   if (!s) s = c->cuda(cudaMemset(c->w32.p, 0, n * sizeof(float)), "zero weights");
-  if (!s) s = c->f32_plan();
+  if (!s && cfg->precision == SV_FP32) s = c->f32_plan(0);
   if (!s) s = c->refresh_weight_copies();
   if (s) {
     c->release_all();

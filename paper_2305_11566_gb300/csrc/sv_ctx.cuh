@@ -202,7 +202,7 @@ struct Ctx {
   template <typename T>
   sv_status refine_direct(const sv_pair& p, const void* coarse_map, bool coarse_int16, const T* eps, T* Y, T* mu_out,
                           T* lv_out, T* const* saved, cudaStream_t st);
-  sv_status f32_plan();
+  sv_status f32_plan(cudaStream_t st);
   sv_status f32_pack(cudaStream_t st);
   sv_status f32_forward(const sv_pair* pairs, int n, const F32Tensors* t, const int16_t* const* coarse_i,
                         const float* const* coarse_f, const float* const* eps, float* const* Y, cudaStream_t st);

@@ -23,8 +23,9 @@ constexpr size_t pad32(size_t v) { return (v + 31) / 32 * 32; }
 
 }  // namespace
 
-sv_status Ctx::f32_plan() {
-  if (cfg.precision != SV_FP32 && cfg.precision != SV_BF16) return SV_OK;
+// Plans the FP32 layers and their packed weights: FP32 contexts when they are created, BF16 contexts
+// (which only train in FP32) at their first training call.
+sv_status Ctx::f32_plan(cudaStream_t st) {
   auto src = [&](int l) { return F32Src{net.w_off(l), net.ks(l), net.cout(l), net.cin(l)}; };
   std::vector<F32PackDesc> descs;
   size_t total = 0;
@@ -57,7 +58,8 @@ sv_status Ctx::f32_plan() {
   sv_status s;
   if ((s = cuda(f32_w.ensure(total * sizeof(float)), "alloc packed FP32 weights"))) return s;
   if ((s = cuda(f32_descs.ensure(descs.size() * sizeof(F32PackDesc)), "alloc pack table"))) return s;
-  return cuda(cudaMemcpy(f32_descs.p, descs.data(), descs.size() * sizeof(F32PackDesc), cudaMemcpyHostToDevice),
+  return cuda(cudaMemcpyAsync(f32_descs.p, descs.data(), descs.size() * sizeof(F32PackDesc), cudaMemcpyHostToDevice,
+                              st),
               "upload pack table");
 }
 
@@ -265,6 +267,7 @@ sv_status Ctx::f32_train_forward(const sv_pair* pairs, const void* const* coarse
 sv_status Ctx::train_forward_bf16(const sv_pair* pairs, const void* const* coarse, const void* const* eps, int n,
                                   void* const* Y, void* const* mu, void* const* lv, cudaStream_t st) {
   sv_status s;
+  if (f32_n_descs == 0 && ((s = f32_plan(st)) || (s = f32_pack(st)))) return s;
   if ((s = train_save_alloc(pairs, n, false, mu, lv))) return s;
   train_pairs.assign(pairs, pairs + n);
   train_coarse.assign(coarse, coarse + n);

@@ -37,7 +37,7 @@ def units():
         src = os.path.join(CSRC, f)
         if f == "zncc_wta.cu":
             for r in range(7, 0, -1):  # the largest units first
-                for m in (2, 1, 0):
+                for m in (3, 2, 1, 0):
                     out.append((src, [f"-DSV_ZNCC_R={r}", f"-DSV_ZNCC_MODE={m}"], f"zncc_wta_r{r}_m{m}.o"))
         else:
             out.append((src, [], f[:-3] + ".o"))

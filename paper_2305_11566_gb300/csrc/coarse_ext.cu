@@ -634,7 +634,7 @@ sv_status Ctx::coarse_ext(const sv_pair* pairs, int n, const sv_coarse_opts& o, 
     if (zncc) {
       LaunchScope ls(*this, with_cost ? "zncc_cost" : "zncc_wta", st);
       if ((s = cuda(launch_zncc_wta((const ZPair*)zpairs.p, (const ZJob*)zjobs.p + job0[i0], job0[i0 + m] - job0[i0],
-                                    cfg.window / 2, z.maxD, st, with_cost ? 2 : 0, z.shape.small),
+                                    cfg.window / 2, z.maxD, st, !with_cost ? 0 : agg ? 3 : 2, z.shape.small),
                     "zncc cost")))
         return s;
     } else {

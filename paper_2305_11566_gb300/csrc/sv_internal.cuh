@@ -94,21 +94,22 @@ inline ZShape zncc_shape(const sv_pair* pairs, int n, int maxD) {
 // Fused downsample + ZNCC + WTA over the given jobs, one entry per window radius
 // r = 1..7 and mode (each compiled in its own translation unit).
 // mode 0: disparities only; 1: also the best / second scores of the pairs that ask for them;
-// 2: also the cost volume (the pairs' cost pointers are set).
+// 2: also the cost volume (the pairs' cost pointers are set); 3: the cost volume only (disp unused).
 // small: jobs of the small shape; in: the pairs by value (p and j unused), or null.
 #define SV_ZNCC_DECL(r, m)                                                                                          \
   cudaError_t launch_zncc_wta_r##r##_m##m(const ZPair* d_pairs, const ZJob* d_jobs, int n_jobs, int maxD, bool small, \
                                           const ZInline* in, cudaStream_t st);
 #define SV_ZNCC_EACH(X) X(1) X(2) X(3) X(4) X(5) X(6) X(7)
-#define SV_ZNCC_DECLS(r) SV_ZNCC_DECL(r, 0) SV_ZNCC_DECL(r, 1) SV_ZNCC_DECL(r, 2)
+#define SV_ZNCC_DECLS(r) SV_ZNCC_DECL(r, 0) SV_ZNCC_DECL(r, 1) SV_ZNCC_DECL(r, 2) SV_ZNCC_DECL(r, 3)
 SV_ZNCC_EACH(SV_ZNCC_DECLS)
 inline cudaError_t launch_zncc_wta(const ZPair* p, const ZJob* j, int n, int r, int maxD, cudaStream_t st,
                                    int mode, bool small, const ZInline* in = nullptr) {
-  switch (r * 3 + mode) {
+  switch (r * 4 + mode) {
 #define SV_ZNCC_CASES(r)                                                          \
-  case r * 3: return launch_zncc_wta_r##r##_m0(p, j, n, maxD, small, in, st);     \
-  case r * 3 + 1: return launch_zncc_wta_r##r##_m1(p, j, n, maxD, small, in, st); \
-  case r * 3 + 2: return launch_zncc_wta_r##r##_m2(p, j, n, maxD, small, in, st);
+  case r * 4: return launch_zncc_wta_r##r##_m0(p, j, n, maxD, small, in, st);     \
+  case r * 4 + 1: return launch_zncc_wta_r##r##_m1(p, j, n, maxD, small, in, st); \
+  case r * 4 + 2: return launch_zncc_wta_r##r##_m2(p, j, n, maxD, small, in, st); \
+  case r * 4 + 3: return launch_zncc_wta_r##r##_m3(p, j, n, maxD, small, in, st);
     SV_ZNCC_EACH(SV_ZNCC_CASES)
   }
   return cudaErrorInvalidValue;

@@ -15,7 +15,7 @@
 //           rho = float(n) * (1/sigma_L) * (1/sigma_R).  The argmax over d is two warp
 //           reductions (__reduce_max_sync on an order-preserving integer key, then
 //           __reduce_min_sync on d among the maxima: lowest d wins ties).
-//           MODE 2 (cost volume): every lane also stores the cost 1 - rho of its candidates (Eq. 1; 2,
+//           MODE 2 and 3 (cost volume): every lane also stores the cost 1 - rho of its candidates (Eq. 1; 2,
 //           the largest value, where x - d < 0) into the pair's volume [h][w][D]: lanes hold
 //           consecutive d, so a warp's stores of one pixel are contiguous.
 #include "sv_internal.cuh"
@@ -72,9 +72,11 @@ __device__ __forceinline__ void stage_box(const uint8_t* __restrict__ img, int p
 // TY output rows; writes sum and 1/sigma for `ncols_out` windows starting at column
 // `c0` of the staged array (staged column c0 + t is the window's left edge), either to
 // sum_out / inv_out or, packed as {sum, bits of 1/sigma}, to packed.
+// packed windows left of the image (the first `outside` of them) get 1/sigma = NaN: a score against
+// them is never larger than another.
 template <int R, int TY>
 __device__ void window_stats(const uint16_t* s, int ncols, int* cs, unsigned* cs2, int* sum_out, float* inv_out,
-                             int2* packed, int ncols_out) {
+                             int2* packed, int ncols_out, int outside = 0) {
   for (int c = threadIdx.x; c < ncols; c += blockDim.x) {
     int a = 0;
     unsigned a2 = 0;
@@ -109,7 +111,7 @@ __device__ void window_stats(const uint16_t* s, int ncols, int* cs, unsigned* cs
     long long v = N * (long long)a2 - (long long)a * a;
     const float inv = v > 0 ? __frsqrt_rn((float)v) : 0.0f;
     if (packed) {
-      packed[e] = make_int2(a, __float_as_int(inv));
+      packed[e] = make_int2(a, t < outside ? 0x7FFFFFFF : __float_as_int(inv));
     } else {
       sum_out[e] = a;
       inv_out[e] = inv;
@@ -135,7 +137,7 @@ __device__ __forceinline__ void get_job(const ZPair* __restrict__ pairs, const Z
   P = in.p[i];
 }
 
-// MODE 0: disparity only; 1: also best / second scores; 2: also the cost volume.
+// MODE 0: disparity only; 1: also best / second scores; 2: also the cost volume; 3: the cost volume only.
 template <int R, int KD, int TX, int TY, int MODE>
 __global__ void __launch_bounds__(kZnccWarps * 32, (KD == 1 || (KD == 2 && R <= 5)) ? 2 : 1)
 zncc_wta_kernel(const ZPair* __restrict__ pairs, const ZJob* __restrict__ jobs, const __grid_constant__ ZInline in) {
@@ -229,9 +231,10 @@ zncc_wta_kernel(const ZPair* __restrict__ pairs, const ZJob* __restrict__ jobs, 
         const long long n = N * (long long)run[k] - (long long)sl * (long long)sr.x;
         const float rho = (float)n * il * __int_as_float(sr.y);
         const bool valid = d < D && d <= x && x < w;
-        if constexpr (MODE == 2) {
+        if constexpr (MODE >= 2) {
           if (d < D && x < w && y < h) P.cost[((size_t)y * w + x) * D + d] = d <= x ? 1.0f - rho : 2.0f;
         }
+        if constexpr (MODE == 3) continue;
         if (valid && rho > bv) {
           if constexpr (MODE == 1) sv = bv;
           bv = rho;
@@ -240,6 +243,7 @@ zncc_wta_kernel(const ZPair* __restrict__ pairs, const ZJob* __restrict__ jobs, 
           sv = rho;
         }
       }
+      if constexpr (MODE == 3) continue;
       const int bk = bv > -3.0f ? order_key(bv) : INT_MIN;
       const int gbest = __reduce_max_sync(0xFFFFFFFFu, bk);
       const unsigned dstar = __reduce_min_sync(0xFFFFFFFFu, (bk == gbest) ? (unsigned)bd : 0x7FFFFFFFu);
@@ -250,6 +254,7 @@ zncc_wta_kernel(const ZPair* __restrict__ pairs, const ZJob* __restrict__ jobs, 
       }
       if (lane == t) { my_d = (int)dstar; my_b = gbest; my_s = gsec; }
     }
+    if constexpr (MODE == 3) continue;
     const int x = xw + lane;
     if (lane < TX && x < w && y < h) {
       const size_t o = (size_t)y * w + x;
@@ -262,18 +267,43 @@ zncc_wta_kernel(const ZPair* __restrict__ pairs, const ZJob* __restrict__ jobs, 
   }
 }
 
-// Disparity ranges of 33-48 (MODE 0, disparities only): the two half-warps own TXH output
+// One level of the half-warp's argmax: lanes OFF apart compare HELD columns, each keeping half of them
+// (TXH of the first level's columns exist), then the next level; one column left: plain reduction.
+template <int HELD, int TXH, int OFF>
+__device__ __forceinline__ void exchange(long long* key, int l) {
+  if constexpr (OFF >= 1) {
+    constexpr int H = HELD > 1 ? HELD / 2 : 1;
+    const bool up = l & OFF;
+#pragma unroll
+    for (int i = 0; i < H; ++i) {
+      if (OFF == 8 && i >= TXH) continue;
+      if (HELD == 1 || (OFF == 8 && i + H >= TXH)) {  // no upper column
+        key[i] = max(key[i], __shfl_xor_sync(0xFFFFFFFFu, key[i], OFF));
+      } else {
+        const long long other = __shfl_xor_sync(0xFFFFFFFFu, up ? key[i] : key[i + H], OFF);
+        key[i] = max(up ? key[i + H] : key[i], other);
+      }
+    }
+    exchange<H, TXH, OFF / 2>(key, l);
+  }
+}
+
+// Disparity ranges of 33-48 (MODE 0, disparities only; COST: MODE 3, the cost volume only): the two half-warps own TXH output
 // columns each (half h: columns xw + h TXH + t) and lane l = lane % 16 the disparities d = l +
 // 16 k, k < 3, so that all 48 candidates of a pixel fill the half's 48 slots (the full-warp
 // layout uses 64 slots for them).  A lane keeps its best candidate as a float (strict ">"
 // over ascending k: lowest d on exact ties); the half's argmax is one max reduction over a
 // 64-bit key, the lane's order key above 63 - d, so that the lowest d wins exact ties, as in
-// the full-warp kernel.  Stages 1 and 2 as in zncc_wta_kernel.
-template <int R, int TXH, int TY>
+// the full-warp kernel.  Stages 1 and 2 as in zncc_wta_kernel.  64 pairs of 1242 x 375, D = 48: 274 -> 250 us
+// with the candidates' validity tests folded into the statistics and the argmax by halving exchanges; the
+// cost volume without the winner-take-all 358 -> 254 us (full-warp layout before).  Bound by the sliding sums'
+// shared-memory loads and their latency at 16 warps an SM.
+template <int R, int TXH, int TY, bool COST>
 __global__ void __launch_bounds__(kZnccWarps * 32, 2)
 zncc_wta_hw_kernel(const ZPair* __restrict__ pairs, const ZJob* __restrict__ jobs, const __grid_constant__ ZInline in) {
   extern __shared__ __align__(16) unsigned char smem[];
-  constexpr int KH = 3, TX = 2 * TXH;
+  constexpr int KH = 3, TX = 2 * TXH, NS = TXH <= 4 ? 4 : 16;  // NS: columns of the exchange
+  static_assert(TXH <= 4 ? TXH == 4 : TXH > 8 && TXH <= 16, "column count of the exchange");
   ZJob job;
   ZPair P;
   get_job(pairs, jobs, in, job, P);
@@ -293,7 +323,7 @@ zncc_wta_hw_kernel(const ZPair* __restrict__ pairs, const ZJob* __restrict__ job
   stage_box<R, TY>(P.R, P.pitch, w, h, rbase, y0, Z.nrc, sR);
   __syncthreads();
   window_stats<R, TY>(sL, Z.nlc, cs, cs2, sumL, invL, nullptr, Z.gx);
-  window_stats<R, TY>(sR, Z.nrc, cs, cs2, nullptr, nullptr, statR, Z.nrs);
+  window_stats<R, TY>(sR, Z.nrc, cs, cs2, nullptr, nullptr, statR, Z.nrs, D - 1 - x0);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, hf = lane >> 4, l = lane & 15;
   const int xw = x0 + warp * TX;
@@ -305,7 +335,7 @@ zncc_wta_hw_kernel(const ZPair* __restrict__ pairs, const ZJob* __restrict__ job
 #pragma unroll
   for (int k = 0; k < KH; ++k) {
     const int d = l + 16 * k;
-    dd[k] = d < D ? d : D - 1;             // reads stay in the staged range; masked below
+    dd[k] = d < D ? d : D - 1;             // a slot beyond D repeats D - 1, whose lower d wins the tie
     rc0[k] = lc0 - dd[k] + (D - 1);
   }
   unsigned colsum[KH][TXH + 2 * R];
@@ -339,36 +369,43 @@ zncc_wta_hw_kernel(const ZPair* __restrict__ pairs, const ZJob* __restrict__ job
       for (int i = 0; i <= 2 * R; ++i) a += colsum[k][i];
       run[k] = a;
     }
-    long long my_key = LLONG_MIN;
+    long long key[NS];
 #pragma unroll
     for (int t = 0; t < TXH; ++t) {
       if (t > 0) {
 #pragma unroll
         for (int k = 0; k < KH; ++k) run[k] += colsum[k][t + 2 * R] - colsum[k][t - 1];
       }
-      const int x = xh + t;
       const int sl = sumL[yi * Z.gx + lc0 + t];
       const float il = invL[yi * Z.gx + lc0 + t];
       float bv = -4.0f;
       int bd = 0;
 #pragma unroll
       for (int k = 0; k < KH; ++k) {
-        const int d = l + 16 * k;
         const int2 sr = statR[yi * Z.nrs + lc0 + t - dd[k] + (D - 1)];  // right window at x - d
         const long long n = N * (long long)run[k] - (long long)sl * (long long)sr.x;
         const float rho = (float)n * il * __int_as_float(sr.y);
-        if (d < D && d <= x && x < w && rho > bv) {
+        if constexpr (COST) {
+          const int d = l + 16 * k, x = xh + t;
+          if (d < D && x < w && y < h) P.cost[((size_t)y * w + x) * D + d] = d <= x ? 1.0f - rho : 2.0f;
+          continue;
+        }
+        if (rho > bv) {
           bv = rho;
-          bd = d;
+          bd = l + 16 * k;
         }
       }
-      long long key = bv > -3.0f ? (long long)order_key(bv) * 4294967296LL + (63 - bd) : LLONG_MIN;
-#pragma unroll
-      for (int off = 8; off >= 1; off >>= 1) key = max(key, __shfl_xor_sync(0xFFFFFFFFu, key, off));
-      if (l == t) my_key = key;
+      if constexpr (COST) continue;
+      key[t] = bv > -3.0f ? (long long)order_key(bv) * 4294967296LL + (63 - bd) : LLONG_MIN;
     }
-    const int x = xh + l;
-    if (l < TXH && x < w && y < h) P.disp[(size_t)y * w + x] = (int16_t)(my_key == LLONG_MIN ? 0 : 63 - (int)(my_key & 63));
+    // The half's argmax of every column: exchanges that halve the columns a lane keeps while they halve
+    // the lanes still to be compared (TXH = 10: 15 exchanges instead of 40); lane l ends with column
+    // l / (16 / NS).
+    if constexpr (COST) continue;
+    exchange<NS, TXH, 8>(key, l);
+    const int t = l / (16 / NS), x = xh + t;
+    if (l % (16 / NS) == 0 && t < TXH && x < w && y < h)
+      P.disp[(size_t)y * w + x] = (int16_t)(key[0] == LLONG_MIN ? 0 : 63 - (int)(key[0] & 63));
   }
 }
 
@@ -381,9 +418,9 @@ cudaError_t launch_shape(const ZPair* p, const ZJob* j, int n, int maxD, const Z
     kern<<<n, kZnccWarps * 32, smem, st>>>(p, j, in);
     return cudaGetLastError();
   };
-  if constexpr (MODE == 0 && KD == 2) {
+  if constexpr ((MODE == 0 || MODE == 3) && KD == 2) {
     // half-warp layout: 48 candidate slots per pixel, the same job geometry
-    if (maxD <= 48) return go(zncc_wta_hw_kernel<R, TX / 2, TY>);
+    if (maxD <= 48) return go(zncc_wta_hw_kernel<R, TX / 2, TY, MODE == 3>);
   }
   return go(zncc_wta_kernel<R, KD, TX, TY, MODE>);
 }

@@ -90,3 +90,33 @@ def test_fused_tail_odd_widths(svlib, form, shape, W, H):
             assert d[:, -2:].mean().item() <= 0.01, (w, h)
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("k,D,W,H", [(5, 33, 262, 80), (9, 40, 322, 97), (3, 48, 200, 64), (15, 47, 420, 130)])
+def test_half_warp_argmax_ties_and_edges(svlib, k, D, W, H):
+    """Disparity ranges of 33-48 run the half-warp layout without scores: textures full of exact
+    ties (periods of 3 and 5 quarter-size pixels, flat areas), where the lowest valid disparity must
+    win, against the full-warp layout with scores and the exact-integer oracle."""
+    rng = np.random.default_rng(k)
+    h, w = H // 4, W // 4
+    rows = rng.integers(0, 255, (h, 15)).astype(np.uint8)
+    left = np.tile(rows[:, :5], (1, w // 5 + 1))[:, :w]
+    right = np.tile(rows[:, :3], (1, w // 3 + 1))[:, :w]
+    right[: h // 2] = left[: h // 2]
+    left[:, w // 2: w // 2 + 20] = 77
+    big = [np.zeros((H, W), np.uint8) for _ in range(2)]
+    for b, s in zip(big, (left, right)):
+        b[: 4 * h, : 4 * w] = np.repeat(np.repeat(s, 4, 0), 4, 1)
+    dp = binding.to_device(synth.Pair(big[0], big[1], np.zeros((H, W), np.float32), np.zeros((H, W), bool), 0), D)
+    ctx = binding.Context(synth.NET_SMALL, k, "fp32")
+    try:
+        plain = ctx.coarse_match([dp])[0]
+        scored, best, _ = ctx.coarse_match([dp], scores=True)
+        many = ctx.coarse_match([dp] * 160)
+        assert torch.equal(plain, scored[0]) and torch.equal(plain, many[159])
+        want, _, _ = oracle.coarse_match(big[0], big[1], k, D)
+        # differences only where FP32 scores cannot tell the oracle's candidates apart
+        d = plain.cpu().numpy() != want
+        assert d.mean() <= 0.02, d.mean()
+    finally:
+        ctx.close()

@@ -11,13 +11,16 @@
 // holds COL output x 4 input channels x 3 kernel columns in registers and slides the three input
 // columns along the row, so a pixel costs it 2 loads of g and 0.5 (nearest x2), 1 or 2 (stride 2) of x
 // for 96 multiply-adds (one thread holding 4 x 2 channels x 9 taps loaded 10 vectors for 72).  g and
-// x of a few rows are staged by cp.async in two buffers.  16 pairs of 1242 x 375, 16/32/64 net: dec3 and dec2
-// 3.5 ms (6.8 before, one pair a launch) at 40 TFLOP/s, the FMA pipes 60 % busy; the whole training step with
-// the input gradients of conv_f32.cu 31.1 -> 11.1 ms.  Summing the folded phase-taps instead ran dec3 and
+// x of a few rows (a whole tile where the input is low-resolution: half the barriers) are staged by cp.async
+// in two buffers; one warp adds the bias gradient from the g it holds anyway (lanes of their own, reading g
+// once more behind the others, cost 5 %).  16 pairs of 1242 x 375, 16/32/64 net: dec3 and dec2 3.27 ms (6.8
+// before, one pair a launch) at 43 TFLOP/s; the whole training step with the input gradients of conv_f32.cu
+// 31.1 -> 10.7 ms.  Summing the folded phase-taps instead ran dec3 and
 // dec2 in 1.6 ms but moves the gradient's bits (see conv_f32.cu).
 #include "conv_f32.cuh"
 
 #include <algorithm>
+#include <type_traits>
 
 #include "sv_internal.cuh"
 
@@ -52,7 +55,7 @@ constexpr int kTR = 8, kTC = 16;  // pixels of a tile
 template <int KIND> struct WK;
 template <> struct WK<FK_S2> { static constexpr int KR = 3, KC = 3, ROWS = 2, XR = 5, XC = 33; };
 template <> struct WK<FK_P1> { static constexpr int KR = 1, KC = 1, ROWS = 4, XR = 4, XC = 16; };
-template <> struct WK<FK_UP2> { static constexpr int KR = 3, KC = 3, ROWS = 4, XR = 4, XC = 10; };
+template <> struct WK<FK_UP2> { static constexpr int KR = 3, KC = 3, ROWS = 8, XR = 6, XC = 10; };
 
 // COL output channels per lane, CGN x IGN lanes of a warp, NB input-channel blocks (warps) per kernel row.
 template <int KIND, int COL_, int CGN_, int IGN_, int NB_>
@@ -90,8 +93,10 @@ wgrad_f32_kernel(const F32WJob* __restrict__ jobs, int n, int Co, int Ci, size_t
   for (int k = 0; k < KC; ++k)
 #pragma unroll
     for (int j = 0; j < COL; ++j) acc[k][j][0] = acc[k][j][1] = 0ull;
-  float4 bacc = make_float4(0.f, 0.f, 0.f, 0.f);  // bias gradient: lanes of the last warp, 4 channels each
-  const bool bias_lane = ci0 == 0 && warp == G::WARPS - 1 && lane < BCO / 4;
+  u64 bacc[COL / 2];  // bias gradient: one warp adds the g it reads anyway
+#pragma unroll
+  for (int j = 0; j < COL / 2; ++j) bacc[j] = 0ull;
+  const bool bias_warp = ci0 == 0 && cib == 0 && ky == K::KR / 2;
 
   auto stage = [&](int step) {
     const int t = t0 + step / STEPS * J.units;
@@ -116,12 +121,17 @@ wgrad_f32_kernel(const F32WJob* __restrict__ jobs, int n, int Co, int Ci, size_t
     }
     cp_commit();
   };
-  auto loadg = [&](const float* g, u64 (&gv)[COL]) {
-    const float4 a = *reinterpret_cast<const float4*>(g + cg * 4);
-    gv[0] = dup2(a.x); gv[1] = dup2(a.y); gv[2] = dup2(a.z); gv[3] = dup2(a.w);
-    if constexpr (COL == 8) {
-      const float4 b = *reinterpret_cast<const float4*>(g + BCO / 2 + cg * 4);
-      gv[4] = dup2(b.x); gv[5] = dup2(b.y); gv[6] = dup2(b.z); gv[7] = dup2(b.w);
+  auto add2 = [](u64& d, u64 a) { asm("add.rn.f32x2 %0, %0, %1;" : "+l"(d) : "l"(a)); };
+  auto loadg = [&](auto bias, const float* g, u64 (&gv)[COL]) {
+#pragma unroll
+    for (int h = 0; h < COL / 4; ++h) {
+      const ulonglong2 q = *reinterpret_cast<const ulonglong2*>(g + h * (BCO / 2) + cg * 4);
+      const float2 u = unpack2(q.x), v = unpack2(q.y);
+      gv[4 * h] = dup2(u.x); gv[4 * h + 1] = dup2(u.y); gv[4 * h + 2] = dup2(v.x); gv[4 * h + 3] = dup2(v.y);
+      if constexpr (decltype(bias)::value) {
+        add2(bacc[2 * h], q.x);
+        add2(bacc[2 * h + 1], q.y);
+      }
     }
   };
   auto madd = [&](u64 (&a)[COL][2], const u64 (&gv)[COL], const ulonglong2& x) {
@@ -146,60 +156,56 @@ wgrad_f32_kernel(const F32WJob* __restrict__ jobs, int n, int Co, int Ci, size_t
     const float* gs = wf_sm + (step & 1) * G::BUF;
     const float* xs = gs + G::GF + cib * G::WCI + ig * 4;
     auto X = [&](int r, int c) { return *reinterpret_cast<const ulonglong2*>(xs + (r * K::XC + c) * BCI); };
+    auto rows = [&](auto bias) {
 #pragma unroll 1
-    for (int r = 0; r < K::ROWS; ++r) {
-      const float* gr = gs + r * kTC * BCO;
-      if constexpr (KIND == FK_UP2) {
-        if (Y0 + r + ky - 1 >= Ho) continue;  // the cropped upsampled row adds nothing
-        const int xr = ((r + ky - 1) >> 1) + 1;
-        ulonglong2 xm = X(xr, 0), x0 = X(xr, 1);
+      for (int r = 0; r < K::ROWS; ++r) {
+        const float* gr = gs + r * kTC * BCO;
+        if constexpr (KIND == FK_UP2) {
+          if (Y0 + r + ky - 1 >= Ho) continue;  // the cropped upsampled row adds nothing
+          const int xr = ((r + ky - 1) >> 1) + 1;
+          ulonglong2 xm = X(xr, 0), x0 = X(xr, 1);
 #pragma unroll 2
-        for (int c = 0; c < kTC / 2; ++c) {
-          const ulonglong2 xp = X(xr, c + 2);
-          u64 gv[COL];
-          loadg(gr + 2 * c * BCO, gv);
-          madd(acc[0], gv, xm);
-          madd(acc[1], gv, x0);
-          if (X0 + 2 * c + 1 < Wo) madd(acc[2], gv, x0);  // (else cropped)
-          loadg(gr + (2 * c + 1) * BCO, gv);
-          madd(acc[0], gv, x0);
-          madd(acc[1], gv, x0);
-          madd(acc[2], gv, xp);
-          xm = x0;
-          x0 = xp;
-        }
-      } else if constexpr (KIND == FK_S2) {
-        const int xr = 2 * r + ky;
-        ulonglong2 xa = X(xr, 0);
+          for (int c = 0; c < kTC / 2; ++c) {
+            const ulonglong2 xp = X(xr, c + 2);
+            u64 gv[COL];
+            loadg(bias, gr + 2 * c * BCO, gv);
+            madd(acc[0], gv, xm);
+            madd(acc[1], gv, x0);
+            if (X0 + 2 * c + 1 < Wo) madd(acc[2], gv, x0);  // (else cropped)
+            loadg(bias, gr + (2 * c + 1) * BCO, gv);
+            madd(acc[0], gv, x0);
+            madd(acc[1], gv, x0);
+            madd(acc[2], gv, xp);
+            xm = x0;
+            x0 = xp;
+          }
+        } else if constexpr (KIND == FK_S2) {
+          const int xr = 2 * r + ky;
+          ulonglong2 xa = X(xr, 0);
 #pragma unroll 2
-        for (int c = 0; c < kTC; ++c) {
-          const ulonglong2 xb = X(xr, 2 * c + 1), xc = X(xr, 2 * c + 2);
-          u64 gv[COL];
-          loadg(gr + c * BCO, gv);
-          madd(acc[0], gv, xa);
-          madd(acc[1], gv, xb);
-          madd(acc[2], gv, xc);
-          xa = xc;
-        }
-      } else {
+          for (int c = 0; c < kTC; ++c) {
+            const ulonglong2 xb = X(xr, 2 * c + 1), xc = X(xr, 2 * c + 2);
+            u64 gv[COL];
+            loadg(bias, gr + c * BCO, gv);
+            madd(acc[0], gv, xa);
+            madd(acc[1], gv, xb);
+            madd(acc[2], gv, xc);
+            xa = xc;
+          }
+        } else {
 #pragma unroll 4
-        for (int c = 0; c < kTC; ++c) {
-          u64 gv[COL];
-          loadg(gr + c * BCO, gv);
-          madd(acc[0], gv, X(r, c));
+          for (int c = 0; c < kTC; ++c) {
+            u64 gv[COL];
+            loadg(bias, gr + c * BCO, gv);
+            madd(acc[0], gv, X(r, c));
+          }
         }
       }
-    }
-    if (bias_lane) {
-#pragma unroll 4
-      for (int p = 0; p < G::NG; ++p) {
-        const float4 g = *reinterpret_cast<const float4*>(gs + p * BCO + 4 * lane);
-        bacc.x += g.x;
-        bacc.y += g.y;
-        bacc.z += g.z;
-        bacc.w += g.w;
-      }
-    }
+    };
+    if (bias_warp)
+      rows(std::true_type());
+    else
+      rows(std::false_type());
     __syncthreads();
   }
   float* out = slots + (size_t)blockIdx.x * slot;
@@ -215,7 +221,11 @@ wgrad_f32_kernel(const F32WJob* __restrict__ jobs, int n, int Co, int Ci, size_t
         *reinterpret_cast<float4*>(out + ((size_t)co * TAPS + ky * KC + k) * Ci + ci) = make_float4(u.x, u.y, v.x, v.y);
       }
   }
-  if (bias_lane) *reinterpret_cast<float4*>(out + (size_t)TAPS * Co * Ci + co0 + 4 * lane) = bacc;
+  if (bias_warp && ig == 0)
+#pragma unroll
+    for (int h = 0; h < COL / 4; ++h)
+      *reinterpret_cast<ulonglong2*>(out + (size_t)TAPS * Co * Ci + co0 + h * (BCO / 2) + cg * 4) =
+          make_ulonglong2(bacc[2 * h], bacc[2 * h + 1]);
 }
 
 // gw[e] += the pairs' sums (e < nWw), gb[e - nWw] likewise: a pair's chains in chain order, the pairs in

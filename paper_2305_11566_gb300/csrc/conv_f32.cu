@@ -5,7 +5,7 @@
 // A block of 128 threads computes TH x TW positions of one output phase x 8 CG output channels;
 // a thread holds 8 consecutive positions x 8 channels in registers.  The input patch is staged
 // channel-planar (CIC channels a step) and the packed weights as [tap][channel][output], both by
-// cp.async into two buffers.  Per channel and window row a thread reads its row segment once
+// cp.async into two buffers, with one barrier a step (two cost the Table I net 1.3 %).  Per channel and window row a thread reads its row segment once
 // and reuses it for the TX taps: 64 TX multiply-adds for 2 TX + 3 vector loads, so the FMA pipe and
 // not shared memory bounds the kernel (one output channel group per thread and one position
 // needed 9 loads for 32 multiply-adds).  The multiply-adds are issued as packed pairs.  8 pairs of
@@ -416,17 +416,15 @@ __device__ __forceinline__ void contract(const Form& form, u64 (&acc)[PX][4], fl
   };
   stage(0);
   for (int ch = 0; ch < nch; ++ch) {
-    if (G::NBUF == 2 && ch + 1 < nch) {
-      stage(ch + 1);
-      cp_wait<1>();
-    } else {
-      cp_wait<0>();
-    }
-    __syncthreads();
+    cp_wait<0>();
+    __syncthreads();  // chunk ch is there, and everyone is done with chunk ch - 1: its buffer may be refilled
+    if (G::NBUF == 2 && ch + 1 < nch) stage(ch + 1);
     const float* b = sm + (ch % G::NBUF) * G::BUF;
     form(acc, b + pa0, b + G::CIC * G::PLANE + cg * 4);
-    __syncthreads();
-    if (G::NBUF == 1 && ch + 1 < nch) stage(ch + 1);
+    if (G::NBUF == 1 && ch + 1 < nch) {
+      __syncthreads();
+      stage(ch + 1);
+    }
   }
 }
 
@@ -823,13 +821,9 @@ f32_y5_kernel(const F32Job* __restrict__ jobs, const float* __restrict__ w, cons
   for (int p = 0; p < PX; ++p) acc[p][0] = acc[p][1] = 0ull;
   stage(0);
   for (int ch = 0; ch < steps; ++ch) {
-    if (ch + 1 < steps) {
-      stage(ch + 1);
-      cp_wait<1>();
-    } else {
-      cp_wait<0>();
-    }
-    __syncthreads();
+    cp_wait<0>();
+    __syncthreads();  // (as in contract)
+    if (ch + 1 < steps) stage(ch + 1);
     const float* pa = sm + (ch & 1) * G::BUF + row * G::PITCH + gx * PX;
     const float* pw = sm + (ch & 1) * G::BUF + G::CIC * G::PLANE;
 #pragma unroll 1
@@ -851,7 +845,6 @@ f32_y5_kernel(const F32Job* __restrict__ jobs, const float* __restrict__ w, cons
           }
         }
       }
-    __syncthreads();
   }
   const float b0 = bias[0];
 #pragma unroll

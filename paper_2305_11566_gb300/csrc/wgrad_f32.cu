@@ -11,9 +11,9 @@
 // holds COL output x 4 input channels x 3 kernel columns in registers and slides the three input
 // columns along the row, so a pixel costs it 2 loads of g and 0.5 (nearest x2), 1 or 2 (stride 2) of x
 // for 96 multiply-adds (one thread holding 4 x 2 channels x 9 taps loaded 10 vectors for 72).  g and
-// x of a few rows (a whole tile where the input is low-resolution: half the barriers) are staged by cp.async
-// in two buffers; one warp adds the bias gradient from the g it holds anyway (lanes of their own, reading g
-// once more behind the others, cost 5 %).  16 pairs of 1242 x 375, 16/32/64 net: dec3 and dec2 3.27 ms (6.8
+// x of a few rows (a whole tile where the input is low-resolution) are staged by cp.async in two buffers, the
+// next step's once the step's one barrier has shown everyone done with the last; one warp adds the bias gradient from the g it holds anyway (lanes of their own, reading g
+// once more behind the others, cost 5 %).  16 pairs of 1242 x 375, 16/32/64 net: dec3 and dec2 3.23 ms (6.8
 // before, one pair a launch) at 43 TFLOP/s; the whole training step with the input gradients of conv_f32.cu
 // 31.1 -> 10.7 ms.  Summing the folded phase-taps instead ran dec3 and
 // dec2 in 1.6 ms but moves the gradient's bits (see conv_f32.cu).
@@ -144,13 +144,9 @@ wgrad_f32_kernel(const F32WJob* __restrict__ jobs, int n, int Co, int Ci, size_t
 
   if (nsteps > 0) stage(0);
   for (int step = 0; step < nsteps; ++step) {
-    if (step + 1 < nsteps) {
-      stage(step + 1);
-      cp_wait<1>();
-    } else {
-      cp_wait<0>();
-    }
-    __syncthreads();
+    cp_wait<0>();
+    __syncthreads();  // this step's rows are there, and everyone is done with the last step's buffer
+    if (step + 1 < nsteps) stage(step + 1);
     const int t = t0 + step / STEPS * J.units;
     const int Y0 = t / tiles_x * kTR + step % STEPS * K::ROWS, X0 = t % tiles_x * kTC;
     const float* gs = wf_sm + (step & 1) * G::BUF;
@@ -206,7 +202,6 @@ wgrad_f32_kernel(const F32WJob* __restrict__ jobs, int n, int Co, int Ci, size_t
       rows(std::true_type());
     else
       rows(std::false_type());
-    __syncthreads();
   }
   float* out = slots + (size_t)blockIdx.x * slot;
   constexpr int TAPS = K::KR * KC;

@@ -37,7 +37,7 @@ def test_sgm_layouts_bit_exact(ctx, D, W, H, npaths):
     assert torch.equal(ctx.coarse_match_ex([dp], o)[0], disp[0])
     # the caller's volume at 4-byte alignment
     h, w = dp.coarse_hw
-    buf = torch.zeros(h * w * D + 1, device="cuda")
+    buf = torch.zeros(h * w * D + 1, dtype=torch.float32, device="cuda")
     d2 = torch.empty_like(disp[0])
     s = binding.lib().sv_coarse_match_ex(ctx.handle, binding._pairs_array([dp]), 1, ctypes.byref(o), binding._ptrs([d2]),
                                          binding._ptrs([buf[1:]]), binding._stream(None))

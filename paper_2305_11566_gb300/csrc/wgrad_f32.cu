@@ -11,12 +11,14 @@
 // holds COL output x 4 input channels x 3 kernel columns in registers and slides the three input
 // columns along the row, so a pixel costs it 2 loads of g and 0.5 (nearest x2), 1 or 2 (stride 2) of x
 // for 96 multiply-adds (one thread holding 4 x 2 channels x 9 taps loaded 10 vectors for 72).  g and
-// x of a few rows (a whole tile where the input is low-resolution) are staged by cp.async in two buffers, the
-// next step's once the step's one barrier has shown everyone done with the last; one warp adds the bias gradient from the g it holds anyway (lanes of their own, reading g
-// once more behind the others, cost 5 %).  16 pairs of 1242 x 375, 16/32/64 net: dec3 and dec2 3.23 ms (6.8
-// before, one pair a launch) at 43 TFLOP/s; the whole training step with the input gradients of conv_f32.cu
-// 31.1 -> 10.7 ms.  Summing the folded phase-taps instead ran dec3 and
-// dec2 in 1.6 ms but moves the gradient's bits (see conv_f32.cu).
+// x of a few rows (a whole tile where the input is low-resolution) are staged by cp.async in two
+// buffers, the next step's once the step's one barrier has shown everyone done with the last; one
+// warp adds the bias gradient from the g it holds anyway (lanes of their own, reading g once more
+// behind the others, cost 5 %).  16 pairs of 1242 x 375, 16/32/64 net: dec3 and dec2 3.23 ms (6.8
+// before, one pair a launch) at 43 TFLOP/s; the whole training step with the input gradients of
+// conv_f32.cu 31.1 -> 10.7 ms.  The FMA pipes are 60 % busy: 96-168 registers a thread leave 12-18
+// warps an SM, in blocks of 3 or 6 that meet at the barrier.  Summing the folded phase-taps instead
+// ran dec3 and dec2 in 1.6 ms but moves the gradient's bits (see conv_f32.cu).
 #include "conv_f32.cuh"
 
 #include <algorithm>
@@ -317,7 +319,9 @@ f32_final_dgrad_kernel(const F32Img* __restrict__ imgs, const float* __restrict_
 // Weight gradient of the final conv: a lane owns one kernel row, 4 input channels and their three
 // kernel columns, and reads d3 and the output gradient of its chain's rows straight from memory (the
 // lanes of a pixel read whole sectors; the three kernel rows and neighbouring tiles meet in the
-// caches).  3 C / 4 lanes run a chain; the bias is one more lane.
+// caches).  3 C / 4 lanes run a chain; a lane of the middle kernel row, which sees every output, adds the
+// bias (a lane of its own walked the tile one dependent load at a time while its warp waited: 16 pairs
+// of 1242 x 375, 16 channels, 317 -> 263 us with its reduction).  Bound by the loads' latency.
 __global__ void __launch_bounds__(256)
 f32_final_wgrad_kernel(const F32Img* __restrict__ imgs, const F32WJob* __restrict__ jobs, int n, int units, int C,
                        int lanes, size_t slot, float* __restrict__ slots) {
@@ -331,17 +335,9 @@ f32_final_wgrad_kernel(const F32Img* __restrict__ imgs, const F32WJob* __restric
   const int tiles_x = (W + kTC - 1) / kTC, ntiles = tiles_x * ((H + kTR - 1) / kTR);
   const float* g = imgs[job].gY;
   float* out = slots + (size_t)u * slot;
-  if (l == 3 * C / 4) {
-    float s = 0.f;
-    for (int t = u - J.unit0; t < ntiles; t += J.units) {
-      const int Y0 = t / tiles_x * kTR, X0 = t % tiles_x * kTC, ye = min(Y0 + kTR, H), xe = min(X0 + kTC, W);
-      for (int y = Y0; y < ye; ++y)
-        for (int x = X0; x < xe; ++x) s += g[(size_t)y * W + x];
-    }
-    out[9 * C] = s;
-    return;
-  }
   const int ky = l / (C / 4), c4 = 4 * (l % (C / 4));
+  const bool bias = l == C / 4;  // (ky 1, channel 0)
+  float bacc = 0.f;
   float4 acc[3] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
   for (int t = u - J.unit0; t < ntiles; t += J.units) {
     const int Y0 = t / tiles_x * kTR, X0 = t % tiles_x * kTC, ye = min(Y0 + kTR, H);
@@ -359,6 +355,9 @@ f32_final_wgrad_kernel(const F32Img* __restrict__ imgs, const F32WJob* __restric
                                               : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
       for (int j = 0; j < kTC; ++j) gv[j] = j < m ? gr[j] : 0.f;
+      if (bias)
+#pragma unroll
+        for (int j = 0; j < kTC; ++j) bacc += gv[j];
 #pragma unroll
       for (int j = 0; j < kTC; ++j)
 #pragma unroll
@@ -372,52 +371,57 @@ f32_final_wgrad_kernel(const F32Img* __restrict__ imgs, const F32WJob* __restric
   }
 #pragma unroll
   for (int k = 0; k < 3; ++k) *reinterpret_cast<float4*>(out + (ky * 3 + k) * C + c4) = acc[k];
+  if (bias) out[9 * C] = bacc;
 }
 
-// Weight and bias gradient of enc1 (2 channels -> C, stride 2): a warp's chain builds the network input
-// (L / 256, U / 256) under its tile in shared memory; a lane owns one kernel row and 4 output
-// channels: 4 x 3 columns x 2 channels.
+// Weight and bias gradient of enc1 (2 channels -> C, stride 2): a warp builds the network input
+// (L / 256, U / 256) under its chain's tile in shared memory; a lane owns one kernel row and 4 output
+// channels: 4 x 3 columns x 2 channels.  Up to 20 channels a chain fills half a warp at most: two
+// chains share it (CW = 2; 16 channels, 16 pairs of 1242 x 375: 324 -> 264 us with its
+// reduction).
 constexpr int kEwWarps = 4, kEwR = 2 * kTR + 1, kEwC = 2 * kTC + 1;
+template <int CW>
 __global__ void __launch_bounds__(32 * kEwWarps)
 f32_enc1_wgrad_kernel(const F32Img* __restrict__ imgs, const F32WJob* __restrict__ jobs, int n, int units, int C,
                       size_t slot, float* __restrict__ slots) {
-  __shared__ float2 sm[kEwWarps][kEwR][kEwC];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, u = blockIdx.x * kEwWarps + warp;
-  if (u >= units) return;
+  constexpr int LW = 32 / CW;  // lanes of a chain
+  __shared__ float2 sm[kEwWarps * CW][kEwR][kEwC];
+  const int chain = threadIdx.x / LW, lane = threadIdx.x % LW, u = blockIdx.x * kEwWarps * CW + chain;
   int job = 0;
   while (job + 1 < n && u >= jobs[job + 1].unit0) ++job;
   const F32WJob& J = jobs[job];
   const F32Img& I = imgs[job];
-  const int tiles_x = (I.W1 + kTC - 1) / kTC, ntiles = tiles_x * ((I.H1 + kTR - 1) / kTR);
+  const int tiles_x = (I.W1 + kTC - 1) / kTC, ntiles = u < units ? tiles_x * ((I.H1 + kTR - 1) / kTR) : 0;
   float* out = slots + (size_t)u * slot;
   const int q0 = C / 4;
-  // 3 q0 (kernel row, 4 channels) tasks, 32 at a time
-  for (int base = 0; base < 3 * q0; base += 32) {
+  // 3 q0 (kernel row, 4 channels) tasks, LW at a time
+  for (int base = 0; base < 3 * q0; base += LW) {
     const int task = base + lane;
     const bool on = task < 3 * q0;
     const int ky = on ? task / q0 : 0, c4 = on ? 4 * (task % q0) : 0;
     float4 acc[6], bacc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
     for (int k = 0; k < 6; ++k) acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int t = u - J.unit0; t < ntiles; t += J.units) {
+    for (int t = u - J.unit0; __any_sync(0xffffffffu, t < ntiles); t += J.units) {
+      const bool live = t < ntiles;  // (the warp's other chain may have a tile more)
       const int Y0 = t / tiles_x * kTR, X0 = t % tiles_x * kTC;
       __syncwarp();
-      for (int e = lane; e < kEwR * kEwC; e += 32) {
+      for (int e = lane; live && e < kEwR * kEwC; e += LW) {
         const int r = e / kEwC, c = e - r * kEwC, vy = 2 * Y0 - 1 + r, vx = 2 * X0 - 1 + c;
         float2 v = make_float2(0.f, 0.f);
         if (vy >= 0 && vx >= 0 && vy < I.H && vx < I.W) {
           v.x = (float)I.L[(size_t)vy * I.pitch + vx] * (1.0f / 256.0f);
           v.y = upsample4_f(I.coarse_f, I.w, I.h, vx, vy) * (1.0f / 256.0f);
         }
-        sm[warp][r][c] = v;
+        sm[chain][r][c] = v;
       }
       __syncwarp();
-      const int ye = min(kTR, I.H1 - Y0), xe = min(kTC, I.W1 - X0);
-      for (int y = 0; on && y < ye; ++y) {
+      const int ye = live && on ? min(kTR, I.H1 - Y0) : 0, xe = min(kTC, I.W1 - X0);
+      for (int y = 0; y < ye; ++y) {
         const float* g = I.ge1 + ((size_t)(Y0 + y) * I.W1 + X0) * C + c4;
-        const float2* xr = sm[warp][2 * y + ky];
+        const float2* xr = sm[chain][2 * y + ky];
         float2 xa = xr[0];
-#pragma unroll 4
+#pragma unroll 8
         for (int x = 0; x < xe; ++x) {
           const float4 gv = *reinterpret_cast<const float4*>(g + (size_t)x * C);
           const float2 xb = xr[2 * x + 1], xc = xr[2 * x + 2];
@@ -435,7 +439,7 @@ f32_enc1_wgrad_kernel(const F32Img* __restrict__ imgs, const F32WJob* __restrict
         }
       }
     }
-    if (on) {
+    if (on && u < units) {
 #pragma unroll
       for (int k = 0; k < 6; ++k) {
         const float v[4] = {acc[k].x, acc[k].y, acc[k].z, acc[k].w};
@@ -541,11 +545,13 @@ cudaError_t launch_f32_final_dgrad(const F32Img* imgs, int n, int maxH, int maxW
 cudaError_t launch_f32_edge_wgrad(const F32WPlan& p, const F32Img* imgs, const F32WJob* d_jobs, int n, float* gw,
                                   float* gb, float* slots, cudaStream_t st) {
   if (p.kind == FK_WENC1) {
-    f32_enc1_wgrad_kernel<<<(p.units + kEwWarps - 1) / kEwWarps, 32 * kEwWarps, 0, st>>>(imgs, d_jobs, n, p.units, p.co,
-                                                                                         p.slot, slots);
+    const bool two = 3 * p.co / 4 <= 16;
+    const int per = kEwWarps * (two ? 2 : 1);
+    (two ? f32_enc1_wgrad_kernel<2> : f32_enc1_wgrad_kernel<1>)<<<(p.units + per - 1) / per, 32 * kEwWarps, 0, st>>>(
+        imgs, d_jobs, n, p.units, p.co, p.slot, slots);
   } else {
-    // a chain takes 3 C / 4 lanes and one for the bias (C <= 256: at most 193)
-    const int lanes = 3 * p.ci / 4 + 1, threads = std::max(lanes, 128), per = threads / lanes;
+    const int lanes = 3 * p.ci / 4,  // of a chain (C <= 256: at most 192)
+              threads = std::max(lanes, 128), per = threads / lanes;
     f32_final_wgrad_kernel<<<(p.units + per - 1) / per, threads, 0, st>>>(imgs, d_jobs, n, p.units, p.ci, lanes, p.slot,
                                                                           slots);
   }

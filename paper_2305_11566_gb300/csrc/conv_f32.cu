@@ -47,6 +47,11 @@ __device__ __forceinline__ void cp4(float* dst, const float* src, bool ok) {
   const int n = ok ? 4 : 0;
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(s), "l"(src), "r"(n));
 }
+__device__ __forceinline__ void cp16z(float* dst, const float* src, bool ok) {
+  const unsigned s = (unsigned)__cvta_generic_to_shared(dst);
+  const int n = ok ? 16 : 0;
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(s), "l"(src), "r"(n));
+}
 __device__ __forceinline__ void cp16(float* dst, const float* src) {
   const unsigned s = (unsigned)__cvta_generic_to_shared(dst);
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s), "l"(src));
@@ -792,13 +797,17 @@ f32_final_ordered_kernel(const F32Img* __restrict__ imgs, const float* __restric
 // FK_Y5: a thread owns 8 input positions along x and their four output phases; the phase pair
 // py = 1 has no tap in window row 0.  Channels go 4 a step (a one-channel source fills its step
 // with zeros); the packed weights are [step][tap][channel][phase].
+// A position's four channels are one 16-byte word, staged by one copy: the wide kinds' channel planes
+// take four 4-byte copies, whose issue slots a kernel of 15 multiply-add pairs per word cannot hide (16
+// pairs of 1242 x 375: 457 -> 300 us).  A gap after every eighth word and rows 4 words apart modulo 8
+// keep a quarter-warp's reads on different banks.  Sources that are no multiple of 4 channels wide or not
+// 16-byte aligned are copied by channels, zeros in the missing ones.
 struct Y5Geo {
-  static constexpr int CIC = 4, TW = 32, TH = 32, S = 1, PR = 34, PC = 34, PITCH = 36;
-  static constexpr int PLANE = (PR * PITCH + 31 - 4) / 32 * 32 + 4, WF = 9 * CIC * 4, BUF = CIC * PLANE + WF;
-  static constexpr bool SPLIT = false;
-  static constexpr int EVEN = 0;
+  static constexpr int CIC = 4, TW = 32, TH = 32, PR = 34, PC = 34, PITCH = 44;  // (in words)
+  static constexpr int PATCH = PR * PITCH * 4, WF = 9 * CIC * 4, BUF = PATCH + WF;
+  __device__ static constexpr int word(int c) { return c + (c >> 3); }
 };
-__global__ void __launch_bounds__(kThreads, 5)
+__global__ void __launch_bounds__(kThreads, 4)
 f32_y5_kernel(const F32Job* __restrict__ jobs, const float* __restrict__ w, const float* __restrict__ bias, int steps,
               float scale, int tiles_x) {
   using G = Y5Geo;
@@ -811,9 +820,23 @@ f32_y5_kernel(const F32Job* __restrict__ jobs, const float* __restrict__ w, cons
   auto stage = [&](int ch) {
     float* b = sm + (ch & 1) * G::BUF;
     if (c0 >= J.ic[s]) { c0 = 0; ++s; }
-    load_patch<G, G::PR, G::PC>(b, J.in[s] + c0, J.ic[s], Y0 - 1, X0 - 1, J.Hi, J.Wi, J.ic[s] - c0);
+    const int ic = J.ic[s], avail = ic - c0;
+    const float* src = J.in[s] + c0;
+    const bool vec = ic % 4 == 0 && reinterpret_cast<size_t>(src) % 16 == 0;
+    for (int e = threadIdx.x; e < G::PR * G::PC; e += kThreads) {
+      const int r = e / G::PC, c = e - r * G::PC, iy = Y0 - 1 + r, ix = X0 - 1 + c;
+      const bool ok = iy >= 0 && ix >= 0 && iy < J.Hi && ix < J.Wi;
+      const float* p = ok ? src + ((size_t)iy * J.Wi + ix) * ic : src;
+      float* d = b + (r * G::PITCH + G::word(c)) * 4;
+      if (vec) {
+        cp16z(d, p, ok);
+      } else {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) cp4(d + q, q < avail ? p + q : p, ok && q < avail);
+      }
+    }
     c0 += G::CIC;
-    if (threadIdx.x < G::WF / 4) cp16(b + G::CIC * G::PLANE + 4 * threadIdx.x, w + (size_t)ch * G::WF + 4 * threadIdx.x);
+    if (threadIdx.x < G::WF / 4) cp16(b + G::PATCH + 4 * threadIdx.x, w + (size_t)ch * G::WF + 4 * threadIdx.x);
     cp_commit();
   };
   u64 acc[PX][2];
@@ -824,17 +847,19 @@ f32_y5_kernel(const F32Job* __restrict__ jobs, const float* __restrict__ w, cons
     cp_wait<0>();
     __syncthreads();  // (as in contract)
     if (ch + 1 < steps) stage(ch + 1);
-    const float* pa = sm + (ch & 1) * G::BUF + row * G::PITCH + gx * PX;
-    const float* pw = sm + (ch & 1) * G::BUF + G::CIC * G::PLANE;
-#pragma unroll 1
-    for (int ci = 0; ci < G::CIC; ++ci)
+    const float* pa = sm + (ch & 1) * G::BUF + (row * G::PITCH + G::word(gx * PX)) * 4;
+    const float* pw = sm + (ch & 1) * G::BUF + G::PATCH;
 #pragma unroll
-      for (int r = 0; r < 3; ++r) {
-        float a[12];
-        load_row<G, 3>(pa + ci * G::PLANE + r * G::PITCH, a);
-        u64 v[10];
+    for (int r = 0; r < 3; ++r) {
+      float4 a[PX + 2];
 #pragma unroll
-        for (int q = 0; q < 10; ++q) v[q] = dup2(a[q]);
+      for (int q = 0; q < PX + 2; ++q)
+        a[q] = *reinterpret_cast<const float4*>(pa + (r * G::PITCH + G::word(q)) * 4);
+#pragma unroll
+      for (int ci = 0; ci < G::CIC; ++ci) {
+        u64 v[PX + 2];
+#pragma unroll
+        for (int q = 0; q < PX + 2; ++q) v[q] = dup2(ci == 0 ? a[q].x : ci == 1 ? a[q].y : ci == 2 ? a[q].z : a[q].w);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
           const ulonglong2 k = *reinterpret_cast<const ulonglong2*>(pw + ((r * 3 + c) * G::CIC + ci) * 4);
@@ -845,6 +870,7 @@ f32_y5_kernel(const F32Job* __restrict__ jobs, const float* __restrict__ w, cons
           }
         }
       }
+    }
   }
   const float b0 = bias[0];
 #pragma unroll

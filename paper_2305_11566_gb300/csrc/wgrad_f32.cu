@@ -16,7 +16,7 @@
 // warp adds the bias gradient from the g it holds anyway (lanes of their own, reading g once more
 // behind the others, cost 5 %).  16 pairs of 1242 x 375, 16/32/64 net: dec3 and dec2 3.23 ms (6.8
 // before, one pair a launch) at 43 TFLOP/s; the whole training step with the input gradients of
-// conv_f32.cu 31.1 -> 10.7 ms.  The FMA pipes are 60 % busy: 96-168 registers a thread leave 12-18
+// conv_f32.cu 31.1 -> 10.6 ms.  The FMA pipes are 60 % busy: 96-168 registers a thread leave 12-18
 // warps an SM, in blocks of 3 or 6 that meet at the barrier.  Summing the folded phase-taps instead
 // ran dec3 and dec2 in 1.6 ms but moves the gradient's bits (see conv_f32.cu).
 #include "conv_f32.cuh"

@@ -52,15 +52,19 @@ sv_status Ctx::f32_plan(cudaStream_t st) {
     add_grad(FK_DS2, L_ENC3);
     add_grad(FK_DS2, L_ENC2);
   }
-  f32_n_descs = (int)descs.size();
-  f32_max_count = 0;
-  for (auto& d : descs) f32_max_count = std::max(f32_max_count, d.count);
+  size_t max_count = 0;
+  for (auto& d : descs) max_count = std::max(max_count, d.count);
   sv_status s;
   if ((s = cuda(f32_w.ensure(total * sizeof(float)), "alloc packed FP32 weights"))) return s;
   if ((s = cuda(f32_descs.ensure(descs.size() * sizeof(F32PackDesc)), "alloc pack table"))) return s;
-  return cuda(cudaMemcpyAsync(f32_descs.p, descs.data(), descs.size() * sizeof(F32PackDesc), cudaMemcpyHostToDevice,
-                              st),
-              "upload pack table");
+  if ((s = cuda(cudaMemcpyAsync(f32_descs.p, descs.data(), descs.size() * sizeof(F32PackDesc), cudaMemcpyHostToDevice,
+                                st),
+                "upload pack table")))
+    return s;
+  // The count says that the plan is there (f32_pack, the first training call): set once it is.
+  f32_n_descs = (int)descs.size();
+  f32_max_count = max_count;
+  return SV_OK;
 }
 
 sv_status Ctx::f32_pack(cudaStream_t st) {
@@ -267,7 +271,10 @@ sv_status Ctx::f32_train_forward(const sv_pair* pairs, const void* const* coarse
 sv_status Ctx::train_forward_bf16(const sv_pair* pairs, const void* const* coarse, const void* const* eps, int n,
                                   void* const* Y, void* const* mu, void* const* lv, cudaStream_t st) {
   sv_status s;
-  if (f32_n_descs == 0 && ((s = f32_plan(st)) || (s = f32_pack(st)))) return s;
+  if (f32_n_descs == 0 && ((s = f32_plan(st)) || (s = f32_pack(st)))) {
+    f32_n_descs = 0;  // the next call plans and packs again
+    return s;
+  }
   if ((s = train_save_alloc(pairs, n, false, mu, lv))) return s;
   train_pairs.assign(pairs, pairs + n);
   train_coarse.assign(coarse, coarse + n);

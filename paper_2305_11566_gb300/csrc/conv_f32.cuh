@@ -69,7 +69,7 @@ struct F32WJob {
   const float* g;  // [Ho][Wo][Co]
   const float* x;  // [Hi][Wi][Ci]
   int Hi, Wi, Ho, Wo;
-  int unit0, units;  // first slot of this pair in the launch, its slots
+  int unit0, units;  // first slot of this pair in its range, its slots
 };
 
 // One packed weight block; see f32_pack_kernel.
@@ -114,21 +114,25 @@ cudaError_t launch_f32_final(const F32Img* imgs, int n, int maxH, int maxW, cons
                              bool ordered, cudaStream_t st);
 
 // Weight gradients: plan (fills the jobs' slot ranges), slots (scratch, p.slot_floats) and launch;
-// gw / gb are added to.
+// gw / gb are added to.  Every pair needs slots of its own, so the pairs go in ranges of at most
+// slot_budget floats of slots (one pair at least), one after the other on the same scratch: the sums are
+// added in pair order either way.
+struct F32WRange { int i0, n, units; };
 struct F32WPlan {
-  int kind = 0, co = 0, ci = 0, units = 0;
+  int kind = 0, co = 0, ci = 0;
   size_t slot = 0, slot_floats = 0;
+  std::vector<F32WRange> ranges;
 };
-F32WPlan f32_wgrad_plan(int kind, int co, int ci, std::vector<F32WJob>& jobs);
-cudaError_t launch_f32_wgrad(const F32WPlan& p, const F32WJob* d_jobs, int n, float* gw, float* gb, float* slots,
+F32WPlan f32_wgrad_plan(int kind, int co, int ci, std::vector<F32WJob>& jobs, size_t slot_budget);
+cudaError_t launch_f32_wgrad(const F32WPlan& p, const F32WJob* d_jobs, float* gw, float* gb, float* slots,
                              cudaStream_t st);
 // Input gradient of the final conv (masked by d3's ReLU).
 cudaError_t launch_f32_final_dgrad(const F32Img* imgs, int n, int maxH, int maxW, const float* w, int C,
                                    cudaStream_t st);
 // Weight gradients of the final conv (kind FK_WFINAL) and of enc1 (FK_WENC1).
 enum { FK_WFINAL = FK_COUNT, FK_WENC1 };
-cudaError_t launch_f32_edge_wgrad(const F32WPlan& p, const F32Img* imgs, const F32WJob* d_jobs, int n, float* gw,
-                                  float* gb, float* slots, cudaStream_t st);
+cudaError_t launch_f32_edge_wgrad(const F32WPlan& p, const F32Img* imgs, const F32WJob* d_jobs, float* gw, float* gb,
+                                  float* slots, cudaStream_t st);
 cudaError_t launch_f32_latent_bwd(const F32Lat* lat, int n, size_t max_n, cudaStream_t st);
 
 }  // namespace sv

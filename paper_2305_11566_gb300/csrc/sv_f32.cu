@@ -19,6 +19,11 @@ namespace {
 // than fill the GPU.
 constexpr size_t kGroupBytes = size_t(2) << 30;
 
+// Bytes of weight-gradient slots a launch may use.  A slot is a copy of the layer's weights and a pair has
+// up to 304 of them: 142 MB a 1242 x 375 pair for dec1 of the 32/64/128 net.  1 GiB holds 7, whose 1680
+// chains fill the GPU several times over.
+constexpr size_t kSlotBytes = size_t(1) << 30;
+
 constexpr size_t pad32(size_t v) { return (v + 31) / 32 * 32; }
 
 }  // namespace
@@ -460,7 +465,7 @@ sv_status Ctx::f32_backward(const void* const* gY, const void* const* gmu_ext, c
     size_t og[L_COUNT], of[L_COUNT], ow[L_COUNT];
     const size_t o_img = tb.put(img), o_lat = tb.put(lat);
     for (int l = 0; l < L_COUNT; ++l) {
-      wp[l] = f32_wgrad_plan(kinds[l], net.cout(l), net.cin(l), wj[l]);
+      wp[l] = f32_wgrad_plan(kinds[l], net.cout(l), net.cin(l), wj[l], kSlotBytes / sizeof(float));
       slots = std::max(slots, wp[l].slot_floats);
       og[l] = tb.put(gj[l]);
       of[l] = tb.put(fj[l]);
@@ -484,8 +489,8 @@ sv_status Ctx::f32_backward(const void* const* gY, const void* const* gmu_ext, c
     };
     auto wgrad = [&](int l) {
       const F32WJob* j = (const F32WJob*)(d + ow[l]);
-      if (l == L_FINAL || l == L_ENC1) return launch_f32_edge_wgrad(wp[l], d_img, j, m, GW(l), GB(l), sl, st);
-      return launch_f32_wgrad(wp[l], j, m, GW(l), GB(l), sl, st);
+      if (l == L_FINAL || l == L_ENC1) return launch_f32_edge_wgrad(wp[l], d_img, j, GW(l), GB(l), sl, st);
+      return launch_f32_wgrad(wp[l], j, GW(l), GB(l), sl, st);
     };
     SV_BW("bwd_final_dgrad", launch_f32_final_dgrad(d_img, m, mH[0], mW[0], W + net.w_off(L_FINAL), net.dec[2], st));
     SV_BW("bwd_final_wgrad", wgrad(L_FINAL));

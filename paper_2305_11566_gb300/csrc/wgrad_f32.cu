@@ -471,39 +471,39 @@ cudaError_t reduce(const F32WPlan& p, const F32WJob* d_jobs, int n, int taps, fl
 }
 
 template <int KIND, int COL, int CGN, int IGN, int NB>
-cudaError_t run_wgrad(const F32WJob* d_jobs, const F32WPlan& p, int n, float* gw, float* gb, float* slots,
-                      cudaStream_t st) {
+cudaError_t run_wgrad(const F32WJob* d_jobs, const F32WPlan& p, const F32WRange& r, float* gw, float* gb,
+                      float* slots, cudaStream_t st) {
   using G = WG<KIND, COL, CGN, IGN, NB>;
   auto kern = wgrad_f32_kernel<KIND, COL, CGN, IGN, NB>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM);
   if (e != cudaSuccess) return e;
-  kern<<<dim3(p.units, (p.co / G::BCO) * ((p.ci + G::BCI - 1) / G::BCI)), G::NT, G::SMEM, st>>>(d_jobs, n, p.co, p.ci,
+  kern<<<dim3(r.units, (p.co / G::BCO) * ((p.ci + G::BCI - 1) / G::BCI)), G::NT, G::SMEM, st>>>(d_jobs, r.n, p.co, p.ci,
                                                                                              p.slot, slots);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  return reduce(p, d_jobs, n, WK<KIND>::KR * WK<KIND>::KC, gw, gb, slots, st);
+  return reduce(p, d_jobs, r.n, WK<KIND>::KR * WK<KIND>::KC, gw, gb, slots, st);
 }
 
 // Channel blocks by the layer's widths: as many output channels as fit a warp's lanes, then input
 // channels up to 12 warps a block.
 template <int KIND>
-cudaError_t wgrad_by_width(const F32WJob* d_jobs, const F32WPlan& p, int n, float* gw, float* gb, float* slots,
-                           cudaStream_t st) {
+cudaError_t wgrad_by_width(const F32WJob* d_jobs, const F32WPlan& p, const F32WRange& r, float* gw, float* gb,
+                           float* slots, cudaStream_t st) {
   if (p.co % 64 == 0) {
-    if (p.ci > 32) return run_wgrad<KIND, 8, 8, 4, 4>(d_jobs, p, n, gw, gb, slots, st);
-    return run_wgrad<KIND, 8, 8, 4, 2>(d_jobs, p, n, gw, gb, slots, st);
+    if (p.ci > 32) return run_wgrad<KIND, 8, 8, 4, 4>(d_jobs, p, r, gw, gb, slots, st);
+    return run_wgrad<KIND, 8, 8, 4, 2>(d_jobs, p, r, gw, gb, slots, st);
   }
   if (p.co % 32 == 0) {
-    if (p.ci > 32) return run_wgrad<KIND, 8, 4, 8, 2>(d_jobs, p, n, gw, gb, slots, st);
-    if (p.ci > 16) return run_wgrad<KIND, 8, 4, 8, 1>(d_jobs, p, n, gw, gb, slots, st);
-    return run_wgrad<KIND, 4, 8, 4, 1>(d_jobs, p, n, gw, gb, slots, st);
+    if (p.ci > 32) return run_wgrad<KIND, 8, 4, 8, 2>(d_jobs, p, r, gw, gb, slots, st);
+    if (p.ci > 16) return run_wgrad<KIND, 8, 4, 8, 1>(d_jobs, p, r, gw, gb, slots, st);
+    return run_wgrad<KIND, 4, 8, 4, 1>(d_jobs, p, r, gw, gb, slots, st);
   }
-  if (p.ci > 32) return run_wgrad<KIND, 4, 4, 8, 2>(d_jobs, p, n, gw, gb, slots, st);
-  return run_wgrad<KIND, 4, 4, 8, 1>(d_jobs, p, n, gw, gb, slots, st);
+  if (p.ci > 32) return run_wgrad<KIND, 4, 4, 8, 2>(d_jobs, p, r, gw, gb, slots, st);
+  return run_wgrad<KIND, 4, 4, 8, 1>(d_jobs, p, r, gw, gb, slots, st);
 }
 
 }  // namespace
 
-F32WPlan f32_wgrad_plan(int kind, int co, int ci, std::vector<F32WJob>& jobs) {
+F32WPlan f32_wgrad_plan(int kind, int co, int ci, std::vector<F32WJob>& jobs, size_t slot_budget) {
   F32WPlan p;
   p.kind = kind;
   p.co = co;
@@ -512,25 +512,40 @@ F32WPlan f32_wgrad_plan(int kind, int co, int ci, std::vector<F32WJob>& jobs) {
   // chains of a pair (part of the summation order: a change moves the gradient's last bits)
   const bool few = co * taps * ci + co <= 512 && (co < 16 || ci < 16);
   const int most = few ? 608 : 304;
+  p.slot = ((size_t)taps * co * ci + co + 31) / 32 * 32;
+  size_t total = 0;
   for (F32WJob& j : jobs) {
     const int tiles = ((j.Wo + kTC - 1) / kTC) * ((j.Ho + kTR - 1) / kTR);
-    j.unit0 = p.units;
     j.units = std::min(tiles, most);
-    p.units += j.units;
+    total += j.units;
   }
-  p.slot = ((size_t)taps * co * ci + co + 31) / 32 * 32;
-  p.slot_floats = p.slot * p.units;
+  // ranges of about equal work, so that no small one is left over
+  const size_t cap = std::max<size_t>(1, slot_budget / p.slot), parts = (total + cap - 1) / cap,
+               share = (total + parts - 1) / std::max<size_t>(1, parts);
+  for (int i = 0; i < (int)jobs.size(); ++i) {
+    const size_t u = p.ranges.empty() ? 0 : p.ranges.back().units;
+    if (p.ranges.empty() || u >= share || u + jobs[i].units > cap) p.ranges.push_back({i, 0, 0});
+    F32WRange& r = p.ranges.back();
+    jobs[i].unit0 = r.units;
+    r.units += jobs[i].units;
+    ++r.n;
+    p.slot_floats = std::max(p.slot_floats, p.slot * r.units);
+  }
   return p;
 }
 
-cudaError_t launch_f32_wgrad(const F32WPlan& p, const F32WJob* d_jobs, int n, float* gw, float* gb, float* slots,
+cudaError_t launch_f32_wgrad(const F32WPlan& p, const F32WJob* d_jobs, float* gw, float* gb, float* slots,
                              cudaStream_t st) {
-  switch (p.kind) {
-    case FK_S2: return wgrad_by_width<FK_S2>(d_jobs, p, n, gw, gb, slots, st);
-    case FK_P1: return wgrad_by_width<FK_P1>(d_jobs, p, n, gw, gb, slots, st);
-    case FK_UP2: return wgrad_by_width<FK_UP2>(d_jobs, p, n, gw, gb, slots, st);
+  for (const F32WRange& r : p.ranges) {
+    cudaError_t e = cudaErrorInvalidValue;
+    switch (p.kind) {
+      case FK_S2: e = wgrad_by_width<FK_S2>(d_jobs + r.i0, p, r, gw, gb, slots, st); break;
+      case FK_P1: e = wgrad_by_width<FK_P1>(d_jobs + r.i0, p, r, gw, gb, slots, st); break;
+      case FK_UP2: e = wgrad_by_width<FK_UP2>(d_jobs + r.i0, p, r, gw, gb, slots, st); break;
+    }
+    if (e != cudaSuccess) return e;
   }
-  return cudaErrorInvalidValue;
+  return cudaSuccess;
 }
 
 cudaError_t launch_f32_final_dgrad(const F32Img* imgs, int n, int maxH, int maxW, const float* w, int C,
@@ -542,22 +557,27 @@ cudaError_t launch_f32_final_dgrad(const F32Img* imgs, int n, int maxH, int maxW
   return cudaGetLastError();
 }
 
-cudaError_t launch_f32_edge_wgrad(const F32WPlan& p, const F32Img* imgs, const F32WJob* d_jobs, int n, float* gw,
-                                  float* gb, float* slots, cudaStream_t st) {
-  if (p.kind == FK_WENC1) {
-    const bool two = 3 * p.co / 4 <= 16;
-    const int per = kEwWarps * (two ? 2 : 1);
-    (two ? f32_enc1_wgrad_kernel<2> : f32_enc1_wgrad_kernel<1>)<<<(p.units + per - 1) / per, 32 * kEwWarps, 0, st>>>(
-        imgs, d_jobs, n, p.units, p.co, p.slot, slots);
-  } else {
-    const int lanes = 3 * p.ci / 4,  // of a chain (C <= 256: at most 192)
-              threads = std::max(lanes, 128), per = threads / lanes;
-    f32_final_wgrad_kernel<<<(p.units + per - 1) / per, threads, 0, st>>>(imgs, d_jobs, n, p.units, p.ci, lanes, p.slot,
-                                                                          slots);
+cudaError_t launch_f32_edge_wgrad(const F32WPlan& p, const F32Img* imgs, const F32WJob* d_jobs, float* gw, float* gb,
+                                  float* slots, cudaStream_t st) {
+  for (const F32WRange& r : p.ranges) {
+    const F32Img* im = imgs + r.i0;
+    const F32WJob* j = d_jobs + r.i0;
+    if (p.kind == FK_WENC1) {
+      const bool two = 3 * p.co / 4 <= 16;
+      const int per = kEwWarps * (two ? 2 : 1);
+      (two ? f32_enc1_wgrad_kernel<2> : f32_enc1_wgrad_kernel<1>)<<<(r.units + per - 1) / per, 32 * kEwWarps, 0, st>>>(
+          im, j, r.n, r.units, p.co, p.slot, slots);
+    } else {
+      const int lanes = 3 * p.ci / 4,  // of a chain (C <= 256: at most 192)
+                threads = std::max(lanes, 128), per = threads / lanes;
+      f32_final_wgrad_kernel<<<(r.units + per - 1) / per, threads, 0, st>>>(im, j, r.n, r.units, p.ci, lanes, p.slot,
+                                                                            slots);
+    }
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = reduce(p, j, r.n, 9, gw, gb, slots, st);
+    if (e != cudaSuccess) return e;
   }
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  return reduce(p, d_jobs, n, 9, gw, gb, slots, st);
+  return cudaSuccess;
 }
 
 cudaError_t launch_f32_latent_bwd(const F32Lat* lat, int n, size_t max_n, cudaStream_t st) {

@@ -1,0 +1,35 @@
+"""The FP32 form where a call's pairs are taken in more than one group or range: bit-equal to the pairs
+taken one by one, since a pair's own sums do not depend on the others and the pairs are added in order."""
+import pytest
+import torch
+
+from paper_2305_11566_gb300 import binding, synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("form", ["fp32", "bf16"])
+def test_weight_gradients_over_slot_ranges(svlib, form):
+    """96 crops of 256 x 128, 32/64/128 net: 1.8 GB of slots for dec2, two ranges of at most 1 GiB."""
+    shape, n, W, H, D = synth.NET_WIDE, 96, 256, 128, 16
+    g = torch.Generator(device="cuda").manual_seed(3)
+    ctx = binding.Context(shape, 7, form)
+    try:
+        ctx.set_weights(synth.he_normal_weights(shape, 7))
+        dp = binding.to_device(synth.make_pair(W, H, 40.0, 5), D)
+        h3, w3 = binding.latent_hw(H, W)
+        coarse = [torch.rand(H // 4, W // 4, device="cuda", generator=g) * (D - 1) for _ in range(n)]
+        eps = [torch.randn(h3, w3, shape.latent, device="cuda", generator=g) for _ in range(n)]
+        gY = [torch.randn(H, W, device="cuda", generator=g) * 1e-4 for _ in range(n)]
+        gl = [torch.randn(h3, w3, shape.latent, device="cuda", generator=g) * 1e-5 for _ in range(n)]
+        ctx.refine_train([dp] * n, coarse, eps)
+        many, _ = ctx.refine_backward(gY, gl, gl, False, coarse)
+        total = torch.zeros_like(many)
+        for i in range(n):
+            ctx.refine_train([dp], coarse[i:i + 1], eps[i:i + 1])
+            one, _ = ctx.refine_backward(gY[i:i + 1], gl[i:i + 1], gl[i:i + 1], False, coarse[i:i + 1])
+            total += one
+        ctx.synchronize()
+        assert many.abs().max() > 0 and torch.equal(many, total)
+    finally:
+        ctx.close()

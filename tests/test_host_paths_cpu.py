@@ -41,3 +41,21 @@ def test_training_after_a_failed_first_call(host, failing):
         assert h.backward() == binding.SV_OK
     finally:
         h.close()
+
+
+def test_weight_gradient_slots_are_bounded(host):
+    """Every pair has weight-gradient slots of its own (19 MB for dec2 of the 32/64/128 net on a 256 x 128
+    crop), so a backward of many pairs takes them in ranges: beside the saved activations it needs the
+    2 GiB of a group's gradients and 1 GiB of slots at most, 4 % for its tables."""
+    h = hostlib.Host(host, synth.NET_WIDE, "fp32", [(256, 128)] * 200, 7, 16)
+    try:
+        assert h.train() == binding.SV_OK, h.error()
+        before = host.host_used()
+        host.host_clear()
+        assert h.backward() == binding.SV_OK, h.error()
+        assert host.host_peak() - before <= 1.04 * (3 << 30), host.host_peak() - before
+        # every pair's slots are summed: 200 pairs of 64 tiles in dec2's 128 x 64 grid
+        dec2 = [g for k, g in h.launches() if "wgrad_f32_kernel" in k and g[0] % 64 == 0]
+        assert sum(g[0] for g in dec2) >= 200 * 64
+    finally:
+        h.close()

@@ -1,6 +1,7 @@
 // sv_ctx.cuh -- the library context behind the opaque sv_ctx handle.
 #pragma once
 
+#include <initializer_list>
 #include <map>
 #include <string>
 #include <vector>
@@ -121,6 +122,7 @@ struct Ctx {
   DevBuf adam_m, adam_v;
   // differentiation form: state saved by the last training forward
   DevBuf train_saved, train_scratch, loss_acc, train_mu;
+  DevBuf train_enc;              // FP32 contexts: e1 .. e3 of the last training forward, where they fit
   DevBuf wgrad_slots;            // per-block partial weight gradients of the FP32 backward
   std::vector<sv_pair> train_pairs;
   std::vector<const void*> train_coarse;
@@ -202,6 +204,7 @@ struct Ctx {
   template <typename T>
   sv_status refine_direct(const sv_pair& p, const void* coarse_map, bool coarse_int16, const T* eps, T* Y, T* mu_out,
                           T* lv_out, T* const* saved, cudaStream_t st);
+  bool give_back(std::initializer_list<DevBuf*> spare);
   sv_status f32_plan(cudaStream_t st);
   sv_status f32_pack(cudaStream_t st);
   sv_status f32_forward(const sv_pair* pairs, int n, const F32Tensors* t, const int16_t* const* coarse_i,
@@ -210,7 +213,7 @@ struct Ctx {
                               void* const* Y, void* const* mu, void* const* lv, cudaStream_t st);
   sv_status f32_backward(const void* const* gY, const void* const* gmu_ext, const void* const* glv_ext, float* gparams,
                          void* const* gcoarse, cudaStream_t st);
-  sv_status train_save_alloc(const sv_pair* pairs, int n, bool encoder, void* const* mu, void* const* lv);
+  sv_status train_save_alloc(const sv_pair* pairs, int n, void* const* mu, void* const* lv);
   sv_status f32_refine(const sv_pair* pairs, const int16_t* const* coarse, int n, float* const* out, cudaStream_t st);
   sv_status refine_infer(const sv_pair* pairs, const int16_t* const* coarse, int n, float* const* out,
                          cudaStream_t st);
@@ -300,7 +303,7 @@ struct Ctx {
     for (auto& b : act) b.release();
     for (auto& b : tc_act) b.release();
     tc_tables.release(); adam_m.release(); adam_v.release();
-    train_saved.release(); train_scratch.release(); loss_acc.release(); train_mu.release(); wgrad_slots.release();
+    train_saved.release(); train_enc.release(); train_scratch.release(); loss_acc.release(); train_mu.release(); wgrad_slots.release();
   }
 };
 

@@ -15,7 +15,7 @@ cudaError_t launch_up4_bwd(const T* gU, const T* gx0, int W, int H, int w, int h
 namespace {
 
 // Bytes of activations one group of pairs may hold: pairs beyond it run as further groups on
-// the same workspace.  A 1242 x 375 pair of the 32/64/128 net needs 134 MB; 2 GiB hold 16, more
+// the same workspace.  Where an allocation of a group fails, smaller groups are tried, down to one pair.  A 1242 x 375 pair of the 32/64/128 net needs 134 MB; 2 GiB hold 16, more
 // than fill the GPU.
 constexpr size_t kGroupBytes = size_t(2) << 30;
 
@@ -190,8 +190,22 @@ static void act_sizes(const NetDims& net, const Levels& lv, size_t out[7]) {
   for (int k = 0; k < 7; ++k) out[k] = pad32(v[k]);
 }
 
+// After an allocation failed: releases the workspaces that the call can do without.  True if there was
+// one (another try may succeed).
+bool Ctx::give_back(std::initializer_list<DevBuf*> spare) {
+  bool any = false;
+  for (DevBuf* b : spare)
+    if (b->p) {
+      b->release();
+      any = true;
+    }
+  if (any) err.clear();
+  return any;
+}
+
 sv_status Ctx::f32_refine(const sv_pair* pairs, const int16_t* const* coarse, int n, float* const* out,
                           cudaStream_t st) {
+  size_t budget = kGroupBytes;
   for (int i0 = 0; i0 < n;) {
     std::vector<F32Tensors> t;
     std::vector<size_t> ofs;
@@ -201,12 +215,20 @@ sv_status Ctx::f32_refine(const sv_pair* pairs, const int16_t* const* coarse, in
       size_t sz[7], sum = 0;
       act_sizes(net, Levels(pairs[i1].height, pairs[i1].width), sz);
       for (size_t v : sz) sum += v;
-      if (i1 > i0 && (total + sum) * sizeof(float) > kGroupBytes) break;
+      if (i1 > i0 && (total + sum) * sizeof(float) > budget) break;
       ofs.push_back(total);
       total += sum;
     }
     sv_status s;
-    if ((s = cuda(f32_act.ensure(total * sizeof(float)), "alloc activations"))) return s;
+    if ((s = cuda(f32_act.ensure(total * sizeof(float)), "alloc activations"))) {
+      if (s != SV_ERR_OOM) return s;
+      if (!give_back({&train_scratch, &wgrad_slots})) {
+        if (i1 - i0 == 1) return s;
+        budget = total * sizeof(float) / 2;
+        err.clear();
+      }
+      continue;
+    }
     for (int i = i0; i < i1; ++i) {
       size_t sz[7];
       act_sizes(net, Levels(pairs[i].height, pairs[i].width), sz);
@@ -224,14 +246,14 @@ sv_status Ctx::f32_refine(const sv_pair* pairs, const int16_t* const* coarse, in
 
 // ---------------------------------------------------------------- training
 
-// Places the tensors the backward needs of every pair in train_saved (encoder: e1 .. e3 too) and
-// the mean head's own output in train_mu.
-sv_status Ctx::train_save_alloc(const sv_pair* pairs, int n, bool encoder, void* const* mu, void* const* lv) {
+// Places the decoder activations and the latent of every pair, which the backward needs, in train_saved
+// and the mean head's own output in train_mu.
+sv_status Ctx::train_save_alloc(const sv_pair* pairs, int n, void* const* mu, void* const* lv) {
   size_t total = 0, lat_total = 0;
   for (int i = 0; i < n; ++i) {
     size_t sz[7];
     act_sizes(net, Levels(pairs[i].height, pairs[i].width), sz);
-    for (int k = encoder ? 0 : 3; k < 7; ++k) total += sz[k];
+    for (int k = 3; k < 7; ++k) total += sz[k];
     total += 2 * sz[3];  // lv, eps
     lat_total += sz[3];
   }
@@ -245,7 +267,6 @@ sv_status Ctx::train_save_alloc(const sv_pair* pairs, int n, bool encoder, void*
     act_sizes(net, Levels(pairs[i].height, pairs[i].width), sz);
     auto take = [&](int k) { float* r = q; q += sz[k]; return r; };
     F32Tensors& t = train_t[i];
-    if (encoder) { t.e1 = take(0); t.e2 = take(1); t.e3 = take(2); }
     t.z = take(3); t.d1 = take(4); t.d2 = take(5); t.d3 = take(6);
     t.lv = take(3); t.eps_copy = take(3);
     t.mu = m;
@@ -256,16 +277,77 @@ sv_status Ctx::train_save_alloc(const sv_pair* pairs, int n, bool encoder, void*
   return SV_OK;
 }
 
+// Places e1 .. e3 of a pair at q.
+static void place_encoder(F32Tensors& t, float* q, const size_t sz[7]) {
+  t.e1 = q;
+  t.e2 = q + sz[0];
+  t.e3 = q + sz[0] + sz[1];
+}
+
+// Keeps the encoder's activations for the backward (train_enc) where they fit.  Else the forward goes
+// through groups of pairs whose encoder activations are let go, and the backward recomputes them as it does
+// for the BF16 form: the same kernels, the same bits.
 sv_status Ctx::f32_train_forward(const sv_pair* pairs, const void* const* coarse, const void* const* eps, int n,
                                  void* const* Y, void* const* mu, void* const* lv, cudaStream_t st) {
   sv_status s;
-  if ((s = train_save_alloc(pairs, n, true, mu, lv))) return s;
+  while ((s = train_save_alloc(pairs, n, mu, lv)))
+    if (s != SV_ERR_OOM || !give_back({&train_scratch, &wgrad_slots, &f32_act, &train_enc})) return s;
+  size_t enc_total = 0;
+  for (int i = 0; i < n; ++i) {
+    size_t sz[7];
+    act_sizes(net, Levels(pairs[i].height, pairs[i].width), sz);
+    enc_total += sz[0] + sz[1] + sz[2];
+  }
+  while ((s = cuda(train_enc.ensure(enc_total * sizeof(float)), "alloc encoder activations")))
+    if (s != SV_ERR_OOM || !give_back({&train_scratch, &wgrad_slots, &f32_act})) break;
+  if (s && s != SV_ERR_OOM) return s;
+  const bool keep = s == SV_OK;
+  err.clear();
+  if (keep) {
+    float* q = (float*)train_enc.p;
+    for (int i = 0; i < n; ++i) {
+      size_t sz[7];
+      act_sizes(net, Levels(pairs[i].height, pairs[i].width), sz);
+      place_encoder(train_t[i], q, sz);
+      q += sz[0] + sz[1] + sz[2];
+    }
+  }
   train_pairs.assign(pairs, pairs + n);
   train_coarse.assign(coarse, coarse + n);
   train_elem = sizeof(float);
-  if ((s = f32_forward(pairs, n, train_t.data(), nullptr, (const float* const*)coarse, (const float* const*)eps,
-                       (float* const*)Y, st)))
-    return s;
+  size_t budget = kGroupBytes;
+  for (int i0 = 0; i0 < n;) {
+    size_t total = 0;
+    int i1 = i0;
+    std::vector<F32Tensors> t;
+    std::vector<size_t> ofs;
+    for (; i1 < n; ++i1) {
+      size_t sz[7];
+      act_sizes(net, Levels(pairs[i1].height, pairs[i1].width), sz);
+      const size_t sum = keep ? 0 : sz[0] + sz[1] + sz[2];
+      if (i1 > i0 && (total + sum) * sizeof(float) > budget) break;
+      t.push_back(train_t[i1]);
+      ofs.push_back(total);
+      total += sum;
+    }
+    if (!keep) {
+      if ((s = cuda(f32_act.ensure(total * sizeof(float)), "alloc encoder activations"))) {
+        if (s != SV_ERR_OOM || i1 - i0 == 1) return s;
+        budget = total * sizeof(float) / 2;
+        err.clear();
+        continue;
+      }
+      for (int i = i0; i < i1; ++i) {
+        size_t sz[7];
+        act_sizes(net, Levels(pairs[i].height, pairs[i].width), sz);
+        place_encoder(t[i - i0], (float*)f32_act.p + ofs[i - i0], sz);
+      }
+    }
+    if ((s = f32_forward(pairs + i0, i1 - i0, t.data(), nullptr, (const float* const*)coarse + i0,
+                         (const float* const*)eps + i0, (float* const*)Y + i0, st)))
+      return s;
+    i0 = i1;
+  }
   train_ready = true;
   return SV_OK;
 }
@@ -280,14 +362,19 @@ sv_status Ctx::train_forward_bf16(const sv_pair* pairs, const void* const* coars
     f32_n_descs = 0;  // the next call plans and packs again
     return s;
   }
-  if ((s = train_save_alloc(pairs, n, false, mu, lv))) return s;
+  auto fitted = [&](auto alloc) {  // (a backward's scratch is not needed before the next backward)
+    sv_status r = alloc();
+    if (r == SV_ERR_OOM && give_back({&train_scratch, &wgrad_slots})) r = alloc();
+    return r;
+  };
+  if ((s = fitted([&] { return train_save_alloc(pairs, n, mu, lv); }))) return s;
   train_pairs.assign(pairs, pairs + n);
   train_coarse.assign(coarse, coarse + n);
   train_elem = sizeof(float);
   std::vector<float*> outs(n);
   for (int i = 0; i < n; ++i) outs[i] = (float*)Y[i];
   TcRun r;
-  if ((s = tc_prepare(pairs, nullptr, n, outs.data(), r, (const float* const*)coarse))) return s;
+  if ((s = fitted([&] { return tc_prepare(pairs, nullptr, n, outs.data(), r, (const float* const*)coarse); }))) return s;
   std::vector<size_t> e3_ofs(n);
   size_t e3_total = 0;
   TcTrainLatent tl{};
@@ -297,7 +384,7 @@ sv_status Ctx::train_forward_bf16(const sv_pair* pairs, const void* const* coars
     e3_total += pad32(tc_len[i][2]);
     tl.max_e3 = std::max(tl.max_e3, tc_len[i][2]);
   }
-  if ((s = cuda(f32_act.ensure(e3_total * sizeof(float)), "alloc latent input"))) return s;
+  if ((s = fitted([&] { return cuda(f32_act.ensure(e3_total * sizeof(float)), "alloc latent input"); }))) return s;
   std::vector<F32Cvt> cvt_e3(n), cvt_d;
   std::vector<F32Job> jm(n), jl(n);
   std::vector<F32Lat> lat(n);
@@ -360,7 +447,7 @@ sv_status Ctx::f32_backward(const void* const* gY, const void* const* gmu_ext, c
   auto GW = [&](int l) { return gparams + net.w_off(l); };
   auto GB = [&](int l) { return gparams + net.b_off(l); };
   if ((s = cuda(cudaMemsetAsync(gparams, 0, net.count() * sizeof(float), st), "zero grads"))) return s;
-  const bool recompute = n > 0 && train_t[0].e1 == nullptr;
+  bool recompute = n > 0 && train_t[0].e1 == nullptr;
   bool want_coarse = false;
   for (int i = 0; gcoarse && i < n; ++i) want_coarse |= gcoarse[i] != nullptr;
   // floats of one pair's gradients: e1 e2 e3 (and the recomputed activations), z, mu, lv, d1 d2 d3, x0
@@ -373,17 +460,36 @@ sv_status Ctx::f32_backward(const void* const* gY, const void* const* gmu_ext, c
     if (want_coarse) t += pad32((size_t)2 * lv.H[0] * lv.W[0]);
     return t;
   };
+  size_t budget = kGroupBytes, slot_budget = kSlotBytes;
   for (int i0 = 0; i0 < n;) {
     size_t total = 0;
     int i1 = i0;
     for (; i1 < n; ++i1) {
       size_t sz[7];
       const size_t f = pair_floats(i1, sz);
-      if (i1 > i0 && (total + f) * sizeof(float) > kGroupBytes) break;
+      if (i1 > i0 && (total + f) * sizeof(float) > budget) break;
       total += f;
     }
     const int m = i1 - i0;
-    if ((s = cuda(train_scratch.ensure(total * sizeof(float)), "alloc backward scratch"))) return s;
+    // The group again: with the forward's workspace given back, half the budget, or for a single pair
+    // the encoder's kept activations given back too.
+    auto again = [&] {
+      if (give_back({&f32_act})) return true;
+      if (m > 1) {
+        budget = total * sizeof(float) / 2;
+      } else {
+        if (recompute || !give_back({&train_enc})) return false;
+        for (F32Tensors& t : train_t) t.e1 = t.e2 = t.e3 = nullptr;
+        recompute = true;
+      }
+      train_scratch.release();
+      err.clear();
+      return true;
+    };
+    if ((s = cuda(train_scratch.ensure(total * sizeof(float)), "alloc backward scratch"))) {
+      if (s == SV_ERR_OOM && (give_back({&wgrad_slots}) || again())) continue;
+      return s;
+    }
     float* q = (float*)train_scratch.p;
     std::vector<F32Img> img(m);
     std::vector<F32Lat> lat(m);
@@ -460,18 +566,31 @@ sv_status Ctx::f32_backward(const void* const* gY, const void* const* gmu_ext, c
     }
     static const int kinds[L_COUNT] = {FK_WENC1, FK_S2, FK_S2, FK_P1, FK_P1, FK_UP2, FK_UP2, FK_UP2, FK_WFINAL};
     F32WPlan wp[L_COUNT];
-    size_t slots = 0;
+    for (;;) {
+      size_t slots = 0;
+      bool split = false;  // the largest ranges can be cut further
+      for (int l = 0; l < L_COUNT; ++l) {
+        wp[l] = f32_wgrad_plan(kinds[l], net.cout(l), net.cin(l), wj[l], slot_budget / sizeof(float));
+        slots = std::max(slots, wp[l].slot_floats);
+      }
+      for (const F32WPlan& w : wp) split = split || (w.slot_floats == slots && (int)w.ranges.size() < m);
+      s = cuda(wgrad_slots.ensure(slots * sizeof(float)), "alloc weight-gradient slots");
+      if (s != SV_ERR_OOM || !split) break;
+      slot_budget = std::min(slot_budget, slots * sizeof(float)) / 2;
+      err.clear();
+    }
+    if (s) {
+      if (s == SV_ERR_OOM && again()) continue;
+      return s;
+    }
     Tables tb;
     size_t og[L_COUNT], of[L_COUNT], ow[L_COUNT];
     const size_t o_img = tb.put(img), o_lat = tb.put(lat);
     for (int l = 0; l < L_COUNT; ++l) {
-      wp[l] = f32_wgrad_plan(kinds[l], net.cout(l), net.cin(l), wj[l], kSlotBytes / sizeof(float));
-      slots = std::max(slots, wp[l].slot_floats);
       og[l] = tb.put(gj[l]);
       of[l] = tb.put(fj[l]);
       ow[l] = tb.put(wj[l]);
     }
-    if ((s = cuda(wgrad_slots.ensure(slots * sizeof(float)), "alloc weight-gradient slots"))) return s;
     if ((s = cuda(f32_tab.ensure(tb.host.size()), "alloc FP32 tables"))) return s;
     if ((s = cuda(cudaMemcpyAsync(f32_tab.p, tb.host.data(), tb.host.size(), cudaMemcpyHostToDevice, st),
                   "upload FP32 tables")))

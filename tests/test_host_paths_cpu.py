@@ -59,3 +59,78 @@ def test_weight_gradient_slots_are_bounded(host):
         assert sum(g[0] for g in dec2) >= 200 * 64
     finally:
         h.close()
+
+
+def pair_bytes(net, W, H, levels):
+    """FP32 bytes of the activations e1 e2 e3 z d1 d2 d3 (those asked for) of one W x H pair."""
+    px = [W * H]
+    for _ in range(3):
+        W, H = (W + 1) // 2, (H + 1) // 2
+        px.append(W * H)
+    ch = (*net.enc, net.latent, *net.dec)
+    at = (1, 2, 3, 3, 2, 1, 0)
+    return 4 * sum(px[at[k]] * ch[k] for k in levels)
+
+
+@pytest.mark.parametrize("room", [1.2, 2.5, 20])
+def test_fp32_refine_in_the_memory_that_is_there(host, room):
+    """Eight frames refine where the activations of one fit (and none where they do not)."""
+    W, H, n = 1242, 375, 8
+    h = hostlib.Host(host, synth.NET_WIDE, "fp32", [(W, H)] * n, 9, 48)
+    one = pair_bytes(synth.NET_WIDE, W, H, range(7))
+    try:
+        host.host_limit(host.host_used() + int(0.9 * one))
+        assert h.refine() == binding.SV_ERR_OOM and "activations" in h.error()
+        host.host_limit(host.host_used() + int(room * one))
+        host.host_clear()
+        assert h.refine() == binding.SV_OK, h.error()
+        assert h.error() == ""
+        finals = [g[2] for k, g in h.launches() if "f32_final_kernel" in k]
+        assert sum(finals) == n and max(finals) <= room
+    finally:
+        h.close()
+
+
+@pytest.mark.parametrize("keep", [False, True])
+def test_fp32_training_in_the_memory_that_is_there(host, keep):
+    """Four frames train where the decoder activations of all, and the gradients, the encoder's
+    activations and the weight-gradient slots of one fit: the encoder is then recomputed.  With room for
+    all of them it is not."""
+    W, H, n, net = 1242, 375, 4, synth.NET_WIDE
+    h = hostlib.Host(host, net, "fp32", [(W, H)] * n, 9, 48)
+    try:
+        saved = n * pair_bytes(net, W, H, (3, 3, 3, 3, 4, 5, 6))  # z, logvar, eps, mu; d1 .. d3
+        enc = pair_bytes(net, W, H, (0, 1, 2))
+        slots = 304 * 4 * (9 * 128 * 128 + 128)
+        work = pair_bytes(net, W, H, range(7)) + 2 * enc + slots  # one pair's backward
+        room = saved + work if not keep else saved + n * (enc + work)
+        base = host.host_used()
+        host.host_limit(base + room + (8 << 20))
+        for _ in range(2):  # the second step finds the first one's workspaces
+            host.host_clear()
+            assert h.train() == binding.SV_OK, h.error()
+            assert h.backward() == binding.SV_OK, h.error()
+            names = [k for k, _ in h.launches()]
+            enc1 = [g[2] for k, g in h.launches() if "f32_enc1_kernel" in k]
+            assert sum(enc1) == (n if keep else 2 * n), enc1
+            assert sum("final_dgrad" in k for k in names) == (1 if keep else n)
+            assert host.host_peak() <= base + room + (8 << 20)
+        h.close()
+        h = hostlib.Host(host, net, "fp32", [(W, H)] * n, 9, 48)
+        host.host_limit(host.host_used() + saved // 2)
+        assert h.train() == binding.SV_ERR_OOM and h.backward() == binding.SV_ERR_STATE
+    finally:
+        h.close()
+
+
+def test_bf16_training_gives_scratch_back(host):
+    """The scratch and the slots of a backward do not keep a larger training forward from its memory."""
+    h = hostlib.Host(host, synth.NET_SMALL, "bf16", [(1242, 375)] * 12, 9, 48)
+    try:
+        assert h.train() == binding.SV_OK and h.backward() == binding.SV_OK
+        for p in h.pairs:
+            p.height += 8  # a little more of everything
+        host.host_limit(host.host_used())
+        assert h.train() == binding.SV_OK, h.error()
+    finally:
+        h.close()

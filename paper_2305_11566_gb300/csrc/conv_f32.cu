@@ -923,8 +923,13 @@ __global__ void f32_convert_kernel(const F32Cvt* __restrict__ jobs) {
 cudaError_t launch_f32_convert(const F32Cvt* jobs, int n, size_t max_n, cudaStream_t st) {
   if (n == 0 || max_n == 0) return cudaSuccess;
   const unsigned gx = (unsigned)std::min<size_t>(1024, (max_n / 8 + 255) / 256);
-  f32_convert_kernel<<<dim3(std::max(1u, gx), n), 256, 0, st>>>(jobs);
-  return cudaGetLastError();
+  constexpr int kMost = 65535;  // jobs of a launch (the grid's y extent)
+  for (int i = 0; i < n; i += kMost) {
+    f32_convert_kernel<<<dim3(std::max(1u, gx), std::min(kMost, n - i)), 256, 0, st>>>(jobs + i);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 cudaError_t launch_f32_reparam(const F32Lat* lat, int n, size_t max_n, cudaStream_t st) {

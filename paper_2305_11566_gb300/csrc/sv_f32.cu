@@ -19,6 +19,9 @@ namespace {
 // than fill the GPU.
 constexpr size_t kGroupBytes = size_t(2) << 30;
 
+// Pairs of a group: the largest z extent of a launch's grid.
+constexpr int kGroupPairs = 65535;
+
 // Bytes of weight-gradient slots a launch may use.  A slot is a copy of the layer's weights and a pair has
 // up to 304 of them: 142 MB a 1242 x 375 pair for dec1 of the 32/64/128 net.  1 GiB holds 7, whose 1680
 // chains fill the GPU several times over.
@@ -211,7 +214,7 @@ sv_status Ctx::f32_refine(const sv_pair* pairs, const int16_t* const* coarse, in
     std::vector<size_t> ofs;
     size_t total = 0;
     int i1 = i0;
-    for (; i1 < n; ++i1) {
+    for (; i1 < n && i1 - i0 < kGroupPairs; ++i1) {
       size_t sz[7], sum = 0;
       act_sizes(net, Levels(pairs[i1].height, pairs[i1].width), sz);
       for (size_t v : sz) sum += v;
@@ -321,7 +324,7 @@ sv_status Ctx::f32_train_forward(const sv_pair* pairs, const void* const* coarse
     int i1 = i0;
     std::vector<F32Tensors> t;
     std::vector<size_t> ofs;
-    for (; i1 < n; ++i1) {
+    for (; i1 < n && i1 - i0 < kGroupPairs; ++i1) {
       size_t sz[7];
       act_sizes(net, Levels(pairs[i1].height, pairs[i1].width), sz);
       const size_t sum = keep ? 0 : sz[0] + sz[1] + sz[2];
@@ -464,7 +467,7 @@ sv_status Ctx::f32_backward(const void* const* gY, const void* const* gmu_ext, c
   for (int i0 = 0; i0 < n;) {
     size_t total = 0;
     int i1 = i0;
-    for (; i1 < n; ++i1) {
+    for (; i1 < n && i1 - i0 < kGroupPairs; ++i1) {
       size_t sz[7];
       const size_t f = pair_floats(i1, sz);
       if (i1 > i0 && (total + f) * sizeof(float) > budget) break;

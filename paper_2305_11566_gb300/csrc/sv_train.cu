@@ -248,8 +248,12 @@ sv_status Ctx::loss(const sv_pair* pairs, int n, const void* const* Y, const flo
     return s;
   {
     LaunchScope _ls(*this, "loss_partial", st);
-    if ((s = cuda(launch_loss_partial<T>(d_jobs, n, 1.0 / npix, kl_w / nlat, (double*)loss_acc.p, st), "loss")))
-      return s;
+    constexpr int kMost = 65535;  // pairs of a launch (the grid's y extent)
+    for (int i = 0; i < n; i += kMost)
+      if ((s = cuda(launch_loss_partial<T>(d_jobs + i, std::min(kMost, n - i), 1.0 / npix, kl_w / nlat,
+                                           (double*)loss_acc.p + per * i, st),
+                    "loss")))
+        return s;
   }
   LaunchScope _ls(*this, "loss_finish", st);
   return cuda(launch_loss_finish<T>((const double*)loss_acc.p, n, 1.0 / npix, 1.0 / nlat, kl_w, (T*)out, st),

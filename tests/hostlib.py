@@ -82,6 +82,10 @@ class Host:
         g = self.buffer(8 * self.params)
         return self.L.sv_refine_backward(self.ctx, self.any, self.any, self.any, ctypes.c_void_p(g), None, None)
 
+    def loss(self):
+        return self.L.sv_loss(self.ctx, self.pairs, self.n, self.any, self.any, self.any, self.any, 1e-3,
+                              ctypes.c_void_p(self.buffer(32)), self.any, self.any, self.any, None)
+
     def launches(self):
         g = (ctypes.c_uint * 3)()
         out = []

@@ -134,3 +134,21 @@ def test_bf16_training_gives_scratch_back(host):
         assert h.train() == binding.SV_OK, h.error()
     finally:
         h.close()
+
+
+@pytest.mark.parametrize("form,n", [("fp32", 70000), ("bf16", 30000)])
+def test_more_pairs_than_a_grid_is_deep(host, form, n):
+    """So many tiny pairs in one call that a launch's grid cannot hold them (FP32), or three saved
+    activations of each (BF16), in y or z."""
+    h = hostlib.Host(host, synth.NET_SMALL, form, [(12, 12)] * n, 3, 3)
+    try:
+        for call in (h.refine, h.train, h.loss, h.backward):
+            host.host_clear()
+            assert call() == binding.SV_OK, (call.__name__, h.error())
+            for name in ("f32_final_kernel", "f32_final_ordered", "loss_partial", "final_dgrad"):
+                depth = [max(g[1:]) for k, g in h.launches() if name in k]
+                assert not depth or sum(depth) == n, (call.__name__, name, depth)
+            convert = [g[1] for k, g in h.launches() if "f32_convert" in k]
+            assert not convert or sum(convert) == 4 * n  # e3, d1, d2, d3
+    finally:
+        h.close()

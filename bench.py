@@ -3,12 +3,13 @@
 
 One step = sv_pipeline over a batch of pairs: coarse ZNCC + WTA on the x4 box-
 downsampled pair (D = 48, 9x9 window) and refinement by the 32/64/128 network to a
-full-resolution disparity map.  Two forms:
-  fp32  the plain method: FP32 CUDA-core convolutions, launched pair by pair;
+full-resolution disparity map.  The forms:
+  fp32  the plain method: FP32 convolutions on the CUDA cores, all pairs of a group per launch;
   bf16  BF16 tcgen05 implicit-GEMM convolutions, all pairs in one persistent launch
-        per layer (when the library has it).
-The JSON line's value is the headline form (bf16 when available, else fp32);
-both forms are listed under "forms".
+        per layer (when the library has it);
+  fp8   the same with E4M3 operands in the quantised layers.
+The JSON line's value is the headline form (bf16 when available, else fp32); the rates of
+all of them are listed under "pairs_per_s".  --details FILE keeps the whole measurement.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl reference]
 
@@ -60,6 +61,8 @@ def parse():
     ap.add_argument("--coarse", action="store_true",
                     help="also time the coarse-stage variants (ZNCC / census cost, SGM / DT aggregation, occlusion "
                          "check and median filter) on the same pairs")
+    ap.add_argument("--details", default="", metavar="FILE",
+                    help="also write the whole measurement (rooflines of every kernel and form) as JSON")
     ap.add_argument("--train-pairs", type=int, default=16)
     ap.add_argument("--no-tune", action="store_true",
                     help="keep the default launch plans (fixed launch order, e.g. for profiler captures)")
@@ -720,11 +723,33 @@ def run_ours(args):
     if coarse is not None:
         line["coarse_variants"] = coarse
     if rank == 0:
-        print(json.dumps(line))
+        if args.details:
+            with open(args.details, "w") as f:
+                json.dump(line, f)
+        print(json.dumps(headline(line)))
     for r in results.values():
         r["ctx"].close()
     if world > 1:
         dist.destroy_process_group()
+
+
+def headline(line):
+    """The printed line: the benchmark's own keys and one number per further leg, short enough for a log's
+    tail (the whole measurement, per kernel and form, is 20 KB; --details FILE keeps it)."""
+    keys = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+            "vs_baseline", "dtype", "data", "config", "cpu_baseline", "e2e", "gpu_launches", "clocks",
+            "delta_epe_px", "wta_flip_fraction")
+    out = {k: line[k] for k in keys}
+    if line["roofline"]:
+        out["roofline"] = {k: line["roofline"].get(k) for k in ("kernel", "bound", "achieved", "peak", "unit", "frac")}
+    rate = {f"form_{f}": r["pairs_per_s"] for f, r in line["forms"].items()}
+    for leg in ("uneven_batch", "table1_net", "train_step"):
+        if line[leg]:
+            rate[leg] = line[leg]["pairs_per_s"]
+    for name, r in line.get("coarse_variants", {}).items():
+        rate[name] = r["pairs_per_s"]
+    out["pairs_per_s"] = {k: round(v, 1) for k, v in rate.items()}
+    return out
 
 
 # Coarse-stage variants timed by --coarse: (name, sv_coarse_opts keywords).  The penalties

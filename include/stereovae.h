@@ -24,6 +24,11 @@
  *     device-side bounded wait that ran out returns SV_ERR_TIMEOUT.  The text of the
  *     last error of a context is available from sv_last_error().
  *   - A context is not thread safe: one host thread at a time.
+ *   - Of the calls that take a context, sv_refine on SV_FP32 contexts, sv_refine_train,
+ *     sv_loss, sv_refine_backward and sv_adam_step may be captured into a caller's own CUDA
+ *     graph, after a call of the same sizes outside the capture has allocated the
+ *     workspaces, and replayed until a larger call on the context makes them grow.  Other
+ *     calls copy tables of their own on the stream and must not be captured.
  *   - Images are uint8, row-major with a row pitch in bytes; pitch % 16 == 0 and
  *     base pointers 16-byte aligned (rows are read with 16-byte vector loads).
  *   - Coarse maps are (height / 4) x (width / 4) (floor), row-major, dense.

@@ -84,6 +84,34 @@ sv_status Ctx::cuda(cudaError_t e, const char* what) {
   return fail(SV_ERR_CUDA, "%s: %s", what, cudaGetErrorString(e));
 }
 
+// Copies a table of this call to the device on the stream.  Where the caller captures the stream, the copy
+// runs at every replay, long after the call's own memory is gone: the graph is then given a copy of the
+// table that lives as long as it does.
+sv_status Ctx::upload(void* dst, const void* table, size_t bytes, const char* what, cudaStream_t st) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  cudaGraph_t graph = nullptr;
+  if (cudaStreamGetCaptureInfo(st, &cs, nullptr, &graph, nullptr, nullptr, nullptr) != cudaSuccess) {
+    cudaGetLastError();  // (the copy reports it)
+    cs = cudaStreamCaptureStatusNone;
+  }
+  if (cs == cudaStreamCaptureStatusActive) {
+    auto* kept = new std::vector<unsigned char>((const unsigned char*)table, (const unsigned char*)table + bytes);
+    table = kept->data();
+    cudaUserObject_t owner = nullptr;
+    cudaError_t e = cudaUserObjectCreate(
+        &owner, kept, [](void* p) { delete (std::vector<unsigned char>*)p; }, 1, cudaUserObjectNoDestructorSync);
+    if (e != cudaSuccess) {
+      delete kept;
+      return cuda(e, what);
+    }
+    if ((e = cudaGraphRetainUserObject(graph, owner, 1, cudaGraphUserObjectMove)) != cudaSuccess) {
+      cudaUserObjectRelease(owner, 1);
+      return cuda(e, what);
+    }
+  }
+  return cuda(cudaMemcpyAsync(dst, table, bytes, cudaMemcpyHostToDevice, st), what);
+}
+
 sv_status Ctx::check_pairs(const sv_pair* pairs, int n_pairs) {
   if (n_pairs < 0) return fail(SV_ERR_INVALID_ARG, "n_pairs < 0");
   if (n_pairs > 0 && !pairs) return fail(SV_ERR_INVALID_ARG, "pairs is NULL");

@@ -205,6 +205,7 @@ struct Ctx {
   sv_status refine_direct(const sv_pair& p, const void* coarse_map, bool coarse_int16, const T* eps, T* Y, T* mu_out,
                           T* lv_out, T* const* saved, cudaStream_t st);
   bool give_back(std::initializer_list<DevBuf*> spare);
+  sv_status upload(void* dst, const void* table, size_t bytes, const char* what, cudaStream_t st);
   sv_status f32_plan(cudaStream_t st);
   sv_status f32_pack(cudaStream_t st);
   sv_status f32_forward(const sv_pair* pairs, int n, const F32Tensors* t, const int16_t* const* coarse_i,

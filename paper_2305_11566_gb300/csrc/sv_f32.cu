@@ -148,9 +148,7 @@ sv_status Ctx::f32_forward(const sv_pair* pairs, int n, const F32Tensors* t, con
   for (int l = 0; l < L_COUNT; ++l) o_job[l] = tb.put(job[l]);
   sv_status s;
   if ((s = cuda(f32_tab.ensure(tb.host.size()), "alloc FP32 tables"))) return s;
-  if ((s = cuda(cudaMemcpyAsync(f32_tab.p, tb.host.data(), tb.host.size(), cudaMemcpyHostToDevice, st),
-                "upload FP32 tables")))
-    return s;
+  if ((s = upload(f32_tab.p, tb.host.data(), tb.host.size(), "upload FP32 tables", st))) return s;
   const unsigned char* d = (const unsigned char*)f32_tab.p;
   const F32Img* d_img = (const F32Img*)(d + o_img);
   const float *W = (const float*)w32.p, *P = (const float*)f32_w.p;
@@ -422,9 +420,7 @@ sv_status Ctx::train_forward_bf16(const sv_pair* pairs, const void* const* coars
   const size_t o_tc = tb.put(r.host), o_e3 = tb.put(cvt_e3), o_m = tb.put(jm), o_l = tb.put(jl), o_lat = tb.put(lat),
                o_d = tb.put(cvt_d);
   if ((s = cuda(tc_tables.ensure(tb.host.size()), "alloc tables"))) return s;
-  if ((s = cuda(cudaMemcpyAsync(tc_tables.p, tb.host.data(), tb.host.size(), cudaMemcpyHostToDevice, st),
-                "upload tables")))
-    return s;
+  if ((s = upload(tc_tables.p, tb.host.data(), tb.host.size(), "upload tables", st))) return s;
   const unsigned char* d = (const unsigned char*)tc_tables.p;
   tl.e3 = (const F32Cvt*)(d + o_e3);
   tl.mu = (const F32Job*)(d + o_m);
@@ -595,9 +591,7 @@ sv_status Ctx::f32_backward(const void* const* gY, const void* const* gmu_ext, c
       ow[l] = tb.put(wj[l]);
     }
     if ((s = cuda(f32_tab.ensure(tb.host.size()), "alloc FP32 tables"))) return s;
-    if ((s = cuda(cudaMemcpyAsync(f32_tab.p, tb.host.data(), tb.host.size(), cudaMemcpyHostToDevice, st),
-                  "upload FP32 tables")))
-      return s;
+    if ((s = upload(f32_tab.p, tb.host.data(), tb.host.size(), "upload FP32 tables", st))) return s;
     const unsigned char* d = (const unsigned char*)f32_tab.p;
     const F32Img* d_img = (const F32Img*)(d + o_img);
     float* sl = (float*)wgrad_slots.p;

@@ -243,9 +243,7 @@ sv_status Ctx::loss(const sv_pair* pairs, int n, const void* const* Y, const flo
                (size_t)lv_.H[3] * lv_.W[3] * net.lat};
   }
   LossJob<T>* d_jobs = (LossJob<T>*)((double*)loss_acc.p + per * n);
-  if ((s = cuda(cudaMemcpyAsync(d_jobs, jobs.data(), sizeof(LossJob<T>) * n, cudaMemcpyHostToDevice, st),
-                "upload loss table")))
-    return s;
+  if ((s = upload(d_jobs, jobs.data(), sizeof(LossJob<T>) * n, "upload loss table", st))) return s;
   {
     LaunchScope _ls(*this, "loss_partial", st);
     constexpr int kMost = 65535;  // pairs of a launch (the grid's y extent)

@@ -216,9 +216,7 @@ sv_status Ctx::t1_forward(const sv_pair* pairs, int n, const int16_t* const* coa
     job(11, {{10, 16}, {4, 16}, {5, 8}, {11, 8}}, 2, 1, T(12));  // D <- D_2 & EN_1 & EN_1_R & D_2_R
     job(12, {{12, 16}, {0, 1}, {2, 32}, {3, 32}}, 1, 0, Y[i]);   // Y <- D & X_0 & FE_1 & FE_2
   }
-  if ((s = cuda(cudaMemcpyAsync(t1_tab.p, host.data(), host.size(), cudaMemcpyHostToDevice, st),
-                "upload Table I tables")))
-    return s;
+  if ((s = upload(t1_tab.p, host.data(), host.size(), "upload Table I tables", st))) return s;
   const T1PairIO* d_io = (const T1PairIO*)t1_tab.p;
   const F32Job* d_jobs = (const F32Job*)((unsigned char*)t1_tab.p + io_bytes);
   const float* W = (const float*)w32.p;

@@ -17,10 +17,12 @@
 namespace {
 struct Launch { std::string name; dim3 grid; };
 struct Copy { const void* src; size_t bytes; std::string content; };
+struct Owned { void* p; cudaHostFn_t destroy; };
 std::map<const void*, std::string> kernels;
 std::map<char*, size_t> blocks;  // live device allocations
 std::vector<Launch> launches;
 std::vector<Copy> copies;
+std::vector<Owned> owned;  // what the captured graph keeps
 size_t used = 0, peak = 0, limit = (size_t)256 << 30;
 long long fail_in = 0, launch_fail_in = 0;  // the fail_in-th allocation (launch) from now fails
 bool capturing = false;
@@ -54,6 +56,13 @@ int host_stale_copies() {
   return n;
 }
 int host_copies() { return (int)copies.size(); }
+// Ends the captured graph's life; returns how many objects it kept.
+int host_drop_graph() {
+  for (auto& o : owned) o.destroy(o.p);
+  const int n = (int)owned.size();
+  owned.clear();
+  return n;
+}
 }
 
 // Freed host memory is overwritten, so that a copy recorded from it shows.
@@ -190,6 +199,19 @@ cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus* s) {
   *s = capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
   return cudaSuccess;
 }
+cudaError_t cudaStreamGetCaptureInfo(cudaStream_t, cudaStreamCaptureStatus* s, unsigned long long*, cudaGraph_t* g,
+                                     const cudaGraphNode_t**, const cudaGraphEdgeData**, size_t*) {
+  *s = capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
+  if (g) *g = nullptr;
+  return cudaSuccess;
+}
+cudaError_t cudaUserObjectCreate(cudaUserObject_t* o, void* p, cudaHostFn_t destroy, unsigned, unsigned) {
+  owned.push_back({p, destroy});
+  *o = nullptr;
+  return cudaSuccess;
+}
+cudaError_t cudaGraphRetainUserObject(cudaGraph_t, cudaUserObject_t, unsigned, unsigned) { return cudaSuccess; }
+cudaError_t cudaUserObjectRelease(cudaUserObject_t, unsigned) { return cudaSuccess; }
 cudaError_t cudaStreamBeginCapture(cudaStream_t, cudaStreamCaptureMode) { return cudaSuccess; }
 cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t* g) { *g = nullptr; return cudaSuccess; }
 cudaError_t cudaGraphInstantiate(cudaGraphExec_t* e, cudaGraph_t, unsigned long long) { *e = nullptr; return cudaSuccess; }

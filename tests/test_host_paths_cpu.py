@@ -152,3 +152,29 @@ def test_more_pairs_than_a_grid_is_deep(host, form, n):
             assert not convert or sum(convert) == 4 * n  # e3, d1, d2, d3
     finally:
         h.close()
+
+
+@pytest.mark.parametrize("form", ["fp32", "bf16", "table1"])
+def test_captured_tables_outlive_their_call(host, form):
+    """Copies recorded in a caller's stream capture read, at replay, what they read at capture; the
+    memory is the graph's."""
+    t1 = form == "table1"
+    h = hostlib.Host(host, form if t1 else synth.NET_SMALL, "fp32" if t1 else form, [(64, 48), (40, 36)])
+    calls = ([h.refine] if form != "bf16" else []) + [h.train] + ([] if t1 else [h.loss, h.backward])
+    try:
+        for call in calls:
+            assert call() == binding.SV_OK, h.error()
+        host.host_clear()
+        host.host_capture(1)
+        for call in calls:
+            assert call() == binding.SV_OK, h.error()
+        host.host_capture(0)
+        assert host.host_copies() >= len(calls)
+        assert host.host_stale_copies() == 0
+        assert host.host_drop_graph() == host.host_copies()
+        for call in calls:  # nothing is kept for a call that is not captured
+            assert call() == binding.SV_OK, h.error()
+        assert host.host_drop_graph() == 0
+    finally:
+        host.host_capture(0)
+        h.close()

@@ -39,6 +39,7 @@
 #include <type_traits>
 #include <cudaTypedefs.h>
 
+#include "strip_plan.h"
 #include "sv_ctx.cuh"
 
 namespace sv {
@@ -1737,50 +1738,6 @@ sv_status Ctx::pack_fp8_weights(cudaStream_t st) {
     if ((s = cuda(cudaGetLastError(), "FP8 unfolded weights"))) return s;
   }
   return SV_OK;
-}
-
-// Strip height of a launch: `lanes` CTAs take the strips in turn, a CTA's time is its strips' rows plus
-// `extra` rows' worth per strip (halo, ring restart), and the launch lasts as long as its busiest CTA.
-// Every column of Hu rows is cut into equal strips, so candidates differ in how many rounds of
-// strips there are and how much of the last round idles.  Four strips per CTA of whatever height, the last
-// one of a column short, left 25-40 % of a launch in its tail (64 pairs of 1242 x 375: enc2 188 us against 137 at
-// 32 rows, dec1 489 against 305 at 4).
-struct StripCols { int Hu; long long cols; };
-static int pick_strip_rows(const std::vector<StripCols>& groups, int lanes, double extra) {
-  int maxHu = 1;
-  for (auto& g : groups) maxHu = std::max(maxHu, g.Hu);
-  int best = maxHu;
-  double best_cost = 1e300;
-  for (int hs = std::min(2, maxHu); hs <= maxHu; hs += hs < 64 ? 1 : hs / 8) {
-    long long strips = 0;
-    int tall = 1;
-    for (auto& g : groups) {
-      const int m = (g.Hu + hs - 1) / hs;
-      strips += m * g.cols;
-      tall = std::max(tall, (g.Hu + m - 1) / m);
-    }
-    const double cost = (double)((strips + lanes - 1) / lanes) * (tall + extra);
-    if (cost < best_cost - 1e-9) {
-      best_cost = cost;
-      best = hs;
-    }
-  }
-  return best;
-}
-static void add_cols(std::vector<StripCols>& groups, int Hu, long long cols) {
-  if (!groups.empty() && groups.back().Hu == Hu)
-    groups.back().cols += cols;
-  else
-    groups.push_back({Hu, cols});
-}
-// The strips of one column: equal heights, or (fixed) hs rows and a shorter last one.
-template <typename F>
-static void cut_column(int Hu, int hs, bool fixed, F&& f) {
-  const int m = (Hu + hs - 1) / hs;
-  for (int t = 0; t < m; ++t) {
-    const int i0 = fixed ? t * hs : (int)((long long)Hu * t / m), i1 = fixed ? std::min(Hu, i0 + hs) : (int)((long long)Hu * (t + 1) / m);
-    f(i0, i1 - i0);
-  }
 }
 
 // Host side of one tensor-core refinement call: activation workspaces (allocated here),

@@ -400,8 +400,9 @@ SV_API sv_status sv_set_option(sv_ctx* ctx, const char* key, long long value);
 
 /* Test hook: copies activation `which` (0 e1, 1 e2, 2 e3, 3 z, 4 d1, 5 d2, 6 d3; NHWC
  * BF16) of pair `pair` of the last SV_BF16 refinement call into host memory `dst`
- * (`bytes` must equal the activation's size).  Synchronous.  d3 is SV_ERR_STATE after a
- * call that fused the final conv (option "fused_final"). */
+ * (`bytes` must equal the activation's size).  Synchronous.  d3 of a call that fused the
+ * final conv (option "fused_final") is SV_ERR_STATE where every output width is even; with
+ * an odd one among them it is computed from d2 by the separate kernel. */
 SV_API sv_status sv_debug_activation(sv_ctx* ctx, int which, int pair, void* dst, size_t bytes);
 
 /* sv_coarse_match without any device allocation, and without a context.

@@ -1865,6 +1865,7 @@ sv_status Ctx::tc_prepare(const sv_pair* pairs, const int16_t* const* coarse, in
   };
   tc_off = off;
   tc_len = lens;
+  tc_pairs.assign(pairs, pairs + n);
   r.host.clear();
   auto put = [&](const void* src, size_t bytes) {
     size_t o = (r.host.size() + 127) / 128 * 128;  // the structs holding tensor maps are 128-byte aligned
@@ -2002,14 +2003,15 @@ sv_status Ctx::tc_prepare(const sv_pair* pairs, const int16_t* const* coarse, in
 }
 
 // Kernel launches of a prepared call; `tables` holds r.host on the device.  Only kernel
-// launches: safe inside a stream capture.
-sv_status Ctx::tc_launch(const TcRun& r, const unsigned char* tables, cudaStream_t st, const TcTrainLatent* tl) {
+// launches: safe inside a stream capture.  dec3_only: the last decoder layer alone, on the d2 that is there.
+sv_status Ctx::tc_launch(const TcRun& r, const unsigned char* tables, cudaStream_t st, const TcTrainLatent* tl,
+                         bool dec3_only) {
   using tc::LayerPair;
   using tc::Strip;
   sv_status s;
   const float* W = (const float*)w32.p;
   const EdgePair* d_edges = (const EdgePair*)(tables + r.edge_ofs);
-  {
+  if (!dec3_only) {
     LaunchScope ls(*this, "edge_enc1", st);
     if ((s = cuda(launch_edge_enc1(d_edges, r.n, r.maxW1, r.maxH1, W + net.w_off(L_ENC1), W + net.b_off(L_ENC1),
                                    net.enc[0], (int*)err_flag.p, spin_limit, enc1_tensor != 0, st),
@@ -2017,7 +2019,7 @@ sv_status Ctx::tc_launch(const TcRun& r, const unsigned char* tables, cudaStream
       return s;
   }
   const bool f8 = cfg.precision == SV_FP8;
-  if (f8 && !enc1_on_tc()) {  // (the tensor-core enc1 writes the codes itself)
+  if (f8 && !enc1_on_tc() && !dec3_only) {  // (the tensor-core enc1 writes the codes itself)
     LaunchScope ls(*this, "e1_to_e4m3", st);
     if ((s = cuda(launch_bf16_to_e4m3((const __nv_bfloat16*)tc_act[0].p, (uint8_t*)tc_act[7].p, r.e1_count, st),
                   "e1 to E4M3")))
@@ -2026,6 +2028,7 @@ sv_status Ctx::tc_launch(const TcRun& r, const unsigned char* tables, cudaStream
   static const char* names[6] = {"tc_enc2", "tc_enc3", "tc_latent", "tc_dec1", "tc_dec2", "tc_dec3"};
   for (size_t li = 0; li < r.plans.size(); ++li) {
     const TcLayerPlan& pl = r.plans[li];
+    if (dec3_only && pl.layer != L_DEC3) continue;
     tc::Params prm{};
     prm.lp = (const LayerPair*)(tables + r.tabs[li].lp_ofs);
     prm.strips = (const Strip*)(tables + r.tabs[li].strip_ofs);
@@ -2106,6 +2109,7 @@ sv_status Ctx::tc_launch(const TcRun& r, const unsigned char* tables, cudaStream
       if (s) return s;
     }
   }
+  if (dec3_only) return SV_OK;
   last_fused = r.fused;
   if (r.fused) return SV_OK;  // the final conv ran inside the fused decoder kernel
   {
@@ -2116,6 +2120,27 @@ sv_status Ctx::tc_launch(const TcRun& r, const unsigned char* tables, cudaStream
       return s;
   }
   return SV_OK;
+}
+
+// d3 of the last call, which the fused tail left on chip: the separate last decoder layer on the call's d2.
+sv_status Ctx::tc_make_d3() {
+  const std::vector<sv_pair> pairs = tc_pairs;
+  const int n = (int)pairs.size(), option = fused_final;
+  std::vector<float*> none(n, nullptr);
+  TcRun r;
+  fused_final = 0;
+  sv_status s = tc_prepare(pairs.data(), nullptr, n, none.data(), r);
+  fused_final = option;
+  if (s) return s;
+  DevBuf tables;
+  s = cuda(tables.ensure(r.host.size()), "alloc tables");
+  if (!s) s = cuda(cudaDeviceSynchronize(), "last call");
+  if (!s) s = cuda(cudaMemcpy(tables.p, r.host.data(), r.host.size(), cudaMemcpyHostToDevice), "upload tables");
+  if (!s) s = tc_launch(r, (const unsigned char*)tables.p, nullptr, nullptr, true);
+  if (!s) s = cuda(cudaStreamSynchronize(nullptr), "last decoder layer");
+  tables.release();
+  if (!s) last_fused = false;  // d3 is there now
+  return s;
 }
 
 sv_status Ctx::refine_tc(const sv_pair* pairs, const int16_t* const* coarse, int n, float* const* out,

@@ -728,9 +728,16 @@ sv_status sv_debug_activation(sv_ctx* ctx, int which, int pair, void* dst, size_
   const int buf = f8 && which == 0 ? 7 : which;
   if (bytes != c->tc_len[pair][which] * es)
     return c->fail(SV_ERR_INVALID_ARG, "activation has %zu bytes", c->tc_len[pair][which] * es);
-  if (which == 6 && c->last_fused)
-    return c->fail(SV_ERR_STATE, "d3 stayed on chip (fused final conv); set option fused_final 0 to keep it");
   DeviceGuard g(c->device);
+  if (which == 6 && c->last_fused) {
+    // A call with an odd output width kept its d3 before it ran fused: it is made from the call's d2.
+    bool odd = false;
+    for (const sv_pair& p : c->tc_pairs) odd = odd || p.width % 2 != 0;
+    if (!odd)
+      return c->fail(SV_ERR_STATE, "d3 stayed on chip (fused final conv); set option fused_final 0 to keep it");
+    const sv_status s = c->tc_make_d3();
+    if (s) return s;
+  }
   return c->cuda(cudaMemcpy(dst, (const unsigned char*)c->tc_act[buf].p + c->tc_off[pair][which] * es, bytes,
                             cudaMemcpyDeviceToHost), "copy activation");
 }

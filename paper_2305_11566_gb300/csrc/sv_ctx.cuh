@@ -74,6 +74,7 @@ struct GraphEntry {
   std::vector<uint64_t> key;
   std::vector<uint64_t> pkey;  // the call signature that led to it (before any preparation)
   std::vector<std::array<size_t, 7>> off, len;  // per-pair activation offsets of the call
+  std::vector<sv_pair> pairs;                   // its pairs (sizes)
   bool fused = false;
   cudaGraphExec_t exec = nullptr;
   void* tables = nullptr;  // device copy of the step's tables (owned)
@@ -166,6 +167,7 @@ struct Ctx {
   long long graph_clock = 0;
   std::vector<std::array<size_t, 7>> tc_off;   // per pair offsets of the last tensor-core call
   std::vector<std::array<size_t, 7>> tc_len;
+  std::vector<sv_pair> tc_pairs;               // its pairs; only their sizes are used after the call
   DevBuf err_flag;                      // device int: first failure code of a kernel
 
   // launch accounting and optional per-kernel event timing
@@ -238,7 +240,9 @@ struct Ctx {
   sv_status refine_tc(const sv_pair* pairs, const int16_t* const* coarse, int n, float* const* out, cudaStream_t st);
   sv_status tc_prepare(const sv_pair* pairs, const int16_t* const* coarse, int n, float* const* out, TcRun& r,
                        const float* const* coarse_f = nullptr);
-  sv_status tc_launch(const TcRun& r, const unsigned char* tables, cudaStream_t st, const TcTrainLatent* tl = nullptr);
+  sv_status tc_launch(const TcRun& r, const unsigned char* tables, cudaStream_t st, const TcTrainLatent* tl = nullptr,
+                      bool dec3_only = false);
+  sv_status tc_make_d3();
   sv_status train_forward_bf16(const sv_pair* pairs, const void* const* coarse, const void* const* eps, int n,
                                void* const* Y, void* const* mu, void* const* lv, cudaStream_t st);
   void coarse_prepare(const sv_pair* pairs, int n, int16_t* const* disp, float* const* best, float* const* second,

@@ -70,6 +70,7 @@ sv_status Ctx::pipeline_graph(const sv_pair* pairs, int n, float* const* out, cu
     g.last_use = ++graph_clock;
     tc_off = g.off;
     tc_len = g.len;
+    tc_pairs = g.pairs;
     last_fused = g.fused;
     sv_status s = cuda(cudaGraphLaunch(g.exec, st), "graph launch");
     if (s) return s;
@@ -116,6 +117,7 @@ sv_status Ctx::pipeline_graph(const sv_pair* pairs, int n, float* const* out, cu
     if (g.key != key) continue;
     g.last_use = graph_clock;
     g.pkey = pkey;
+    last_fused = g.fused;
     if ((s = cuda(cudaGraphLaunch(g.exec, st), "graph launch"))) return s;
     launches += g.kernels;
     if (prof_on)
@@ -137,6 +139,7 @@ sv_status Ctx::pipeline_graph(const sv_pair* pairs, int n, float* const* out, cu
   g.pkey = pkey;
   g.off = tc_off;
   g.len = tc_len;
+  g.pairs = tc_pairs;
   g.fused = r.fused;
   g.last_use = graph_clock;
   const size_t zp_bytes = sizeof(ZPair) * z.pairs.size(), zj_bytes = sizeof(ZJob) * z.jobs.size();

@@ -27,7 +27,7 @@ namespace sv {
 namespace {
 
 constexpr int kThreads = 128;
-constexpr int PX = 8;  // positions per thread, along x
+constexpr int PX = 8;  // positions per thread, along x (FK_DUP2 launches that leave SMs idle take 4)
 
 typedef unsigned long long u64;
 
@@ -77,10 +77,10 @@ constexpr int kind_cic(int kind) { return kind == FK_P1 ? 16 : kind == FK_S1_5 |
 
 constexpr int imax(int a, int b) { return a > b ? a : b; }
 
-template <int KIND, int CG_, int CIC_>
+template <int KIND, int CG_, int CIC_, int PX_ = 8>
 struct Geo {
   using K = Kind<KIND>;
-  static constexpr int CG = CG_, CIC = CIC_, BN = 8 * CG, S = K::S;
+  static constexpr int CG = CG_, CIC = CIC_, BN = 8 * CG, S = K::S, PX = PX_;
   static constexpr int TW = CG >= 4 ? 16 : 32, GX = TW / PX, TH = kThreads / CG / GX;
   static constexpr int PR = (TH - 1) * S + K::TY, PC = (TW - 1) * S + K::TX;
   static constexpr int NV = ((PX - 1) * S + K::TX + 3) / 4;  // float4 loads of a thread's row segment
@@ -97,9 +97,9 @@ struct Geo {
 // FK_S2: the patch's even and odd columns are staged apart (a tap's stride-2 reads of 8 positions
 // are then consecutive), in one buffer: the 8 channels of a step and their weights take 38 KB, and
 // four blocks share an SM.
-template <int CG_, int CIC_>
-struct Geo<FK_S2, CG_, CIC_> {
-  static constexpr int CG = CG_, CIC = CIC_, BN = 8 * CG, S = 2;
+template <int CG_, int CIC_, int PX_>
+struct Geo<FK_S2, CG_, CIC_, PX_> {
+  static constexpr int CG = CG_, CIC = CIC_, BN = 8 * CG, S = 2, PX = PX_;
   static constexpr int TW = CG >= 4 ? 16 : 32, GX = TW / PX, TH = kThreads / CG / GX;
   static constexpr int PR = 2 * TH + 1, PC = 2 * TW + 1;
   // row: odd columns 2x - 1 (TW + 1 of them, to a multiple of 4, + 4 read past the last), then even
@@ -111,9 +111,9 @@ struct Geo<FK_S2, CG_, CIC_> {
 };
 
 // FK_DUP2: columns 2x - 1 .. 2x + 2 of the upsampled grid, split by parity, in one buffer.
-template <int CG_, int CIC_>
-struct Geo<FK_DUP2, CG_, CIC_> {
-  static constexpr int CG = CG_, CIC = CIC_, BN = 8 * CG, S = 2;
+template <int CG_, int CIC_, int PX_>
+struct Geo<FK_DUP2, CG_, CIC_, PX_> {
+  static constexpr int CG = CG_, CIC = CIC_, BN = 8 * CG, S = 2, PX = PX_;
   static constexpr int TW = CG >= 4 ? 16 : 32, GX = TW / PX, TH = kThreads / CG / GX;
   static constexpr int PR = 2 * TH + 2, PC = 2 * TW + 2;
   static constexpr int EVEN = TW + 4, PITCH = 2 * EVEN;
@@ -125,9 +125,9 @@ struct Geo<FK_DUP2, CG_, CIC_> {
 
 // FK_UP2X: the patch holds the input pixels under the tile, (TH / 2 + 2) x (TW / 2 + 2); column 0 sits
 // at offset 3, so that a thread's four input pixels are one aligned vector.
-template <int CG_, int CIC_>
-struct Geo<FK_UP2X, CG_, CIC_> {
-  static constexpr int CG = CG_, CIC = CIC_, BN = 8 * CG, S = 1;
+template <int CG_, int CIC_, int PX_>
+struct Geo<FK_UP2X, CG_, CIC_, PX_> {
+  static constexpr int CG = CG_, CIC = CIC_, BN = 8 * CG, S = 1, PX = PX_;
   static constexpr int TW = CG >= 4 ? 16 : 32, GX = TW / PX, TH = kThreads / CG / GX;
   static constexpr int PR = TH / 2 + 2, PC = TW / 2 + 2, PITCH = TW / 2 + 8;
   static constexpr int PLANE = (PR * PITCH + 31 - 4) / 32 * 32 + 4;
@@ -183,11 +183,11 @@ __device__ __forceinline__ void load_row(const float* p, float* a) {
 
 // acc[p][..] += a[p S + c] * w: weights of one tap and channel, 4 + 4 outputs of this thread.
 template <class G, int OFS>
-__device__ __forceinline__ void tap(u64 (&acc)[PX][4], const float* a, const float* w) {
+__device__ __forceinline__ void tap(u64 (&acc)[G::PX][4], const float* a, const float* w) {
   const ulonglong2 w0 = *reinterpret_cast<const ulonglong2*>(w);
   const ulonglong2 w1 = *reinterpret_cast<const ulonglong2*>(w + G::BN / 2);
 #pragma unroll
-  for (int p = 0; p < PX; ++p) {
+  for (int p = 0; p < G::PX; ++p) {
     const u64 v = dup2(a[p * G::S + OFS]);
     fma2(acc[p][0], v, w0.x);
     fma2(acc[p][1], v, w0.y);
@@ -197,11 +197,11 @@ __device__ __forceinline__ void tap(u64 (&acc)[PX][4], const float* a, const flo
 }
 // The same with position `drop` left out (-1: none).
 template <class G, int OFS>
-__device__ __forceinline__ void tap_but(u64 (&acc)[PX][4], const float* a, const float* w, int drop) {
+__device__ __forceinline__ void tap_but(u64 (&acc)[G::PX][4], const float* a, const float* w, int drop) {
   const ulonglong2 w0 = *reinterpret_cast<const ulonglong2*>(w);
   const ulonglong2 w1 = *reinterpret_cast<const ulonglong2*>(w + G::BN / 2);
 #pragma unroll
-  for (int p = 0; p < PX; ++p) {
+  for (int p = 0; p < G::PX; ++p) {
     const u64 v = dup2(p == drop ? 0.f : a[p * G::S + OFS]);
     fma2(acc[p][0], v, w0.x);
     fma2(acc[p][1], v, w0.y);
@@ -211,7 +211,7 @@ __device__ __forceinline__ void tap_but(u64 (&acc)[PX][4], const float* a, const
 }
 
 template <class G, int TY, int TX, int C = 0>
-__device__ __forceinline__ void taps_of_row(u64 (&acc)[PX][4], const float* a, const float* w) {
+__device__ __forceinline__ void taps_of_row(u64 (&acc)[G::PX][4], const float* a, const float* w) {
   if constexpr (C < TX) {
     tap<G, C>(acc, a, w + C * G::CIC * G::BN);
     taps_of_row<G, TY, TX, C + 1>(acc, a, w);
@@ -222,8 +222,8 @@ __device__ __forceinline__ void taps_of_row(u64 (&acc)[PX][4], const float* a, c
 template <class G, int TY, int TX>
 struct Window {
   static constexpr int PR = (G::TH - 1) * G::S + TY, PC = (G::TW - 1) * G::S + TX, TAPS = TY * TX;
-  __device__ __forceinline__ void operator()(u64 (&acc)[PX][4], const float* pa, const float* pw) const {
-    constexpr int NV = ((PX - 1) * G::S + TX + 3) / 4;
+  __device__ __forceinline__ void operator()(u64 (&acc)[G::PX][4], const float* pa, const float* pw) const {
+    constexpr int NV = ((G::PX - 1) * G::S + TX + 3) / 4;
 #pragma unroll 1
     for (int ci = 0; ci < G::CIC; ++ci, pa += G::PLANE, pw += G::BN)
 #pragma unroll
@@ -242,8 +242,8 @@ struct UpEdge {
   static constexpr int PR = G::PR, PC = G::PC, TAPS = 9;
   int py, px, drop;
   bool last_row;
-  __device__ __forceinline__ void operator()(u64 (&acc)[PX][4], const float* pa, const float* pw) const {
-    constexpr int NV = (PX + 1 + 3) / 4, WS = G::CIC * G::BN;
+  __device__ __forceinline__ void operator()(u64 (&acc)[G::PX][4], const float* pa, const float* pw) const {
+    constexpr int NV = (G::PX + 1 + 3) / 4, WS = G::CIC * G::BN;
 #pragma unroll 1
     for (int ci = 0; ci < G::CIC; ++ci, pa += G::PLANE, pw += G::BN)
 #pragma unroll 1
@@ -270,11 +270,11 @@ struct UpEdge {
 // same bits as one thread per pixel does.  So these kinds run the unsummed nine taps (dec2 of 8 pairs of
 // 256 x 128: 229 us against 105 us for the summed 2x2 form, which inference uses).
 template <class G, int OFS>
-__device__ __forceinline__ void tap_unit(u64 (&acc)[PX][4], const float* a, const float* w) {
+__device__ __forceinline__ void tap_unit(u64 (&acc)[G::PX][4], const float* a, const float* w) {
   const ulonglong2 w0 = *reinterpret_cast<const ulonglong2*>(w);
   const ulonglong2 w1 = *reinterpret_cast<const ulonglong2*>(w + G::BN / 2);
 #pragma unroll
-  for (int p = 0; p < PX; ++p) {
+  for (int p = 0; p < G::PX; ++p) {
     const u64 v = dup2(a[p + OFS]);
     fma2(acc[p][0], v, w0.x);
     fma2(acc[p][1], v, w0.y);
@@ -283,15 +283,16 @@ __device__ __forceinline__ void tap_unit(u64 (&acc)[PX][4], const float* a, cons
   }
 }
 // All channels of a step for one tap; drop: position left out (EDGE tiles).
-template <class G, int OFS, int NV, bool EDGE = false>
-__device__ __forceinline__ void columns(u64 (&acc)[PX][4], const float* pa, const float* w, int drop = -1) {
+template <class G, int OFS, bool EDGE = false>
+__device__ __forceinline__ void columns(u64 (&acc)[G::PX][4], const float* pa, const float* w, int drop = -1) {
+  constexpr int NV = (G::PX + OFS + 3) / 4;
 #pragma unroll 2
   for (int ci = 0; ci < G::CIC; ++ci) {
     float a[4 * NV];
     load_row<G, NV>(pa + ci * G::PLANE, a);
     if constexpr (EDGE) {
 #pragma unroll
-      for (int p = 0; p < PX; ++p) a[p + OFS] = p == drop ? 0.f : a[p + OFS];
+      for (int p = 0; p < G::PX; ++p) a[p + OFS] = p == drop ? 0.f : a[p + OFS];
     }
     tap_unit<G, OFS>(acc, a, w + ci * G::BN);
   }
@@ -300,13 +301,13 @@ __device__ __forceinline__ void columns(u64 (&acc)[PX][4], const float* pa, cons
 template <class G>
 struct OrderedS2 {
   static constexpr int PR = G::PR, PC = G::PC, TAPS = 9;
-  __device__ __forceinline__ void operator()(u64 (&acc)[PX][4], const float* pa, const float* pw) const {
+  __device__ __forceinline__ void operator()(u64 (&acc)[G::PX][4], const float* pa, const float* pw) const {
     constexpr int WS = G::CIC * G::BN;
 #pragma unroll 1
     for (int ky = 0; ky < 3; ++ky, pa += G::PITCH, pw += 3 * WS) {
-      columns<G, 0, 2>(acc, pa, pw);
-      columns<G, 0, 2>(acc, pa + G::EVEN, pw + WS);
-      columns<G, 1, 3>(acc, pa, pw + 2 * WS);
+      columns<G, 0>(acc, pa, pw);
+      columns<G, 0>(acc, pa + G::EVEN, pw + WS);
+      columns<G, 1>(acc, pa, pw + 2 * WS);
     }
   }
 };
@@ -318,7 +319,7 @@ template <class G, bool EDGE>
 struct OrderedDup {
   static constexpr int PR = G::PR, PC = G::PC, TAPS = 9;
   int na, drop;  // na: 1 where a = 1 is cropped
-  __device__ __forceinline__ void operator()(u64 (&acc)[PX][4], const float* pa, const float* pw) const {
+  __device__ __forceinline__ void operator()(u64 (&acc)[G::PX][4], const float* pa, const float* pw) const {
     constexpr int WS = G::CIC * G::BN;
 #pragma unroll 1
     for (int a = 0; a < (EDGE ? na : 2); ++a) {
@@ -326,16 +327,16 @@ struct OrderedDup {
 #pragma unroll 1
       for (int ky = 0; ky < 3; ++ky) {
         const float *q = p - ky * G::PITCH, *w = pw + ky * 3 * WS;
-        columns<G, 1, 3>(acc, q, w);
-        columns<G, 0, 2>(acc, q + G::EVEN, w + WS);
-        columns<G, 0, 2>(acc, q, w + 2 * WS);
+        columns<G, 1>(acc, q, w);
+        columns<G, 0>(acc, q + G::EVEN, w + WS);
+        columns<G, 0>(acc, q, w + 2 * WS);
       }
 #pragma unroll 1
       for (int ky = 0; ky < 3; ++ky) {
         const float *q = p - ky * G::PITCH, *w = pw + ky * 3 * WS;
-        columns<G, 1, 3, EDGE>(acc, q + G::EVEN, w, drop);
-        columns<G, 1, 3, EDGE>(acc, q, w + WS, drop);
-        columns<G, 0, 2, EDGE>(acc, q + G::EVEN, w + 2 * WS, drop);
+        columns<G, 1, EDGE>(acc, q + G::EVEN, w, drop);
+        columns<G, 1, EDGE>(acc, q, w + WS, drop);
+        columns<G, 0, EDGE>(acc, q + G::EVEN, w + 2 * WS, drop);
       }
     }
   }
@@ -345,12 +346,12 @@ struct OrderedDup {
 template <class G, int TY, int TX>
 struct OrderedDs {
   static constexpr int PR = G::TH - 1 + TY, PC = G::TW - 1 + TX, TAPS = TY * TX;
-  __device__ __forceinline__ void operator()(u64 (&acc)[PX][4], const float* pa, const float* pw) const {
+  __device__ __forceinline__ void operator()(u64 (&acc)[G::PX][4], const float* pa, const float* pw) const {
     constexpr int WS = G::CIC * G::BN;
 #pragma unroll
     for (int r = TY - 1; r >= 0; --r) {
-      if (TX == 2) columns<G, 1, 3>(acc, pa + r * G::PITCH, pw + (r * TX + 1) * WS);
-      columns<G, 0, 2>(acc, pa + r * G::PITCH, pw + r * TX * WS);
+      if (TX == 2) columns<G, 1>(acc, pa + r * G::PITCH, pw + (r * TX + 1) * WS);
+      columns<G, 0>(acc, pa + r * G::PITCH, pw + r * TX * WS);
     }
   }
 };
@@ -362,7 +363,7 @@ template <class G>
 struct OrderedUp {
   static constexpr int PR = G::PR, PC = G::PC, TAPS = 9;
   int vy0, rows, drop;
-  __device__ __forceinline__ void operator()(u64 (&acc)[PX][4], const float* pa, const float* pw) const {
+  __device__ __forceinline__ void operator()(u64 (&acc)[G::PX][4], const float* pa, const float* pw) const {
     constexpr int WS = G::CIC * G::BN;
 #pragma unroll 1
     for (int ky = 0; ky < rows; ++ky) {
@@ -377,7 +378,7 @@ struct OrderedUp {
     }
   }
   template <int KX>
-  __device__ __forceinline__ void column(u64 (&acc)[PX][4], const float* p, const float* w) const {
+  __device__ __forceinline__ void column(u64 (&acc)[G::PX][4], const float* p, const float* w) const {
     const float4 f = *reinterpret_cast<const float4*>(p);
     const ulonglong2 w0 = *reinterpret_cast<const ulonglong2*>(w);
     const ulonglong2 w1 = *reinterpret_cast<const ulonglong2*>(w + G::BN / 2);
@@ -390,7 +391,7 @@ struct OrderedUp {
     v[o + 3] = dup2(f.w);
     if (KX == 2) v[4] = dup2(p[4]);
 #pragma unroll
-    for (int q = 0; q < PX; ++q) {
+    for (int q = 0; q < G::PX; ++q) {
       u64 x = v[KX == 1 ? q >> 1 : (q + 1) >> 1];
       if (KX == 2 && q == drop) x = 0ull;
       fma2(acc[q][0], x, w0.x);
@@ -403,7 +404,7 @@ struct OrderedUp {
 
 // Runs the channel chunks through the staging buffers; pa0: the thread's place in a patch.
 template <class G, class Form>
-__device__ __forceinline__ void contract(const Form& form, u64 (&acc)[PX][4], float* sm, const F32Job& J,
+__device__ __forceinline__ void contract(const Form& form, u64 (&acc)[G::PX][4], float* sm, const F32Job& J,
                                          const float* w, int K, int iy0, int ix0, int pa0, int cg) {
   const int nch = K / G::CIC;
   constexpr int WF = Form::TAPS * G::CIC * G::BN;
@@ -439,9 +440,9 @@ __device__ __forceinline__ float activate(float v, int act) {
   return v;
 }
 
-template <int KIND, int CG, int CIC>
+template <int KIND, int CG, int CIC, int PXV>
 __global__ void __launch_bounds__(kThreads, 4) f32_conv_kernel(const F32Job* __restrict__ jobs, const F32Args A) {
-  using G = Geo<KIND, CG, CIC>;
+  using G = Geo<KIND, CG, CIC, PXV>;
   extern __shared__ __align__(16) float f32_sm[];
   constexpr int PH = Kind<KIND>::PH, OS = PH == 4 ? 2 : 1;
   const F32Job& J = jobs[blockIdx.z];
@@ -452,21 +453,21 @@ __global__ void __launch_bounds__(kThreads, 4) f32_conv_kernel(const F32Job* __r
   const int Y0 = (blockIdx.x / A.tiles_x) * G::TH, X0 = (blockIdx.x % A.tiles_x) * G::TW;
   if (Y0 >= GH || X0 >= GW) return;
   const int cg = threadIdx.x % CG, pg = threadIdx.x / CG, gx = pg % G::GX, row = pg / G::GX;
-  const int y = Y0 + row, xb = X0 + gx * PX, n0 = nblk * G::BN + cg * 4;
-  u64 acc[PX][4];
+  const int y = Y0 + row, xb = X0 + gx * G::PX, n0 = nblk * G::BN + cg * 4;
+  u64 acc[G::PX][4];
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const u64 b = KIND == FK_P1 && A.bias_first
                       ? *reinterpret_cast<const u64*>(A.bias + n0 + (q >> 1) * (G::BN / 2) + 2 * (q & 1))
                       : 0ull;
 #pragma unroll
-    for (int p = 0; p < PX; ++p) acc[p][q] = b;
+    for (int p = 0; p < G::PX; ++p) acc[p][q] = b;
   }
   const float* wm = A.packed + A.w[phase];
   auto run = [&](auto form, const float* base, int dy, int dx) {
     using Form = decltype(form);
     contract<G>(form, acc, f32_sm, J, base + (size_t)nblk * Form::TAPS * A.K * G::BN, A.K, Y0 * G::S + dy,
-                X0 * G::S + dx, row * G::S * G::PITCH + gx * PX * (G::SPLIT ? 1 : G::S), cg);
+                X0 * G::S + dx, row * G::S * G::PITCH + gx * G::PX * (G::SPLIT ? 1 : G::S), cg);
   };
   if constexpr (KIND == FK_S2) {
     run(OrderedS2<G>{}, wm, -1, -1);
@@ -474,7 +475,7 @@ __global__ void __launch_bounds__(kThreads, 4) f32_conv_kernel(const F32Job* __r
     const int rows = min(3, Ho - (y - 1));
     const int drop = (Wo & 1) && X0 + G::TW >= GW ? GW - 1 - xb : -1;
     contract<G>(OrderedUp<G>{row + 1, rows, drop}, acc, f32_sm, J, wm + (size_t)nblk * 9 * A.K * G::BN, A.K, Y0 / 2 - 1,
-                X0 / 2 - 1, gx * (PX / 2) + 4, cg);
+                X0 / 2 - 1, gx * (G::PX / 2) + 4, cg);
   } else if constexpr (KIND == FK_P1) {
     run(Window<G, 1, 1>{}, wm, 0, 0);
   } else if constexpr (KIND == FK_S1_5 || KIND == FK_S2_5) {
@@ -508,7 +509,7 @@ __global__ void __launch_bounds__(kThreads, 4) f32_conv_kernel(const F32Job* __r
   for (int q = 0; q < 8; ++q)
     bs[q] = A.bias && !(KIND == FK_P1 && A.bias_first) ? A.bias[n0 + (q >> 2) * (G::BN / 2) + (q & 3)] : 0.f;
 #pragma unroll
-  for (int p = 0; p < PX; ++p) {
+  for (int p = 0; p < G::PX; ++p) {
     const int x = xb + p;
     if (x >= GW) break;
     const size_t o = ((size_t)(y * OS + py) * Wo + x * OS + px) * A.N + n0;
@@ -534,18 +535,27 @@ __global__ void __launch_bounds__(kThreads, 4) f32_conv_kernel(const F32Job* __r
   }
 }
 
-template <int KIND, int CG, int CIC>
+template <int KIND, int CG, int CIC, int PXV = PX>
 cudaError_t run_conv(const F32Layer& l, const F32Job* jobs, int n, int maxHo, int maxWo, const float* packed,
                      const float* bias, int act, cudaStream_t st) {
-  using G = Geo<KIND, CG, CIC>;
+  using G = Geo<KIND, CG, CIC, PXV>;
   constexpr int PH = Kind<KIND>::PH, OS = PH == 4 ? 2 : 1;
   F32Args a{packed, {l.w[0], l.w[1], l.w[2], l.w[3]}, l.wb, bias, l.K, l.N, l.N / G::BN, 0, act & 3, act & 8 ? 1 : 0, act & 4 ? 1 : 0};
   a.tiles_x = ((maxWo + OS - 1) / OS + G::TW - 1) / G::TW;
   const int tiles_y = ((maxHo + OS - 1) / OS + G::TH - 1) / G::TH;
-  auto kern = f32_conv_kernel<KIND, CG, CIC>;
+  const dim3 grid(a.tiles_x * tiles_y, PH * a.nb, n);
+  // FK_DUP2 launches of blocks for half the SMs at most: half the positions per thread.  A thread's chain
+  // (36 taps x K channels, one after the other) is then all the time there is, and half as long with half
+  // the independent sums; larger launches need the 8 positions' reuse of loads.  One pair: 36 x 36,
+  // 32/64/128 net, dec1 289 -> 207 us, dec2 141 -> 99; 256 x 128, 16/32/64 net, 138 -> 97 and 78 -> 55.
+  if constexpr (KIND == FK_DUP2 && PXV == PX) {
+    if (2LL * grid.x * grid.y * grid.z <= 152)
+      return run_conv<KIND, CG, CIC, 4>(l, jobs, n, maxHo, maxWo, packed, bias, act, st);
+  }
+  auto kern = f32_conv_kernel<KIND, CG, CIC, PXV>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM);
   if (e != cudaSuccess) return e;
-  kern<<<dim3(a.tiles_x * tiles_y, PH * a.nb, n), kThreads, G::SMEM, st>>>(jobs, a);
+  kern<<<grid, kThreads, G::SMEM, st>>>(jobs, a);
   return cudaGetLastError();
 }
 
@@ -599,7 +609,7 @@ __global__ void f32_pack_kernel(const F32PackDesc* __restrict__ descs, const flo
 
 template <int CG_>
 struct Enc1Geo {
-  static constexpr int CG = CG_, CIC = 2, BN = 8 * CG, S = 2;
+  static constexpr int CG = CG_, CIC = 2, BN = 8 * CG, S = 2, PX = 8;
   static constexpr int TW = CG >= 4 ? 16 : 32, GX = TW / PX, TH = kThreads / CG / GX;
   static constexpr int PR = 2 * TH + 1, PC = 2 * TW + 1, PITCH = (TW - PX) * 2 + 20, PLANE = PR * PITCH;
   static constexpr int BUF = 2 * PLANE + 18 * BN;

@@ -9,9 +9,11 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("form", ["fp32", "bf16"])
-def test_weight_gradients_over_slot_ranges(svlib, form):
-    """96 crops of 256 x 128, 32/64/128 net: 1.8 GB of slots for dec2, two ranges of at most 1 GiB."""
-    shape, n, W, H, D = synth.NET_WIDE, 96, 256, 128, 16
+@pytest.mark.parametrize("n,W,H", [(96, 256, 128), (60, 131, 77)], ids=["slots", "odd"])
+def test_gradients_of_many_pairs(svlib, form, n, W, H):
+    """96 crops of 256 x 128, 32/64/128 net: 1.8 GB of slots for dec2, two ranges of at most 1 GiB.  And odd
+    crops; a pair alone also takes the input gradients' form for launches that leave SMs idle."""
+    shape, D = synth.NET_WIDE, 16
     g = torch.Generator(device="cuda").manual_seed(3)
     ctx = binding.Context(shape, 7, form)
     try:
@@ -23,12 +25,13 @@ def test_weight_gradients_over_slot_ranges(svlib, form):
         gY = [torch.randn(H, W, device="cuda", generator=g) * 1e-4 for _ in range(n)]
         gl = [torch.randn(h3, w3, shape.latent, device="cuda", generator=g) * 1e-5 for _ in range(n)]
         ctx.refine_train([dp] * n, coarse, eps)
-        many, _ = ctx.refine_backward(gY, gl, gl, False, coarse)
+        many, many_c = ctx.refine_backward(gY, gl, gl, True, coarse)
         total = torch.zeros_like(many)
         for i in range(n):
             ctx.refine_train([dp], coarse[i:i + 1], eps[i:i + 1])
-            one, _ = ctx.refine_backward(gY[i:i + 1], gl[i:i + 1], gl[i:i + 1], False, coarse[i:i + 1])
+            one, one_c = ctx.refine_backward(gY[i:i + 1], gl[i:i + 1], gl[i:i + 1], True, coarse[i:i + 1])
             total += one
+            assert torch.equal(many_c[i], one_c[0])
         ctx.synchronize()
         assert many.abs().max() > 0 and torch.equal(many, total)
     finally:

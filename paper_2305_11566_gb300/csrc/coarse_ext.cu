@@ -9,8 +9,8 @@
 //              the box sums, clamped windows), census_cost (Hamming distance of the codes of
 //              (x, y) and (x - d, y); kc^2 - 1 where x - d < 0)
 //   aggregation A [h][w][D]
-//     SGM      sgm_axis: Eq. 4 along both directions of one axis per launch, 8 lanes per path
-//              line, each holding V consecutive disparities, so that the d - 1 and d + 1 terms are
+//     SGM      sgm_axis: Eq. 4 along both directions of one axis per launch, 8 or 16 lanes per
+//              path line, each holding V consecutive disparities, so that the d - 1 and d + 1 terms are
 //              registers but for one shuffle each way; the directions add into A in order
 //              (Eq. 5, deterministic); the last one also takes the winner-take-all of the sum
 //              (Eq. 6).  The pairs of a call go through cost and paths in parts of bounded
@@ -18,11 +18,9 @@
 //     DT       dt_weights (the edge weights of an iteration), dt_rows / dt_cols: the recursive
 //              domain-transform filter on every disparity slice, guided by the left box sums, one
 //              thread per (row, d) or (column, d)
-//   wta        Eq. 6 on a volume: 8 lanes per pixel, argmin over d, lowest d on ties
+//   wta        Eq. 6 on a volume: 8 or 16 lanes per pixel, argmin over d, lowest d on ties
 //   smp        single-matching-phase check (Eq. 7, read as uniqueness of the target column),
 //              one block per row; median3: 3 x 3 median filter, one thread per pixel
-#include <type_traits>
-
 #include "sv_ctx.cuh"
 
 namespace sv {
@@ -132,8 +130,8 @@ __device__ __forceinline__ void load_d(const float* p, int d0, int D, float (&v)
   }
 }
 
-// Lowest d among the smallest values over the 8 lanes of a group, in every lane.
-template <int V>
+// Lowest d among the smallest values over the LG lanes of a group, in every lane.
+template <int V, int LG>
 __device__ __forceinline__ int group_argmin(const float (&v)[V], int d0, int D) {
   int key = INT_MAX, bd = 0x7FFFFFFF;
 #pragma unroll
@@ -142,7 +140,7 @@ __device__ __forceinline__ int group_argmin(const float (&v)[V], int d0, int D) 
     if (kk < key) { key = kk; bd = d0 + k; }
   }
 #pragma unroll
-  for (int o = 1; o < 8; o <<= 1) {
+  for (int o = 1; o < LG; o <<= 1) {
     const int ok = __shfl_xor_sync(0xffffffffu, key, o), od = __shfl_xor_sync(0xffffffffu, bd, o);
     if (ok < key || (ok == key && od < bd)) { key = ok; bd = od; }
   }
@@ -151,10 +149,10 @@ __device__ __forceinline__ int group_argmin(const float (&v)[V], int d0, int D) 
 
 // One direction of Eq. 4 along a line of `len` pixels, `step` floats (and qstep pixels) apart, from pixel
 // q0 on.  FIRST: A = L, else A += L.  The costs and sums of the next PF pixels are loaded ahead.
-template <int V, bool VEC, bool FIRST>
+template <int V, int LG, bool VEC, bool FIRST>
 __device__ __forceinline__ void sgm_line(const XPair& p, int q0, int qstep, int len, int l, bool active, bool last,
                                          bool keep, float P1, float P2) {
-  constexpr int PF = V <= 8 ? 8 : 4;
+  constexpr int PF = 8;
   const unsigned FULL = 0xffffffffu;
   const float INF = __int_as_float(0x7f800000);
   const int D = p.D, d0 = l * V;
@@ -182,9 +180,9 @@ __device__ __forceinline__ void sgm_line(const XPair& p, int q0, int qstep, int 
 #pragma unroll
         for (int k = 0; k < V; ++k) cur[k] = c[j][k];
       } else {
-        float lo = __shfl_up_sync(FULL, prev[V - 1], 1, 8), hi = __shfl_down_sync(FULL, prev[0], 1, 8);
+        float lo = __shfl_up_sync(FULL, prev[V - 1], 1, LG), hi = __shfl_down_sync(FULL, prev[0], 1, LG);
         if (l == 0) lo = INF;
-        if (l == 7) hi = INF;
+        if (l == LG - 1) hi = INF;
         const float mp = m + P2;
 #pragma unroll
         for (int k = 0; k < V; ++k) {
@@ -197,7 +195,7 @@ __device__ __forceinline__ void sgm_line(const XPair& p, int q0, int qstep, int 
 #pragma unroll
       for (int k = 1; k < V; ++k) mn = fminf(mn, cur[k]);
 #pragma unroll
-      for (int x = 1; x < 8; x <<= 1) mn = fminf(mn, __shfl_xor_sync(FULL, mn, x));
+      for (int x = 1; x < LG; x <<= 1) mn = fminf(mn, __shfl_xor_sync(FULL, mn, x));
       m = mn;
       float tot[V];
 #pragma unroll
@@ -218,7 +216,7 @@ __device__ __forceinline__ void sgm_line(const XPair& p, int q0, int qstep, int 
         }
       }
       if (last) {
-        const int bd = group_argmin<V>(tot, d0, D);
+        const int bd = group_argmin<V, LG>(tot, d0, D);
         if (active && l == 0) p.wta[q0 + s * qstep] = (int16_t)bd;
       }
       // the slot's next pixel, PF ahead
@@ -232,30 +230,31 @@ __device__ __forceinline__ void sgm_line(const XPair& p, int q0, int qstep, int 
 }
 
 // Eq. 4 along rows (axis 0: left to right, then right to left) or columns (axis 1: top to bottom, then
-// bottom to top), 8 lanes per line and 4 lines per warp; ndir: 1 or both directions.  first: the
+// bottom to top), LG lanes per line and 32 / LG lines per warp; ndir: 1 or both directions.  first: the
 // axis's first direction writes A, every other adds; last: the axis's last direction also takes the
 // winner-take-all into wta; keep: it stores A too (else only the map).  A lane's values of the
 // second direction are the ones it stored in the first.  (One warp per line with the lanes over d
 // spent 10 shuffles on a line's minimum and used 48 of 64 lane slots at D = 48.)  Four paths of 64
 // pairs of 1242 x 375, D = 48: 1294 -> 577 us; reading and writing the volumes once per direction takes
 // 470 us at the measured 6.8 TB/s.
-template <int V, bool VEC>
+template <int V, int LG, bool VEC>
 __global__ void __launch_bounds__(128) sgm_axis_kernel(const XPair* __restrict__ P, int axis, int ndir, int first,
                                                        int last, int keep, float P1, float P2) {
   const XPair& p = P[blockIdx.y];
   const int w = p.w, h = p.h, nlines = axis == 0 ? h : w, len = axis == 0 ? w : h;
-  const int base = (blockIdx.x * 4 + (threadIdx.x >> 5)) * 4;
+  constexpr int NL = 32 / LG;
+  const int base = (blockIdx.x * 4 + (threadIdx.x >> 5)) * NL;
   if (base >= nlines) return;  // whole warp
-  const int l = threadIdx.x & 7, line0 = base + (threadIdx.x >> 3 & 3);
+  const int l = threadIdx.x % LG, line0 = base + threadIdx.x / LG % NL;
   const bool active = line0 < nlines;
   const int line = min(line0, nlines - 1);
   const int qstep = axis == 0 ? 1 : w, q0 = axis == 0 ? line * w : line;
   const bool one = ndir == 1;
   if (first)
-    sgm_line<V, VEC, true>(p, q0, qstep, len, l, active, last && one, keep, P1, P2);
+    sgm_line<V, LG, VEC, true>(p, q0, qstep, len, l, active, last && one, keep, P1, P2);
   else
-    sgm_line<V, VEC, false>(p, q0, qstep, len, l, active, last && one, keep, P1, P2);
-  if (!one) sgm_line<V, VEC, false>(p, q0 + (len - 1) * qstep, -qstep, len, l, active, last, keep, P1, P2);
+    sgm_line<V, LG, VEC, false>(p, q0, qstep, len, l, active, last && one, keep, P1, P2);
+  if (!one) sgm_line<V, LG, VEC, false>(p, q0 + (len - 1) * qstep, -qstep, len, l, active, last, keep, P1, P2);
 }
 
 // The weights of one DT iteration, once for all disparities: a^t between a pixel and its left / upper
@@ -338,18 +337,19 @@ __global__ void dt_cols_kernel(const XPair* __restrict__ P) {
   dt_line(end, end, -row, p.WY + x + (size_t)(h - 1) * w, -(ptrdiff_t)w, h, end[0]);
 }
 
-// Eq. 6 on a volume (vol_sel 0: C, 1: A): 8 lanes per pixel, lowest d among the minima.
-template <int V, bool VEC>
+// Eq. 6 on a volume (vol_sel 0: C, 1: A): LG lanes per pixel, lowest d among the minima.
+template <int V, int LG, bool VEC>
 __global__ void __launch_bounds__(256) vol_wta_kernel(const XPair* __restrict__ P, int vol_sel) {
   const XPair& p = P[blockIdx.y];
-  const int D = p.D, npix = p.w * p.h, l = threadIdx.x & 7;
+  constexpr int NP = 32 / LG;  // pixels of a warp
+  const int D = p.D, npix = p.w * p.h, l = threadIdx.x % LG;
   const float* A = vol_sel ? p.A : p.C;
-  const int stride = gridDim.x * 32;
-  for (int q0 = blockIdx.x * 32 + (threadIdx.x >> 5) * 4; q0 < npix; q0 += stride) {  // whole warps
-    const int q = q0 + (threadIdx.x >> 3 & 3);
+  const int stride = gridDim.x * 8 * NP;
+  for (int q0 = (blockIdx.x * 8 + (threadIdx.x >> 5)) * NP; q0 < npix; q0 += stride) {  // whole warps
+    const int q = q0 + threadIdx.x / LG % NP;
     float v[V];
     load_d<V, VEC, false>(A + (size_t)min(q, npix - 1) * D, l * V, D, v);
-    const int bd = group_argmin<V>(v, l * V, D);
+    const int bd = group_argmin<V, LG>(v, l * V, D);
     if (l == 0 && q < npix) p.wta[q] = (int16_t)bd;
   }
 }
@@ -444,36 +444,46 @@ cudaError_t launch_census_codes(const XPair* T, int kc, int maxw, int maxh, int 
   return cudaGetLastError();
 }
 
-// Disparities per lane for the largest range of the call; vec: every pair's volumes can be read in
-// pairs of floats.
+// Disparities per lane and lanes per line (or pixel) for the largest range of the call; vec: every pair's
+// volumes can be read in pairs of floats.  Ranges above 64 take 16 lanes: 12 or 16 disparities in one of 8
+// lanes hold so many registers that too few lines are in flight (four paths, D = 128: one 640 x 128 pair
+// 331 us with 8 lanes, 165 with 16; 16 census pairs of 1242 x 375 1038, 669).
+template <int V_, int LG_, bool VEC_>
+struct Range {
+  static constexpr int V = V_, LG = LG_;
+  static constexpr bool VEC = VEC_;
+};
 template <typename F>
 cudaError_t by_range(int maxD, bool vec, F&& f) {
-#define SV_RANGE(v)                                                                     \
-  if (maxD <= 8 * v) {                                                                  \
-    if (vec)                                                                            \
-      f(std::integral_constant<int, v>(), std::true_type());                            \
-    else                                                                                \
-      f(std::integral_constant<int, v>(), std::false_type());                           \
-    return cudaGetLastError();                                                          \
+#define SV_RANGE(v, lg)               \
+  if (maxD <= lg * v) {               \
+    if (vec)                          \
+      f(Range<v, lg, true>());        \
+    else                              \
+      f(Range<v, lg, false>());       \
+    return cudaGetLastError();        \
   }
-  SV_RANGE(2) SV_RANGE(4) SV_RANGE(6) SV_RANGE(8) SV_RANGE(12) SV_RANGE(16)
+  SV_RANGE(2, 8) SV_RANGE(4, 8) SV_RANGE(6, 8) SV_RANGE(8, 8) SV_RANGE(6, 16) SV_RANGE(8, 16)
 #undef SV_RANGE
   return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_sgm_axis(const XPair* T, int maxD, bool vec, int nlines, int n, int axis, int ndir, int first,
                             int last, int keep, float P1, float P2, cudaStream_t st) {
-  const dim3 g((nlines + 15) / 16, n);
-  return by_range(maxD, vec, [&](auto v, auto vc) {
-    sgm_axis_kernel<decltype(v)::value, decltype(vc)::value><<<g, 128, 0, st>>>(T, axis, ndir, first, last, keep, P1,
-                                                                                P2);
+  return by_range(maxD, vec, [&](auto r) {
+    using R = decltype(r);
+    constexpr int lines = 4 * 32 / R::LG;  // of a block
+    sgm_axis_kernel<R::V, R::LG, R::VEC><<<dim3((nlines + lines - 1) / lines, n), 128, 0, st>>>(
+        T, axis, ndir, first, last, keep, P1, P2);
   });
 }
 
 cudaError_t launch_vol_wta(const XPair* T, int maxD, bool vec, int n, int maxpix, int vol_sel, cudaStream_t st) {
-  const dim3 g(std::min(8 * 152, (maxpix + 31) / 32), n);
-  return by_range(maxD, vec, [&](auto v, auto vc) {
-    vol_wta_kernel<decltype(v)::value, decltype(vc)::value><<<g, 256, 0, st>>>(T, vol_sel);
+  return by_range(maxD, vec, [&](auto r) {
+    using R = decltype(r);
+    constexpr int pixels = 8 * 32 / R::LG;  // of a block
+    vol_wta_kernel<R::V, R::LG, R::VEC><<<dim3(std::min(8 * 152, (maxpix + pixels - 1) / pixels), n), 256, 0, st>>>(
+        T, vol_sel);
   });
 }
 

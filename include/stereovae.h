@@ -111,6 +111,8 @@ typedef struct {
   int enc_ch[3];  /* encoder widths, each a multiple of 16, <= 256 */
   int latent_ch;  /* latent (mean / logvar) width, multiple of 16, <= 256 */
   int dec_ch[3];  /* decoder widths, each a multiple of 16, <= 256 */
+  /* (SV_BF16 and SV_FP8: sv_create returns SV_ERR_UNSUPPORTED where a layer's rows do not fit in
+   * shared memory, e.g. a 144-channel stride-2 layer) */
   int precision;  /* sv_precision */
   int flags;      /* 0 or SV_NET_TABLE1 */
 } sv_config;

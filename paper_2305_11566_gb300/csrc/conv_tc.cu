@@ -1600,7 +1600,8 @@ __global__ void to_bf16_kernel(const float* __restrict__ a, __nv_bfloat16* __res
 
 // f8: the FP8 form, whose operands are E4M3 bytes: a layer of cin channels is planned as cin / 2
 // BF16-sized channels (the same bytes), N at most 128, bias and scale beside the weights.
-static void plan_layers(const NetDims& net, std::vector<TcLayerPlan>& plans, size_t& total, bool f8 = false) {
+// False: some layer is so wide that not even the rows of one tile fit in shared memory.
+static bool plan_layers(const NetDims& net, std::vector<TcLayerPlan>& plans, size_t& total, bool f8 = false) {
   plans.clear();
   total = 0;
   const int layers[6] = {L_ENC2, L_ENC3, L_MU, L_DEC1, L_DEC2, L_DEC3};
@@ -1620,6 +1621,7 @@ static void plan_layers(const NetDims& net, std::vector<TcLayerPlan>& plans, siz
       size_t sm = tc::smem_bytes(pl.mode, NT, pl.cin, ring, false, f8);
       if (sm <= kSmemLimit) break;
       if (ring > RA) { --ring; continue; }
+      if (NT == 0) return false;
       NT /= 2;
       ring = RA + STEP;
     }
@@ -1641,12 +1643,14 @@ static void plan_layers(const NetDims& net, std::vector<TcLayerPlan>& plans, siz
   unfolded_offsets(net, total, unf);
   for (auto& pl : plans)
     if (pl.mode == tc::TM_UP2) pl.fix_wofs = unf[pl.layer == L_DEC1 ? 0 : pl.layer == L_DEC2 ? 1 : 2];
+  return true;
 }
 
 sv_status Ctx::pack_bf16_weights(cudaStream_t st) {
   std::vector<TcLayerPlan> plans;
   size_t total;
-  plan_layers(net, plans, total);
+  if (!plan_layers(net, plans, total))
+    return fail(SV_ERR_UNSUPPORTED, "a layer is too wide for the tensor-core form's shared memory");
   size_t unf[3];
   const size_t all = unfolded_offsets(net, total, unf);
   sv_status s = cuda(wbf.ensure(all * sizeof(__nv_bfloat16)), "alloc packed weights");
@@ -1690,7 +1694,8 @@ sv_status Ctx::pack_bf16_weights(cudaStream_t st) {
 sv_status Ctx::pack_fp8_weights(cudaStream_t st) {
   std::vector<TcLayerPlan> plans;
   size_t total;
-  plan_layers(net, plans, total, true);
+  if (!plan_layers(net, plans, total, true))
+    return fail(SV_ERR_UNSUPPORTED, "a layer is too wide for the tensor-core form's shared memory");
   const int dl[3] = {L_DEC1, L_DEC2, L_DEC3};
   size_t unf_bytes = 0, nscale = 0;
   for (int k = 0; k < 3; ++k) {
@@ -1749,11 +1754,13 @@ sv_status Ctx::tc_prepare(const sv_pair* pairs, const int16_t* const* coarse, in
   using tc::Strip;
   size_t wtotal;
   const bool f8 = cfg.precision == SV_FP8;
-  plan_layers(net, r.plans, wtotal, f8);
+  if (!plan_layers(net, r.plans, wtotal, f8))
+    return fail(SV_ERR_UNSUPPORTED, "a layer is too wide for the tensor-core form's shared memory");
   if (f8) {  // the FP8 form's last decoder layer runs as in the BF16 form (BF16 pack, BF16 d2)
     std::vector<TcLayerPlan> bfp;
     size_t bft;
-    plan_layers(net, bfp, bft, false);
+    if (!plan_layers(net, bfp, bft, false))
+      return fail(SV_ERR_UNSUPPORTED, "a layer is too wide for the tensor-core form's shared memory");
     for (size_t li = 0; li < r.plans.size(); ++li)
       if (r.plans[li].layer == L_DEC3) r.plans[li] = bfp[li];
   }

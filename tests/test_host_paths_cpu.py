@@ -178,3 +178,19 @@ def test_captured_tables_outlive_their_call(host, form):
     finally:
         host.host_capture(0)
         h.close()
+
+
+@pytest.mark.parametrize("form", ["bf16", "fp8"])
+def test_networks_too_wide_for_the_tensor_core_form(host, form):
+    """Widths whose staged rows alone exceed shared memory are refused when the context is created (planning
+    them had no end); FP32 takes them."""
+    wide = synth.NetShape((256, 256, 256), 256, (256, 256, 256))
+    ctx = hostlib.ctypes.c_void_p()
+    cfg = binding.make_config(wide, 9, form)
+    assert host.sv_create(hostlib.ctypes.byref(cfg), 0, hostlib.ctypes.byref(ctx)) == binding.SV_ERR_UNSUPPORTED
+    assert not ctx.value
+    h = hostlib.Host(host, wide, "fp32", [(64, 48)])
+    try:
+        assert h.refine() == binding.SV_OK, h.error()
+    finally:
+        h.close()

@@ -14,21 +14,22 @@ def test_replay_equals_eager(svlib, form):
     t1 = form == "table1"
     shape = form if t1 else synth.NET_SMALL
     g = torch.Generator(device="cuda").manual_seed(1)
+    f32 = {"device": "cuda", "dtype": torch.float32}
     ctx = binding.Context(shape, 3, "fp32" if t1 else form)
     try:
-        ctx.set_weights(torch.randn(ctx.n_params, device="cuda", generator=g) * 0.05)
+        ctx.set_weights(torch.randn(ctx.n_params, **f32, generator=g) * 0.05)
         dps = [binding.to_device(synth.make_pair(W, H, 20.0, 3 + W), D) for W, H in sizes]
         maps = [torch.empty(H // 4, W // 4, device="cuda", dtype=torch.int16) for W, H in sizes]
-        coarse = [torch.empty(H // 4, W // 4, device="cuda") for W, H in sizes]
-        eps = [torch.empty(*binding.latent_hw(H, W), ctx.latent, device="cuda") for W, H in sizes]
-        gt = [torch.empty(H, W, device="cuda") for W, H in sizes]
+        coarse = [torch.empty(H // 4, W // 4, **f32) for W, H in sizes]
+        eps = [torch.empty(*binding.latent_hw(H, W), ctx.latent, **f32) for W, H in sizes]
+        gt = [torch.empty(H, W, **f32) for W, H in sizes]
 
         def fresh():
             for m, c, e, t in zip(maps, coarse, eps, gt):
                 m.copy_(torch.randint(0, D, m.shape, device="cuda", generator=g))
-                c.copy_(torch.rand(c.shape, device="cuda", generator=g) * (D - 1))
-                e.copy_(torch.randn(e.shape, device="cuda", generator=g))
-                t.copy_(torch.rand(t.shape, device="cuda", generator=g) * 20)
+                c.copy_(torch.rand(c.shape, **f32, generator=g) * (D - 1))
+                e.copy_(torch.randn(e.shape, **f32, generator=g))
+                t.copy_(torch.rand(t.shape, **f32, generator=g) * 20)
 
         def calls():
             out = list(ctx.refine(dps, maps)) if form != "bf16" else []

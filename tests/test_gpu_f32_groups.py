@@ -15,15 +15,16 @@ def test_gradients_of_many_pairs(svlib, form, n, W, H):
     crops; a pair alone also takes the input gradients' form for launches that leave SMs idle."""
     shape, D = synth.NET_WIDE, 16
     g = torch.Generator(device="cuda").manual_seed(3)
+    f32 = {"device": "cuda", "dtype": torch.float32, "generator": g}
     ctx = binding.Context(shape, 7, form)
     try:
         ctx.set_weights(synth.he_normal_weights(shape, 7))
         dp = binding.to_device(synth.make_pair(W, H, 40.0, 5), D)
         h3, w3 = binding.latent_hw(H, W)
-        coarse = [torch.rand(H // 4, W // 4, device="cuda", generator=g) * (D - 1) for _ in range(n)]
-        eps = [torch.randn(h3, w3, shape.latent, device="cuda", generator=g) for _ in range(n)]
-        gY = [torch.randn(H, W, device="cuda", generator=g) * 1e-4 for _ in range(n)]
-        gl = [torch.randn(h3, w3, shape.latent, device="cuda", generator=g) * 1e-5 for _ in range(n)]
+        coarse = [torch.rand(H // 4, W // 4, **f32) * (D - 1) for _ in range(n)]
+        eps = [torch.randn(h3, w3, shape.latent, **f32) for _ in range(n)]
+        gY = [torch.randn(H, W, **f32) * 1e-4 for _ in range(n)]
+        gl = [torch.randn(h3, w3, shape.latent, **f32) * 1e-5 for _ in range(n)]
         ctx.refine_train([dp] * n, coarse, eps)
         many, many_c = ctx.refine_backward(gY, gl, gl, True, coarse)
         total = torch.zeros_like(many)
@@ -34,5 +35,23 @@ def test_gradients_of_many_pairs(svlib, form, n, W, H):
             assert torch.equal(many_c[i], one_c[0])
         ctx.synchronize()
         assert many.abs().max() > 0 and torch.equal(many, total)
+    finally:
+        ctx.close()
+
+
+def test_refine_around_a_group_boundary(svlib):
+    """A 1242 x 375 pair of the 32/64/128 net has 134.4 MB of activations, so 2 GiB hold 15: pairs 14 and 15
+    of a call are the last of one group and the first of the next."""
+    shape, W, H, D, n = synth.NET_WIDE, 1242, 375, 48, 17
+    g = torch.Generator(device="cuda").manual_seed(4)
+    ctx = binding.Context(shape, 9, "fp32")
+    try:
+        ctx.set_weights(synth.he_normal_weights(shape, 7))
+        dp = binding.to_device(synth.make_pair(W, H, 190.0, 5), D)
+        maps = [torch.randint(0, D, (H // 4, W // 4), device="cuda", generator=g, dtype=torch.int16) for _ in range(n)]
+        many = ctx.refine([dp] * n, maps)
+        for i in (13, 14, 15, 16):
+            assert torch.equal(many[i], ctx.refine([dp], [maps[i]])[0])
+        ctx.synchronize()
     finally:
         ctx.close()

@@ -85,9 +85,10 @@ def peaks():
 # capture, per pair; valid only while the kernel's sources are unchanged since the capture
 # (checked by content hash), else the roofline reports traffic as null.
 MEASURED_TRAFFIC = {
-    "tc_dec3_final": {"bytes_per_pair": (240.199424e6 + 21.983744e6) / 16,
-                      "sources": {"paper_2305_11566_gb300/csrc/conv_tc.cu": "08bfb139ec14",
-                                  "paper_2305_11566_gb300/csrc/sv_ctx.cuh": "08fb6e322a2a",
+    "tc_dec3_final": {"bytes_per_pair": (240.308480e6 + 21.908480e6) / 16,
+                      "sources": {"paper_2305_11566_gb300/csrc/conv_tc.cu": "58e0d5487ba1",
+                                  "paper_2305_11566_gb300/csrc/strip_plan.h": "20ddee9ba96e",
+                                  "paper_2305_11566_gb300/csrc/sv_ctx.cuh": "0f2badce3fde",
                                   "paper_2305_11566_gb300/csrc/sv_internal.cuh": "6aea9b8c4f23"},
                       "capture": "profiles/dec3_final_fused_16x1242x375.md (16 pairs, scaled by pairs)"},
 }
@@ -179,7 +180,9 @@ def levels(h, w):
 
 
 def upfix_pixels(Ho, Wo):
-    """Border pixels of a cropped nearest-x2 + 3x3 layer recomputed by the border-fix kernel."""
+    """Border pixels of a cropped nearest-x2 + 3x3 layer recomputed by the border-fix kernel.  (Priced below
+    at the FP32 rate that the training form's kernel runs at; inference computes them on warp MMA, where a few
+    hundred pixels a pair are bound by latency.)"""
     return (Wo if Ho & 1 else 0) + ((Ho - (Ho & 1)) if Wo & 1 else 0)
 
 

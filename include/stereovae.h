@@ -65,7 +65,10 @@ typedef enum {
 /* Arithmetic of the refinement convolutions.
  * SV_FP32: FP32 convolutions on the CUDA cores (the plain method).
  * SV_BF16: implicit-GEMM convolutions on the tcgen05 tensor cores, BF16 operands,
- *          FP32 accumulation; the last conv and the residual stay FP32.
+ *          FP32 accumulation; the residual and the last conv's sums stay FP32.  Where the
+ *          last conv is fused into the last decoder layer (option "fused_final", even and
+ *          odd output widths), its FP32 weights are the sum of two BF16 parts (to about
+ *          2^-16 of each); else, and in training, they are FP32.
  * SV_FP64_CHECK: FP64 CUDA-core convolutions, for gradient checks on small crops.
  * SV_FP8: the quantised refinement the paper names as future work (Sec. V), inference
  *          only: the quantised layers enc2, enc3, latent, dec1 and dec2 take E4M3 operands
@@ -260,7 +263,7 @@ SV_API sv_status sv_pipeline(sv_ctx* ctx, const sv_pair* pairs, int n_pairs, flo
 /* Training forward of n_pairs pairs: z = mu + eps * exp(logvar / 2) (the
  * reparameterisation of Eq. 8 in its standard form).  Saves in the context what
  * sv_refine_backward needs (activations and the latent; SV_BF16 and SV_FP64_CHECK contexts
- * recompute the encoder there).  On SV_BF16 contexts the encoder and decoder convolutions run on
+ * recompute the encoder there, SV_FP32 contexts where its activations do not fit).  On SV_BF16 contexts the encoder and decoder convolutions run on
  * the tensor cores (BF16 operands, FP32 accumulation, FP32 master weights) and the
  * backward runs in FP32; SV_FP32 runs FP32 throughout, SV_FP64_CHECK FP64.  Element type of coarse, eps, disp_out, mu_out and logvar_out
  * is float for SV_FP32 / SV_BF16 contexts and double for SV_FP64_CHECK contexts.

@@ -3,8 +3,8 @@
 // every pair of a call.
 //
 //   cost volume C [h][w][D]
-//     ZNCC     1 - rho of Eq. 1-3, written by the coarse matcher itself (zncc_wta.cu, the
-//              cost-writing instance) while it computes its own winner-take-all;
+//     ZNCC     1 - rho of Eq. 1-3, written by the coarse matcher itself (zncc_wta.cu): the cost
+//              alone where an aggregation follows, beside its own winner-take-all where not;
 //     census   box4 (4 x 4 box sums of L and R), census_codes (kc x kc census bit strings of
 //              the box sums, clamped windows), census_cost (Hamming distance of the codes of
 //              (x, y) and (x - d, y); kc^2 - 1 where x - d < 0)

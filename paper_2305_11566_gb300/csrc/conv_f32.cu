@@ -148,14 +148,13 @@ struct F32Args {
 
 // The patch rows iy0 .. of one channel chunk, channel-planar; zero outside the input.
 template <class G, int PR, int PC>
-__device__ __forceinline__ void load_patch(float* dst, const float* src, int C, int iy0, int ix0, int Hi, int Wi,
-                                           int nc = G::CIC) {  // nc: channels that exist (the others are zero)
+__device__ __forceinline__ void load_patch(float* dst, const float* src, int C, int iy0, int ix0, int Hi, int Wi) {
   constexpr int SL = kThreads / G::CIC, CW = SL < 32 ? SL : 32, RG = SL / CW;
   const int t = threadIdx.x, ci = t % G::CIC, cc = (t / G::CIC) % CW, rg = t / (G::CIC * CW);
   const ptrdiff_t step = (ptrdiff_t)RG * Wi * C;
   for (int c = cc; c < PC; c += CW) {
     const int ix = ix0 + c;
-    const bool cok = (unsigned)ix < (unsigned)Wi && ci < nc;
+    const bool cok = (unsigned)ix < (unsigned)Wi;
     ptrdiff_t o = ((ptrdiff_t)(iy0 + rg) * Wi + ix) * C + ci;
     const int cd = G::SPLIT ? (c & 1 ? G::EVEN : 0) + (c >> 1) : c;  // (patch column 0 is odd)
     float* d = dst + ci * G::PLANE + rg * G::PITCH + cd;

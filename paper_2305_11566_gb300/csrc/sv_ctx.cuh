@@ -109,7 +109,7 @@ struct Ctx {
   DevBuf f32_act, f32_tab;       // FP32 form: activations of one group of pairs, job tables
   F32Layer f32_l[L_COUNT];       // forward layers
   F32Layer f32_t[L_COUNT];       // decoder layers of the training forward
-  F32Layer f32_g[L_COUNT];       // input gradients (L_MU: both latent heads)
+  F32Layer f32_g[L_COUNT];       // input gradients
   F32Layer t1_l[13];             // the Table I network's 5 x 5 layers
   int f32_n_descs = 0;
   size_t f32_max_count = 0;
@@ -155,7 +155,7 @@ struct Ctx {
   int split_rows = 1;                   // 1: layers without a spare staged row stage channel blocks
   int host_copy = 1;                    // sv_pipeline_host: 0 copy calls, 1 gather kernel in, 2 kernels both ways
   bool last_fused = false;              // the last tensor-core call did not materialise d3
-  int tc_ctas_per_sm = 0;               // 0: deepest row ring (one CTA per SM); k: ring sized for k
+  int tc_ctas_per_sm = 0;               // 0: chosen per layer by what fits; k: row ring sized for k CTAs per SM
   int tc_rows_override[6] = {0, 0, 0, 0, 0, 0};  // per tensor-core layer, set by the autotuner
   int tc_nt_override[6] = {0, 0, 0, 0, 0, 0};
   int tc_ctas_override[6] = {0, 0, 0, 0, 0, 0};  // CTAs per SM the ring is sized for (0: tc_ctas_per_sm)

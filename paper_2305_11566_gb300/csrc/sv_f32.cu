@@ -15,8 +15,8 @@ cudaError_t launch_up4_bwd(const T* gU, const T* gx0, int W, int H, int w, int h
 namespace {
 
 // Bytes of activations one group of pairs may hold: pairs beyond it run as further groups on
-// the same workspace.  Where an allocation of a group fails, smaller groups are tried, down to one pair.  A 1242 x 375 pair of the 32/64/128 net needs 134 MB; 2 GiB hold 16, more
-// than fill the GPU.
+// the same workspace.  Where an allocation of a group fails, smaller groups are tried, down to one pair.
+// A 1242 x 375 pair of the 32/64/128 net needs 134 MB; 2 GiB hold 15, more than fill the GPU.
 constexpr size_t kGroupBytes = size_t(2) << 30;
 
 // Pairs of a group: the largest z extent of a launch's grid.

@@ -1,5 +1,5 @@
-// sv_forms.cu -- inference entry points of the context: plain refinement (per-pair
-// launches on CUDA cores, FP32 or FP64), the tensor-core form, and the pipeline.
+// sv_forms.cu -- inference entry points of the context: which form refines (the Table I network,
+// the tensor-core forms or FP32, each batched over the pairs of a call), and the pipeline.
 #include <algorithm>
 #include <vector>
 

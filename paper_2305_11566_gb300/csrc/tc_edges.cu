@@ -9,9 +9,13 @@
 //                persistent grid whose blocks walk the (pair, tile) list.
 //   edge_final   last conv (3x3, C -> 1) + bias + U (residual), BF16 input, FP32 output;
 //                register-blocked packed-FP32 form for C = 16, 32, 64, 128.
-//   edge_up2fix  exact recomputation of the last row / column of an odd-sized (cropped)
+//   edge_up2fix_mma   exact recomputation of the last row / column of an odd-sized (cropped)
 //                nearest-x2 + 3x3 conv output, which the 4-phase tensor-core form folds
-//                wrongly: segments of 64 border pixels x 32 channels per block.
+//                wrongly: 16 border pixels x 32 channels per block on warp MMA, BF16 or E4M3.
+//   edge_up2fix  the same for the training forward, on CUDA-core FMA in one fixed order:
+//                segments of 64 border pixels x 32 channels per block.
+//   fused_edge_cols   the last two output columns of odd widths after the fused dec3 + final
+//                kernel of conv_tc.cu.
 #include <cuda_fp8.h>
 
 #include "sv_ctx.cuh"
